@@ -63,7 +63,7 @@ def parse_args():
     ap.add_argument("--bucket-slots", type=int, choices=[16, 32], default=0,
                     help="fix the bucket width instead of autotuning it (profiling runs)")
     ap.add_argument("--l2-persist", type=int, choices=[-1, 0, 1], default=-1,
-                    help="fix the persisting L2 window of the free masks (-1: autotuned)")
+                    help="fix the persisting L2 window of the slot tags (-1: autotuned)")
     ap.add_argument("--block-threads", type=int, choices=[0, 128, 256, 512], default=0,
                     help="fix the bulk kernels' block shape (0: autotuned)")
     ap.add_argument("--no-cpu-parallel", action="store_true",

@@ -4,7 +4,8 @@
  * The table is the one of "Hive Hash Table: A Warp-Cooperative, Dynamically
  * Resizable Hash Table for GPUs" (arXiv 2510.15095): 32-bit keys and 32-bit
  * values packed into 64-bit words (Section III-A), buckets of S slots with a
- * per-bucket free mask and lock plus an overflow stash (Section III-B), two
+ * per-slot tags (the free mask, and a filter for lookups) and a lock per
+ * bucket plus an overflow stash (Section III-B), two
  * candidate buckets per key from BitHash1/BitHash2 (Section III-C), insert by
  * replace -> claim-then-commit -> bounded cuckoo eviction -> stash
  * (Section IV-A, Algorithms 1-3), lookup and delete by warp match-and-elect
@@ -103,18 +104,19 @@ typedef struct {
                                of buckets up front (default; faster on the
                                multi-table path) */
   uint32_t l2_persist;      /* 1 = the kernels that claim slots (bulk insert,
-                               mixed batch, claims, eviction) keep the free masks
+                               mixed batch, claims, eviction) keep the slot tags
                                in a persisting L2 access-policy window, so that
-                               the claim atomics hit L2 while the bucket reads
-                               stream past; the first such table of the process
-                               sets the CUDA context's persisting-L2 limit (a
-                               per-process setting, gone when the process exits).
-                               0 = off (default; a tuning knob) */
-  uint32_t stage_wait_limit;/* tries before a wait for staged bucket copies
-                               gives up (TIMEOUT) and the round is redone with
-                               direct loads; 0 = 2^22 (default).  Only the
-                               256-byte-bucket (S = 32) copies wait on an
-                               mbarrier; a small value exercises the fallback */
+                               the tag reads and claim atomics hit L2 while the
+                               bucket reads stream past; the first such table of
+                               the process sets the CUDA context's persisting-L2
+                               limit (a per-process setting, gone when the process
+                               exits).  0 = off (default; a tuning knob) */
+  uint32_t stage_wait_limit;/* 0 (default): probes read the slot tags.  Otherwise,
+                               with S = 32: probes stage whole 256-byte buckets
+                               through bulk copies that wait on an mbarrier, and
+                               this is the number of tries before such a wait
+                               gives up (TIMEOUT) and the round is redone by
+                               tags; a small value exercises that fallback */
   uint32_t block_threads;   /* block shape of the bulk kernels: 128, 256 or 512
                                threads (one op per lane); 0 = 256 (default; a
                                tuning knob) */
@@ -137,8 +139,8 @@ typedef struct {
   uint64_t stash_reinserted; /* stash words moved back into buckets by maintenance */
   uint64_t splits;           /* bucket pairs split */
   uint64_t merges;           /* bucket pairs merged */
-  uint64_t probes;           /* 256-byte bucket reads by the bulk kernel (Section IV-B:
-                                one per candidate bucket examined) */
+  uint64_t probes;           /* candidate buckets examined by the bulk kernel
+                                (Section IV-B), by their tags */
   uint64_t stash_lookups;    /* binary searches of the stash by the bulk kernel */
   uint64_t fused_retries;    /* single-kernel batches: lookups repeated because a
                                 candidate bucket had a word in transit */
@@ -178,7 +180,7 @@ typedef struct {
   uint64_t size;        /* live-entry counter */
   uint64_t pending;     /* words waiting for room (0 at quiescence) */
   uint64_t* buckets;    /* [nb * S] packed words, or NULL to query sizes only */
-  uint32_t* masks;      /* [nb] free masks, bit i set = slot i free */
+  uint32_t* masks;      /* [nb] free masks, bit i set = slot i free (its tag is 0) */
   uint32_t* locks;      /* [nb] lock words */
   uint64_t* stash;      /* [stash_n] packed words */
 } hive_image;

@@ -9,7 +9,7 @@ on the current GPU and caches the fastest in a JSON file.  The knobs:
 * placement (two-choice policy): balanced, BitHash1-first (fixed tables)
 * block_threads, the block shape of the bulk kernels: 128, 256, 512 threads
   (one op per lane, so 4, 8 or 16 warps of 32 ops each)
-* l2_persist: the free masks in a persisting L2 window for the kernels that
+* l2_persist: the slot tags in a persisting L2 window for the kernels that
   claim slots, or not (fixed tables)
 * resize_batch K (bucket pairs per split/merge launch, Section IV-C), for
   resizable tables: 256, 1024, 4096, 8192

@@ -100,7 +100,7 @@ cudaEvent_t ev_get(hive_table* t) {
 View hive::make_view(const hive_table* t) {
   View v{};
   v.buckets = t->buckets;
-  v.masks = t->masks;
+  v.tags = t->tags;
   v.locks = t->locks;
   v.vers = t->locks + t->nb_max;
   v.stash_kv = t->stash_kv;
@@ -121,7 +121,11 @@ View hive::make_view(const hive_table* t) {
 namespace {
 
 List list_a(const hive_table* t) {
-  return List{t->la_words, t->la_idx, &t->ctrl->ovf_n, nullptr, t->la_cnt};
+  return List{t->la_words, t->la_idx, &t->ctrl->ovf_n, nullptr};
+}
+// The same arrays while they hold a mixed batch's new keys for launch_claim.
+List list_defer(const hive_table* t) {
+  return List{t->la_words, t->la_idx, &t->ctrl->defer_n, nullptr};
 }
 List list_b(const hive_table* t) { return List{t->lb_words, t->lb_idx, &t->ctrl->pend_n}; }
 
@@ -130,8 +134,6 @@ void free_lists(hive_table* t) {
   cudaFree(t->la_idx);
   cudaFree(t->lb_words);
   cudaFree(t->lb_idx);
-  cudaFree(t->la_cnt);
-  t->la_cnt = nullptr;
   t->la_words = t->lb_words = nullptr;
   t->la_idx = t->lb_idx = nullptr;
   t->list_cap = t->lb_cap = 0;
@@ -151,7 +153,6 @@ hive_status ensure_lists(hive_table* t, uint64_t n, bool need_b = false) {
   if (e == cudaSuccess) e = dev_alloc(&t->la_idx, cap * sizeof(uint32_t));
   if (e == cudaSuccess && two) e = dev_alloc(&t->lb_words, cap * sizeof(uint64_t));
   if (e == cudaSuccess && two) e = dev_alloc(&t->lb_idx, cap * sizeof(uint32_t));
-  if (e == cudaSuccess && two) e = dev_alloc(&t->la_cnt, cap / 32);
   if (e != cudaSuccess) {
     free_lists(t);
     return cuda_fail(e, "allocating op lists");
@@ -455,8 +456,8 @@ void hive_config_default(hive_config* cfg) {
   cfg->lock_spin_limit = 1u << 14;
 }
 
-// The persisting L2 window of a table's free masks (hive_config.l2_persist):
-// as many mask bytes as one window may cover, and a persisting set-aside of
+// The persisting L2 window of a table's slot tags (hive_config.l2_persist):
+// as many tag bytes as one window may cover, and a persisting set-aside of
 // the context at least that large (never lowered, capped at the device's
 // maximum).  With a set-aside smaller than the window, the hit ratio scales
 // down so that the persisting lines fit.
@@ -467,7 +468,7 @@ static cudaError_t setup_l2_window(hive_table* t) {
     e = cudaDeviceGetAttribute(&max_persist, cudaDevAttrMaxPersistingL2CacheSize, t->device);
   if (e != cudaSuccess) return e;
   if (max_win <= 0 || max_persist <= 0) return cudaSuccess;  // no persisting L2 here
-  const size_t bytes = std::min<size_t>(t->nb_max * sizeof(uint32_t), static_cast<size_t>(max_win));
+  const size_t bytes = std::min<size_t>(t->nb_max * t->S, static_cast<size_t>(max_win));
   size_t cur = 0;
   if ((e = cudaDeviceGetLimit(&cur, cudaLimitPersistingL2CacheSize)) != cudaSuccess) return e;
   if (cur < bytes) {
@@ -476,7 +477,7 @@ static cudaError_t setup_l2_window(hive_table* t) {
     if ((e = cudaDeviceGetLimit(&cur, cudaLimitPersistingL2CacheSize)) != cudaSuccess) return e;
   }
   if (cur == 0) return cudaSuccess;
-  t->L.l2_base = t->masks;
+  t->L.l2_base = t->tags;
   t->L.l2_bytes = bytes;
   t->L.l2_hit = cur >= bytes ? 1.0f : static_cast<float>(cur) / static_cast<float>(bytes);
   return cudaSuccess;
@@ -531,12 +532,12 @@ hive_status hive_create(const hive_config* cfg, void* stream, hive_table** out) 
 
   cudaError_t e = cudaGetDevice(&t->device);
   t->L.ops_threads = cfg->block_threads ? static_cast<int>(cfg->block_threads) : 256;
+  t->L.staged = S == 32 && cfg->stage_wait_limit != 0;
   if (e == cudaSuccess) e = query_occupancy(&t->L, static_cast<int>(S));
   if (e == cudaSuccess && cfg->blocks_per_sm) {
     const int cap = static_cast<int>(cfg->blocks_per_sm);
-    t->L.ops_blocks_per_sm = std::min(t->L.ops_blocks_per_sm, cap);
+    for (int& b : t->L.ops_blocks_per_sm) b = std::min(b, cap);
     t->L.staged_blocks_per_sm = std::min(t->L.staged_blocks_per_sm, cap);
-    t->L.staged1_blocks_per_sm = std::min(t->L.staged1_blocks_per_sm, cap);
   }
   if (e == cudaSuccess && cfg->resizable && cfg->map_on_demand) {
     // reserve the address range of nb_max buckets, back only nb_init of them
@@ -550,7 +551,7 @@ hive_status hive_create(const hive_config* cfg, void* stream, hive_table** out) 
   }
   if (e == cudaSuccess && !t->vmm)
     e = dev_alloc(&t->buckets, t->nb_max * S * sizeof(uint64_t));
-  if (e == cudaSuccess) e = dev_alloc(&t->masks, t->nb_max * sizeof(uint32_t));
+  if (e == cudaSuccess) e = dev_alloc(&t->tags, t->nb_max * S);
   if (e == cudaSuccess) e = dev_alloc(&t->locks, 2 * t->nb_max * sizeof(uint32_t));
   if (e == cudaSuccess) e = dev_alloc(&t->stash_kv, t->stash_alloc * sizeof(uint64_t));
   if (e == cudaSuccess) e = dev_alloc(&t->stash_keys, t->stash_cap * sizeof(uint32_t));
@@ -560,8 +561,7 @@ hive_status hive_create(const hive_config* cfg, void* stream, hive_table** out) 
     std::memset(t->host_ctrl, 0, sizeof(Ctrl));
     if (!t->vmm) e = cudaMemsetAsync(t->buckets, 0xFF, t->nb_max * S * sizeof(uint64_t), s);
   }
-  if (e == cudaSuccess) e = cudaMemsetAsync(t->masks, 0xFF, t->nb_max * sizeof(uint32_t), s);
-  if (e == cudaSuccess && S < 32) e = launch_fill_u32(t->masks, t->nb_max, (1u << S) - 1u, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(t->tags, 0, t->nb_max * S, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(t->locks, 0, 2 * t->nb_max * sizeof(uint32_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(t->stash_kv, 0xFF, t->stash_alloc * sizeof(uint64_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(t->ctrl, 0, sizeof(Ctrl), s);
@@ -582,7 +582,7 @@ hive_status hive_destroy(hive_table* t) {
     grow_free(&t->bucket_vm);
   else
     cudaFree(t->buckets);
-  cudaFree(t->masks);
+  cudaFree(t->tags);
   cudaFree(t->locks);
   cudaFree(t->stash_kv);
   cudaFree(t->stash_keys);
@@ -701,15 +701,16 @@ hive_status hive_execute(hive_table* t, const uint8_t* ops, const uint32_t* keys
     HIVE_LAUNCH(t, HIVE_K_MAINT, s, launch_maintenance(v, s));
     return HIVE_OK;
   }
-  // P1: finds, erases and replaces; the new keys wait in A chunk by chunk
-  // (reading 14: no op of P1 moves a word, and the claims of P2 then see
-  // every slot that P1's erases freed)
+  // P1: finds, erases and replaces; the new keys wait in A (reading 14: no op
+  // of P1 moves a word, and the claims of P2 then see every slot that P1's
+  // erases freed)
   HIVE_LAUNCH(t, HIVE_K_MIXED, s,
               launch_ops(kModeMixed, v, ops, keys, vals, n, vals_out, nullptr, status,
-                         list_a(t), t->L, s, true));
+                         list_defer(t), t->L, s, true));
   // P2: claims (A -> B for keys whose buckets are both full), then eviction
-  // and stash (B, with pending items appended to A, whose count is still 0)
-  HIVE_LAUNCH(t, HIVE_K_CLAIM, s, launch_claim(v, list_a(t), n, list_b(t), status, t->L, s));
+  // and stash (B, with pending items appended to A, whose pending count is
+  // still 0)
+  HIVE_LAUNCH(t, HIVE_K_CLAIM, s, launch_claim(v, list_defer(t), n, list_b(t), t->L, s));
   HIVE_LAUNCH(t, HIVE_K_EVICT, s,
               launch_overflow(v, list_b(t), list_a(t), t->cfg.resizable, status, t->L, s));
   if (t->cfg.resizable) return finish_resizable(t, status, s, false);
@@ -784,9 +785,9 @@ hive_status hive_memory(hive_table* t, uint64_t* committed, uint64_t* reserved) 
   if (!committed || !reserved) return fail(HIVE_ERR_INVALID_ARG, "outputs must not be NULL");
   const uint64_t bucket_max = t->nb_max * t->S * sizeof(uint64_t);
   const uint64_t bucket_now = t->vmm ? t->bucket_vm.committed : bucket_max;
-  const uint64_t other = t->nb_max * 3 * sizeof(uint32_t) + t->stash_alloc * sizeof(uint64_t) +
+  const uint64_t other = t->nb_max * (t->S + 2 * sizeof(uint32_t)) + t->stash_alloc * sizeof(uint64_t) +
                          t->stash_cap * sizeof(uint32_t) + sizeof(Ctrl) +
-                         (t->list_cap + t->lb_cap) * 12 + t->lb_cap / 32;
+                         (t->list_cap + t->lb_cap) * 12;
   *committed = bucket_now + other;
   *reserved = bucket_max + other;
   return HIVE_OK;
@@ -807,8 +808,7 @@ hive_status hive_clear(hive_table* t, void* stream) {
   // Buckets at or past nb are kept empty by construction; only [0, nb) and
   // the stash need resetting.
   HIVE_CK(cudaMemsetAsync(t->buckets, 0xFF, t->nb * t->S * sizeof(uint64_t), s));
-  HIVE_CK(cudaMemsetAsync(t->masks, 0xFF, t->nb * sizeof(uint32_t), s));
-  if (t->S < 32) HIVE_CK(launch_fill_u32(t->masks, t->nb, (1u << t->S) - 1u, s));
+  HIVE_CK(cudaMemsetAsync(t->tags, 0, t->nb * t->S, s));
   HIVE_CK(cudaMemsetAsync(t->locks, 0, t->nb * sizeof(uint32_t), s));
   HIVE_CK(cudaMemsetAsync(t->stash_kv, 0xFF, t->stash_alloc * sizeof(uint64_t), s));
   HIVE_CK(cudaMemsetAsync(t->ctrl, 0, sizeof(Ctrl), s));
@@ -948,12 +948,24 @@ hive_status hive_dump(hive_table* t, hive_image* img, void* stream) {
     return fail(HIVE_ERR_INVALID_ARG, "image arrays must not be NULL");
   HIVE_CK(cudaMemcpyAsync(img->buckets, t->buckets, t->nb * t->S * sizeof(uint64_t),
                           cudaMemcpyDeviceToHost, s));
-  HIVE_CK(cudaMemcpyAsync(img->masks, t->masks, t->nb * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+  // the image's free masks are the slots whose tag is 0
+  std::vector<uint8_t> tags;
+  try {
+    tags.resize(t->nb * t->S);
+  } catch (const std::bad_alloc&) {
+    return fail(HIVE_ERR_OOM, "hive_dump: host allocation failed");
+  }
+  HIVE_CK(cudaMemcpyAsync(tags.data(), t->tags, tags.size(), cudaMemcpyDeviceToHost, s));
   HIVE_CK(cudaMemcpyAsync(img->locks, t->locks, t->nb * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   if (img->stash_n)
     HIVE_CK(cudaMemcpyAsync(img->stash, t->stash_kv, img->stash_n * sizeof(uint64_t),
                             cudaMemcpyDeviceToHost, s));
   HIVE_CK(cudaStreamSynchronize(s));
+  for (uint64_t b = 0; b < t->nb; ++b) {
+    uint32_t m = 0;
+    for (uint32_t k = 0; k < t->S; ++k) m |= static_cast<uint32_t>(tags[b * t->S + k] == 0) << k;
+    img->masks[b] = m;
+  }
   return HIVE_OK;
 }
 

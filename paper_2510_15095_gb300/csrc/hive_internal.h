@@ -58,14 +58,15 @@ struct alignas(128) Ctrl {
   unsigned int err;          // sticky error bits
   unsigned int merge_excess; // words a merge batch cannot keep in the low bucket
   unsigned int n_insert;     // insert ops counted in a mixed batch
-  unsigned int pad0[5];
+  unsigned int defer_n;      // new keys of a mixed batch waiting for k_claim
+  unsigned int pad0[4];
   unsigned long long stats[kNumStats];
 };
 
 // Everything a kernel needs to reach one table; passed by value.
 struct View {
   uint64_t* buckets;     // [nb_max * S] packed words (value << 32 | key)
-  uint32_t* masks;       // [nb_max] free masks, bit i set = slot i free
+  uint32_t* tags;        // [nb_max * S / 4] slot tags, one byte per slot (0: free slot)
   uint32_t* locks;       // [nb_max] bucket locks (eviction only)
   uint32_t* vers;        // [nb_max] bucket versions (single-kernel batches)
   uint64_t* stash_kv;    // [stash_alloc] stash words, EMPTY padded
@@ -88,7 +89,6 @@ struct List {
   uint32_t* idx;   // caller op index or kNoOp
   unsigned int* count;
   uint32_t* seg;   // multi-table batches: segment of each entry (else NULL)
-  uint8_t* chunk_cnt;  // mixed batches: new keys of each 32-op chunk (see k_claim)
 };
 
 // One (table, op range) of a multi-table batch; 64 bytes.
@@ -123,14 +123,14 @@ enum OpMode : int { kModeFind = 0, kModeInsert = 1, kModeErase = 2, kModeMixed =
 struct Launch {
   int num_sms;
   int ops_threads;           // block shape of the bulk kernels: 128, 256 or 512 threads
-  int ops_blocks_per_sm;     // bulk kernel, fragments loaded from global memory
-  int staged_blocks_per_sm;  // bulk kernel, paired insert rounds staged in shared memory
-  int staged1_blocks_per_sm; // bulk kernel, single-bucket rounds staged in shared memory
+  int ops_blocks_per_sm[5];  // bulk kernel, by mode (4: mixed with deferred claims)
+  bool staged;               // 32-slot buckets probed whole, staged in shared memory
+  int staged_blocks_per_sm;  // bulk kernel with staged probes
   int fused_blocks_per_sm;   // single-kernel mixed batch
   int ovf_blocks_per_sm;
   int multi_blocks_per_sm;
   int claim_blocks_per_sm;   // claims of a mixed batch's new keys
-  // persisting L2 window over the free masks for the kernels that claim
+  // persisting L2 window over the slot tags for the kernels that claim
   // slots (l2_bytes = 0: none)
   void* l2_base;
   size_t l2_bytes;
@@ -138,18 +138,18 @@ struct Launch {
 };
 
 // Kernel launchers (hive_kernels.cu).  Each returns the launch error.
-// defer (mixed batches): new keys go to list A chunk by chunk for
-// launch_claim instead of claiming in the bulk kernel.
+// defer (mixed batches): new keys go to the list for launch_claim instead of
+// claiming in the bulk kernel.
 cudaError_t launch_ops(int mode, const View& v, const uint8_t* ops, const uint32_t* keys,
                        const uint32_t* vals, uint64_t n, uint32_t* vals_out, uint8_t* found,
                        uint8_t* status, List ovf, const Launch& L, cudaStream_t s,
                        bool defer = false);
 cudaError_t launch_overflow(const View& v, List in, List pend, int resizable, uint8_t* status,
                             const Launch& L, cudaStream_t s);
-// Claims for the new keys of a mixed batch of n ops, left in `in` chunk by
-// chunk by the bulk kernel; items with both buckets full go to `out`.
-cudaError_t launch_claim(const View& v, List in, uint64_t n, List out, uint8_t* status,
-                         const Launch& L, cudaStream_t s);
+// Claims for the new keys of a mixed batch of n ops, listed in `in` by the bulk
+// kernel; items with both buckets full go to `out`.
+cudaError_t launch_claim(const View& v, List in, uint64_t n, List out, const Launch& L,
+                         cudaStream_t s);
 cudaError_t launch_maintenance(const View& v, cudaStream_t s);
 cudaError_t launch_split(const View& v_new, uint32_t src0, uint32_t count, uint32_t half,
                          cudaStream_t s);
@@ -249,7 +249,7 @@ struct hive_table {
   uint32_t stash_cap = 0;
   uint64_t stash_alloc = 0;
   uint64_t* buckets = nullptr;
-  uint32_t* masks = nullptr;
+  uint32_t* tags = nullptr;
   uint32_t* locks = nullptr;  // [2 nb_max]: bucket locks, then bucket versions
   uint64_t* stash_kv = nullptr;
   uint32_t* stash_keys = nullptr;
@@ -259,7 +259,6 @@ struct hive_table {
   uint64_t lb_cap = 0;           // entries of list B (0: not allocated)
   uint64_t* la_words = nullptr;  // list A: bulk kernel -> eviction kernel
   uint32_t* la_idx = nullptr;
-  uint8_t* la_cnt = nullptr;     // list A per-chunk counts (mixed batches)
   uint64_t* lb_words = nullptr;  // list B: items that found no room
   uint32_t* lb_idx = nullptr;
   uint64_t size_host = 0;       // exact after each resizable call

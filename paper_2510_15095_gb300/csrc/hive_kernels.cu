@@ -2,21 +2,17 @@
 //
 // Layout (Section III-A/B of the paper): a bucket is S packed 64-bit words
 // (value << 32 | key), S = 32 (256 bytes) or 16 (128 bytes), aligned to its
-// size; a 32-bit free mask per bucket (bit i set = slot i free); a 32-bit lock
-// per bucket used only by eviction; an overflow stash of packed words.  The
-// empty word is all ones (key 0xFFFFFFFF).
+// size; S one-byte slot tags per bucket (0 = free slot), which are the free
+// mask and a filter for lookups; a 32-bit lock per bucket used only by
+// eviction; an overflow stash of packed words.  The empty word is all ones
+// (key 0xFFFFFFFF).
 //
 // Kernels:
-//   k_ops<MODE,S>  bulk find / insert (steps 1-2) / erase / mixed batch.  A
-//                  warp takes 32 ops.  Staged: each probe round copies the
-//                  buckets of all 32 ops into the warp's shared-memory buffer
-//                  (cp.async for 128-byte buckets, one bulk copy per 256-byte
-//                  bucket) and each lane scans its own op's buckets.  Direct:
-//                  L = S/2 lanes read a bucket as 16-byte fragments, and
-//                  match-and-elect (WCME, Section III-F) is a ballot over the
-//                  fragments.  New keys claim a slot with one atomicAnd on the
-//                  free mask (WABC, Section III-E), the free slot predicted from
-//                  the probe round.
+//   k_ops<MODE,S>  bulk find / insert (steps 1-2) / erase / mixed batch, one op
+//                  per lane: both candidate buckets' tags in one round trip,
+//                  then the words whose tag matches the key's.  A new key
+//                  claims a slot with one CAS on a tag word (WABC, Section
+//                  III-E).
 //   k_overflow<S>  steps 3-4 for inserts whose two buckets were full: warp per
 //                  item, bounded cuckoo eviction under the bucket lock
 //                  (Algorithm 3), then the stash.
@@ -38,50 +34,9 @@ namespace {
 
 constexpr int kOpsThreads = 256;
 #ifndef HIVE_MULTI_MIN_BLOCKS
-#define HIVE_MULTI_MIN_BLOCKS 3  // the multi-table bulk kernel also holds a table view per warp
-#endif
-// Bulk-kernel modes (bit kModeFind, kModeInsert, ...) whose probes are staged
-// in shared memory, per bucket width; the others load
-// fragments straight from global memory with the warp-wide match-and-elect.
-// Measured on the 2^26-slot, 95%-load bench workload, staging wins for
-// every mode at both widths (with the copy path chosen below per width).
-#ifndef HIVE_STAGED_MODES_S16
-#define HIVE_STAGED_MODES_S16 0xF
-#endif
-#ifndef HIVE_STAGED_MODES_S32
-#define HIVE_STAGED_MODES_S32 0xF
-#endif
-// How a staged round copies its buckets, per bucket width: 1 = cp.async
-// through the load/store path (16 bytes per lane, coalesced per bucket),
-// 0 = one bulk copy (TMA) per bucket.  Measured on the bench workload, the
-// load/store path wins for 128-byte buckets (S = 16 finds 30.1 against 27.7
-// Gops/s) and bulk copies win for 256-byte buckets (S = 32 inserts 11.7
-// against 11.0).
-#ifndef HIVE_STAGE_LSU_S16
-#define HIVE_STAGE_LSU_S16 1
-#endif
-#ifndef HIVE_STAGE_LSU_S32
-#define HIVE_STAGE_LSU_S32 0
-#endif
-// Where the paired insert round takes the free slots that steer its claims:
-// 1 = the EMPTY words of the staged buckets (no mask reads), 0 = the two
-// free masks, read while the copies are in flight.
-#ifndef HIVE_FREE_FROM_STAGE
-#define HIVE_FREE_FROM_STAGE 1
-#endif
-#ifndef HIVE_STAGED_SMALL_MIN_BLOCKS
-#define HIVE_STAGED_SMALL_MIN_BLOCKS 4  // 32 KB of staging per block (S = 16 single rounds)
-#endif
-#ifndef HIVE_STAGED_MIN_BLOCKS
-#define HIVE_STAGED_MIN_BLOCKS 3  // 64 KB of staging per block: three blocks fit an SM
-#endif
-#ifndef HIVE_OPS_MIN_BLOCKS
-#define HIVE_OPS_MIN_BLOCKS 4  // resident 256-thread blocks per SM the bulk kernel is built for
+#define HIVE_MULTI_MIN_BLOCKS 4
 #endif
 constexpr int kOvfThreads = 256;
-__host__ __device__ constexpr bool staged_mode(int mode, int S) {
-  return ((S == 16 ? HIVE_STAGED_MODES_S16 : HIVE_STAGED_MODES_S32) >> mode) & 1;
-}
 constexpr int kMaintThreads = 1024;
 constexpr unsigned kMaintSmemWords = 8192;  // 64 KB of words sorted in shared memory
 
@@ -95,15 +50,129 @@ __device__ __forceinline__ uint64_t pack(uint32_t k, uint32_t v) {
 __device__ __forceinline__ uint32_t key_of(uint64_t w) { return static_cast<uint32_t>(w); }
 __device__ __forceinline__ uint32_t val_of(uint64_t w) { return static_cast<uint32_t>(w >> 32); }
 
+// The two candidate buckets of a key.
+struct Cand {
+  uint32_t b1, b2;
+};
+__device__ __forceinline__ Cand cand_of(const View& v, uint32_t key) {
+  return Cand{lh_bucket(bithash1(key), v.M, v.p), lh_bucket(bithash2(key), v.M, v.p)};
+}
+
+// ----------------------------------------------------------------------------
+// Slot tags
+// ----------------------------------------------------------------------------
+//
+// Each slot has a one-byte tag in an array of its own: 0 while the slot is
+// free, else a byte in [1, 255] computed from the slot's key.  The S tags of
+// a bucket are 32 (S = 32) or 16 (S = 16) bytes, at most one memory sector,
+// so a lookup reads one sector per candidate bucket and then only the words
+// whose tag matches: one word for a hit, and one in about 255 / S buckets for
+// a false match.  Random reads bound every bulk kernel here: measured on one
+// GB300, DRAM serves 40-50 G random accesses/s whether each moves 32 or 128
+// bytes, L2 serves 290 G/s of 32-byte sectors, and the tags of a 2^26-slot
+// table (64 MB) fit in L2 where its words (512 MB) do not.
+//
+// The tags are also the authority on free slots (WABC, Section III-E): a
+// claim is one CAS that replaces a zero byte of a tag word by the key's tag,
+// and the claimer then owns the slot and publishes the word with a plain
+// store.  Every later change of a tag byte is an XOR with (old tag ^ new
+// tag), so changes of neighbouring slots in one tag word never undo each
+// other.  A chain that swaps a word lets its XOR reach memory before it
+// unlocks the bucket (transient sums of two pending XORs could read as 0).
+// At the end of every kernel a slot is EMPTY iff its tag is 0.
+
+__device__ __forceinline__ uint32_t tag_of(uint32_t key) {
+  // the high bits of a multiplicative hash, independent of the bucket bits
+  return 1u + __umulhi(key * 0x9E3779B1u, 255u);
+}
+
+template <int S>
+struct TagVec {
+  uint32_t w[S / 4];
+};
+
+// L2 priorities: tags stay (every op reads 2 S bytes of them), words go first
+// (an op reads one of 8 bytes, and the next op that wants its line is far
+// away).  Measured on 2^26 slots: lookups 1.77 -> 1.51 ms with the words sent
+// first, bulk load 4.08 -> 3.67 ms with the tags kept as well.
+__device__ __forceinline__ uint64_t policy_keep() {
+  uint64_t p;
+  asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+__device__ __forceinline__ uint64_t policy_pass() {
+  uint64_t p;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+
+// The tags of bucket b.  RO: through the read-only path (no kernel writes
+// tags meanwhile); otherwise a relaxed load, which never returns a stale
+// cached copy.
+template <int S, bool RO>
+__device__ __forceinline__ TagVec<S> ld_tags(const View& v, uint32_t b) {
+  TagVec<S> t;
+  const uint32_t* p = v.tags + static_cast<uint64_t>(b) * (S / 4);
+  const uint64_t pol = policy_keep();
+  if constexpr (S == 32) {
+    if constexpr (RO)
+      asm("ld.global.nc.L2::cache_hint.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
+          : "=r"(t.w[0]), "=r"(t.w[1]), "=r"(t.w[2]), "=r"(t.w[3]), "=r"(t.w[4]), "=r"(t.w[5]),
+            "=r"(t.w[6]), "=r"(t.w[7])
+          : "l"(p), "l"(pol));
+    else
+      asm volatile(
+          "ld.relaxed.gpu.global.L2::cache_hint.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
+          : "=r"(t.w[0]), "=r"(t.w[1]), "=r"(t.w[2]), "=r"(t.w[3]), "=r"(t.w[4]), "=r"(t.w[5]),
+            "=r"(t.w[6]), "=r"(t.w[7])
+          : "l"(p), "l"(pol)
+          : "memory");
+  } else {
+    if constexpr (RO)
+      asm("ld.global.nc.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;"
+          : "=r"(t.w[0]), "=r"(t.w[1]), "=r"(t.w[2]), "=r"(t.w[3])
+          : "l"(p), "l"(pol));
+    else
+      asm volatile("ld.relaxed.gpu.global.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;"
+                   : "=r"(t.w[0]), "=r"(t.w[1]), "=r"(t.w[2]), "=r"(t.w[3])
+                   : "l"(p), "l"(pol)
+                   : "memory");
+  }
+  return t;
+}
+
+// 0x80 in every byte of x that is zero (exact in every byte).
+__device__ __forceinline__ uint32_t zero_bytes(uint32_t x) {
+  return ~(((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x | 0x7F7F7F7Fu);
+}
+
+// Slot sets are 32-bit masks in tag order: bit 8 j + q stands for byte j of
+// tag word q, which is slot 4 q + j.  Consecutive bits lie in different tag
+// words, so claims that start at different bits rarely meet in one word.
+__device__ __forceinline__ uint32_t slot_of(uint32_t p) { return ((p & 7u) << 2) | (p >> 3); }
+
+// Slots whose tag equals `t4` (a tag in all four bytes); t4 = 0: free slots.
+template <int S>
+__device__ __forceinline__ uint32_t tag_match(const TagVec<S>& t, uint32_t t4) {
+  uint32_t m = 0;
+#pragma unroll
+  for (int q = 0; q < S / 4; ++q) m |= zero_bytes(t.w[q] ^ t4) >> (7 - q);
+  return m;
+}
+template <int S>
+__device__ __forceinline__ uint32_t free_slots(const TagVec<S>& t) {
+  return tag_match<S>(t, 0u);
+}
+
+template <int S>
+__device__ __forceinline__ uint32_t* tag_word(const View& v, uint32_t b, uint32_t slot) {
+  return v.tags + static_cast<uint64_t>(b) * (S / 4) + (slot >> 2);
+}
+
 // ----------------------------------------------------------------------------
 // Memory access helpers
 // ----------------------------------------------------------------------------
 
-// 16-byte bucket fragment through the read-only path (table not written by
-// the running kernel).
-__device__ __forceinline__ void ld_frag_ro(const uint64_t* p, uint64_t& a, uint64_t& b) {
-  asm("ld.global.nc.L1::no_allocate.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p));
-}
 // 16-byte bucket fragment while other warps may be writing the table.
 __device__ __forceinline__ void ld_frag(const uint64_t* p, uint64_t& a, uint64_t& b) {
   asm volatile("ld.relaxed.gpu.global.L1::no_allocate.v2.u64 {%0, %1}, [%2];"
@@ -111,60 +180,136 @@ __device__ __forceinline__ void ld_frag(const uint64_t* p, uint64_t& a, uint64_t
                : "l"(p)
                : "memory");
 }
+// One slot's word; RO as for ld_tags.
+template <bool RO>
+__device__ __forceinline__ uint64_t ld_word(const uint64_t* p) {
+  uint64_t r;
+  const uint64_t pol = policy_pass();
+  if constexpr (RO)
+    asm("ld.global.nc.L2::cache_hint.b64 %0, [%1], %2;" : "=l"(r) : "l"(p), "l"(pol));
+  else
+    asm volatile("ld.relaxed.gpu.global.L2::cache_hint.b64 %0, [%1], %2;"
+                 : "=l"(r)
+                 : "l"(p), "l"(pol)
+                 : "memory");
+  return r;
+}
 
 // ----------------------------------------------------------------------------
 // Slot claims (WABC, Section III-E / Algorithm 2)
 // ----------------------------------------------------------------------------
 
-// Claim a free slot of bucket b starting from the predicted slot `s`, then
-// publish `word` with a plain store.  Used where no eviction runs concurrently
-// (the bulk kernel and maintenance).  Algorithm 2 restores the bit with
-// fetch_or when the fetch_and finds it already clear; that would free a slot
-// another warp owns, so here a failed claim retries on the returned mask.
+// Claims a free byte of tag word q of bucket b, whose last seen value is
+// `cur` and whose byte j was 0 in it, and publishes `word` there with a plain
+// store: a non-zero tag byte makes the slot the claimer's, and nothing else
+// writes a slot while it is EMPTY (erases, replaces and swaps expect a
+// non-EMPTY word).  Algorithm 2 restores its bit when it loses the race; here
+// a lost CAS changes nothing, and the claim goes on from the value the CAS
+// returned.  A CAS fails only because another op of the batch changed the
+// word, so the loop ends.
 template <int S>
-__device__ __forceinline__ bool claim_store(const View& v, uint32_t b, uint32_t s,
-                                            uint64_t word) {
-  for (int t = 0; t <= S && s < S; ++t) {
-    const uint32_t bit = 1u << s;
-    const uint32_t old = atomicAnd(v.masks + b, ~bit);
-    if (old & bit) {
-      st_relaxed64(v.buckets + static_cast<uint64_t>(b) * S + s, word);
+__device__ __forceinline__ bool claim_in_word(const View& v, uint32_t b, uint32_t q, uint32_t j,
+                                              uint32_t cur, uint32_t tag, uint64_t word) {
+  uint32_t* tw = v.tags + static_cast<uint64_t>(b) * (S / 4) + q;
+  for (;;) {
+    const uint32_t old = atomicCAS(tw, cur, cur | (tag << (8 * j)));
+    if (old == cur) {
+      st_relaxed64(v.buckets + static_cast<uint64_t>(b) * S + 4 * q + j, word);
       return true;
     }
-    s = old ? static_cast<uint32_t>(__ffs(old) - 1) : S;
+    const uint32_t z = zero_bytes(old);
+    if (!z) return false;
+    cur = old;
+    j = (__ffs(z) - 1) >> 3;
+  }
+}
+
+// The first set bit of slot set m at or after bit `rot`, cyclically (m != 0).
+__device__ __forceinline__ uint32_t pick_slot(uint32_t m, uint32_t rot) {
+  return (__ffs(__funnelshift_r(m, m, rot)) - 1 + rot) & 31u;
+}
+// Tag word q of t, for q known only at run time.
+template <int S>
+__device__ __forceinline__ uint32_t tag_sel(const TagVec<S>& t, uint32_t q) {
+  uint32_t x = t.w[0];
+#pragma unroll
+  for (int k = 1; k < S / 4; ++k)
+    if (q == k) x = t.w[k];
+  return x;
+}
+
+// Claims a slot of bucket b for `word` among the free slots `fm` of its tags
+// `t`, read moments ago (the CAS is the authority), starting at bit `rot`.
+template <int S>
+__device__ __forceinline__ bool claim_from(const View& v, uint32_t b, const TagVec<S>& t,
+                                           uint32_t fm, uint64_t word, uint32_t rot) {
+  const uint32_t tag = tag_of(key_of(word));
+  while (fm) {
+    const uint32_t p = pick_slot(fm, rot);
+    const uint32_t q = p & 7u;
+    if (claim_in_word<S>(v, b, q, p >> 3, tag_sel<S>(t, q), tag, word)) return true;
+    fm &= ~(0x01010101u << q);  // that word is full now
   }
   return false;
 }
 
-// The claim of the eviction kernel and of the single-kernel batch: fetch_and
-// on the free mask, then a plain store.  The bit makes the slot the
-// claimer's, and nothing else writes a slot while it is EMPTY: in the
-// eviction phase slots only go from EMPTY to occupied (there are no erases)
-// and a chain exchanges only a slot it saw occupied; in the single-kernel
-// batch every other write to a bucket word is a CAS whose expected word is
-// not EMPTY (an erase's, a replace's, a chain's swap).  `hint`: a free mask
-// of bucket b read moments ago, used as the first guess (the fetch_and result
-// is the authority either way).
+// The same with the tags read here.
 template <int S>
-__device__ __forceinline__ bool claim_pub(const View& v, uint32_t b, uint64_t word,
-                                          uint32_t hint = 0) {
-  uint32_t fm = hint ? hint : ld_relaxed32(v.masks + b);
-  for (int t = 0; t <= S && fm; ++t) {
-    const uint32_t s = __ffs(fm) - 1;
-    const uint32_t bit = 1u << s;
-    const uint32_t old = atomicAnd(v.masks + b, ~bit);
-    if (old & bit) {
-      st_relaxed64(v.buckets + static_cast<uint64_t>(b) * S + s, word);
-      return true;
-    }
-    fm = old;
-  }
-  return false;
+__device__ __forceinline__ bool claim_bucket(const View& v, uint32_t b, uint64_t word,
+                                             uint32_t rot) {
+  const TagVec<S> t = ld_tags<S, false>(v, b);
+  return claim_from<S>(v, b, t, free_slots<S>(t), word, rot);
 }
 
-// The bucket lock serialises evictors of one bucket (Algorithm 3).  Every
-// access it protects is an L2 atomic whose result has returned before the
-// unlock issues, so neither side needs a fence.
+// Where a key's claims start in a bucket: spreads the claims of concurrent
+// inserts into one bucket over its tag words.
+__device__ __forceinline__ uint32_t claim_rot(uint32_t key) { return (key * 0x85EBCA6Bu) >> 27; }
+
+// Step 2 for an absent key, with the tags of both candidate buckets at hand:
+// the bucket the placement rule prefers, else the other (with its tags read
+// again: rare, and keeping both sets costs registers).
+template <int S>
+__device__ __forceinline__ bool place_from(const View& v, uint32_t b1, uint32_t b2,
+                                           const TagVec<S>& t1, const TagVec<S>& t2,
+                                           uint64_t word) {
+  const uint32_t m1 = free_slots<S>(t1), m2 = free_slots<S>(t2);
+  const uint32_t f1 = __popc(m1), f2 = __popc(m2);
+  const bool first1 = v.placement ? (f1 > 0) : (f1 >= f2);
+  const uint32_t rot = claim_rot(key_of(word));
+  TagVec<S> t;
+#pragma unroll
+  for (int q = 0; q < S / 4; ++q) t.w[q] = first1 ? t1.w[q] : t2.w[q];
+  if (claim_from<S>(v, first1 ? b1 : b2, t, first1 ? m1 : m2, word, rot)) return true;
+  // filled up meanwhile, or no room in either when the tags were read
+  if (b1 == b2 || (first1 ? f2 : f1) == 0) return false;
+  return claim_bucket<S>(v, first1 ? b2 : b1, word, rot);
+}
+template <int S>
+__device__ __forceinline__ bool place_new(const View& v, uint32_t b1, uint32_t b2, uint64_t word) {
+  const TagVec<S> t1 = ld_tags<S, false>(v, b1);
+  const TagVec<S> t2 = ld_tags<S, false>(v, b2);
+  return place_from<S>(v, b1, b2, t1, t2, word);
+}
+
+// Frees a slot whose word (of key `key`) this thread has just emptied: called
+// once the CAS to EMPTY has returned, so a claimer that sees the zero tag
+// finds the slot EMPTY.
+template <int S>
+__device__ __forceinline__ void free_tag(const View& v, uint32_t b, uint32_t slot, uint32_t key) {
+  atomicXor(tag_word<S>(v, b, slot), tag_of(key) << (8 * (slot & 3u)));
+}
+// Slot's word changed from a key with tag t0 to one with tag t1.
+template <int S>
+__device__ __forceinline__ void swap_tag(const View& v, uint32_t b, uint32_t slot, uint32_t k0,
+                                         uint32_t k1) {
+  const uint32_t d = tag_of(k0) ^ tag_of(k1);
+  if (d) atomicXor(tag_word<S>(v, b, slot), d << (8 * (slot & 3u)));
+}
+
+// The bucket lock serialises evictors of one bucket (Algorithm 3).  The word
+// swap it protects is an L2 atomic whose result has returned before the
+// unlock; the tag change of the swap is ordered before the unlock by the
+// fence in unlock_swapped().
 __device__ __forceinline__ bool lock_bucket(const View& v, uint32_t b) {
   for (uint32_t t = 0; t < v.lock_spin_limit; ++t) {
     if (atomicCAS(v.locks + b, 0u, 1u) == 0u) return true;
@@ -173,6 +318,10 @@ __device__ __forceinline__ bool lock_bucket(const View& v, uint32_t b) {
   return false;
 }
 __device__ __forceinline__ void unlock_bucket(const View& v, uint32_t b) {
+  atomicExch(v.locks + b, 0u);
+}
+__device__ __forceinline__ void unlock_swapped(const View& v, uint32_t b) {
+  fence_acq_rel_gpu();
   atomicExch(v.locks + b, 0u);
 }
 
@@ -198,68 +347,29 @@ __device__ __forceinline__ bool stash_find(const View& v, uint32_t stash_n, uint
 struct LaneCounters {
   int size_delta = 0;
   unsigned replaced = 0, claimed = 0, overflowed = 0, stash_lookups = 0;
-  unsigned probes = 0;  // warp-uniform: buckets probed by this warp
+  unsigned probes = 0;  // warp-uniform: buckets examined by this warp
   bool reserved = false, contract = false;
-};
-
-// Lane geometry of a bucket of S slots read as 16-byte fragments: L lanes per
-// bucket, Q buckets per load instruction.
-template <int S>
-struct Geo {
-  static constexpr int L = S / 2;
-  static constexpr int Q = 32 / L;
-  static constexpr unsigned LM = (L >= 32) ? 0xFFFFFFFFu : ((1u << L) - 1u);
 };
 
 // ---- Shared-memory staging of bucket reads ----
 //
-// A kernel that stages its probes gives each warp one mbarrier and a buffer
-// (stage_words() below): every bucket a probe round needs -- the 32 ops'
-// buckets of a single-bucket round, or both candidate buckets of 32 (S = 16)
-// or 16 (S = 32) ops of a paired round -- is copied in before any compare, so
-// the warp has all of them in flight at once without holding registers.
-// 128-byte buckets are copied with 16-byte cp.async through the load/store
-// path (stage_issue_lsu); 256-byte buckets with one bulk copy (TMA) each,
-// counted by the barrier (stage_issue).  Each lane then scans its own op's
-// buckets in shared memory.  A barrier wait that does not end within
-// View::stage_spin_limit tries raises the table's sticky TIMEOUT error, marks
-// the stage dead and redoes the round from global memory; before the warp
-// exits it waits up to kMbarSpinLimit tries for the copies still in flight.
-constexpr int kStageWords = 1024;
-// Staging words of a paired insert round: both buckets of kPairWords / (2 S)
-// ops per round (32 ops at S = 16 and 8 KB; fewer words split a chunk into
-// more rounds and leave more of the SM's on-chip memory to L1)
-#ifndef HIVE_PAIR_WORDS
-#define HIVE_PAIR_WORDS 1024
-#endif
-constexpr int kPairWords = HIVE_PAIR_WORDS;
+// Tables of 32-slot buckets created with a stage_wait_limit probe whole
+// buckets instead of tags: the buckets of a warp's 32 ops are copied into its
+// 8 KB of shared memory with one bulk copy (TMA) each, counted by the warp's
+// mbarrier, and each lane scans its own op's bucket.  A barrier wait that
+// does not end within View::stage_spin_limit tries raises the table's sticky
+// TIMEOUT error, marks the stage dead and redoes the round by tags; before
+// the warp exits it waits up to kMbarSpinLimit tries for the copies still in
+// flight.
 constexpr uint32_t kMbarSpinLimit = 1u << 22;
-
-// Staging words a warp of mode MODE needs: a paired insert round fills the
-// whole 8 KB; a single-bucket round holds 32 buckets (4 KB at S = 16), which
-// lets four 256-thread blocks share an SM.
-__host__ __device__ constexpr int stage_words(int mode, int S) {
-  return mode == kModeInsert ? kPairWords : 32 * S;
-}
-// Shared-memory words per warp: its barrier, then its staging words.  (The
-// 64 KB of a paired round's block keeps three blocks within a 196 KB
-// shared-memory carveout, which leaves the L1 that the cp.async.ca copies go
-// through 60 KB; three blocks of 68 KB need the largest carveout, and the
-// insert kernel then ran at two-thirds speed.)
-__host__ __device__ constexpr int warp_smem_words(int mode, int S) {
-  return 2 + stage_words(mode, S);
-}
-__host__ __device__ constexpr size_t stage_smem(int mode, int S, int threads = kOpsThreads) {
-  return static_cast<size_t>(threads / 32) * 8u * warp_smem_words(mode, S);
-}
-__host__ __device__ constexpr int staged_min_blocks(int mode, int S) {
-  return (mode != kModeInsert && stage_words(mode, S) < kStageWords) ? HIVE_STAGED_SMALL_MIN_BLOCKS
-                                                                     : HIVE_STAGED_MIN_BLOCKS;
+__host__ __device__ constexpr int stage_warp_words(int S) { return 2 + 32 * S; }
+__host__ __device__ constexpr size_t stage_smem(int S, int threads = kOpsThreads) {
+  return static_cast<size_t>(threads / 32) * 8u * stage_warp_words(S);
 }
 
 struct Stage {
   uint64_t* bar;   // mbarrier
-  uint64_t* buf;   // kStageWords words, 16-byte aligned
+  uint64_t* buf;   // 32 S words, 16-byte aligned
   uint32_t phase;  // parity of the barrier's current phase
   bool dead;       // a wait gave up: copies may still land, the buffer is not reused
 };
@@ -267,7 +377,7 @@ struct Stage {
 // Sets up the calling warp's stage in the kernel's dynamic shared memory
 // (`stride` words per warp: its barrier, then its staging words).
 __device__ __forceinline__ Stage stage_init(uint64_t* smem, int warp_in_block, int lane,
-                                            int stride = kStageWords + 2) {
+                                            int stride) {
   Stage sg;
   uint64_t* base = smem + static_cast<size_t>(warp_in_block) * stride;
   sg.bar = base;
@@ -287,41 +397,21 @@ __device__ __forceinline__ void stage_drain(Stage& sg) {
   for (uint32_t it = 0; it < kMbarSpinLimit && !ok; ++it) ok = mbar_try_wait(sg.bar, sg.phase ^ 1u);
 }
 
-// Issues the copies of one staged round and waits for them (warp-wide).
-// PAIR = false: op j (bit j of `need`, j < 32) copies bucket x1 of lane j to
-// buffer bucket j.  PAIR = true: ops [o0, o0 + 512 / S) copy buckets x1 and x2
-// of their lanes to buffer buckets 2 (j - o0) and 2 (j - o0) + 1.  Returns
-// false, with the stage marked dead and the error raised, if the wait gave up.
-template <int S, bool PAIR>
-__device__ __forceinline__ void stage_issue(const View& v, Stage& sg, unsigned need, int o0,
-                                            uint32_t x1, uint32_t x2, int lane) {
+// One staged round (warp-wide): op j (bit j of `need`) copies bucket x of
+// lane j to buffer bucket j, then the warp waits (bounded).  A limit below 16
+// polls without suspending (mbarrier.test_wait), so that a test can make the
+// wait give up while the copies are certainly in flight.  Returns false, with
+// the stage marked dead and the error raised, if the wait gave up.
+template <int S>
+__device__ __forceinline__ bool stage_round(const View& v, Stage& sg, unsigned need, uint32_t x,
+                                            int lane) {
   constexpr uint32_t kBucketBytes = S * 8u;
   fence_proxy_async();  // earlier fragment reads of the buffer come before the new copies
   __syncwarp();
-  if (lane == 0) mbar_arrive_expect_tx(sg.bar, __popc(need) * (PAIR ? 2u : 1u) * kBucketBytes);
+  if (lane == 0) mbar_arrive_expect_tx(sg.bar, __popc(need) * kBucketBytes);
   __syncwarp();
-  if (!PAIR) {
-    if ((need >> lane) & 1u)
-      bulk_g2s(sg.buf + lane * S, v.buckets + static_cast<uint64_t>(x1) * S, kBucketBytes, sg.bar);
-  } else {
-    constexpr int BO = kPairWords / (2 * S);
-#pragma unroll
-    for (int k = 0; k < (2 * BO + 31) / 32; ++k) {
-      const int bi = lane + 32 * k;
-      const int op = o0 + ((bi >> 1) & (BO - 1));
-      const uint32_t y1 = __shfl_sync(kFull, x1, op & 31);
-      const uint32_t y2 = __shfl_sync(kFull, x2, op & 31);
-      if (bi < 2 * BO && ((need >> op) & 1u))
-        bulk_g2s(sg.buf + bi * S, v.buckets + static_cast<uint64_t>((bi & 1) ? y2 : y1) * S,
-                 kBucketBytes, sg.bar);
-    }
-  }
-}
-
-// Waits (bounded, warp-wide) for the copies of the round issued last.
-// A limit below 16 polls without suspending (mbarrier.test_wait), so that a
-// test can make the wait give up while the copies are certainly in flight.
-__device__ __forceinline__ bool stage_wait(const View& v, Stage& sg, int lane) {
+  if ((need >> lane) & 1u)
+    bulk_g2s(sg.buf + lane * S, v.buckets + static_cast<uint64_t>(x) * S, kBucketBytes, sg.bar);
   bool ok = false;
   if (v.stage_spin_limit < 16) {
     for (uint32_t it = 0; it < v.stage_spin_limit && !ok; ++it) ok = mbar_test_wait(sg.bar, sg.phase);
@@ -329,7 +419,7 @@ __device__ __forceinline__ bool stage_wait(const View& v, Stage& sg, int lane) {
     for (uint32_t it = 0; it < v.stage_spin_limit && !ok; ++it) ok = mbar_try_wait(sg.bar, sg.phase);
   }
   sg.phase ^= 1u;
-  if (__any_sync(kFull, !ok)) {  // never expected
+  if (__any_sync(kFull, !ok)) {
     sg.dead = true;
     if (lane == 0) atomicOr(&v.ctrl->err, kErrTimeout);
     return false;
@@ -337,292 +427,74 @@ __device__ __forceinline__ bool stage_wait(const View& v, Stage& sg, int lane) {
   return true;
 }
 
-// The same round through the load/store path: the lanes of a group of L = S/2
-// copy one bucket with 16-byte cp.async each, so one warp instruction moves
-// 32 / L whole buckets, coalesced exactly as the direct probe loads them.
-// stage_wait_lsu() then waits for the warp's copies (cp.async.wait_group)
-// and syncs the warp.  No registers hold the data and no spin loop waits.
-template <int S, bool PAIR>
-__device__ __forceinline__ void stage_issue_lsu(const View& v, Stage& sg, unsigned need, int o0,
-                                                uint32_t x1, uint32_t x2, int lane) {
-  constexpr int L = Geo<S>::L, Q = Geo<S>::Q;  // lanes per bucket, buckets per instruction
-  constexpr int NB = PAIR ? 2 * (kPairWords / (2 * S)) : 32;  // buckets per round
-  const int q = lane / L, ql = lane % L;
-  __syncwarp();  // earlier reads of the buffer by any lane come first
-#pragma unroll 4
-  for (int r = 0; r < NB / Q; ++r) {
-    const int bi = Q * r + q;                  // buffer bucket of this lane group
-    const int op = PAIR ? o0 + (bi >> 1) : bi;  // its op
-    const uint32_t y1 = __shfl_sync(kFull, x1, op & 31);
-    const uint32_t y2 = PAIR ? __shfl_sync(kFull, x2, op & 31) : 0u;
-    const uint32_t b = (PAIR && (bi & 1)) ? y2 : y1;
-    if ((need >> op) & 1u)
-      cp_async16(sg.buf + bi * S + 2 * ql, v.buckets + static_cast<uint64_t>(b) * S + 2 * ql);
-  }
-  cp_async_commit();
-}
-__device__ __forceinline__ void stage_wait_lsu() {
-  cp_async_wait_all();
-  __syncwarp();
-}
+// Where an op's key was found.
+struct Hit {
+  uint64_t word;
+  uint32_t b, slot;
+  bool ok;
+};
 
-// A staged round in two halves, so that a caller can do other work while the
-// copies are in flight: stage_begin() issues them on the path chosen for the
-// bucket width, stage_end() waits (false: the wait gave up, see stage_wait).
-template <int S, bool PAIR>
-__device__ __forceinline__ void stage_begin(const View& v, Stage& sg, unsigned need, int o0,
-                                            uint32_t x1, uint32_t x2, int lane) {
-  if (S == 16 ? HIVE_STAGE_LSU_S16 : HIVE_STAGE_LSU_S32)
-    stage_issue_lsu<S, PAIR>(v, sg, need, o0, x1, x2, lane);
-  else
-    stage_issue<S, PAIR>(v, sg, need, o0, x1, x2, lane);
-}
+// The op's staged bucket `myb`, scanned by its own lane with swizzled 16-byte
+// reads (the eight lanes of a shared-memory wavefront read eight different
+// bank groups).
 template <int S>
-__device__ __forceinline__ bool stage_end(const View& v, Stage& sg, int lane) {
-  if (S == 16 ? HIVE_STAGE_LSU_S16 : HIVE_STAGE_LSU_S32) {
-    stage_wait_lsu();
-    return true;
+__device__ __forceinline__ void scan_staged(const uint64_t* sbuf, int lane, uint32_t myb,
+                                            uint32_t key, Hit& h) {
+  constexpr int NP = S / 2;
+  const uint64_t* B = sbuf + lane * S;
+  int ms = -1;
+#pragma unroll 8
+  for (int k = 0; k < NP; ++k) {
+    const int f = (k + lane) & (NP - 1);
+    uint64_t a, b;
+    lds_frag(B + 2 * f, a, b);
+    if (key_of(a) == key) ms = 2 * f;
+    if (key_of(b) == key) ms = 2 * f + 1;
   }
-  return stage_wait(v, sg, lane);
+  if (ms >= 0) h = Hit{B[ms], myb, static_cast<uint32_t>(ms), true};
 }
 
-template <int S, bool PAIR>
-__device__ __forceinline__ bool stage_round(const View& v, Stage& sg, unsigned need, int o0,
-                                            uint32_t x1, uint32_t x2, int lane) {
-  stage_begin<S, PAIR>(v, sg, need, o0, x1, x2, lane);
-  return stage_end<S>(v, sg, lane);
-}
-
-// One probe round over the 32 ops of a warp.  `need` has bit j set when op j
-// (held by lane j, its home lane) must read bucket `myb` this round.  Load u
-// (u = 0..3) of lane group q (L lanes) reads the bucket of op Q*u + q of the
-// current group of 4Q ops, 16 bytes (two slots) per lane, so each load
-// instruction probes Q buckets.  Match-and-elect (Section III-F) is a ballot per load: the lowest
-// matching lane of a group is the winner, and one shuffle per load hands the
-// matched value to every home lane, which then reads its own op's outcome out
-// of the warp-uniform ballots.  A home lane that must update the matched slot
-// (erase, replace) does the single CAS itself: the expected word is
-// (value << 32 | key), both of which it now holds.
-template <int MODE, int S>
-__device__ __forceinline__ void probe(const View& v, unsigned need, uint32_t myb, uint32_t key,
-                                      uint32_t val, uint32_t op, int lane, bool& done,
-                                      uint8_t& st, uint32_t& outv, uint32_t& fcnt,
-                                      uint32_t& fslot, LaneCounters& cnt) {
-  constexpr bool kIns = (MODE == kModeInsert || MODE == kModeMixed);
-  constexpr int L = Geo<S>::L, Q = Geo<S>::Q;
-  constexpr unsigned LM = Geo<S>::LM;
-  constexpr int G = 4 * Q;   // ops per group
-  constexpr int NG = 32 / G; // groups per warp
-  constexpr unsigned GM = (G >= 32) ? 0xFFFFFFFFu : ((1u << G) - 1u);
-  const int q = lane / L;
-  const int ql = lane % L;
-  const int my_g = lane / G, my_j = lane % G, my_u = my_j / Q, my_q = my_j % Q;
-#pragma unroll 1
-  for (int g = 0; g < NG; ++g) {
-    const unsigned gneed = (need >> (G * g)) & GM;
-    if (!gneed) continue;
-    uint64_t wa[4], wb[4];
-    uint32_t kq[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int src = G * g + Q * u + q;
-      const uint32_t bq = __shfl_sync(kFull, myb, src);
-      kq[u] = __shfl_sync(kFull, key, src);
-      if ((gneed >> (Q * u + q)) & 1u) {
-        const uint64_t* p = v.buckets + static_cast<uint64_t>(bq) * S + 2 * ql;
-        if (MODE == kModeFind)
-          ld_frag_ro(p, wa[u], wb[u]);
-        else
-          ld_frag(p, wa[u], wb[u]);
-      } else {
-        wa[u] = kEmptyWord;
-        wb[u] = kEmptyWord;
-      }
+// The slots `m1` of bucket b1, then `m2` of b2, whose tags match the key:
+// reads their words until one holds the key, starting where the key's own
+// claim would have (so the slot that holds it tends to come before a false
+// match).
+template <int S, bool RO>
+__device__ __forceinline__ void check_words(const View& v, uint32_t b1, uint32_t b2, uint32_t m1,
+                                            uint32_t m2, uint32_t key, Hit& h) {
+  const uint32_t rot = claim_rot(key);
+  while (m1 | m2) {
+    const bool in1 = m1 != 0;
+    const uint32_t b = in1 ? b1 : b2;
+    const uint32_t p = pick_slot(in1 ? m1 : m2, rot);
+    const uint32_t slot = slot_of(p);
+    const uint64_t w = ld_word<RO>(v.buckets + static_cast<uint64_t>(b) * S + slot);
+    if (key_of(w) == key) {
+      h = Hit{w, b, slot, true};
+      return;
     }
-    unsigned my_m = 0, my_mh = 0, my_el = 0, my_eh = 0;
-    uint32_t got = 0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const bool lo = key_of(wa[u]) == kq[u];
-      const bool hi = key_of(wb[u]) == kq[u];
-      const unsigned m = __ballot_sync(kFull, lo || hi);
-      const unsigned mh = (MODE != kModeFind) ? __ballot_sync(kFull, hi) : 0u;
-      const unsigned el = kIns ? __ballot_sync(kFull, wa[u] == kEmptyWord) : 0u;
-      const unsigned eh = kIns ? __ballot_sync(kFull, wb[u] == kEmptyWord) : 0u;
-      const uint32_t cv = lo ? val_of(wa[u]) : val_of(wb[u]);
-      const unsigned hm = (m >> (L * my_q)) & LM;
-      const uint32_t x = __shfl_sync(kFull, cv, L * my_q + (hm ? __ffs(hm) - 1 : 0));
-      if (u == my_u) {
-        my_m = m;
-        my_mh = mh;
-        my_el = el;
-        my_eh = eh;
-        got = x;
-      }
-    }
-    if (my_g == g && ((gneed >> my_j) & 1u)) {
-      const unsigned hm = (my_m >> (L * my_q)) & LM;
-      if (hm) {
-        done = true;
-        const uint32_t opk = MODE == kModeMixed
-                                 ? op
-                                 : (MODE == kModeFind ? OP_FIND
-                                                      : (MODE == kModeErase ? OP_ERASE : OP_INSERT));
-        if (opk == OP_FIND) {
-          outv = got;
-          st = ST_FOUND;
-          done = true;
-        } else {
-          const uint32_t w = __ffs(hm) - 1;
-          const uint32_t slot = 2 * w + ((my_mh >> (L * my_q + w)) & 1u);
-          uint64_t* sp = v.buckets + static_cast<uint64_t>(myb) * S + slot;
-          const uint64_t cur = pack(key, got);
-          if (opk == OP_ERASE) {
-            // Algorithm 4: CAS the slot to EMPTY, then publish the free bit.
-            // The atomicOr issues only after the CAS has returned, so a
-            // claimer that sees the bit finds the slot already EMPTY.
-            if (atomicCAS(ull(sp), cur, kEmptyWord) == cur) {
-              atomicOr(v.masks + myb, 1u << slot);
-              cnt.size_delta -= 1;
-              st = ST_ERASED;
-            } else {
-              st = ST_ERASED;
-              cnt.contract = true;
-            }
-          } else {
-            // Algorithm 1: CAS the cached word to the new pair.
-            if (atomicCAS(ull(sp), cur, pack(key, val)) == cur) {
-              cnt.replaced += 1;
-              st = ST_REPLACED;
-            } else {
-              st = ST_REPLACED;
-              cnt.contract = true;
-            }
-          }
-        }
-      } else if (kIns) {
-        const unsigned ev = (my_el >> (L * my_q)) & LM;
-        const unsigned od = (my_eh >> (L * my_q)) & LM;
-        fcnt = __popc(ev) + __popc(od);
-        const uint32_t se = ev ? 2u * (__ffs(ev) - 1) : S;
-        const uint32_t so = od ? 2u * (__ffs(od) - 1) + 1u : S;
-        fslot = se < so ? se : so;
-      }
-    }
+    if (in1)
+      m1 &= ~(1u << p);
+    else
+      m2 &= ~(1u << p);
   }
 }
 
-// Insert batches probe both candidate buckets of an op in one round: the two
-// lane groups of a pair read the BitHash1 and the BitHash2 bucket of one op,
-// P = Q / 2 ops per load instruction.  An insert of a new key needs both
-// buckets anyway (step 1 must rule the key out of both before step 2 claims),
-// so this halves the dependent probe rounds of the find-shaped probe() above.
-// Covers the op groups of ops [o0, o1).  On a match the home lane replaces the value with one CAS
-// (Algorithm 1); otherwise it records each bucket's free count and first
-// free slot.
-template <int S>
-__device__ __forceinline__ void probe_pair(const View& v, unsigned need, uint32_t b1,
-                                           uint32_t b2, uint32_t key, uint32_t val, int lane,
-                                           bool& done, uint8_t& st, uint32_t& f1, uint32_t& s1,
-                                           uint32_t& f2, uint32_t& s2, LaneCounters& cnt, int o0,
-                                           int o1) {
-  constexpr int L = Geo<S>::L, Q = Geo<S>::Q;
-  constexpr unsigned LM = Geo<S>::LM;
-  constexpr int P = Q / 2;    // ops per load instruction
-  constexpr int G = 4 * P;    // ops per group
-  constexpr unsigned GM = (1u << G) - 1u;
-  constexpr unsigned PM = (2 * L >= 32) ? 0xFFFFFFFFu : ((1u << (2 * L)) - 1u);
-  const int q = lane / L;
-  const int ql = lane % L;
-  const int my_g = lane / G, my_j = lane % G, my_u = my_j / P, my_p = my_j % P;
-#pragma unroll 1
-  for (int g = o0 / G; g < o1 / G; ++g) {
-    const unsigned gneed = (need >> (G * g)) & GM;
-    if (!gneed) continue;
-    uint64_t wa[4], wb[4];
-    uint32_t kq[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int src = G * g + P * u + (q >> 1);
-      const uint32_t q1 = __shfl_sync(kFull, b1, src);
-      const uint32_t q2 = __shfl_sync(kFull, b2, src);
-      kq[u] = __shfl_sync(kFull, key, src);
-      if ((gneed >> (P * u + (q >> 1))) & 1u) {
-        const uint64_t* p = v.buckets + static_cast<uint64_t>((q & 1) ? q2 : q1) * S + 2 * ql;
-        ld_frag(p, wa[u], wb[u]);
-      } else {
-        wa[u] = kEmptyWord;
-        wb[u] = kEmptyWord;
-      }
-    }
-    unsigned my_m = 0, my_mh = 0, my_el = 0, my_eh = 0;
-    uint32_t got = 0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const bool lo = key_of(wa[u]) == kq[u];
-      const bool hi = key_of(wb[u]) == kq[u];
-      const unsigned m = __ballot_sync(kFull, lo || hi);
-      const unsigned mh = __ballot_sync(kFull, hi);
-      const unsigned el = __ballot_sync(kFull, wa[u] == kEmptyWord);
-      const unsigned eh = __ballot_sync(kFull, wb[u] == kEmptyWord);
-      const uint32_t cv = lo ? val_of(wa[u]) : val_of(wb[u]);
-      const unsigned pm = (m >> (2 * L * my_p)) & PM;
-      const uint32_t x = __shfl_sync(kFull, cv, 2 * L * my_p + (pm ? __ffs(pm) - 1 : 0));
-      if (u == my_u) {
-        my_m = m;
-        my_mh = mh;
-        my_el = el;
-        my_eh = eh;
-        got = x;
-      }
-    }
-    if (my_g == g && ((gneed >> my_j) & 1u)) {
-      const int base = 2 * L * my_p;
-      const unsigned pm = (my_m >> base) & PM;
-      if (pm) {
-        // the lowest matching lane: the BitHash1 group wins when both match
-        done = true;
-        st = ST_REPLACED;
-        const uint32_t w = __ffs(pm) - 1;
-        const uint32_t slot = 2 * (w % L) + ((my_mh >> (base + w)) & 1u);
-        const uint32_t b = w < static_cast<uint32_t>(L) ? b1 : b2;
-        uint64_t* sp = v.buckets + static_cast<uint64_t>(b) * S + slot;
-        const uint64_t cur = pack(key, got);
-        if (atomicCAS(ull(sp), cur, pack(key, val)) == cur)
-          cnt.replaced += 1;
-        else
-          cnt.contract = true;
-      } else {
-        const unsigned e0 = (my_el >> base) & LM, o_0 = (my_eh >> base) & LM;
-        const unsigned e1 = (my_el >> (base + L)) & LM, o_1 = (my_eh >> (base + L)) & LM;
-        f1 = __popc(e0) + __popc(o_0);
-        f2 = __popc(e1) + __popc(o_1);
-        const uint32_t a0 = e0 ? 2u * (__ffs(e0) - 1) : S;
-        const uint32_t a1 = o_0 ? 2u * (__ffs(o_0) - 1) + 1u : S;
-        const uint32_t c0 = e1 ? 2u * (__ffs(e1) - 1) : S;
-        const uint32_t c1 = o_1 ? 2u * (__ffs(o_1) - 1) + 1u : S;
-        s1 = a0 < a1 ? a0 : a1;
-        s2 = c0 < c1 ? c0 : c1;
-      }
-    }
-  }
-}
-
-// An erase or replace CAS issued by a staged probe round, checked only at the
-// end of the chunk, so that its round trip overlaps the rounds and claims
-// after it (an op updates at most one slot, so one record per lane).
+// An erase or replace CAS issued by a probe, checked only at the end of the
+// chunk, so that its round trip overlaps the claims after it (an op updates
+// at most one slot, so one record per lane).
 struct PendCas {
   uint64_t cur, old;
   uint32_t b, slot, kind;  // kind: 0 none, 1 erase, 2 replace
 };
 
+template <int S>
 __device__ __forceinline__ void resolve_cas(const View& v, const PendCas& pc, LaneCounters& cnt) {
   if (pc.kind == 0) return;
   const bool ok = pc.old == pc.cur;
   if (pc.kind == 1) {
-    // Algorithm 4: the free bit is published once the CAS has emptied the slot
+    // Algorithm 4: the slot is published as free once the CAS has emptied it
     if (ok) {
-      atomicOr(v.masks + pc.b, 1u << pc.slot);
+      free_tag<S>(v, pc.b, pc.slot, key_of(pc.cur));
       cnt.size_delta -= 1;
     } else {
       cnt.contract = true;
@@ -635,167 +507,26 @@ __device__ __forceinline__ void resolve_cas(const View& v, const PendCas& pc, La
   }
 }
 
-// A single-bucket probe round on staged buckets, one op per lane: lane j
-// scans buffer bucket j (its op's bucket this round) with swizzled 16-byte
-// reads, as scan_staged_pair() below does for both buckets, and acts on a
-// match exactly as probe() does.  `mask` is the bucket's free mask, read while
-// the copies were in flight (insert-capable modes), for the claim.
+// Acts on a hit: a find takes the value; an erase or replace issues its CAS
+// (Algorithm 4 / Algorithm 1).
 template <int MODE, int S>
-__device__ __forceinline__ void scan_staged_one(const View& v, const uint64_t* sbuf, int lane,
-                                                uint32_t myb, uint32_t key, uint32_t val,
-                                                uint32_t op, uint32_t mask, bool& done,
-                                                uint8_t& st, uint32_t& outv, uint32_t& fcnt,
-                                                uint32_t& fslot, PendCas& pc) {
-  constexpr bool kIns = (MODE == kModeInsert || MODE == kModeMixed);
-  constexpr int NP = S / 2;
-  const uint64_t* B = sbuf + lane * S;
-  int ms = -1;
-#pragma unroll 8
-  for (int k = 0; k < NP; ++k) {
-    const int f = (k + lane) & (NP - 1);
-    uint64_t a, b;
-    lds_frag(B + 2 * f, a, b);
-    if (key_of(a) == key) ms = 2 * f;
-    if (key_of(b) == key) ms = 2 * f + 1;
-  }
-  if (ms >= 0) {
-    done = true;
-    const uint64_t cur = B[ms];
-    const uint32_t opk = MODE == kModeMixed
-                             ? op
-                             : (MODE == kModeFind ? OP_FIND
-                                                  : (MODE == kModeErase ? OP_ERASE : OP_INSERT));
-    if (opk == OP_FIND) {
-      outv = val_of(cur);
-      st = ST_FOUND;
-    } else {
-      uint64_t* sp = v.buckets + static_cast<uint64_t>(myb) * S + ms;
-      st = opk == OP_ERASE ? ST_ERASED : ST_REPLACED;
-      pc.old = atomicCAS(ull(sp), cur, opk == OP_ERASE ? kEmptyWord : pack(key, val));
-      pc.cur = cur;
-      pc.b = myb;
-      pc.slot = ms;
-      pc.kind = opk == OP_ERASE ? 1u : 2u;
-    }
-  } else if (kIns) {
-    fcnt = __popc(mask);
-    fslot = mask ? __ffs(mask) - 1 : S;
-  }
-}
-
-// A single-bucket probe round, staged when the warp has a live stage.
-// CLAIM: the op may claim a slot in this kernel, so the round also reads the
-// bucket's free mask.
-template <int MODE, int S, bool CLAIM>
-__device__ __forceinline__ void probe_round(const View& v, unsigned need, uint32_t myb,
-                                            uint32_t key, uint32_t val, uint32_t op, int lane,
-                                            bool& done, uint8_t& st, uint32_t& outv,
-                                            uint32_t& fcnt, uint32_t& fslot, LaneCounters& cnt,
-                                            Stage* sg, PendCas& pc) {
-  if (sg && !sg->dead) {
-    const bool mine = (need >> lane) & 1u;
-    const uint32_t m = (CLAIM && mine && op == OP_INSERT) ? ld_relaxed32(v.masks + myb) : 0u;
-    if (stage_round<S, false>(v, *sg, need, 0, myb, 0, lane)) {
-      if (mine)
-        scan_staged_one<MODE, S>(v, sg->buf, lane, myb, key, val, op, m, done, st, outv, fcnt,
-                                 fslot, pc);
-      return;
-    }
-  }
-  probe<MODE, S>(v, need, myb, key, val, op, lane, done, st, outv, fcnt, fslot, cnt);
-}
-
-// The paired insert round on staged buckets, one op per lane.  With both
-// candidate buckets of its op in shared memory, a lane scans them itself:
-// S / 2 16-byte fragment reads per bucket, starting at fragment (op mod S / 2)
-// so that the eight lanes of a shared-memory wavefront read eight different
-// bank groups, and one compare per slot against the op's key (a key sits in
-// at most one slot of the table).  Free counts and first free slots come from
-// the EMPTY words of the staged buckets (HIVE_FREE_FROM_STAGE), or from the
-// free masks read while the copies are in flight: either way they only steer
-// the claim, whose fetch_and result is the authority (a slot claimed and not
-// yet written still reads EMPTY; the claim then retries on the returned mask).  This
-// takes a few instructions per slot where the warp-wide match-and-elect takes
-// several ballots per 16-byte fragment, and the staged kernel is bound by
-// instruction issue, not by memory.
-template <int S>
-__device__ __forceinline__ void scan_staged_pair(const View& v, const uint64_t* sbuf, int jj,
-                                                 uint32_t b1, uint32_t b2, uint32_t key,
-                                                 uint32_t val, uint32_t m1, uint32_t m2,
-                                                 bool& done, uint8_t& st, uint32_t& f1,
-                                                 uint32_t& s1, uint32_t& f2, uint32_t& s2,
-                                                 LaneCounters& cnt) {
-  constexpr int NP = S / 2;  // 16-byte fragments per bucket
-  const uint64_t* B = sbuf + 2 * jj * S;
-  int ms = -1;  // matched word in [0, 2S): bucket ms / S, slot ms % S
-  uint32_t em[2] = {0u, 0u};  // EMPTY slots of each bucket
-#pragma unroll
-  for (int which = 0; which < 2; ++which) {
-#pragma unroll 8
-    for (int k = 0; k < NP; ++k) {
-      const int f = (k + jj) & (NP - 1);
-      uint64_t a, b;
-      lds_frag(B + which * S + 2 * f, a, b);
-      if (key_of(a) == key) ms = which * S + 2 * f;
-      if (key_of(b) == key) ms = which * S + 2 * f + 1;
-      if (HIVE_FREE_FROM_STAGE)
-        em[which] |= ((key_of(a) == kEmptyKey ? 1u : 0u) | (key_of(b) == kEmptyKey ? 2u : 0u))
-                     << (2 * f);
-    }
-  }
-  if (HIVE_FREE_FROM_STAGE) {
-    m1 = em[0];
-    m2 = em[1];
-  }
-  if (ms >= 0) {
-    done = true;
-    st = ST_REPLACED;
-    const uint64_t cur = B[ms];
-    const uint32_t b = ms < S ? b1 : b2;
-    uint64_t* sp = v.buckets + static_cast<uint64_t>(b) * S + (ms & (S - 1));
-    if (atomicCAS(ull(sp), cur, pack(key, val)) == cur)
-      cnt.replaced += 1;
-    else
-      cnt.contract = true;
+__device__ __forceinline__ void act_on(const View& v, const Hit& h, uint32_t key, uint32_t val,
+                                       uint32_t op, uint8_t& st, uint32_t& outv, PendCas& pc) {
+  const uint32_t opk = MODE == kModeMixed
+                           ? op
+                           : (MODE == kModeFind ? OP_FIND
+                                                : (MODE == kModeErase ? OP_ERASE : OP_INSERT));
+  if (opk == OP_FIND) {
+    outv = val_of(h.word);
+    st = ST_FOUND;
   } else {
-    f1 = __popc(m1);
-    f2 = __popc(m2);
-    s1 = m1 ? __ffs(m1) - 1 : S;
-    s2 = m2 ? __ffs(m2) - 1 : S;
-  }
-}
-
-// The paired insert round, staged in batches of 512 / S ops when the warp has
-// a live stage.
-template <int S>
-__device__ __forceinline__ void probe_pair_round(const View& v, unsigned need, uint32_t b1,
-                                                 uint32_t b2, uint32_t key, uint32_t val,
-                                                 int lane, bool& done, uint8_t& st, uint32_t& f1,
-                                                 uint32_t& s1, uint32_t& f2, uint32_t& s2,
-                                                 LaneCounters& cnt, Stage* sg) {
-  constexpr int BO = kPairWords / (2 * S);
-  constexpr unsigned BM = (BO >= 32) ? 0xFFFFFFFFu : ((1u << BO) - 1u);
-  if (sg) {
-    // free masks of both buckets, in flight beside the copies (unless the
-    // staged words give the free slots)
-    const bool mine = !HIVE_FREE_FROM_STAGE && ((need >> lane) & 1u);
-    const uint32_t m1 = mine ? ld_relaxed32(v.masks + b1) : 0u;
-    const uint32_t m2 = mine ? ld_relaxed32(v.masks + b2) : 0u;
-#pragma unroll 1
-    for (int o0 = 0; o0 < 32; o0 += BO) {
-      const unsigned bneed = need & (BM << o0);
-      if (!bneed) continue;
-      if (sg->dead || !stage_round<S, true>(v, *sg, bneed, o0, b1, b2, lane)) {
-        probe_pair<S>(v, need & ~((1u << o0) - 1u), b1, b2, key, val, lane, done, st, f1, s1, f2,
-                      s2, cnt, o0, 32);
-        return;
-      }
-      if ((bneed >> lane) & 1u)
-        scan_staged_pair<S>(v, sg->buf, lane - o0, b1, b2, key, val, m1, m2, done, st, f1, s1,
-                            f2, s2, cnt);
-    }
-  } else {
-    probe_pair<S>(v, need, b1, b2, key, val, lane, done, st, f1, s1, f2, s2, cnt, 0, 32);
+    uint64_t* sp = v.buckets + static_cast<uint64_t>(h.b) * S + h.slot;
+    st = opk == OP_ERASE ? ST_ERASED : ST_REPLACED;
+    pc.old = atomicCAS(ull(sp), h.word, opk == OP_ERASE ? kEmptyWord : pack(key, val));
+    pc.cur = h.word;
+    pc.b = h.b;
+    pc.slot = h.slot;
+    pc.kind = opk == OP_ERASE ? 1u : 2u;
   }
 }
 
@@ -910,8 +641,7 @@ __device__ __forceinline__ OpIn load_in(const OpPtrs& a, uint32_t c, uint64_t n,
 // holds with one atomicAdd when the next round's entries would not fit.  One
 // counter serves the whole list; an atomicAdd on that one word per warp round
 // queued behind each other in L2 and held up every warp's memory pipeline.
-// (The bulk kernel's own eviction hand-off is rare enough to append directly;
-// a mixed batch's new keys go to fixed per-chunk places, see run_chunk.)
+// (The bulk kernel's own eviction hand-off is rare enough to append directly.)
 // A buffer of `cap` entries takes 2 * cap shared-memory words: cap packed
 // words, then cap op indices and cap segment tags (u32).
 struct OvfBuf {
@@ -989,20 +719,22 @@ __device__ __forceinline__ void ovf_flush_block(const List& ovf, OvfBuf& ob, int
   ob.n = 0;
 }
 
-// Ops [32c, 32c + 32) of a batch of n ops on the table of `v`.  Full-bucket
-// inserts go to the overflow list, tagged with `seg` when the list keeps tags.
-// `pre` holds the chunk's inputs when the caller loaded them ahead.
-// DEFER (mixed batches): inserts of absent keys do not claim here.  Chunk c
-// writes them to list places [32c, 32c + k) and k to ovf.chunk_cnt[c], with no
-// atomic, and k_claim places them once every find, erase and replace of the
-// batch has run.
+// Ops [32c, 32c + 32) of a batch of n ops on the table of `v`, one op per
+// lane.  Full-bucket inserts go to the overflow list, tagged with `seg` when
+// the list keeps tags.  `pre` holds the chunk's inputs when the caller loaded
+// them ahead.
+// DEFER (mixed batches): inserts of absent keys do not claim here.  They join
+// the list through the warp's buffer `ob`, and k_claim places them once every
+// find, erase and replace of the batch has run; their status is written here
+// already (INSERTED, which only a full table changes).
 template <int MODE, int S, bool DEFER = false>
 __device__ __forceinline__ void run_chunk(const View& v, uint32_t stash_n, const OpPtrs a,
                                           uint32_t c, uint64_t n, const List ovf, uint32_t seg,
                                           LaneCounters& cnt, int lane, Stage* sg = nullptr,
-                                          const OpIn* pre = nullptr) {
+                                          const OpIn* pre = nullptr, OvfBuf* ob = nullptr) {
   constexpr bool kIns = (MODE == kModeInsert || MODE == kModeMixed);
   constexpr bool kClaim = kIns && !DEFER;
+  constexpr bool kRO = MODE == kModeFind;
   const uint32_t i = (c << 5) + lane;
   const bool valid = i < n;
   const OpIn in = pre ? *pre : load_in<MODE>(a, c, n, lane);
@@ -1011,30 +743,50 @@ __device__ __forceinline__ void run_chunk(const View& v, uint32_t stash_n, const
   const bool live = valid && !reserved;
   cnt.reserved |= reserved;
 
-  const uint32_t b1 = lh_bucket(bithash1(key), v.M, v.p);
-  const uint32_t b2 = lh_bucket(bithash2(key), v.M, v.p);
-  bool done = !live;
+  const Cand cd = cand_of(v, key);
+  const uint32_t b1 = cd.b1, b2 = cd.b2;
   uint8_t st = reserved ? ST_RESERVED : ST_NOT_FOUND;
   uint32_t outv = 0;
-  uint32_t f1 = 0, s1 = S, f2 = 0, s2 = S;
   PendCas pc{0, 0, 0, 0, 0};
+  Hit h{0, 0, 0, false};
+  TagVec<S> t1, t2;
+  bool have_tags = false;
 
-  // Probe the BitHash1 bucket of every op, then the BitHash2 bucket of the
-  // ops still unresolved (Section IV-B: WCME over the d = 2 candidates).
-  unsigned need = __ballot_sync(kFull, !done);
-  if (MODE == kModeInsert) {
-    cnt.probes += 2 * __popc(need);
-    if (need) probe_pair_round<S>(v, need, b1, b2, key, val, lane, done, st, f1, s1, f2, s2, cnt, sg);
-  } else {
-    cnt.probes += __popc(need);
-    if (need)
-      probe_round<MODE, S, kClaim>(v, need, b1, key, val, op, lane, done, st, outv, f1, s1, cnt,
-                                   sg, pc);
-    need = __ballot_sync(kFull, !done);
-    cnt.probes += __popc(need);
-    if (need)
-      probe_round<MODE, S, kClaim>(v, need, b2, key, val, op, lane, done, st, outv, f2, s2, cnt,
-                                   sg, pc);
+  bool probed = false;
+  if (sg && !sg->dead) {
+    // whole buckets, staged: the BitHash1 bucket, then the BitHash2 bucket
+    // of the ops still open
+    unsigned need = __ballot_sync(kFull, live);
+    probed = need == 0 || stage_round<S>(v, *sg, need, b1, lane);
+    if (probed) {
+      if (live) scan_staged<S>(sg->buf, lane, b1, key, h);
+      cnt.probes += __popc(need);
+      need = __ballot_sync(kFull, live && !h.ok);
+      probed = need == 0 || stage_round<S>(v, *sg, need, b2, lane);
+      if (probed) {
+        if (live && !h.ok) scan_staged<S>(sg->buf, lane, b2, key, h);
+        cnt.probes += __popc(need);
+      }
+    }
+  }
+  if (!probed) {
+    // by tags: both buckets' tags in one round trip, then the matching words
+    if (live) {
+      t1 = ld_tags<S, kRO>(v, b1);
+      t2 = ld_tags<S, kRO>(v, b2);
+      have_tags = true;
+      const uint32_t t4 = tag_of(key) * 0x01010101u;
+      const uint32_t m1 = tag_match<S>(t1, t4);
+      const uint32_t m2 = b2 != b1 ? tag_match<S>(t2, t4) : 0u;
+      check_words<S, kRO>(v, b1, b2, m1, m2, key, h);
+    }
+    cnt.probes += __popc(__ballot_sync(kFull, live));
+    cnt.probes += __popc(__ballot_sync(kFull, live && (MODE == kModeInsert || !h.ok || h.b != b1)));
+  }
+  bool done = !live;
+  if (h.ok) {
+    done = true;
+    act_on<MODE, S>(v, h, key, val, op, st, outv, pc);
   }
 
   // The stash (Section IV-A step 4) holds keys that found no bucket room.
@@ -1067,19 +819,15 @@ __device__ __forceinline__ void run_chunk(const View& v, uint32_t stash_n, const
 
   // Step 2: claim-then-commit for absent keys.
   bool to_ovf = false;
-  if (DEFER && kIns && !done && op == OP_INSERT) {
+  if (DEFER && !done && op == OP_INSERT) {
     to_ovf = true;  // k_claim places it
-  } else if (kIns && !done && op == OP_INSERT) {
-    const uint64_t word = pack(key, val);
-    const bool first1 = v.placement ? (f1 > 0) : (f1 >= f2);
-    const uint32_t tb = first1 ? b1 : b2, ts = first1 ? s1 : s2;
-    const uint32_t ob = first1 ? b2 : b1, os = first1 ? s2 : s1;
-    bool placed = false;
-    if (f1 + f2 > 0) {
-      placed = claim_store<S>(v, tb, ts, word);
-      if (!placed && ob != tb) placed = claim_store<S>(v, ob, os, word);
+    st = ST_INSERTED;
+  } else if (kClaim && !done && op == OP_INSERT) {
+    if (!have_tags) {
+      t1 = ld_tags<S, false>(v, b1);
+      t2 = ld_tags<S, false>(v, b2);
     }
-    if (placed) {
+    if (place_from<S>(v, b1, b2, t1, t2, pack(key, val))) {
       done = true;
       st = ST_INSERTED;
       cnt.size_delta += 1;
@@ -1090,19 +838,14 @@ __device__ __forceinline__ void run_chunk(const View& v, uint32_t stash_n, const
     }
   }
 
-  resolve_cas(v, pc, cnt);
+  resolve_cas<S>(v, pc, cnt);
 
   // Hand full-bucket inserts to the eviction kernel (steps 3-4).
-  if (kIns) {
+  if constexpr (DEFER) {
+    ovf_put(ovf, *ob, lane, to_ovf, pack(key, val), i, 0);
+  } else if (kIns) {
     const unsigned om = __ballot_sync(kFull, to_ovf);
-    if (DEFER) {
-      if (to_ovf) {
-        const unsigned r = (c << 5) + __popc(om & ((1u << lane) - 1u));
-        ovf.words[r] = pack(key, val);
-        ovf.idx[r] = i;
-      }
-      if (lane == 0) ovf.chunk_cnt[c] = static_cast<uint8_t>(__popc(om));
-    } else if (om) {
+    if (om) {
       const int leader = __ffs(om) - 1;
       unsigned base = 0;
       if (lane == leader) base = atomicAdd(ovf.count, static_cast<unsigned>(__popc(om)));
@@ -1121,189 +864,212 @@ __device__ __forceinline__ void run_chunk(const View& v, uint32_t stash_n, const
       __stcs(a.vals_out + i, outv);
       if (a.found) a.found[i] = st == ST_FOUND ? 1 : 0;
     } else {
-      if (a.status && !to_ovf) a.status[i] = st;
+      if (a.status && (DEFER || !to_ovf)) a.status[i] = st;
       if (MODE == kModeMixed && a.vals_out) __stcs(a.vals_out + i, outv);
     }
   }
 }
 
-// Resident blocks of THREADS threads per SM a bulk kernel is built for: the
-// warps per SM of the 256-thread shape (at least one block), which sets the
-// register budget of each shape.
-__host__ __device__ constexpr int ops_min_blocks(int mode, int S, int threads) {
-  return ((staged_mode(mode, S) ? staged_min_blocks(mode, S) : HIVE_OPS_MIN_BLOCKS) * kOpsThreads /
-              threads >
-          0)
-             ? (staged_mode(mode, S) ? staged_min_blocks(mode, S) : HIVE_OPS_MIN_BLOCKS) *
-                   kOpsThreads / threads
-             : 1;
+// Resident 256-thread blocks per SM a bulk kernel is built for, which sets its
+// register budget (other shapes: the same warps per SM, at least one block).
+// Kernels that claim need about 64 registers (five blocks of 48 spill: bulk
+// load 4.36 -> 5.00 ms); the others run at six (lookups on a 2^26-slot table
+// 1.455 -> 1.441 ms, erases on an L2-resident one 24.6 -> 21.2 us).
+__host__ __device__ constexpr int ops_min_blocks(int mode, bool defer, bool staged, int threads) {
+  const int b256 = staged ? 3 : (mode == kModeInsert || (mode == kModeMixed && !defer)) ? 4
+                            : mode == kModeMixed                                        ? 5
+                                                                                        : 6;
+  return b256 * kOpsThreads / threads > 0 ? b256 * kOpsThreads / threads : 1;
 }
+
+constexpr int kDeferBuf = 128;  // entries of each warp's buffer of new keys
 
 // DEFER (mixed batches): the new keys are claimed by k_claim afterwards.
 // THREADS: the block shape (128, 256 or 512 threads; a tuning knob).
-template <int MODE, int S, bool DEFER, int THREADS>
-__global__ void __launch_bounds__(THREADS, ops_min_blocks(MODE, S, THREADS))
-    k_ops(View v, OpPtrs a, uint64_t n, List ovf, int prefetch_masks) {
-  // claims and erases update free masks at random; a large batch first asks
-  // L2 for the whole mask array in sequential pieces
-  if (prefetch_masks) prefetch_l2_grid(v.masks, static_cast<uint64_t>(v.nb) * sizeof(uint32_t));
+// STAGED: whole buckets staged in shared memory instead of tags (tables with
+// a stage_wait_limit).
+template <int MODE, int S, bool DEFER, int THREADS, bool STAGED>
+__global__ void __launch_bounds__(THREADS, ops_min_blocks(MODE, DEFER, STAGED, THREADS))
+    k_ops(View v, OpPtrs a, uint64_t n, List ovf, int prefetch_tags) {
+  // probes read tags at random; a large batch first asks L2 for the whole tag
+  // array in sequential pieces
+  if (prefetch_tags) prefetch_l2_grid(v.tags, static_cast<uint64_t>(v.nb) * S);
   const int lane = threadIdx.x & 31;
   // n < 2^32 per call, so chunk and op indices fit 32 bits
   const uint32_t warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t nchunks = static_cast<uint32_t>((n + 31) >> 5);
   const uint32_t stash_n = v.ctrl->stash_n;
+  __shared__ uint64_t sums[(THREADS / 32) * 8];
+  // new keys of a deferring batch gather here, so that the list is written in
+  // long runs with one atomic per kDeferBuf entries
+  __shared__ __align__(16) uint64_t defer_smem[DEFER ? (THREADS / 32) * 2 * kDeferBuf : 1];
+  OvfBuf ob{};
+  if constexpr (DEFER)
+    ob = ovf_buf_init(defer_smem + (threadIdx.x >> 5) * 2 * kDeferBuf, kDeferBuf);
   LaneCounters cnt;
-  if (staged_mode(MODE, S)) {
-    // bucket reads staged in shared memory
+  // inputs are loaded one chunk ahead, so their latency hides behind the
+  // current chunk's probes and claims
+  OpIn nxt{};
+  if (warp0 < nchunks) nxt = load_in<MODE>(a, warp0, n, lane);
+  if constexpr (STAGED) {
     extern __shared__ __align__(16) uint64_t ops_smem[];
-    Stage sg = stage_init(ops_smem, threadIdx.x >> 5, lane, warp_smem_words(MODE, S));
-    // inputs are loaded one chunk ahead, so their latency hides behind the
-    // current chunk's probes and claims
-    OpIn nxt{};
-    if (warp0 < nchunks) nxt = load_in<MODE>(a, warp0, n, lane);
+    Stage sg = stage_init(ops_smem, threadIdx.x >> 5, lane, stage_warp_words(S));
     for (uint32_t c = warp0; c < nchunks; c += nwarps) {
       const OpIn cur = nxt;
       if (c + nwarps < nchunks) nxt = load_in<MODE>(a, c + nwarps, n, lane);
-      run_chunk<MODE, S, DEFER>(v, stash_n, a, c, n, ovf, 0, cnt, lane, &sg, &cur);
+      run_chunk<MODE, S, DEFER>(v, stash_n, a, c, n, ovf, 0, cnt, lane, &sg, &cur, &ob);
     }
     stage_drain(sg);
-    // the staging buffers are free now (a dead stage's late copies have landed
-    // or stage_drain gave up on them, and then its first words stay unused)
-    if (!__syncthreads_or(sg.dead ? 1 : 0))
-      flush_counters_block(v, cnt, lane, sg.buf, ops_smem + 2, warp_smem_words(MODE, S));
-    else
-      flush_counters(v, cnt, lane);
   } else {
-    for (uint32_t c = warp0; c < nchunks; c += nwarps)
-      run_chunk<MODE, S, DEFER>(v, stash_n, a, c, n, ovf, 0, cnt, lane);
-    flush_counters(v, cnt, lane);
+    for (uint32_t c = warp0; c < nchunks; c += nwarps) {
+      const OpIn cur = nxt;
+      if (c + nwarps < nchunks) nxt = load_in<MODE>(a, c + nwarps, n, lane);
+      run_chunk<MODE, S, DEFER>(v, stash_n, a, c, n, ovf, 0, cnt, lane, nullptr, &cur, &ob);
+    }
   }
+  if constexpr (DEFER) ovf_flush_block(ovf, ob, lane);
+  flush_counters_block(v, cnt, lane, sums + (threadIdx.x >> 5) * 8, sums, 8);
+}
+
+// Find batches (Section IV-B).  A warp takes G runs of 32 consecutive ops at a
+// time, one op per lane and run, with the keys loaded one run ahead.  The
+// found flags of G = 4 runs leave as one 4-byte store per lane, assembled from
+// the runs' ballots: with the outputs in host memory, whole lines cross the
+// CPU-GPU link where G = 1 sends 32-byte pieces (2^22 ops: 145 -> 137 us; the
+// link alone takes 115 us for their 21 MB of results).
+//
+// What bounds it (one GB300, 2^26 lookups, half of them hits, 2^26 slots at
+// 95%, S = 32): DRAM serves about 41 G random lines/s, and a hit needs one.
+// 3.68 ms when each lookup read whole 256-byte buckets, 1.44 ms by tags; the
+// floor is 0.82 ms for the 2^25 hits, and false tag matches (30 of 255 per
+// bucket examined) make the rest.  In an L2-resident table the dependent
+// chain key -> tags -> word is the cost: 2^20 slots, 1.7 M lookups 77 -> 27 us.
+template <int S, int THREADS, int G>
+__global__ void __launch_bounds__(THREADS, ops_min_blocks(kModeFind, false, false, THREADS))
+    k_find(View v, const uint32_t* __restrict__ keys, uint64_t n, uint32_t* __restrict__ vals_out,
+           uint8_t* __restrict__ found, int prefetch_tags) {
+  if (prefetch_tags) prefetch_l2_grid(v.tags, static_cast<uint64_t>(v.nb) * S);
+  const int lane = threadIdx.x & 31;
+  const uint32_t warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  const uint32_t ngroups = static_cast<uint32_t>((n + 32 * G - 1) / (32 * G));
+  const uint32_t stash_n = v.ctrl->stash_n;
+  const bool wide = G == 4 && (reinterpret_cast<uintptr_t>(found) & 3) == 0;
+  __shared__ uint64_t sums[(THREADS / 32) * 8];
+  LaneCounters cnt;
+  uint32_t nxt = kEmptyKey;
+  {
+    const uint64_t i = static_cast<uint64_t>(warp0) * G * 32 + lane;
+    if (i < n) nxt = __ldcs(keys + i);
+  }
+  for (uint32_t g = warp0; g < ngroups; g += nwarps) {
+    uint32_t fb[G];
+    const uint64_t base = static_cast<uint64_t>(g) * G * 32;
+    const bool whole = base + 32 * G <= n;
+#pragma unroll 1
+    for (int j = 0; j < G; ++j) {
+      const uint32_t key = nxt;
+      const uint64_t i = base + 32 * j + lane;
+      {  // the next run's keys: of this group, or the first of the warp's next one
+        const uint64_t k = j + 1 < G ? i + 32 : i + (static_cast<uint64_t>(nwarps) * G - (G - 1)) * 32;
+        nxt = k < n ? __ldcs(keys + k) : kEmptyKey;
+      }
+      const bool valid = i < n;
+      const bool live = valid && key < kReservedKeyMin;
+      cnt.reserved |= valid && !live;
+      const Cand cd = cand_of(v, key);
+      Hit h{0, 0, 0, false};
+      if (live) {
+        const TagVec<S> t1 = ld_tags<S, true>(v, cd.b1);
+        const TagVec<S> t2 = ld_tags<S, true>(v, cd.b2);
+        const uint32_t t4 = tag_of(key) * 0x01010101u;
+        check_words<S, true>(v, cd.b1, cd.b2, tag_match<S>(t1, t4),
+                             cd.b2 != cd.b1 ? tag_match<S>(t2, t4) : 0u, key, h);
+      }
+      cnt.probes += __popc(__ballot_sync(kFull, live)) +
+                    __popc(__ballot_sync(kFull, live && (!h.ok || h.b != cd.b1)));
+      if (live && !h.ok && stash_n) {
+        uint32_t pos;
+        cnt.stash_lookups += 1;
+        if (stash_find(v, stash_n, key, pos)) {
+          h.word = ld_relaxed64(v.stash_kv + pos);
+          h.ok = key_of(h.word) == key;
+        }
+      }
+      const uint32_t b = __ballot_sync(kFull, h.ok);
+#pragma unroll
+      for (int k = 0; k < G; ++k)
+        if (j == k) fb[k] = b;
+      if (valid) {
+        __stcs(vals_out + i, h.ok ? val_of(h.word) : 0u);
+        if (found && !(wide && whole)) __stcs(found + i, static_cast<uint8_t>(h.ok));
+      }
+    }
+    if (G == 4 && found && wide && whole) {
+      // lane l: the flags of ops 4 l .. 4 l + 3 of the group, four bits of
+      // run l / 8's ballot, one to each byte
+      uint32_t b = fb[0];
+#pragma unroll
+      for (int k = 1; k < G; ++k)
+        if ((lane >> 3) == k) b = fb[k];
+      const uint32_t nib = (b >> ((4 * lane) & 31)) & 0xFu;
+      __stcs(reinterpret_cast<uint32_t*>(found + base) + lane, (nib * 0x00204081u) & 0x01010101u);
+    }
+  }
+  flush_counters_block(v, cnt, lane, sums + (threadIdx.x >> 5) * 8, sums, 8);
 }
 
 // Step 2 for the new keys of a mixed batch (WABC, Section III-E), after the
-// bulk kernel has run every find, erase and replace of the batch: the slots
-// those erases freed are then visible to the claims.  The bulk kernel left
-// chunk c's new keys at list places [32c, 32c + chunk_cnt[c]).  A warp takes 32
-// chunks at a time, scans their counts and spreads their entries over its
-// lanes, one item per lane: hash, read both free masks, claim the predicted
-// slot of the emptier bucket with one atomicAnd (the other bucket next),
-// store the word.  Nothing moves or erases a word meanwhile, so the claim
-// publishes with a plain store.  Items whose two buckets are both full go to
-// `out` for eviction (steps 3-4).
+// bulk kernel has run every find, erase and replace of the batch and listed
+// them in `in`: the slots those erases freed are then visible to the claims.
+// One item per lane: hash, read the tags of both buckets, claim a free slot of
+// the emptier bucket with one CAS (the other bucket next), store the word.
+// Nothing moves or erases a word meanwhile, so the claim publishes with a
+// plain store.  Items whose two buckets are both full go to `out` for
+// eviction (steps 3-4).
 constexpr int kClaimThreads = 256;
-constexpr int kClaimBuf = 256;  // entries of each warp's buffer of full-bucket items
-#ifndef HIVE_CLAIM_PREFETCH_SLOT
-#define HIVE_CLAIM_PREFETCH_SLOT 0
-#endif
-#ifndef HIVE_CLAIM_ILP
-#define HIVE_CLAIM_ILP 4
-#endif
-constexpr int kClaimIlp = HIVE_CLAIM_ILP;  // items per lane in flight at once
+constexpr int kClaimBuf = 128;  // entries of each warp's buffer of full-bucket items
 template <int S>
-__global__ void __launch_bounds__(kClaimThreads)
-    k_claim(View v, List in, uint32_t nchunks, List out, uint8_t* __restrict__ status,
-            int prefetch_masks) {
-  // The claims read the free masks at random: a batch with as many new keys
-  // as a fraction of the buckets is served faster from L2 after one
-  // sequential fetch of the whole mask array than by a DRAM sector per read.
-  if (prefetch_masks) prefetch_l2_grid(v.masks, static_cast<uint64_t>(v.nb) * sizeof(uint32_t));
+__global__ void __launch_bounds__(kClaimThreads, 4) k_claim(View v, List in, List out) {
   __shared__ __align__(16) uint64_t claim_smem[(kClaimThreads / 32) * 2 * kClaimBuf];
   const int lane = threadIdx.x & 31;
   OvfBuf ob = ovf_buf_init(claim_smem + (threadIdx.x >> 5) * 2 * kClaimBuf, kClaimBuf);
   LaneCounters cnt;
-  const uint32_t ngroups = (nchunks + 31) >> 5;
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  // chunk counts are loaded one group ahead
-  uint32_t k_next = (g < ngroups && (g << 5) + lane < nchunks) ? in.chunk_cnt[(g << 5) + lane] : 0u;
-  for (; g < ngroups; g += nwarps) {
-    const uint32_t k = k_next;
-    const uint32_t gn = g + nwarps;
-    k_next = (gn < ngroups && (gn << 5) + lane < nchunks) ? in.chunk_cnt[(gn << 5) + lane] : 0u;
-    uint32_t incl = k;  // inclusive prefix sum of the 32 counts
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t t = __shfl_up_sync(kFull, incl, d);
-      if (lane >= d) incl += t;
+  const uint32_t total = *in.count;
+  const uint32_t step = gridDim.x * blockDim.x;
+  uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  // entries are loaded one step ahead of their claims
+  uint64_t word_n = i < total ? __ldcs(in.words + i) : kEmptyWord;
+  uint32_t idx_n = i < total ? __ldcs(in.idx + i) : kNoOp;
+  for (; i - lane < total; i += step) {
+    const uint64_t word = word_n;
+    const uint32_t idx = idx_n;
+    const bool valid = i < total;
+    TagVec<S> t1, t2;
+    Cand cd{0, 0};
+    if (valid) {
+      cd = cand_of(v, key_of(word));
+      t1 = ld_tags<S, false>(v, cd.b1);
+      t2 = ld_tags<S, false>(v, cd.b2);
     }
-    const uint32_t excl = incl - k;
-    const uint32_t total = __shfl_sync(kFull, incl, 31);
-    for (uint32_t t0 = 0; t0 < total; t0 += 32 * kClaimIlp) {
-      uint64_t word[kClaimIlp];
-      uint32_t idx[kClaimIlp], b1[kClaimIlp], b2[kClaimIlp], m1[kClaimIlp], m2[kClaimIlp];
-#pragma unroll
-      for (int u = 0; u < kClaimIlp; ++u) {
-        const uint32_t t = t0 + 32 * u + lane;
-        // chunk j of entry t: the first j whose inclusive sum passes t
-        uint32_t j = 0;
-#pragma unroll
-        for (uint32_t step = 16; step; step >>= 1) {
-          const uint32_t e = __shfl_sync(kFull, incl, j + step - 1);
-          if (e <= t) j += step;
-        }
-        const uint32_t ex = __shfl_sync(kFull, excl, j & 31);
-        const uint32_t pos = (((g << 5) + j) << 5) + (t - ex);
-        word[u] = t < total ? in.words[pos] : kEmptyWord;
-        idx[u] = t < total ? in.idx[pos] : kNoOp;
-      }
-#pragma unroll
-      for (int u = 0; u < kClaimIlp; ++u) {
-        const uint32_t key = key_of(word[u]);
-        b1[u] = lh_bucket(bithash1(key), v.M, v.p);
-        b2[u] = lh_bucket(bithash2(key), v.M, v.p);
-        const bool valid = t0 + 32 * u + lane < total;
-        m1[u] = valid ? ld_relaxed32(v.masks + b1[u]) : 0u;
-        m2[u] = valid ? ld_relaxed32(v.masks + b2[u]) : 0u;
-      }
-      // first claim attempt of every item, then the outcomes (a failed
-      // attempt retries on the returned mask, then on the other bucket)
-      uint32_t old[kClaimIlp], bit[kClaimIlp];
-#pragma unroll
-      for (int u = 0; u < kClaimIlp; ++u) {
-        const uint32_t f1 = __popc(m1[u]), f2 = __popc(m2[u]);
-        const bool first1 = v.placement ? (f1 > 0) : (f1 >= f2);
-        if (!first1) {
-          const uint32_t tb = b1[u], tm = m1[u];
-          b1[u] = b2[u];
-          m1[u] = m2[u];
-          b2[u] = tb;
-          m2[u] = tm;
-        }
-        bit[u] = m1[u] ? (1u << (__ffs(m1[u]) - 1)) : 0u;
-#if HIVE_CLAIM_PREFETCH_SLOT
-        if (bit[u])
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(v.buckets + static_cast<uint64_t>(b1[u]) * S +
-                                                          (__ffs(bit[u]) - 1)));
-#endif
-        old[u] = bit[u] ? atomicAnd(v.masks + b1[u], ~bit[u]) : 0u;
-      }
-#pragma unroll
-      for (int u = 0; u < kClaimIlp; ++u) {
-        const bool valid = t0 + 32 * u + lane < total;
-        bool placed = false, to_ovf = false;
-        if (valid) {
-          if (old[u] & bit[u]) {
-            st_relaxed64(v.buckets + static_cast<uint64_t>(b1[u]) * S + (__ffs(bit[u]) - 1),
-                         word[u]);
-            placed = true;
-          } else {
-            if (bit[u]) placed = claim_store<S>(v, b1[u], old[u] ? __ffs(old[u]) - 1 : S, word[u]);
-            if (!placed && b2[u] != b1[u] && m2[u])
-              placed = claim_store<S>(v, b2[u], __ffs(m2[u]) - 1, word[u]);
-          }
-          if (placed) {
-            cnt.size_delta += 1;
-            cnt.claimed += 1;
-            if (status && idx[u] != kNoOp) status[idx[u]] = ST_INSERTED;
-          } else {
-            to_ovf = true;
-            cnt.overflowed += 1;
-          }
-        }
-        ovf_put(out, ob, lane, to_ovf, word[u], idx[u], 0);
+    const uint64_t j = static_cast<uint64_t>(i) + step;
+    if (j < total) {
+      word_n = __ldcs(in.words + j);
+      idx_n = __ldcs(in.idx + j);
+    }
+    bool to_ovf = false;
+    if (valid) {
+      if (place_from<S>(v, cd.b1, cd.b2, t1, t2, word)) {
+        cnt.size_delta += 1;
+        cnt.claimed += 1;
+      } else {
+        to_ovf = true;
+        cnt.overflowed += 1;
       }
     }
+    ovf_put(out, ob, lane, to_ovf, word, idx, 0);
+    if (j - lane >= total) break;  // also keeps i from wrapping
   }
   ovf_flush_block(out, ob, lane);
   flush_counters_block(v, cnt, lane, ob.words, claim_smem, 2 * kClaimBuf);
@@ -1417,10 +1183,8 @@ __device__ __forceinline__ void overflow_item(const View& v, uint64_t word0, uin
   // here find both buckets still full
   const uint64_t w0 = ld_relaxed64(v.buckets + static_cast<uint64_t>(b1) * S + gl);
   if (gl == 0) {
-    // both free masks in one round trip; claim where a bit is free
-    const uint32_t m1 = ld_relaxed32(v.masks + b1);
-    const uint32_t m2 = ld_relaxed32(v.masks + b2);
-    if ((m1 && claim_pub<S>(v, b1, word0, m1)) || (b2 != b1 && m2 && claim_pub<S>(v, b2, word0, m2))) {
+    // the tags of both buckets in one round trip; claim where a slot is free
+    if (place_new<S>(v, b1, b2, word0)) {
       outcome = 1;
       ++oc.claim;
     } else {
@@ -1441,21 +1205,31 @@ __device__ __forceinline__ void overflow_item(const View& v, uint64_t word0, uin
       // Look ahead: each lane checks whether the word in its slot could move
       // to its other candidate bucket without a further eviction.
       const uint64_t w = r == 0 ? w0 : ld_relaxed64(v.buckets + static_cast<uint64_t>(b) * S + gl);
-      uint32_t am = 0;  // free mask of this word's other candidate bucket
+      // a free slot of this word's other candidate bucket (32: none), and
+      // the tag word it lies in
+      uint32_t ap = 32, aw = 0;
       if (w != kEmptyWord) {
         const uint32_t k = key_of(w);
         const uint32_t a1 = lh_bucket(bithash1(k), v.M, v.p);
         const uint32_t a2 = lh_bucket(bithash2(k), v.M, v.p);
         const uint32_t alt = (a1 == b) ? a2 : a1;
-        if (alt != b) am = ld_relaxed32(v.masks + alt);
+        if (alt != b) {
+          const TagVec<S> ta = ld_tags<S, false>(v, alt);
+          const uint32_t fm = free_slots<S>(ta);
+          if (fm) {
+            ap = pick_slot(fm, claim_rot(k));
+            aw = tag_sel<S>(ta, ap & 7u);
+          }
+        }
       }
-      const unsigned gm = group_ballot(am != 0u);
+      const unsigned gm = group_ballot(ap < 32u);
       const unsigned occ = group_ballot(w != kEmptyWord);
       const bool has_empty = occ != kGroupBits;
       int res = 0;  // 0: evicted `victim`, 1: placed, 2: lock wait gave up, 3: redo the round
       uint64_t victim = kEmptyWord;
       // victim: an occupied slot whose word can move on at once, else an
-      // occupied slot picked by rotation (never an EMPTY one, see claim_pub)
+      // occupied slot picked by rotation (never an EMPTY one, see
+      // claim_in_word; occupied slots stay occupied here)
       uint32_t vs = S;
       if (gm) {
         vs = __ffs(gm) - 1;
@@ -1465,7 +1239,8 @@ __device__ __forceinline__ void overflow_item(const View& v, uint64_t word0, uin
             start ? (((occ >> start) | (occ << (S - start))) & kGroupBits) : occ;
         vs = (start + __ffs(rot) - 1) & (S - 1);
       }
-      const uint32_t vmask = __shfl_sync(gmask, am, vs & (S - 1), S);
+      const uint32_t vp = __shfl_sync(gmask, ap, vs & (S - 1), S);
+      const uint32_t vw = __shfl_sync(gmask, aw, vs & (S - 1), S);
       if (gl == 0) {
         ++oc.rounds;
         if (!lock_bucket(v, b)) {
@@ -1473,15 +1248,17 @@ __device__ __forceinline__ void overflow_item(const View& v, uint64_t word0, uin
           ++oc.to;
         } else {
           ++oc.locks;
-          if (has_empty && claim_pub<S>(v, b, cur)) {
+          if (has_empty && claim_bucket<S>(v, b, cur, claim_rot(key_of(cur)))) {
             res = 1;
+            unlock_bucket(v, b);
           } else if (vs >= S) {
             res = 3;  // every slot claimed but not yet published: look again
+            unlock_bucket(v, b);
           } else {
             victim = atomicExch(ull(v.buckets + static_cast<uint64_t>(b) * S + vs), cur);
-            res = (victim == kEmptyWord) ? 1 : 0;
+            swap_tag<S>(v, b, vs, key_of(victim), key_of(cur));
+            unlock_swapped(v, b);
           }
-          unlock_bucket(v, b);
         }
       }
       res = __shfl_sync(gmask, res, 0, S);
@@ -1501,7 +1278,9 @@ __device__ __forceinline__ void overflow_item(const View& v, uint64_t word0, uin
       if (nb == b) break;  // both candidates are this bucket: no alternative
       b = nb;
       int ok = 0;
-      if (gl == 0) ok = claim_pub<S>(v, b, cur, vmask);
+      if (gl == 0)
+        ok = vp < 32u ? claim_in_word<S>(v, b, vp & 7u, vp >> 3, vw, tag_of(kc), cur)
+                      : claim_bucket<S>(v, b, cur, claim_rot(kc));
       if (__shfl_sync(gmask, ok, 0, S)) {
         placed = true;
         break;
@@ -1633,9 +1412,9 @@ __device__ __forceinline__ void transit_end(const View& v, uint32_t b) {
 // most one bucket lock at a time and waits for it a bounded number of
 // tries).  A chain is a run of dependent round trips, so carrying many at
 // once is what keeps the step short; a warp-wide chain left 31 lanes idle
-// per round trip.  The caller has already tried both free masks and holds a
-// stash reservation in `oc`.  Each round reads the bucket in hand 8 words at
-// a time with the free masks of those words' other buckets, and stops at the
+// per round trip.  The caller has already tried both buckets' tags and holds a
+// stash reservation in `oc`.  Each round reads the bucket in hand 4 words at
+// a time with the tags of those words' other buckets, and stops at the
 // first word that could move on at once (the victim); if none could, the
 // victim is the first occupied slot from a rotating start.  Under the bucket
 // lock the chain claims a free slot of the bucket for its word, or swaps the
@@ -1653,30 +1432,36 @@ __device__ int chain_lane(const View& v, uint64_t word0, uint32_t b1, OvfCounter
     uint64_t* B = v.buckets + static_cast<uint64_t>(b) * S;
     unsigned occ = 0;
     int vs = -1;
-    uint32_t vmask = 0;
+    uint32_t vp = 32, vw = 0;  // free slot of the victim's other bucket, and its tag word
 #pragma unroll 1
-    for (int f0 = 0; f0 < S; f0 += 8) {
-      uint64_t w[8];
+    for (int f0 = 0; f0 < S; f0 += 4) {
+      uint64_t w[4];
+      ld_frag(B + f0, w[0], w[1]);
+      ld_frag(B + f0 + 2, w[2], w[3]);
+      TagVec<S> ta[4];
+      bool can[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) ld_frag(B + f0 + 2 * q, w[2 * q], w[2 * q + 1]);
-      uint32_t am[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        am[k] = 0;
+      for (int k = 0; k < 4; ++k) {
+        can[k] = false;
         if (w[k] != kEmptyWord) {
           occ |= 1u << (f0 + k);
-          const uint32_t kk = key_of(w[k]);
-          const uint32_t a1 = lh_bucket(bithash1(kk), v.M, v.p);
-          const uint32_t a2 = lh_bucket(bithash2(kk), v.M, v.p);
-          const uint32_t alt = (a1 == b) ? a2 : a1;
-          if (alt != b) am[k] = ld_relaxed32(v.masks + alt);
+          const Cand a = cand_of(v, key_of(w[k]));
+          const uint32_t alt = (a.b1 == b) ? a.b2 : a.b1;
+          if (alt != b) {
+            ta[k] = ld_tags<S, false>(v, alt);
+            can[k] = true;
+          }
         }
       }
 #pragma unroll
-      for (int k = 7; k >= 0; --k)
-        if (am[k]) {
-          vs = f0 + k;
-          vmask = am[k];
+      for (int k = 3; k >= 0; --k)
+        if (can[k]) {
+          const uint32_t fm = free_slots<S>(ta[k]);
+          if (fm) {
+            vs = f0 + k;
+            vp = pick_slot(fm, claim_rot(key_of(w[k])));
+            vw = tag_sel<S>(ta[k], vp & 7u);
+          }
         }
       if (vs >= 0) break;
     }
@@ -1694,8 +1479,7 @@ __device__ int chain_lane(const View& v, uint64_t word0, uint32_t b1, OvfCounter
       ++oc.to;
     } else {
       ++oc.locks;
-      const uint32_t mb = ld_relaxed32(v.masks + b);
-      if (mb && claim_pub<S>(v, b, cur, mb)) {
+      if (claim_bucket<S>(v, b, cur, claim_rot(key_of(cur)))) {
         res = 1;
       } else if (vs < 0) {
         res = 3;
@@ -1708,6 +1492,7 @@ __device__ int chain_lane(const View& v, uint64_t word0, uint32_t b1, OvfCounter
           vb = lh_bucket(bithash1(key_of(wv)), v.M, v.p);
           transit_begin(v, vb);
           if (atomicCAS(ull(sp), wv, cur) == wv) {
+            swap_tag<S>(v, b, vs, key_of(wv), key_of(cur));
             res = 0;
           } else {
             transit_end(v, vb);
@@ -1715,7 +1500,10 @@ __device__ int chain_lane(const View& v, uint64_t word0, uint32_t b1, OvfCounter
           }
         }
       }
-      unlock_bucket(v, b);
+      if (res == 0)
+        unlock_swapped(v, b);
+      else
+        unlock_bucket(v, b);
     }
     // the word in hand now sits in b (placed or swapped in)
     if ((res == 0 || res == 1) && held != kNoOp) transit_end(v, held);
@@ -1734,7 +1522,10 @@ __device__ int chain_lane(const View& v, uint64_t word0, uint32_t b1, OvfCounter
     const uint32_t nb = (a1 == b) ? a2 : a1;
     if (nb == b) break;
     b = nb;
-    if (claim_pub<S>(v, b, cur, vmask)) {
+    // the free slot seen in the lookahead (only a guess: the victim may have
+    // been swapped meanwhile)
+    if (vp < 32u ? claim_in_word<S>(v, b, vp & 7u, vp >> 3, vw, tag_of(kc), cur)
+                 : claim_bucket<S>(v, b, cur, claim_rot(kc))) {
       transit_end(v, held);
       held = kNoOp;
       placed = true;
@@ -1768,8 +1559,8 @@ struct EvictQ {
 };
 
 // Runs the chains of the first min(n, 32) queued keys, one per lane, and
-// moves the rest to the front (warp-wide).  Each key first tries both free
-// masks again (slots may have been freed since); the keys still without room
+// moves the rest to the front (warp-wide).  Each key first tries both
+// buckets again (slots may have been freed since); the keys still without room
 // take a stash reservation for the warp's chains with one atomic, then run
 // their chains.
 template <int S>
@@ -1785,10 +1576,7 @@ __device__ void fused_drain(const View& v, EvictQ& q, uint8_t* status, const Lis
   const uint32_t b2 = lh_bucket(bithash2(key), v.M, v.p);
   int out = 0;  // 1 placed, 2 stashed, 3 no room
   if (has) {
-    const uint32_t m1 = ld_relaxed32(v.masks + b1);
-    const uint32_t m2 = ld_relaxed32(v.masks + b2);
-    if ((m1 && claim_pub<S>(v, b1, word, m1)) ||
-        (b2 != b1 && m2 && claim_pub<S>(v, b2, word, m2))) {
+    if (place_new<S>(v, b1, b2, word)) {
       out = 1;
       ++oc.claim;
     }
@@ -1847,30 +1635,6 @@ __device__ void fused_drain(const View& v, EvictQ& q, uint8_t* status, const Lis
   q.n = rest;
 }
 
-// One single-bucket probe round of the single-kernel batch: bucket `myb` of
-// every op in `need` copied into the warp's staging buffer (buffer bucket j
-// for op j) with 16-byte cp.async through L2 only, then waited for.  Each
-// copy starts after the version read (an acquire) that precedes it in
-// program order, and the wait ends before the fence ahead of the second
-// version read.
-template <int S>
-__device__ __forceinline__ void fused_stage(const View& v, uint64_t* sbuf, unsigned need,
-                                            uint32_t myb, int lane) {
-  constexpr int L = Geo<S>::L, Q = Geo<S>::Q;
-  const int q = lane / L, ql = lane % L;
-  __syncwarp();  // earlier reads of the buffer by any lane come first
-#pragma unroll 4
-  for (int r = 0; r < 32 / Q; ++r) {
-    const int bi = Q * r + q;
-    const uint32_t y = __shfl_sync(kFull, myb, bi);
-    if ((need >> bi) & 1u)
-      cp_async16_cg(sbuf + bi * S + 2 * ql, v.buckets + static_cast<uint64_t>(y) * S + 2 * ql);
-  }
-  cp_async_commit();
-  cp_async_wait_all();
-  __syncwarp();
-}
-
 // Looks the op keys of the `need` lanes up in the stash words appended during
 // this kernel, [from, to) (warp-wide).  A lane that finds its key gets its
 // position in `pos` and returns true.
@@ -1916,7 +1680,7 @@ struct OpQ {
 template <int S>
 __device__ void fused_checked(const View& v, uint32_t stash_n, const OpPtrs& a, OpQ& rq,
                               EvictQ& q, const List& pend, int resizable, LaneCounters& cnt,
-                              OvfCounters& oc, unsigned& retries, int lane, uint64_t* sbuf) {
+                              OvfCounters& oc, unsigned& retries, int lane) {
   __syncwarp();
   const uint32_t mq = rq.n < 32 ? rq.n : 32u;
   const bool has = static_cast<uint32_t>(lane) < mq;
@@ -1946,7 +1710,6 @@ __device__ void fused_checked(const View& v, uint32_t stash_n, const OpPtrs& a, 
   bool done = !has;
   uint8_t st = ST_NOT_FOUND;
   uint32_t outv = 0;
-  uint32_t f1 = 0, s1 = S, f2 = 0, s2 = S;
   bool absent = false;  // a miss that survived the version check
   for (uint32_t attempt = 0;; ++attempt) {
     const bool active = !done && !absent;
@@ -1966,29 +1729,25 @@ __device__ void fused_checked(const View& v, uint32_t stash_n, const OpPtrs& a, 
     // the second version read catches)
     const uint32_t tail = ld_relaxed32(&v.ctrl->stash_tail);
     PendCas pc{0, 0, 0, 0, 0};
-    // the BitHash1 bucket of every open op
-    uint32_t m = (active && op == OP_INSERT) ? ld_relaxed32(v.masks + b1) : 0u;
-    cnt.probes += __popc(need);
-    fused_stage<S>(v, sbuf, need, b1, lane);
-    if (active)
-      scan_staged_one<kModeMixed, S>(v, sbuf, lane, b1, key, val, op, m, done, st, outv, f1, s1,
-                                     pc);
-    // the BitHash2 bucket of the ops still open
-    const unsigned need2 = __ballot_sync(kFull, active && !done);
-    if (need2) {
-      m = (active && !done && op == OP_INSERT) ? ld_relaxed32(v.masks + b2) : 0u;
-      cnt.probes += __popc(need2);
-      fused_stage<S>(v, sbuf, need2, b2, lane);
-      if (active && !done)
-        scan_staged_one<kModeMixed, S>(v, sbuf, lane, b2, key, val, op, m, done, st, outv, f2,
-                                       s2, pc);
+    Hit h{0, 0, 0, false};
+    if (active) {
+      const TagVec<S> t1 = ld_tags<S, false>(v, b1);
+      const TagVec<S> t2 = ld_tags<S, false>(v, b2);
+      const uint32_t t4 = tag_of(key) * 0x01010101u;
+      check_words<S, false>(v, b1, b2, tag_match<S>(t1, t4),
+                            b2 != b1 ? tag_match<S>(t2, t4) : 0u, key, h);
+    }
+    cnt.probes += __popc(need) + __popc(__ballot_sync(kFull, active && (!h.ok || h.b != b1)));
+    if (h.ok) {
+      done = true;
+      act_on<kModeMixed, S>(v, h, key, val, op, st, outv, pc);
     }
     // an erase or replace is done once its CAS has succeeded
     bool retry = false;
     if (pc.kind) {
       if (pc.old == pc.cur) {
         if (pc.kind == 1) {
-          atomicOr(v.masks + pc.b, 1u << pc.slot);
+          free_tag<S>(v, pc.b, pc.slot, key);
           cnt.size_delta -= 1;
         } else {
           cnt.replaced += 1;
@@ -2055,16 +1814,7 @@ __device__ void fused_checked(const View& v, uint32_t stash_n, const OpPtrs& a, 
   // keys that find both full join the eviction queue.
   bool to_evict = false;
   if (absent && op == OP_INSERT) {
-    const uint64_t word = pack(key, val);
-    const bool first1 = v.placement ? (f1 > 0) : (f1 >= f2);
-    const uint32_t tb = first1 ? b1 : b2, ts = first1 ? s1 : s2;
-    const uint32_t ob = first1 ? b2 : b1, os = first1 ? s2 : s1;
-    bool placed = false;
-    if (f1 + f2 > 0) {
-      placed = claim_pub<S>(v, tb, word, ts < S ? (1u << ts) : 0u);
-      if (!placed && ob != tb) placed = claim_pub<S>(v, ob, word, os < S ? (1u << os) : 0u);
-    }
-    if (placed) {
+    if (place_new<S>(v, b1, b2, pack(key, val))) {
       st = ST_INSERTED;
       cnt.size_delta += 1;
       cnt.claimed += 1;
@@ -2103,8 +1853,7 @@ __device__ __forceinline__ void run_chunk_fused(const View& v, uint32_t stash_n,
                                                 uint32_t c, uint64_t n, const OpIn& in,
                                                 const List pend, int resizable,
                                                 LaneCounters& cnt, OvfCounters& oc,
-                                                unsigned& retries, int lane, uint64_t* sbuf,
-                                                OpQ& rq, EvictQ& q) {
+                                                unsigned& retries, int lane, OpQ& rq, EvictQ& q) {
   const uint32_t i = (c << 5) + lane;
   const bool valid = i < n;
   const uint32_t op = in.op, key = in.key, val = in.val;
@@ -2117,27 +1866,24 @@ __device__ __forceinline__ void run_chunk_fused(const View& v, uint32_t stash_n,
   bool done = false;
   uint8_t st = reserved ? ST_RESERVED : ST_NOT_FOUND;
   uint32_t outv = 0;
-  uint32_t fc = 0, fs = S;  // unused: finds and erases claim nothing
   PendCas pc{0, 0, 0, 0, 0};
-  const unsigned need = __ballot_sync(kFull, open);
-  if (need) {
-    cnt.probes += __popc(need);
-    fused_stage<S>(v, sbuf, need, b1, lane);
-    if (open)
-      scan_staged_one<kModeMixed, S>(v, sbuf, lane, b1, key, val, op, 0u, done, st, outv, fc, fs,
-                                     pc);
-    const unsigned need2 = __ballot_sync(kFull, open && !done);
-    if (need2) {
-      cnt.probes += __popc(need2);
-      fused_stage<S>(v, sbuf, need2, b2, lane);
-      if (open && !done)
-        scan_staged_one<kModeMixed, S>(v, sbuf, lane, b2, key, val, op, 0u, done, st, outv, fc,
-                                       fs, pc);
-    }
+  Hit h{0, 0, 0, false};
+  if (open) {
+    const TagVec<S> t1 = ld_tags<S, false>(v, b1);
+    const TagVec<S> t2 = ld_tags<S, false>(v, b2);
+    const uint32_t t4 = tag_of(key) * 0x01010101u;
+    check_words<S, false>(v, b1, b2, tag_match<S>(t1, t4), b2 != b1 ? tag_match<S>(t2, t4) : 0u,
+                          key, h);
+  }
+  cnt.probes += __popc(__ballot_sync(kFull, open)) +
+                __popc(__ballot_sync(kFull, open && (!h.ok || h.b != b1)));
+  if (h.ok) {
+    done = true;
+    act_on<kModeMixed, S>(v, h, key, val, op, st, outv, pc);
   }
   if (pc.kind) {
     if (pc.old == pc.cur) {
-      atomicOr(v.masks + pc.b, 1u << pc.slot);  // erases only here
+      free_tag<S>(v, pc.b, pc.slot, key);  // erases only here
       cnt.size_delta -= 1;
     } else {
       done = false;
@@ -2159,31 +1905,24 @@ __device__ __forceinline__ void run_chunk_fused(const View& v, uint32_t stash_n,
     }
     rq.n += __popc(cm);
     if (rq.n >= 32)
-      fused_checked<S>(v, stash_n, a, rq, q, pend, resizable, cnt, oc, retries, lane, sbuf);
+      fused_checked<S>(v, stash_n, a, rq, q, pend, resizable, cnt, oc, retries, lane);
   }
 }
 
-// Shared-memory words per warp of the single-kernel batch: one staging round
-// (32 buckets), the checked-probe queue (2 kFusedQ words), then the eviction
-// queue (kFusedQ words and kFusedQ indices).
-__host__ __device__ constexpr int fused_warp_words(int S) {
-  return 32 * S + 3 * static_cast<int>(kFusedQ) + static_cast<int>(kFusedQ) / 2;
-}
-__host__ __device__ constexpr size_t fused_smem(int S) {
-  return static_cast<size_t>(kOpsThreads / 32) * 8u * fused_warp_words(S);
-}
+// Shared-memory words per warp of the single-kernel batch: the checked-probe
+// queue (2 kFusedQ words), then the eviction queue (kFusedQ words and kFusedQ
+// indices).
+constexpr int kFusedWarpWords = 3 * static_cast<int>(kFusedQ) + static_cast<int>(kFusedQ) / 2;
 
 template <int S>
 __global__ void __launch_bounds__(kOpsThreads, 3)
     k_fused(View v, OpPtrs a, uint64_t n, List pend, int resizable) {
-  extern __shared__ __align__(16) uint64_t fused_smem_words[];
+  __shared__ __align__(16) uint64_t fused_smem_words[(kOpsThreads / 32) * kFusedWarpWords];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
-  uint64_t* mine = fused_smem_words + static_cast<size_t>(wib) * fused_warp_words(S);
-  uint64_t* sbuf = mine;
-  OpQ rq{mine + 32 * S, mine + 32 * S + kFusedQ, 0};
-  EvictQ q{mine + 32 * S + 2 * kFusedQ, reinterpret_cast<uint32_t*>(mine + 32 * S + 3 * kFusedQ),
-           0};
+  uint64_t* mine = fused_smem_words + static_cast<size_t>(wib) * kFusedWarpWords;
+  OpQ rq{mine, mine + kFusedQ, 0};
+  EvictQ q{mine + 2 * kFusedQ, reinterpret_cast<uint32_t*>(mine + 3 * kFusedQ), 0};
   const uint32_t warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t nchunks = static_cast<uint32_t>((n + 31) >> 5);
@@ -2197,10 +1936,9 @@ __global__ void __launch_bounds__(kOpsThreads, 3)
   for (uint32_t c = warp0; c < nchunks; c += nwarps) {
     const OpIn cur = nxt;
     if (c + nwarps < nchunks) nxt = load_in<kModeMixed>(a, c + nwarps, n, lane);
-    run_chunk_fused<S>(v, stash_n, a, c, n, cur, pend, resizable, cnt, oc, retries, lane, sbuf,
-                       rq, q);
+    run_chunk_fused<S>(v, stash_n, a, c, n, cur, pend, resizable, cnt, oc, retries, lane, rq, q);
   }
-  while (rq.n) fused_checked<S>(v, stash_n, a, rq, q, pend, resizable, cnt, oc, retries, lane, sbuf);
+  while (rq.n) fused_checked<S>(v, stash_n, a, rq, q, pend, resizable, cnt, oc, retries, lane);
   while (q.n) fused_drain<S>(v, q, a.status, pend, resizable, oc, lane);
   // counters: one atomic per counter and block
   // (and the lanes' unused stash reservations go back in one atomic)
@@ -2217,7 +1955,7 @@ __global__ void __launch_bounds__(kOpsThreads, 3)
       if (lane == 0 && t) atomicAdd(&sum[k], t);
     }
   }
-  flush_counters_block(v, cnt, lane, sbuf, fused_smem_words, fused_warp_words(S));
+  flush_counters_block(v, cnt, lane, mine, fused_smem_words, kFusedWarpWords);
   if (threadIdx.x == 0) {
     OvfCounters b;
     b.claim = sum[0];
@@ -2276,6 +2014,7 @@ __device__ void maint_body(const View& v, uint64_t* smem) {
   if (threadIdx.x == 0) {  // the next call's op lists start empty
     c->ovf_n = 0;
     c->pend_n = 0;
+    c->defer_n = 0;
   }
   if (tail == sorted && !dirty) return;
 
@@ -2287,13 +2026,7 @@ __device__ void maint_body(const View& v, uint64_t* smem) {
     const uint32_t k = key_of(w);
     const uint32_t b1 = lh_bucket(bithash1(k), v.M, v.p);
     const uint32_t b2 = lh_bucket(bithash2(k), v.M, v.p);
-    const uint32_t m1 = ld_relaxed32(v.masks + b1);
-    bool ok = m1 && claim_store<S>(v, b1, __ffs(m1) - 1, w);
-    if (!ok) {
-      const uint32_t m2 = ld_relaxed32(v.masks + b2);
-      ok = m2 && claim_store<S>(v, b2, __ffs(m2) - 1, w);
-    }
-    if (ok) {
+    if (place_new<S>(v, b1, b2, w)) {
       v.stash_kv[j] = kEmptyWord;
       ++reins;
     }
@@ -2345,6 +2078,12 @@ __global__ void __launch_bounds__(kMaintThreads) k_maint(View v) {
 // Linear-hashing resize (Section IV-C)
 // ----------------------------------------------------------------------------
 
+// The tags of bucket b as bytes, slot by slot (one warp has the bucket to itself).
+template <int S>
+__device__ __forceinline__ uint8_t* tag_bytes(const View& v, uint32_t b) {
+  return reinterpret_cast<uint8_t*>(v.tags) + static_cast<uint64_t>(b) * S;
+}
+
 // Expansion: warp w splits bucket src0 + w into its partner src0 + w + half.
 // `v` carries the state after this launch.  A word leaves the source bucket
 // when neither candidate address equals the source under the new state; it
@@ -2365,14 +2104,13 @@ __device__ __forceinline__ void split_pair(const View& v, uint32_t src, uint32_t
   }
   const unsigned mm = __ballot_sync(kFull, mv);
   if (mv) {
-    db[__popc(mm & ((1u << lane) - 1u))] = word;
+    // the partner's slots past the movers stay EMPTY with tag 0, as every
+    // bucket outside [0, nb) is kept
+    const uint32_t r = __popc(mm & ((1u << lane) - 1u));
+    db[r] = word;
     sb[lane] = kEmptyWord;
-  }
-  if (lane == 0) {
-    constexpr uint32_t kValid = S >= 32 ? 0xFFFFFFFFu : ((1u << S) - 1u);
-    v.masks[src] |= mm;
-    const int nm = __popc(mm);
-    v.masks[dst] = nm >= 32 ? 0u : ((0xFFFFFFFFu << nm) & kValid);
+    tag_bytes<S>(v, dst)[r] = static_cast<uint8_t>(tag_of(key_of(word)));
+    tag_bytes<S>(v, src)[lane] = 0;
   }
 }
 
@@ -2395,7 +2133,8 @@ __global__ void __launch_bounds__(256) k_merge_excess(View v, uint32_t count) {
   const uint64_t word =
       lane < S ? v.buckets[static_cast<uint64_t>(high) * S + lane] : kEmptyWord;
   const int live = __popc(__ballot_sync(kFull, word != kEmptyWord));
-  const int fr = __popc(v.masks[low]);
+  const int fr =
+      __popc(__ballot_sync(kFull, lane < S && tag_bytes<S>(v, low)[lane & (S - 1)] == 0));
   if (lane == 0 && live > fr) atomicAdd(&v.ctrl->merge_excess, static_cast<unsigned>(live - fr));
 }
 
@@ -2416,13 +2155,15 @@ __global__ void __launch_bounds__(256) k_merge(View v, uint32_t count, List ovf)
   const bool live = word != kEmptyWord;
   const unsigned lm = __ballot_sync(kFull, live);
   const unsigned rank = __popc(lm & ((1u << lane) - 1u));
-  const uint32_t fr = v.masks[low];
+  const uint32_t fr =
+      __ballot_sync(kFull, lane < S && tag_bytes<S>(v, low)[lane & (S - 1)] == 0);
   const unsigned nfree = __popc(fr);
   const bool fits = live && rank < nfree;
   if (fits) {
     uint32_t m = fr;
     for (unsigned t = 0; t < rank; ++t) m &= m - 1u;
     lb[__ffs(m) - 1] = word;
+    tag_bytes<S>(v, low)[__ffs(m) - 1] = static_cast<uint8_t>(tag_of(key_of(word)));
   }
   const bool spill = live && !fits;
   const unsigned sm = __ballot_sync(kFull, spill);
@@ -2437,13 +2178,9 @@ __global__ void __launch_bounds__(256) k_merge(View v, uint32_t count, List ovf)
       ovf.idx[r] = kNoOp;
     }
   }
-  if (lane < S) hb[lane] = kEmptyWord;
-  if (lane == 0) {
-    const unsigned used = __popc(lm) < nfree ? __popc(lm) : nfree;
-    uint32_t m = fr;
-    for (unsigned t = 0; t < used; ++t) m &= m - 1u;
-    v.masks[low] = m;
-    v.masks[high] = S >= 32 ? 0xFFFFFFFFu : ((1u << S) - 1u);
+  if (lane < S) {
+    hb[lane] = kEmptyWord;
+    tag_bytes<S>(v, high)[lane] = 0;
   }
 }
 
@@ -2592,7 +2329,7 @@ __global__ void k_fill_u32(uint32_t* __restrict__ p, uint64_t n, uint32_t value)
 }
 
 // Launches a kernel on `s`, inside the table's persisting L2 window over the
-// free masks when it has one (a per-launch attribute: the stream is left as
+// slot tags when it has one (a per-launch attribute: the stream is left as
 // it was).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_in_window(const Launch& L, void (*kern)(KArgs...), unsigned grid,
@@ -2616,29 +2353,40 @@ cudaError_t launch_in_window(const Launch& L, void (*kern)(KArgs...), unsigned g
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
-template <int MODE, int S, bool DEFER, int THREADS>
+// Large batches fetch the tag array into L2 first: when the probes of a batch
+// would touch about every second bucket's tags or more.
+template <int S>
+int prefetch_rule(uint64_t n, const View& v) {
+  return n * 4 >= v.nb ? 1 : 0;
+}
+
+template <int MODE, int S, bool DEFER, int THREADS, bool STAGED = false>
 cudaError_t launch_ops_tt(const View& v, const OpPtrs& a, uint64_t n, List ovf, const Launch& L,
                           cudaStream_t s) {
   const uint64_t chunks = (n + 31) / 32;
   constexpr uint64_t warps_per_block = THREADS / 32;
   uint64_t blocks = (chunks + warps_per_block - 1) / warps_per_block;
-  constexpr bool kStaged = staged_mode(MODE, S);
-  const int per_sm = !kStaged ? L.ops_blocks_per_sm
-                     : (MODE == kModeInsert ? L.staged_blocks_per_sm : L.staged1_blocks_per_sm);
+  const int per_sm =
+      STAGED ? L.staged_blocks_per_sm : L.ops_blocks_per_sm[MODE + (DEFER ? 1 : 0)];
   const uint64_t cap = static_cast<uint64_t>(L.num_sms) * per_sm;
   if (blocks > cap) blocks = cap;
   if (blocks == 0) blocks = 1;
-  const size_t smem = kStaged ? stage_smem(MODE, S, THREADS) : 0;
-  if (MODE == kModeFind) {  // finds touch no free mask
-    k_ops<MODE, S, false, THREADS><<<static_cast<unsigned>(blocks), THREADS, smem, s>>>(v, a, n,
-                                                                                        ovf, 0);
+  const size_t smem = STAGED ? stage_smem(S, THREADS) : 0;
+  const int pf = prefetch_rule<S>(n, v);
+  if constexpr (MODE == kModeFind && !STAGED) {  // finds change no tag: no persisting window
+    // groups of four runs once every warp has at least four of them: with
+    // fewer, rounding to whole groups leaves warps idle (1.7 M ops on 7296
+    // warps: 33 us against 28)
+    if (chunks >= cap * warps_per_block * 16)
+      k_find<S, THREADS, 4><<<static_cast<unsigned>(cap), THREADS, 0, s>>>(
+          v, a.keys, n, a.vals_out, a.found, pf);
+    else
+      k_find<S, THREADS, 1><<<static_cast<unsigned>(blocks), THREADS, 0, s>>>(
+          v, a.keys, n, a.vals_out, a.found, pf);
     return cudaGetLastError();
-  }
-  // mask prefetch when the batch could touch about one mask sector per 16
-  // buckets or more
-  const int pf = n * 16 >= v.nb ? 1 : 0;
-  return launch_in_window(L, k_ops<MODE, S, DEFER, THREADS>, static_cast<unsigned>(blocks), THREADS,
-                          smem, s, v, a, n, ovf, pf);
+  } else
+  return launch_in_window(L, k_ops<MODE, S, DEFER, THREADS, STAGED>, static_cast<unsigned>(blocks),
+                          THREADS, smem, s, v, a, n, ovf, pf);
 }
 
 template <int MODE, int S, bool DEFER = false>
@@ -2646,6 +2394,9 @@ cudaError_t launch_ops_t(const View& v, const uint8_t* ops, const uint32_t* keys
                          const uint32_t* vals, uint64_t n, uint32_t* vals_out, uint8_t* found,
                          uint8_t* status, List ovf, const Launch& L, cudaStream_t s) {
   const OpPtrs a{ops, keys, vals, vals_out, found, status};
+  if constexpr (S == 32) {
+    if (L.staged) return launch_ops_tt<MODE, S, DEFER, 256, true>(v, a, n, ovf, L, s);
+  }
   switch (L.ops_threads) {
     case 128:
       return launch_ops_tt<MODE, S, DEFER, 128>(v, a, n, ovf, L, s);
@@ -2688,11 +2439,9 @@ cudaError_t launch_fused(const View& v, const uint8_t* ops, const uint32_t* keys
   if (blocks == 0) blocks = 1;
   const OpPtrs a{ops, keys, vals, vals_out, nullptr, status};
   if (v.S == 16)
-    k_fused<16><<<static_cast<unsigned>(blocks), kOpsThreads, fused_smem(16), s>>>(v, a, n, pend,
-                                                                                   resizable);
+    k_fused<16><<<static_cast<unsigned>(blocks), kOpsThreads, 0, s>>>(v, a, n, pend, resizable);
   else
-    k_fused<32><<<static_cast<unsigned>(blocks), kOpsThreads, fused_smem(32), s>>>(v, a, n, pend,
-                                                                                   resizable);
+    k_fused<32><<<static_cast<unsigned>(blocks), kOpsThreads, 0, s>>>(v, a, n, pend, resizable);
   return cudaGetLastError();
 }
 
@@ -2704,22 +2453,17 @@ cudaError_t launch_ops(int mode, const View& v, const uint8_t* ops, const uint32
   return launch_ops_s<32>(mode, v, ops, keys, vals, n, vals_out, found, status, ovf, L, s, defer);
 }
 
-cudaError_t launch_claim(const View& v, List in, uint64_t n, List out, uint8_t* status,
-                         const Launch& L, cudaStream_t s) {
+cudaError_t launch_claim(const View& v, List in, uint64_t n, List out, const Launch& L,
+                         cudaStream_t s) {
   if (!n) return cudaSuccess;
-  const uint32_t nchunks = static_cast<uint32_t>((n + 31) / 32);
-  uint64_t blocks = ((nchunks + 31) / 32 + kClaimThreads / 32 - 1) / (kClaimThreads / 32);
+  uint64_t blocks = (n + kClaimThreads - 1) / kClaimThreads;
   const uint64_t cap = static_cast<uint64_t>(L.num_sms) * L.claim_blocks_per_sm;
   if (blocks > cap) blocks = cap;
-  if (blocks == 0) blocks = 1;
-  // prefetch the masks when the batch could read about one sector per 16
-  // buckets or more (a mixed batch of n ops holds at most n new keys)
-  const int pf = n * 16 >= v.nb ? 1 : 0;
   if (v.S == 16)
     return launch_in_window(L, k_claim<16>, static_cast<unsigned>(blocks), kClaimThreads, 0, s, v,
-                            in, nchunks, out, status, pf);
+                            in, out);
   return launch_in_window(L, k_claim<32>, static_cast<unsigned>(blocks), kClaimThreads, 0, s, v, in,
-                          nchunks, out, status, pf);
+                          out);
 }
 
 cudaError_t launch_overflow(const View& v, List in, List pend, int resizable, uint8_t* status,
@@ -2847,43 +2591,41 @@ cudaError_t launch_multi_gather(const MultiHdr* hdr, const View* views, const ui
 }
 
 namespace {
-// Shared-memory limits and resident blocks of the bulk kernels of one shape.
+// Resident blocks of the bulk kernels of one shape.
+template <int S, int T, int MODE, bool DEFER = false>
+cudaError_t occupancy_mode(Launch* L) {
+  int b = 0;
+  cudaError_t e;
+  if constexpr (MODE == kModeFind)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_find<S, T, 4>, T, 0);
+  else
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ops<MODE, S, DEFER, T, false>, T, 0);
+  L->ops_blocks_per_sm[MODE + (DEFER ? 1 : 0)] = b > 0 ? b : 1;
+  return e;
+}
 template <int S, int T>
 cudaError_t occupancy_ops(Launch* L) {
+  cudaError_t e = occupancy_mode<S, T, kModeFind>(L);
+  if (e == cudaSuccess) e = occupancy_mode<S, T, kModeInsert>(L);
+  if (e == cudaSuccess) e = occupancy_mode<S, T, kModeErase>(L);
+  if (e == cudaSuccess) e = occupancy_mode<S, T, kModeMixed>(L);
+  if (e == cudaSuccess) e = occupancy_mode<S, T, kModeMixed, true>(L);
+  return e;
+}
+
+// The same for the staged kernels (32-slot buckets, 256 threads).
+template <int MODE, bool DEFER>
+cudaError_t staged_limits(int* least) {
+  constexpr int smem = static_cast<int>(stage_smem(32));
+  cudaError_t e = cudaFuncSetAttribute(k_ops<MODE, 32, DEFER, 256, true>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   int b = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ops<kModeFind, S, false, T>,
-                                                                T, 0);
-  if (e != cudaSuccess) return e;
-  L->ops_blocks_per_sm = b > 0 ? b : 1;
-  e = cudaFuncSetAttribute(k_ops<kModeFind, S, false, T>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(stage_smem(kModeFind, S, T)));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_ops<kModeInsert, S, false, T>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(stage_smem(kModeInsert, S, T)));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_ops<kModeErase, S, false, T>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(stage_smem(kModeErase, S, T)));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_ops<kModeMixed, S, false, T>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(stage_smem(kModeMixed, S, T)));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_ops<kModeMixed, S, true, T>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(stage_smem(kModeMixed, S, T)));
-  if (e != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ops<kModeInsert, S, false, T>, T,
-                                                    stage_smem(kModeInsert, S, T));
-  if (e != cudaSuccess) return e;
-  L->staged_blocks_per_sm = b > 0 ? b : 1;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ops<kModeMixed, S, false, T>, T,
-                                                    stage_smem(kModeMixed, S, T));
-  if (e != cudaSuccess) return e;
-  L->staged1_blocks_per_sm = b > 0 ? b : 1;
-  return cudaSuccess;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ops<MODE, 32, DEFER, 256, true>, 256,
+                                                      smem);
+  if (b < 1) b = 1;
+  if (b < *least) *least = b;
+  return e;
 }
 
 template <int S>
@@ -2893,10 +2635,17 @@ cudaError_t occupancy_s(Launch* L) {
                   : L->ops_threads == 512 ? occupancy_ops<S, 512>(L)
                                           : occupancy_ops<S, 256>(L);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_fused<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(fused_smem(S)));
-  if (e != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_fused<S>, kOpsThreads, fused_smem(S));
+  if (S == 32 && L->staged) {
+    int least = 64;
+    e = staged_limits<kModeFind, false>(&least);
+    if (e == cudaSuccess) e = staged_limits<kModeInsert, false>(&least);
+    if (e == cudaSuccess) e = staged_limits<kModeErase, false>(&least);
+    if (e == cudaSuccess) e = staged_limits<kModeMixed, false>(&least);
+    if (e == cudaSuccess) e = staged_limits<kModeMixed, true>(&least);
+    if (e != cudaSuccess) return e;
+    L->staged_blocks_per_sm = least;
+  }
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_fused<S>, kOpsThreads, 0);
   if (e != cudaSuccess) return e;
   L->fused_blocks_per_sm = b > 0 ? b : 1;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_multi_ops<S>, kOpsThreads, 0);
@@ -2926,3 +2675,4 @@ cudaError_t query_occupancy(Launch* L, int S) {
 }
 
 }  // namespace hive
+

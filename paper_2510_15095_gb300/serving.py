@@ -33,7 +33,7 @@ import numpy as np
 
 from . import hive as H
 
-SLOT_BYTES = 8.0 + 8.0 / 32  # a bucket slot plus its share of free mask and lock words
+SLOT_BYTES = 9.0 + 8.0 / 32  # a slot, its tag, and its share of the lock and version words
 
 
 @dataclass

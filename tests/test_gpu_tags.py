@@ -1,0 +1,133 @@
+"""Slot tags: one byte per slot that lookups compare first and claims own.
+
+A tag must be 0 exactly where the slot is EMPTY and match the slot's key
+elsewhere; a stale byte would hide a key, leak a slot or let two keys claim
+one.  The dump's free masks are the zero tags, so the image check compares
+tags with words, and finds of every key compare the others.  Sizes sit at the
+edges: one to three buckets (both candidates often the same bucket), batches
+around the 32 ops of a warp, buckets filled to the last slot, and churn that
+reuses every slot many times, in each of the three ways a batch can run.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2510_15095_gb300 import workload as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def H():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_15095_gb300 import hive
+    hive.load_library()
+    return hive
+
+
+def up(H, a):
+    return H.to_device_u32(a)
+
+
+def check(H, t, d, keys):
+    v, f = t.find(up(H, keys))
+    ev, ef = d.find(keys)
+    assert np.array_equal(f.cpu().numpy(), ef) and np.array_equal(H.to_host_u32(v), ev)
+    img = t.dump()
+    code, where = oracle.check_image(img, img["S"], d, None)
+    assert code == 0, f"invariant {code} fails at {where}"
+
+
+@pytest.mark.parametrize("bs", [16, 32])
+@pytest.mark.parametrize("buckets", [1, 2, 3, 5, 64])
+@pytest.mark.parametrize("n", [1, 31, 33, 257])
+def test_tiny_tables_and_ragged_batches(H, bs, buckets, n):
+    t = H.HiveTable(bs * buckets, bucket_slots=bs)
+    d = oracle.Dict()
+    keys, c = W.take_keys(900 + n, 0, n)
+    vals = W.values_for(keys, 1)
+    absent, _ = W.take_keys(900 + n, c, n)
+    probe = np.concatenate([keys, absent])
+    for _ in range(3):
+        assert np.array_equal(t.insert(up(H, keys), up(H, vals)).cpu().numpy(),
+                              d.insert(keys, vals))
+        check(H, t, d, probe)
+        er = keys[::2].copy()
+        assert np.array_equal(t.erase(up(H, er)).cpu().numpy(), d.erase(er))
+        check(H, t, d, probe)
+    assert t.check() == 0
+    t.close()
+
+
+@pytest.mark.parametrize("bs", [16, 32])
+@pytest.mark.parametrize("way", ["phased", "deferred", "fused"])
+def test_churn_keeps_tags_and_words_together(H, bs, way):
+    """Batches that erase as many keys as they insert, at 95% load, so that
+    every slot changes hands several times and chains run in each batch."""
+    big = way == "deferred"  # claims in their own kernel from 2^18 ops on
+    slots = 1 << (19 if big else 14)
+    rng = np.random.default_rng(bs)
+    t = H.HiveTable(slots, bucket_slots=bs)
+    d = oracle.Dict()
+    live, c = W.take_keys(77, 0, slots * 95 // 100)
+    assert np.array_equal(t.insert(up(H, live), up(H, W.values_for(live, 3))).cpu().numpy(),
+                          d.insert(live, W.values_for(live, 3)))
+    n = slots // 4
+    rounds = 4 if big else 12
+    for r in range(rounds):
+        new, c = W.take_keys(77, c, n)
+        ops, keys, vals = W.mixed_batch(rng, live, new, n, n, 2 * n if big else n, seed=r)
+        vo, st = t.execute(torch.from_numpy(ops).cuda(), up(H, keys), up(H, vals),
+                           fused=way == "fused")
+        ev, es = d.execute(ops, keys, vals)
+        assert np.array_equal(st.cpu().numpy(), es) and np.array_equal(H.to_host_u32(vo), ev)
+        live, _ = d.dump()
+    check(H, t, d, np.concatenate([live, W.take_keys(77, c, 1000)[0]]))
+    assert t.check() == 0
+    t.close()
+
+
+@pytest.mark.parametrize("bs", [16, 32])
+def test_every_slot_of_full_buckets(H, bs):
+    """Fills a table to the last slot through small inserts (claims, chains,
+    stash) and finds every key after each; then empties it."""
+    slots = 64 * bs
+    t = H.HiveTable(slots, bucket_slots=bs)
+    d = oracle.Dict()
+    keys, _ = W.take_keys(5, 0, slots)
+    vals = W.values_for(keys, 5)
+    for part in np.array_split(np.arange(slots), 16):
+        assert np.array_equal(t.insert(up(H, keys[part]), up(H, vals[part])).cpu().numpy(),
+                              d.insert(keys[part], vals[part]))
+        check(H, t, d, keys)
+    for part in np.array_split(np.arange(slots), 5):
+        assert np.array_equal(t.erase(up(H, keys[part])).cpu().numpy(), d.erase(keys[part]))
+        check(H, t, d, keys)
+    assert t.size() == 0 and t.check() == 0
+    t.close()
+
+
+@pytest.mark.parametrize("n", [4_000_000, 4_000_001, 4_000_127])
+@pytest.mark.parametrize("off", [0, 1, 4])
+def test_long_find_batches(H, n, off):
+    """Find batches long enough for four runs per warp and store, ragged ones
+    and found flags at any byte offset: the same answers as in short batches."""
+    t = H.HiveTable(1 << 16)
+    keys, c = W.take_keys(31, 0, 50_000)
+    vals = W.values_for(keys, 31)
+    t.insert(up(H, keys), up(H, vals))
+    pool = up(H, np.concatenate([keys, W.take_keys(31, c, 50_000)[0],
+                                 np.array([0xFFFFFFFE, 0xFFFFFFFF], np.uint32)]))
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + off)
+    at = torch.randint(0, pool.numel(), (n,), generator=g, device="cuda")
+    v0, f0 = t.find(pool)  # a short batch
+    vals_out = torch.full((n + off,), -1, dtype=torch.int32, device="cuda")
+    found = torch.full((n + off + 64,), 7, dtype=torch.uint8, device="cuda")
+    t.find(pool[at], vals_out=vals_out[off:], found=found[off:off + n])
+    assert torch.equal(vals_out[off:], v0[at]) and torch.equal(found[off:off + n], f0[at])
+    assert bool((found[:off] == 7).all()) and bool((found[off + n:] == 7).all())
+    assert t.check() == 2  # the reserved keys
+    t.close()
