@@ -242,16 +242,35 @@ hive_status grow_for(hive_table* t, uint64_t n_ins, cudaStream_t s) {
   return HIVE_OK;
 }
 
+// Before a mixed batch of n ops: grows for its inserts.  They are counted only
+// if n new keys would grow the table; fewer then would not either, and the
+// call does not wait for the GPU here.
+hive_status grow_for_mixed(hive_table* t, const uint8_t* ops, uint64_t n, cudaStream_t s) {
+  if (t->nb >= t->nb_max || !over_grow(t, t->size_host + n, t->nb)) return HIVE_OK;
+  HIVE_CK(cudaMemsetAsync(&t->ctrl->n_insert, 0, sizeof(unsigned), s));
+  HIVE_LAUNCH(t, HIVE_K_COUNT, s, launch_count_inserts(ops, n, &t->ctrl->n_insert, s));
+  hive_status st = readback(t, s);
+  if (st != HIVE_OK) return st;
+  return grow_for(t, t->host_ctrl->n_insert, s);
+}
+
 // After P1+P2 on a resizable table: place items that found no room by growing,
 // then run maintenance, read the size back, and contract while under the lower
 // threshold.  `status` receives FULL for ops that still find no room at
 // nb_max.  The pending items are in list B, or in list A with !pending_in_b.
 hive_status finish_resizable(hive_table* t, uint8_t* status, cudaStream_t s,
                              bool pending_in_b = true) {
+  // Maintenance goes ahead of the read-back that says whether items are
+  // pending: it does nothing if there are, and in the usual case the call
+  // waits for the GPU once.
+  HIVE_LAUNCH(t, HIVE_K_MAINT, s,
+              launch_maintenance(make_view(t), s,
+                                 kMaintStash | (pending_in_b ? kMaintUnlessPend : kMaintUnlessOvf)));
   hive_status st = readback(t, s);
   if (st != HIVE_OK) return st;
-  bool in_b = pending_in_b;
+  bool in_b = pending_in_b, again = false;
   while ((in_b ? t->host_ctrl->pend_n : t->host_ctrl->ovf_n) != 0) {
+    again = true;
     bool did = false;
     st = split_step(t, s, &did);
     if (st != HIVE_OK) return st;
@@ -268,13 +287,11 @@ hive_status finish_resizable(hive_table* t, uint8_t* status, cudaStream_t s,
     in_b = !in_b;
     if (!did) break;
   }
-  if (t->host_ctrl->stash_n) {
-    st = mark_stash_dirty(t, s);
+  if (again) {
+    HIVE_LAUNCH(t, HIVE_K_MAINT, s, launch_maintenance(make_view(t), s, kMaintStash));
+    st = readback(t, s);
     if (st != HIVE_OK) return st;
   }
-  HIVE_LAUNCH(t, HIVE_K_MAINT, s, launch_maintenance(make_view(t), s));
-  st = readback(t, s);
-  if (st != HIVE_OK) return st;
   t->size_host = t->host_ctrl->size;
 
   return contract_table(t, s);
@@ -680,12 +697,7 @@ hive_status hive_execute(hive_table* t, const uint8_t* ops, const uint32_t* keys
       (st = check_contract_device(ops, HIVE_OP_FIND, keys, n, kReservedKeyMin, s)) != HIVE_OK)
     return st;
   if ((st = ensure_lists(t, n, true)) != HIVE_OK) return st;
-  if (t->cfg.resizable) {
-    HIVE_CK(cudaMemsetAsync(&t->ctrl->n_insert, 0, sizeof(unsigned), s));
-    HIVE_LAUNCH(t, HIVE_K_COUNT, s, launch_count_inserts(ops, n, &t->ctrl->n_insert, s));
-    if ((st = readback(t, s)) != HIVE_OK) return st;
-    if ((st = grow_for(t, t->host_ctrl->n_insert, s)) != HIVE_OK) return st;
-  }
+  if (t->cfg.resizable && (st = grow_for_mixed(t, ops, n, s)) != HIVE_OK) return st;
   const View v = make_view(t);
   // Both op lists are empty here: every mutating call ends with the
   // maintenance kernel, which resets their counts.
@@ -731,12 +743,7 @@ hive_status hive_execute_fused(hive_table* t, const uint8_t* ops, const uint32_t
       (st = check_contract_device(ops, HIVE_OP_FIND, keys, n, kReservedKeyMin, s)) != HIVE_OK)
     return st;
   if ((st = ensure_lists(t, n)) != HIVE_OK) return st;
-  if (t->cfg.resizable) {
-    HIVE_CK(cudaMemsetAsync(&t->ctrl->n_insert, 0, sizeof(unsigned), s));
-    HIVE_LAUNCH(t, HIVE_K_COUNT, s, launch_count_inserts(ops, n, &t->ctrl->n_insert, s));
-    if ((st = readback(t, s)) != HIVE_OK) return st;
-    if ((st = grow_for(t, t->host_ctrl->n_insert, s)) != HIVE_OK) return st;
-  }
+  if (t->cfg.resizable && (st = grow_for_mixed(t, ops, n, s)) != HIVE_OK) return st;
   // inserts that find no room at all go to list B, the pending list that
   // finish_resizable drains
   HIVE_LAUNCH(t, HIVE_K_FUSED, s,

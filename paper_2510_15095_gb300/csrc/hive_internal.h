@@ -150,7 +150,13 @@ cudaError_t launch_overflow(const View& v, List in, List pend, int resizable, ui
 // kernel; items with both buckets full go to `out`.
 cudaError_t launch_claim(const View& v, List in, uint64_t n, List out, const Launch& L,
                          cudaStream_t s);
-cudaError_t launch_maintenance(const View& v, cudaStream_t s);
+// mode: kMaint* bits.
+enum : int {
+  kMaintStash = 1,       // look at every stash word, also if none changed
+  kMaintUnlessPend = 2,  // do nothing while the pending list (pend_n) holds items
+  kMaintUnlessOvf = 4    // do nothing while list A (ovf_n) holds items
+};
+cudaError_t launch_maintenance(const View& v, cudaStream_t s, int mode = 0);
 cudaError_t launch_split(const View& v_new, uint32_t src0, uint32_t count, uint32_t half,
                          cudaStream_t s);
 cudaError_t launch_merge_excess(const View& v_new, uint32_t count, cudaStream_t s);

@@ -1998,14 +1998,18 @@ __device__ void block_bitonic(uint64_t* a, unsigned P) {
 }
 
 // One CTA maintains the stash of the table of `v`; `smem` holds
-// kMaintSmemWords words.
+// kMaintSmemWords words.  `mode` (kMaint*): what a resizable table's call
+// asks for before the host has seen the batch's outcome.
 template <int S>
-__device__ void maint_body(const View& v, uint64_t* smem) {
+__device__ void maint_body(const View& v, uint64_t* smem, int mode = 0) {
   __shared__ unsigned s_reins, s_live;
   Ctrl* c = v.ctrl;
+  // items wait for growth: the host grows, places them and asks again
+  if ((mode & kMaintUnlessPend) && c->pend_n) return;
+  if ((mode & kMaintUnlessOvf) && c->ovf_n) return;
   const unsigned tail = c->stash_tail;
   const unsigned sorted = c->stash_n;
-  const unsigned dirty = c->stash_dirty;
+  const unsigned dirty = c->stash_dirty || ((mode & kMaintStash) && sorted);
   if (threadIdx.x == 0) {
     s_reins = 0;
     s_live = 0;
@@ -2069,9 +2073,9 @@ __device__ void maint_body(const View& v, uint64_t* smem) {
 }
 
 template <int S>
-__global__ void __launch_bounds__(kMaintThreads) k_maint(View v) {
+__global__ void __launch_bounds__(kMaintThreads) k_maint(View v, int mode) {
   extern __shared__ uint64_t smem[];
-  maint_body<S>(v, smem);
+  maint_body<S>(v, smem, mode);
 }
 
 // ----------------------------------------------------------------------------
@@ -2184,13 +2188,34 @@ __global__ void __launch_bounds__(256) k_merge(View v, uint32_t count, List ovf)
   }
 }
 
-__global__ void k_count_inserts(const uint8_t* __restrict__ ops, uint64_t n, unsigned* out) {
+// Inserts among the op codes of a batch: 16 codes per load (the bytes before
+// the first 16-byte boundary and after the last one by single loads) and one
+// atomic per block.  Reads n bytes once: 2^22 codes in 5 us (25 with a byte
+// per load and an atomic per warp).
+__global__ void __launch_bounds__(256)
+    k_count_inserts(const uint8_t* __restrict__ ops, uint64_t n, unsigned* out) {
+  const uint64_t tid = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const uint64_t step = static_cast<uint64_t>(gridDim.x) * blockDim.x;
+  uint64_t head = (16 - (reinterpret_cast<uintptr_t>(ops) & 15)) & 15;
+  if (head > n) head = n;
+  const uint64_t nv = (n - head) / 16;
+  const uint64_t tail0 = head + 16 * nv;
   unsigned c = 0;
-  for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-       i += static_cast<uint64_t>(gridDim.x) * blockDim.x)
-    c += ops[i] == OP_INSERT;
+  if (tid < head) c += ops[tid] == OP_INSERT;
+  if (tid < n - tail0) c += ops[tail0 + tid] == OP_INSERT;
+  const uint4* p = reinterpret_cast<const uint4*>(ops + head);
+  for (uint64_t i = tid; i < nv; i += step) {
+    const uint4 x = __ldg(p + i);  // op code 0 is an insert
+    c += __popc(zero_bytes(x.x)) + __popc(zero_bytes(x.y)) + __popc(zero_bytes(x.z)) +
+         __popc(zero_bytes(x.w));
+  }
+  __shared__ unsigned sum;
+  if (threadIdx.x == 0) sum = 0;
+  __syncthreads();
   c = __reduce_add_sync(kFull, c);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(&sum, c);
+  __syncthreads();
+  if (threadIdx.x == 0 && sum) atomicAdd(out, sum);
 }
 
 // ----------------------------------------------------------------------------
@@ -2476,12 +2501,12 @@ cudaError_t launch_overflow(const View& v, List in, List pend, int resizable, ui
                           status);
 }
 
-cudaError_t launch_maintenance(const View& v, cudaStream_t s) {
+cudaError_t launch_maintenance(const View& v, cudaStream_t s, int mode) {
   constexpr size_t smem = kMaintSmemWords * sizeof(uint64_t);
   if (v.S == 16)
-    k_maint<16><<<1, kMaintThreads, smem, s>>>(v);
+    k_maint<16><<<1, kMaintThreads, smem, s>>>(v, mode);
   else
-    k_maint<32><<<1, kMaintThreads, smem, s>>>(v);
+    k_maint<32><<<1, kMaintThreads, smem, s>>>(v, mode);
   return cudaGetLastError();
 }
 
@@ -2518,8 +2543,9 @@ cudaError_t launch_merge(const View& v_new, uint32_t count, List ovf, cudaStream
 
 cudaError_t launch_count_inserts(const uint8_t* ops, uint64_t n, unsigned* out, cudaStream_t s) {
   if (!n) return cudaSuccess;
-  uint64_t blocks = (n + 255) / 256;
-  if (blocks > 4096) blocks = 4096;
+  uint64_t blocks = (n / 16 + 255) / 256;
+  if (blocks > 152 * 4) blocks = 152 * 4;
+  if (blocks == 0) blocks = 1;
   k_count_inserts<<<static_cast<unsigned>(blocks), 256, 0, s>>>(ops, n, out);
   return cudaGetLastError();
 }
