@@ -454,7 +454,7 @@ typedef struct {
   uint32_t M, p;        /* linear-hashing address state (p > 0 when nb is not a power of two) */
   uint32_t layout;
   uint32_t* buckets;    /* [nb * 32] entries, 0xFFFFFFFF = empty (caller-allocated) */
-  uint32_t* masks;      /* [nb] free masks */
+  uint32_t* masks;      /* [nb] free masks (zero tags) */
   uint32_t* locks;      /* [nb] */
   uint32_t* stash;      /* [stash_cap] sorted live prefix of stash_n entries */
   uint64_t stash_n, stash_cap, size, pending;

@@ -10,6 +10,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <vector>
 
 #include "hive.h"
 #include "hive_internal.h"
@@ -24,7 +25,7 @@ struct hive32_table {
   uint32_t stash_cap = 0;
   uint64_t stash_alloc = 0;
   uint32_t* buckets = nullptr;
-  uint32_t* masks = nullptr;
+  uint32_t* tags = nullptr;
   uint32_t* locks = nullptr;
   uint32_t* stash_kv = nullptr;
   uint32_t* stash_keys = nullptr;
@@ -62,7 +63,7 @@ constexpr uint64_t kMaxBuckets32 = 1ull << 31;
 View32 view32(const hive32_table* t) {
   View32 v{};
   v.buckets = t->buckets;
-  v.masks = t->masks;
+  v.tags = t->tags;
   v.locks = t->locks;
   v.stash_kv = t->stash_kv;
   v.stash_keys = t->stash_keys;
@@ -142,7 +143,7 @@ hive_status run32(hive32_table* t, int mode, const uint8_t* ops, const uint32_t*
 
 void free32(hive32_table* t) {
   cudaFree(t->buckets);
-  cudaFree(t->masks);
+  cudaFree(t->tags);
   cudaFree(t->locks);
   cudaFree(t->stash_kv);
   cudaFree(t->stash_keys);
@@ -197,14 +198,14 @@ hive_status hive32_create(const hive32_config* cfg, void* stream, hive32_table**
     e = cudaDeviceGetAttribute(&t->num_sms, cudaDevAttrMultiProcessorCount, t->device);
   if (e == cudaSuccess) e = setup32(static_cast<int>(cfg->layout), &t->blocks_per_sm);
   if (e == cudaSuccess) e = cudaMalloc(&t->buckets, nb * kS * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&t->masks, nb * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&t->tags, nb * kS);
   if (e == cudaSuccess) e = cudaMalloc(&t->locks, nb * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&t->stash_kv, t->stash_alloc * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&t->stash_keys, t->stash_cap * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&t->ctrl, sizeof(Ctrl));
   if (e == cudaSuccess) e = cudaMallocHost(&t->host_ctrl, sizeof(Ctrl));
   if (e == cudaSuccess) e = cudaMemsetAsync(t->buckets, 0xFF, nb * kS * sizeof(uint32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(t->masks, 0xFF, nb * sizeof(uint32_t), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(t->tags, 0, nb * kS, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(t->locks, 0, nb * sizeof(uint32_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(t->stash_kv, 0xFF, t->stash_alloc * sizeof(uint32_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(t->ctrl, 0, sizeof(Ctrl), s);
@@ -267,7 +268,7 @@ hive_status hive32_clear(hive32_table* t, void* stream) {
   if (st != HIVE_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   H32_CK(cudaMemsetAsync(t->buckets, 0xFF, t->nb * kS * sizeof(uint32_t), s));
-  H32_CK(cudaMemsetAsync(t->masks, 0xFF, t->nb * sizeof(uint32_t), s));
+  H32_CK(cudaMemsetAsync(t->tags, 0, t->nb * kS, s));
   H32_CK(cudaMemsetAsync(t->locks, 0, t->nb * sizeof(uint32_t), s));
   H32_CK(cudaMemsetAsync(t->stash_kv, 0xFF, t->stash_alloc * sizeof(uint32_t), s));
   H32_CK(cudaMemsetAsync(t->ctrl, 0, sizeof(Ctrl), s));
@@ -329,12 +330,24 @@ hive_status hive32_dump(hive32_table* t, hive32_image* img, void* stream) {
     return fail32(HIVE_ERR_INVALID_ARG, "image arrays must all be given");
   H32_CK(cudaMemcpyAsync(img->buckets, t->buckets, t->nb * kS * sizeof(uint32_t),
                          cudaMemcpyDeviceToHost, s));
-  H32_CK(cudaMemcpyAsync(img->masks, t->masks, t->nb * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+  // the image's free masks are the slots whose tag is 0
+  std::vector<uint8_t> tags;
+  try {
+    tags.resize(t->nb * kS);
+  } catch (const std::bad_alloc&) {
+    return fail32(HIVE_ERR_OOM, "hive32_dump: host allocation failed");
+  }
+  H32_CK(cudaMemcpyAsync(tags.data(), t->tags, tags.size(), cudaMemcpyDeviceToHost, s));
   H32_CK(cudaMemcpyAsync(img->locks, t->locks, t->nb * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   if (img->stash_n)
     H32_CK(cudaMemcpyAsync(img->stash, t->stash_kv, img->stash_n * sizeof(uint32_t),
                            cudaMemcpyDeviceToHost, s));
   H32_CK(cudaStreamSynchronize(s));
+  for (uint64_t b = 0; b < t->nb; ++b) {
+    uint32_t m = 0;
+    for (uint32_t k = 0; k < kS; ++k) m |= static_cast<uint32_t>(tags[b * kS + k] == 0) << k;
+    img->masks[b] = m;
+  }
   return HIVE_OK;
 }
 

@@ -184,7 +184,7 @@ cudaError_t query_occupancy(Launch* L, int S);
 // ---- tables with 32-bit entries (hive32_*) ----
 struct View32 {
   uint32_t* buckets;     // [nb * 32] entries
-  uint32_t* masks;       // [nb] free masks
+  uint32_t* tags;        // [nb * 8] slot tags, one byte per slot (0: free slot)
   uint32_t* locks;       // [nb] bucket locks (eviction only)
   uint32_t* stash_kv;    // [stash_alloc] stash entries, EMPTY padded
   uint32_t* stash_keys;  // [stash_cap] keys of the sorted prefix

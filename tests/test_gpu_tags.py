@@ -131,3 +131,38 @@ def test_long_find_batches(H, n, off):
     assert bool((found[:off] == 7).all()) and bool((found[off + n:] == 7).all())
     assert t.check() == 2  # the reserved keys
     t.close()
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("buckets", [1, 2, 3, 64])
+@pytest.mark.parametrize("n", [1, 33, 700])
+def test_small_tables_with_32_bit_entries(H, layout, buckets, n):
+    """The same edges on tables with 32-bit entries: a 16-bit map and a set."""
+    from test_gpu_hive32 import check_image as check_image32
+
+    n = min(n, buckets * 32)
+    rng = np.random.default_rng(n)
+    if layout == 0:
+        every = rng.permutation(0xFFFE).astype(np.uint32)
+        keys, absent = every[:n].copy(), every[n:2 * n].copy()
+        vals = rng.integers(0, 1 << 16, n).astype(np.uint32)
+    else:
+        keys, c = W.take_keys(600 + n, 0, n)
+        absent, _ = W.take_keys(600 + n, c, n)
+        vals = np.zeros(n, np.uint32)
+    t = H.Hive32Table(buckets * 32, layout)
+    d = oracle.Dict()
+    probe = np.concatenate([keys, absent])
+    for _ in range(3):
+        assert np.array_equal(t.insert(up(H, keys), up(H, vals)).cpu().numpy(),
+                              d.insert(keys, vals))
+        for phase in range(2):
+            v, f = t.find(up(H, probe))
+            ev, ef = d.find(probe)
+            assert np.array_equal(f.cpu().numpy(), ef) and np.array_equal(H.to_host_u32(v), ev)
+            check_image32(t, d)
+            if phase == 0:
+                er = keys[::2].copy()
+                assert np.array_equal(t.erase(up(H, er)).cpu().numpy(), d.erase(er))
+    assert t.check() == 0
+    t.close()
