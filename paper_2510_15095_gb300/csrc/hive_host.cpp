@@ -162,6 +162,69 @@ hive_status ensure_lists(hive_table* t, uint64_t n, bool need_b = false) {
   return HIVE_OK;
 }
 
+void free_part(hive_table* t) {
+  cudaFree(t->part_words);
+  cudaFree(t->part_slots);
+  cudaFree(t->part_off);
+  t->part_words = nullptr;
+  t->part_slots = nullptr;
+  t->part_off = nullptr;
+  t->part_cap = 0;
+}
+
+// Bulk inserts store their words region by region (launch_insert_part) when
+// the table's words are well beyond L2 and the batch brings two ops or more to
+// each 128-byte line of them.  Measured on one GB300 (first batch of a bulk
+// load, plain -> by region): 2^24 slots 489 -> 590 us and 2^25 slots 1148 ->
+// 1114 us, where L2 still collects most lines by itself; 2^26 slots 3244 ->
+// 2262 us at 15 ops a line, 1689 -> 1266 us at eight, and 607 -> 533 us for a
+// second batch of two ops a line.  A region is 4 MB of words (8 MB: 1384 us in
+// place of 1266), and as much larger as the limit on their number asks.
+constexpr uint64_t kPartMinBytes = 256ull << 20;
+constexpr uint64_t kPartOpsPerLine = 2;
+constexpr uint32_t kPartMinShift = 19, kPartMaxShift = 22;  // 2^19 slots: 4 MB
+uint32_t part_shift(const hive_table* t) {
+  uint32_t shift = kPartMinShift;
+  while ((t->nb * t->S - 1) >> shift >= kPartMaxRegions) ++shift;
+  return shift;
+}
+bool want_part(const hive_table* t, uint64_t n) {
+  const uint64_t slots = t->nb * t->S;
+  return slots * sizeof(uint64_t) > kPartMinBytes && n * 16 >= slots * kPartOpsPerLine &&
+         !t->L.staged && part_shift(t) <= kPartMaxShift;
+}
+// The list of such an insert.  False (and the plain way is taken) when there
+// is no memory for it, or when the stream is being captured and it would have
+// to be allocated.
+bool ensure_part(hive_table* t, uint64_t n, cudaStream_t s, PartList* out) {
+  if (n > t->part_cap) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      return false;
+    }
+    if (t->part_cap) {
+      if (cudaDeviceSynchronize() != cudaSuccess) return false;  // the next launch reports it
+      free_part(t);
+    }
+    const uint64_t tiles = part_tiles(n);
+    cudaError_t e = dev_alloc(&t->part_words, n * sizeof(uint64_t));
+    if (e == cudaSuccess) e = dev_alloc(&t->part_slots, n * sizeof(uint32_t));
+    if (e == cudaSuccess)
+      e = dev_alloc(&t->part_off, tiles * (kPartMaxRegions + 1) * sizeof(uint16_t));
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      free_part(t);
+      return false;
+    }
+    t->part_cap = n;
+  }
+  const uint32_t shift = part_shift(t);
+  *out = PartList{t->part_words, t->part_slots, t->part_off,
+                  static_cast<uint32_t>((t->nb * t->S - 1) >> shift) + 1, shift};
+  return true;
+}
+
 hive_status readback(hive_table* t, cudaStream_t s) {
   HIVE_CK(cudaMemcpyAsync(t->host_ctrl, t->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
   HIVE_CK(cudaStreamSynchronize(s));
@@ -606,6 +669,7 @@ hive_status hive_destroy(hive_table* t) {
   cudaFree(t->ctrl);
   if (t->host_ctrl) cudaFreeHost(t->host_ctrl);
   free_lists(t);
+  free_part(t);
   free_staging(t);
   for (const auto& r : t->recs) {
     cudaEventDestroy(r.a);
@@ -630,9 +694,14 @@ hive_status hive_insert(hive_table* t, const uint32_t* keys, const uint32_t* val
   if ((st = ensure_lists(t, n)) != HIVE_OK) return st;
   if (t->cfg.resizable && (st = grow_for(t, n, s)) != HIVE_OK) return st;
   const View v = make_view(t);
-  HIVE_LAUNCH(t, HIVE_K_INSERT, s,
-              launch_ops(kModeInsert, v, nullptr, keys, vals, n, nullptr, nullptr, status,
-                         list_a(t), t->L, s));
+  PartList pl{};
+  if (want_part(t, n) && ensure_part(t, n, s, &pl))
+    HIVE_LAUNCH(t, HIVE_K_INSERT, s,
+                launch_insert_part(v, keys, vals, n, status, list_a(t), pl, t->L, s));
+  else
+    HIVE_LAUNCH(t, HIVE_K_INSERT, s,
+                launch_ops(kModeInsert, v, nullptr, keys, vals, n, nullptr, nullptr, status,
+                           list_a(t), t->L, s));
   HIVE_LAUNCH(t, HIVE_K_EVICT, s,
               launch_overflow(v, list_a(t), list_b(t), t->cfg.resizable, status, t->L, s));
   if (t->cfg.resizable) return finish_resizable(t, status, s);
@@ -794,7 +863,9 @@ hive_status hive_memory(hive_table* t, uint64_t* committed, uint64_t* reserved) 
   const uint64_t bucket_now = t->vmm ? t->bucket_vm.committed : bucket_max;
   const uint64_t other = t->nb_max * (t->S + 2 * sizeof(uint32_t)) + t->stash_alloc * sizeof(uint64_t) +
                          t->stash_cap * sizeof(uint32_t) + sizeof(Ctrl) +
-                         (t->list_cap + t->lb_cap) * 12;
+                         (t->list_cap + t->lb_cap) * 12 +
+                         t->part_cap * 12 +
+                         part_tiles(t->part_cap) * (kPartMaxRegions + 1) * sizeof(uint16_t);
   *committed = bucket_now + other;
   *reserved = bucket_max + other;
   return HIVE_OK;

@@ -59,7 +59,8 @@ struct alignas(128) Ctrl {
   unsigned int merge_excess; // words a merge batch cannot keep in the low bucket
   unsigned int n_insert;     // insert ops counted in a mixed batch
   unsigned int defer_n;      // new keys of a mixed batch waiting for k_claim
-  unsigned int pad0[4];
+  unsigned int part_next;    // next group of tiles of a store by region
+  unsigned int pad0[3];
   unsigned long long stats[kNumStats];
 };
 
@@ -89,6 +90,18 @@ struct List {
   uint32_t* idx;   // caller op index or kNoOp
   unsigned int* count;
   uint32_t* seg;   // multi-table batches: segment of each entry (else NULL)
+};
+
+// Claimed words of a bulk insert, waiting to be stored region by region (see
+// k_insert_part): tile t's pairs lie from t * tile ops on, sorted by region;
+// off[t * (regions + 1) + r] is where region r starts within the tile.
+constexpr uint32_t kPartMaxRegions = 128;
+struct PartList {
+  uint64_t* words;
+  uint32_t* slots;   // slot index in the table
+  uint16_t* off;
+  uint32_t regions;  // <= kPartMaxRegions
+  uint32_t shift;    // slot index >> shift = region
 };
 
 // One (table, op range) of a multi-table batch; 64 bytes.
@@ -146,6 +159,11 @@ cudaError_t launch_ops(int mode, const View& v, const uint8_t* ops, const uint32
                        bool defer = false);
 cudaError_t launch_overflow(const View& v, List in, List pend, int resizable, uint8_t* status,
                             const Launch& L, cudaStream_t s);
+// A bulk insert in two kernels: claims, then stores by region.
+cudaError_t launch_insert_part(const View& v, const uint32_t* keys, const uint32_t* vals,
+                               uint64_t n, uint8_t* status, List ovf, const PartList& pl,
+                               const Launch& L, cudaStream_t s);
+uint64_t part_tiles(uint64_t n);
 // Claims for the new keys of a mixed batch of n ops, listed in `in` by the bulk
 // kernel; items with both buckets full go to `out`.
 cudaError_t launch_claim(const View& v, List in, uint64_t n, List out, const Launch& L,
@@ -267,6 +285,11 @@ struct hive_table {
   uint32_t* la_idx = nullptr;
   uint64_t* lb_words = nullptr;  // list B: items that found no room
   uint32_t* lb_idx = nullptr;
+  // list of a bulk insert that stores by region (allocated on first use)
+  uint64_t part_cap = 0;         // ops it holds
+  uint64_t* part_words = nullptr;
+  uint32_t* part_slots = nullptr;
+  uint16_t* part_off = nullptr;
   uint64_t size_host = 0;       // exact after each resizable call
   uint64_t splits = 0, merges = 0;
   bool merge_deferred = false;

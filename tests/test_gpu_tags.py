@@ -166,3 +166,34 @@ def test_small_tables_with_32_bit_entries(H, layout, buckets, n):
                 assert np.array_equal(t.erase(up(H, er)).cpu().numpy(), d.erase(er))
     assert t.check() == 0
     t.close()
+
+
+@pytest.mark.parametrize("bs", [16, 32])
+def test_bulk_inserts_stored_by_region(H, bs):
+    """Tables beyond 256 MB of words take large inserts in two kernels: claims,
+    then stores by region.  Ragged batches with new and present keys, reserved
+    keys and a status array, on a table whose last region is a partial one;
+    the same finds, sizes and image as the CPU dictionary's."""
+    slots = (1 << 25) + (1 << 20) + 32 * 77
+    n = slots // 8 + 4097  # two ops a line and a ragged tile
+    t = H.HiveTable(slots, bucket_slots=bs)
+    keys, c = W.take_keys(71, 0, n)
+    vals = W.values_for(keys, 71)
+    st = t.insert(up(H, keys), up(H, vals))
+    assert bool((st == H.INSERTED).all())
+    new, c = W.take_keys(71, c, n // 2)
+    k2 = np.concatenate([keys[: n // 2], new, np.array([0xFFFFFFFF, 0xFFFFFFFE], np.uint32)])
+    v2 = W.values_for(k2, 72)
+    order = np.random.default_rng(3).permutation(k2.size)
+    k2, v2 = k2[order], v2[order]
+    st = t.insert(up(H, k2), up(H, v2)).cpu().numpy()
+    want = np.where(order < n // 2, H.REPLACED, H.INSERTED)
+    want[order >= k2.size - 2] = H.RESERVED_KEY
+    assert np.array_equal(st, want)
+    assert t.size() == n + n // 2 and t.check() == 2  # the reserved keys
+    d = oracle.Dict()
+    d.insert(keys, vals)
+    d.insert(k2, v2)
+    check(H, t, d, np.concatenate([keys[:100_000], new[:100_000],
+                                   W.take_keys(71, c, 100_000)[0]]))
+    t.close()
