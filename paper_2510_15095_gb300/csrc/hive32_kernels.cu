@@ -65,10 +65,11 @@ __device__ __forceinline__ void flush32_block(const View32& v, const Counters32&
   const unsigned rp = __reduce_add_sync(kFull, c.replaced);
   const unsigned cl = __reduce_add_sync(kFull, c.claimed);
   const unsigned of = __reduce_add_sync(kFull, c.overflowed);
+  const unsigned pr = __reduce_add_sync(kFull, c.probes);
   const unsigned rs = __ballot_sync(kFull, c.reserved);
   const unsigned ct = __ballot_sync(kFull, c.contract);
   if (lane == 0) {
-    mine[0] = c.probes;
+    mine[0] = pr;
     mine[1] = static_cast<uint64_t>(static_cast<int64_t>(sd));
     mine[2] = rp;
     mine[3] = cl;
@@ -262,8 +263,10 @@ __device__ __forceinline__ void run_chunk32(const View32& v, uint32_t stash_n, c
     }
   }
   const bool hit = slot < kS32;
-  cnt.probes += __popc(__ballot_sync(kFull, live)) +
-                __popc(__ballot_sync(kFull, live && (MODE == kModeInsert || !hit || hb != b1)));
+  if (MODE != kModeInsert) {
+    cnt.probes += live;
+    cnt.probes += live && (!hit || hb != b1);
+  }
   if (hit) {
     done = true;
     act32<LAYOUT>(v, op, v.buckets + static_cast<uint64_t>(hb) * kS32 + slot, hb, slot, cur, key,
@@ -344,6 +347,8 @@ __global__ void __launch_bounds__(kOps32Threads, (MODE == kModeInsert || MODE ==
     if (c + nwarps < nchunks) nxt = load32<MODE>(a, c + nwarps, n, lane);
     run_chunk32<MODE, LAYOUT>(v, stash_n, a, c, n, ovf, cnt, in, lane);
   }
+  // an insert examines both buckets of every live op, which ends in one of these
+  if (MODE == kModeInsert) cnt.probes = 2 * (cnt.replaced + cnt.claimed + cnt.overflowed);
   flush32_block(v, cnt, lane);
 }
 

@@ -215,9 +215,16 @@ __device__ __forceinline__ bool stash_find(const View& v, uint32_t stash_n, uint
 struct LaneCounters {
   int size_delta = 0;
   unsigned replaced = 0, claimed = 0, overflowed = 0, stash_lookups = 0;
-  unsigned probes = 0;  // warp-uniform: buckets examined by this warp
+  unsigned probes = 0;  // buckets examined
   bool reserved = false, contract = false;
 };
+
+// An insert examines both candidate buckets of every live op, and every live
+// op ends replaced, claimed or handed on: counting the probes once at the end
+// keeps a counter out of the loop.
+__device__ __forceinline__ void count_insert_probes(LaneCounters& cnt) {
+  cnt.probes = 2 * (cnt.replaced + cnt.claimed + cnt.overflowed);
+}
 
 // ---- Shared-memory staging of bucket reads ----
 //
@@ -326,9 +333,9 @@ __device__ __forceinline__ void scan_staged(const uint64_t* sbuf, int lane, uint
 // reads their words until one holds the key, starting where the key's own
 // claim would have (so the slot that holds it tends to come before a false
 // match).
-template <int S, bool RO>
+template <int S, bool RO, class F>
 __device__ __forceinline__ void check_words(const View& v, uint32_t b1, uint32_t b2, uint32_t m1,
-                                            uint32_t m2, uint32_t key, Hit& h) {
+                                            uint32_t m2, uint32_t key, Hit& h, F on_hit) {
   const uint32_t rot = claim_rot(key);
   while (m1 | m2) {
     const bool in1 = m1 != 0;
@@ -338,6 +345,7 @@ __device__ __forceinline__ void check_words(const View& v, uint32_t b1, uint32_t
     const uint64_t w = ld_word<RO>(v.buckets + static_cast<uint64_t>(b) * S + slot);
     if (key_of(w) == key) {
       h = Hit{w, b, slot, true};
+      on_hit();
       return;
     }
     if (in1)
@@ -345,6 +353,12 @@ __device__ __forceinline__ void check_words(const View& v, uint32_t b1, uint32_t
     else
       m2 &= ~(1u << p);
   }
+}
+
+template <int S, bool RO>
+__device__ __forceinline__ void check_words(const View& v, uint32_t b1, uint32_t b2, uint32_t m1,
+                                            uint32_t m2, uint32_t key, Hit& h) {
+  check_words<S, RO>(v, b1, b2, m1, m2, key, h, [] {});
 }
 
 // An erase or replace CAS issued by a probe, checked only at the end of the
@@ -418,9 +432,9 @@ __device__ __forceinline__ void flush_counters(const View& v, LaneCounters& cnt,
   const unsigned rs = __ballot_sync(kFull, cnt.reserved);
   const unsigned ct = __ballot_sync(kFull, cnt.contract);
   const unsigned sl = __reduce_add_sync(kFull, cnt.stash_lookups);
+  const unsigned pr = __reduce_add_sync(kFull, cnt.probes);
   if (lane == 0) {
-    if (cnt.probes)
-      atomicAdd(&v.ctrl->stats[kStProbes], static_cast<unsigned long long>(cnt.probes));
+    if (pr) atomicAdd(&v.ctrl->stats[kStProbes], static_cast<unsigned long long>(pr));
     if (sl) atomicAdd(&v.ctrl->stats[kStStashLookups], static_cast<unsigned long long>(sl));
     if (sd) atomicAdd(&v.ctrl->size, static_cast<unsigned long long>(static_cast<long long>(sd)));
     if (rp) atomicAdd(&v.ctrl->stats[kStReplaced], static_cast<unsigned long long>(rp));
@@ -446,11 +460,12 @@ __device__ __forceinline__ void flush_counters_block(const View& v, LaneCounters
   const unsigned cl = __reduce_add_sync(kFull, cnt.claimed);
   const unsigned of = __reduce_add_sync(kFull, cnt.overflowed);
   const unsigned sl = __reduce_add_sync(kFull, cnt.stash_lookups);
+  const unsigned pr = __reduce_add_sync(kFull, cnt.probes);
   const unsigned rs = __ballot_sync(kFull, cnt.reserved);
   const unsigned ct = __ballot_sync(kFull, cnt.contract);
   __syncwarp();
   if (lane == 0) {
-    scratch[0] = cnt.probes;
+    scratch[0] = pr;
     scratch[1] = sl;
     scratch[2] = static_cast<uint64_t>(static_cast<int64_t>(sd));
     scratch[3] = rp;
@@ -618,7 +633,7 @@ __device__ __forceinline__ void run_chunk(const View& v, uint32_t stash_n, const
   PendCas pc{0, 0, 0, 0, 0};
   Hit h{0, 0, 0, false};
   TagVec<S> t1, t2;
-  bool have_tags = false;
+  bool have_tags = false, acted = false;
 
   bool probed = false;
   if (sg && !sg->dead) {
@@ -628,12 +643,12 @@ __device__ __forceinline__ void run_chunk(const View& v, uint32_t stash_n, const
     probed = need == 0 || stage_round<S>(v, *sg, need, b1, lane);
     if (probed) {
       if (live) scan_staged<S>(sg->buf, lane, b1, key, h);
-      cnt.probes += __popc(need);
+      if (MODE != kModeInsert) cnt.probes += live;
       need = __ballot_sync(kFull, live && !h.ok);
       probed = need == 0 || stage_round<S>(v, *sg, need, b2, lane);
       if (probed) {
+        if (MODE != kModeInsert) cnt.probes += live && !h.ok;
         if (live && !h.ok) scan_staged<S>(sg->buf, lane, b2, key, h);
-        cnt.probes += __popc(need);
       }
     }
   }
@@ -646,16 +661,18 @@ __device__ __forceinline__ void run_chunk(const View& v, uint32_t stash_n, const
       const uint32_t t4 = tag_of(key) * 0x01010101u;
       const uint32_t m1 = tag_match<S>(t1, t4);
       const uint32_t m2 = b2 != b1 ? tag_match<S>(t2, t4) : 0u;
-      check_words<S, kRO>(v, b1, b2, m1, m2, key, h);
+      // an erase or replace issues its CAS at once, while the word's line is in L2
+      check_words<S, kRO>(v, b1, b2, m1, m2, key, h,
+                          [&] { act_on<MODE, S>(v, h, key, val, op, st, outv, pc); });
+      acted = h.ok;
     }
-    cnt.probes += __popc(__ballot_sync(kFull, live));
-    cnt.probes += __popc(__ballot_sync(kFull, live && (MODE == kModeInsert || !h.ok || h.b != b1)));
+    if (MODE != kModeInsert) {  // insert batches: see count_insert_probes()
+      cnt.probes += live;
+      cnt.probes += live && (!h.ok || h.b != b1);
+    }
   }
-  bool done = !live;
-  if (h.ok) {
-    done = true;
-    act_on<MODE, S>(v, h, key, val, op, st, outv, pc);
-  }
+  bool done = !live || h.ok;
+  if (h.ok && !acted) act_on<MODE, S>(v, h, key, val, op, st, outv, pc);
 
   // The stash (Section IV-A step 4) holds keys that found no bucket room.
   if (!done && stash_n) {
@@ -797,6 +814,7 @@ __global__ void __launch_bounds__(THREADS, ops_min_blocks(MODE, DEFER, STAGED, T
     }
   }
   if constexpr (DEFER) ovf_flush_block(ovf, ob, lane);
+  if constexpr (MODE == kModeInsert) count_insert_probes(cnt);
   flush_counters_block(v, cnt, lane, sums + (threadIdx.x >> 5) * 8, sums, 8);
 }
 
@@ -855,8 +873,8 @@ __global__ void __launch_bounds__(THREADS, ops_min_blocks(kModeFind, false, fals
         check_words<S, true>(v, cd.b1, cd.b2, tag_match<S>(t1, t4),
                              cd.b2 != cd.b1 ? tag_match<S>(t2, t4) : 0u, key, h);
       }
-      cnt.probes += __popc(__ballot_sync(kFull, live)) +
-                    __popc(__ballot_sync(kFull, live && (!h.ok || h.b != cd.b1)));
+      cnt.probes += live;
+      cnt.probes += live && (!h.ok || h.b != cd.b1);
       if (live && !h.ok && stash_n) {
         uint32_t pos;
         cnt.stash_lookups += 1;
@@ -982,7 +1000,6 @@ __global__ void __launch_bounds__(kPartThreads, 4)
           }
         }
       }
-      cnt.probes += 2 * __popc(__ballot_sync(kFull, live));
       if (sid != kNoOp) {
         words[o] = pack(key, val);
         rank[o] = static_cast<uint16_t>(atomicAdd(&hist[sid >> pl.shift], 1u));
@@ -1037,6 +1054,7 @@ __global__ void __launch_bounds__(kPartThreads, 4)
     }
     __syncthreads();
   }
+  count_insert_probes(cnt);
   flush_counters_block(v, cnt, lane, sums + (tid >> 5) * 8, sums, 8);
 }
 
@@ -1791,7 +1809,8 @@ __device__ void fused_checked(const View& v, uint32_t stash_n, const OpPtrs& a, 
       check_words<S, false>(v, b1, b2, tag_match<S>(t1, t4),
                             b2 != b1 ? tag_match<S>(t2, t4) : 0u, key, h);
     }
-    cnt.probes += __popc(need) + __popc(__ballot_sync(kFull, active && (!h.ok || h.b != b1)));
+    cnt.probes += active;
+    cnt.probes += active && (!h.ok || h.b != b1);
     if (h.ok) {
       done = true;
       act_on<kModeMixed, S>(v, h, key, val, op, st, outv, pc);
@@ -1929,8 +1948,8 @@ __device__ __forceinline__ void run_chunk_fused(const View& v, uint32_t stash_n,
     check_words<S, false>(v, b1, b2, tag_match<S>(t1, t4), b2 != b1 ? tag_match<S>(t2, t4) : 0u,
                           key, h);
   }
-  cnt.probes += __popc(__ballot_sync(kFull, open)) +
-                __popc(__ballot_sync(kFull, open && (!h.ok || h.b != b1)));
+  cnt.probes += open;
+  cnt.probes += open && (!h.ok || h.b != b1);
   if (h.ok) {
     done = true;
     act_on<kModeMixed, S>(v, h, key, val, op, st, outv, pc);

@@ -98,17 +98,28 @@ __device__ __forceinline__ uint32_t zero_bytes(uint32_t x) {
 // words, so claims that start at different bits rarely meet in one word.
 __device__ __forceinline__ uint32_t slot_of(uint32_t p) { return ((p & 7u) << 2) | (p >> 3); }
 
-// Slots whose tag equals `t4` (a tag in all four bytes); t4 = 0: free slots.
+// Slots that may hold the tag in all four bytes of `t4`: every slot whose tag
+// equals it, and possibly the slot after one of these when its tag differs
+// from it in the lowest bit only (the borrow of the byte below reaches it).
+// One operation less per tag word than the exact test; a lookup compares
+// the words' keys anyway.
 template <int S>
 __device__ __forceinline__ uint32_t tag_match(const TagVec<S>& t, uint32_t t4) {
   uint32_t m = 0;
 #pragma unroll
-  for (int q = 0; q < S / 4; ++q) m |= zero_bytes(t.w[q] ^ t4) >> (7 - q);
-  return m;
+  for (int q = 0; q < S / 4; ++q) {
+    const uint32_t x = t.w[q] ^ t4;
+    m = (m >> 1) + ((x - 0x01010101u) & ~x & 0x80808080u);
+  }
+  return S == 32 ? m : m >> 4;
 }
+// Slots whose tag is 0 (exact: a claim may only take a zero byte).
 template <int S>
 __device__ __forceinline__ uint32_t free_slots(const TagVec<S>& t) {
-  return tag_match<S>(t, 0u);
+  uint32_t m = 0;
+#pragma unroll
+  for (int q = 0; q < S / 4; ++q) m = (m >> 1) + zero_bytes(t.w[q]);
+  return S == 32 ? m : m >> 4;
 }
 
 // The first set bit of slot set m at or after bit `rot`, cyclically (m != 0).
