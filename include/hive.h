@@ -395,8 +395,9 @@ hive_status hive_multi_destroy(hive_multi* m);
  * the exact sizes (synchronous groups).  A scheduler that admits work by
  * memory uses these, and hive_capacity() of each table, instead of counting
  * inserts itself: erases make the bounds fall again.  Host-side; it queries
- * the batches' events and never waits.  INVALID_ARG for NULL pointers or
- * n_tables above the group's. */
+ * the batches' events and never waits, except that a synchronous group of
+ * fixed tables waits here for its newest batch.  INVALID_ARG for NULL pointers
+ * or n_tables above the group's. */
 hive_status hive_multi_bounds(hive_multi* m, uint64_t* out, uint32_t n_tables);
 
 /* Insert into a FIXED-capacity table without allocating anything.  The paper

@@ -1,7 +1,9 @@
-"""Builds libhive_gb300.so in-tree with nvcc for sm_103a (GB300).
+"""Builds libhive_gb300.so in-tree with nvcc for sm_103a (GB300), and the
+native call path of the Python binding (hive_binding.so) with g++.
 
-Two translation units compile in parallel: the kernels (CUDA) and the host
-library (C++ using the CUDA runtime).  The CUDA runtime is linked statically.
+The translation units compile in parallel: the kernels (CUDA), the host
+library (C++ using the CUDA runtime, linked statically) and the binding, which
+uses the installed torch's headers.
 """
 from __future__ import annotations
 
@@ -18,6 +20,8 @@ LIB = os.path.join(OUT_DIR, "libhive_gb300.so")
 SOURCES = ["hive_kernels.cu", "hive32_kernels.cu", "hive_host.cpp", "hive32.cpp", "hive_multi.cpp",
            "hive_hostio.cpp", "hive_vmm.cpp", "hive_contract.cpp", "hive_noalloc.cu"]
 HEADERS = ["hive_internal.h", "hive_device.cuh", "hive_tags.cuh"]
+BINDING = os.path.join(OUT_DIR, "hive_binding.so")
+BINDING_SRC = "hive_binding.cpp"
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -27,13 +31,39 @@ def nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS]
+    t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
+    deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS + [BINDING_SRC]]
     deps.append(os.path.join(ROOT, "include", "hive.h"))
     deps.append(os.path.abspath(__file__))
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def build_binding() -> str:
+    """hive_binding.so: a CPython module compiled against the installed torch."""
+    import sysconfig
+
+    import torch
+
+    base = os.path.dirname(torch.__file__)
+    inc = os.path.join(base, "include")
+    lib = os.path.join(base, "lib")
+    cuda = os.path.dirname(os.path.dirname(nvcc())) if os.sep in nvcc() else "/usr/local/cuda"
+    tmp = BINDING + f".{os.getpid()}.tmp"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           "-I", os.path.join(ROOT, "include"), "-isystem", inc,
+           "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"),
+           "-isystem", os.path.join(cuda, "include"),
+           "-isystem", sysconfig.get_paths()["include"],
+           os.path.join(CSRC, BINDING_SRC), "-o", tmp, "-L", lib,
+           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", f"-Wl,-rpath,{lib}"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed for {BINDING_SRC}:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, BINDING)
+    return BINDING
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
@@ -55,8 +85,10 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
             sys.stderr.write(r.stderr)
         return obj
 
-    with ThreadPoolExecutor(len(SOURCES)) as ex:
+    with ThreadPoolExecutor(len(SOURCES) + 1) as ex:
+        binding = ex.submit(build_binding)
         objs = list(ex.map(compile_one, SOURCES))
+        binding.result()
     tmp = LIB + f".{os.getpid()}.tmp"
     cmd = [nvcc(), *ARCH, "-shared", "-o", tmp, *objs]
     r = subprocess.run(cmd, capture_output=True, text=True)

@@ -88,6 +88,10 @@ struct hive_multi {
   unsigned long long* d_gather = nullptr;
   unsigned long long* h_gather = nullptr;
   std::vector<uint64_t> ub;  // asynchronous mode: upper bound of each size
+  // synchronous groups of fixed tables: tables whose gathered size is still to
+  // be taken, and whether there are any
+  std::vector<char> stale;
+  bool untaken = false;
   cudaGraphExec_t graph = nullptr;
   cudaStream_t cap_stream = nullptr;
   std::vector<MultiJob> jobs;
@@ -181,6 +185,21 @@ void refresh_bounds(hive_multi* m) {
     if (sl.seq && sl.seq <= newest->seq) sl.applied = true;
 }
 
+// Synchronous group of fixed tables: waits for the newest batch and takes the
+// gathered sizes of the tables that batches have touched since.
+cudaError_t take_sizes(hive_multi* m) {
+  if (!m->untaken) return cudaSuccess;
+  const cudaError_t e = cudaEventSynchronize(m->slot[(m->seq - 1) & 1].done);
+  if (e != cudaSuccess) return e;
+  for (size_t t = 0; t < m->tables.size(); ++t)
+    if (m->stale[t]) {
+      m->tables[t]->size_host = m->ub[t] = m->h_gather[2 * t];
+      m->stale[t] = 0;
+    }
+  m->untaken = false;
+  return cudaSuccess;
+}
+
 void release(hive_multi* m) {
   if (m->graph) cudaGraphExecDestroy(m->graph);
   if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
@@ -226,6 +245,7 @@ hive_status hive_multi_create(hive_table* const* tables, uint32_t n_tables, uint
     m->tables.push_back(tables[i]);
     m->any_resizable |= tables[i]->cfg.resizable != 0;
     m->ub.push_back(tables[i]->size_host);
+    m->stale.push_back(0);
   }
   m->max_segs = max_segments;
   m->max_ops = max_ops;
@@ -270,7 +290,10 @@ hive_status hive_multi_destroy(hive_multi* m) {
 hive_status hive_multi_bounds(hive_multi* m, uint64_t* out, uint32_t n_tables) {
   if (!m || !out) return mfail(HIVE_ERR_INVALID_ARG, "group and out must not be NULL");
   if (n_tables > m->tables.size()) return mfail(HIVE_ERR_INVALID_ARG, "n_tables above the group's");
-  if (m->async) refresh_bounds(m);
+  if (m->async)
+    refresh_bounds(m);
+  else if (!m->any_resizable)
+    MCK(take_sizes(m));
   for (uint32_t t = 0; t < n_tables; ++t) out[t] = m->async ? m->ub[t] : m->tables[t]->size_host;
   return HIVE_OK;
 }
@@ -426,6 +449,13 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
     m->ub[t] += ins[t];
   }
 
+  // nothing of a group of fixed tables depends on the batch's outcome
+  // (hive_multi_bounds takes the sizes when it is asked)
+  if (!m->async && !m->any_resizable) {
+    for (uint32_t t : touched) m->stale[t] = 1;
+    m->untaken = true;
+    return HIVE_OK;
+  }
   if (m->async) return HIVE_OK;
 
   // exact mode: take the sizes and contract (one synchronisation for all tables)

@@ -17,6 +17,7 @@ import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "_build", "libhive_gb300.so")
+BINDING_PATH = os.path.join(_HERE, "_build", "hive_binding.so")
 
 # Status codes (include/hive.h)
 HIVE_OK = 0
@@ -168,6 +169,35 @@ def load_library(path: str = LIB_PATH):
         return L
 
 
+_native = None  # the native call path (csrc/hive_binding.cpp)
+_fn = {}        # addresses of the C ABI's functions, for the native call path
+
+
+def _load_native(L):
+    """Load hive_binding.so: the calls of plain tensors in native code.  It
+    returns NotImplemented for anything else, which the Python code below then
+    handles or refuses."""
+    global _native
+    with _lock:
+        if _native is not None:
+            return _native
+        import importlib.util
+
+        import torch  # noqa: F401  (the module links against it)
+
+        if not os.path.exists(BINDING_PATH):
+            raise RuntimeError(f"{BINDING_PATH} is not built; run __graft_entry__.build()")
+        for name in ("hive_insert", "hive_insert_noalloc", "hive_find", "hive_erase",
+                     "hive_execute", "hive_execute_fused", "hive_multi_execute", "hive32_insert",
+                     "hive32_find", "hive32_erase", "hive32_execute"):
+            _fn[name] = C.cast(getattr(L, name), C.c_void_p).value
+        spec = importlib.util.spec_from_file_location("hive_binding", BINDING_PATH)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        _native = mod
+        return _native
+
+
 def _raise(L, code):
     if code != HIVE_OK:
         raise HiveError(code, L.hive_last_error().decode(errors="replace"))
@@ -247,12 +277,15 @@ class HiveTable:
         h = C.c_void_p()
         _raise(self._L, self._L.hive_create(C.byref(cfg), _stream_ptr(stream), C.byref(h)))
         self._h = h
+        self._hp = h.value
+        self._N = _load_native(self._L)
 
     # -- lifetime ---------------------------------------------------------
     def close(self):
         if getattr(self, "_h", None):
             self._L.hive_destroy(self._h)
             self._h = None
+            self._hp = 0
 
     def __del__(self):
         try:
@@ -269,6 +302,11 @@ class HiveTable:
     # -- operations -------------------------------------------------------
     def insert(self, keys, vals, status=True, stream=None):
         """Insert/Replace.  Returns the per-op status tensor (uint8) or None."""
+        r = self._N.insert(_fn["hive_insert"], self._hp, keys, vals, status, stream)
+        if r is not NotImplemented:
+            if r[0]:
+                _raise(self._L, r[0])
+            return r[1]
         torch = _torch()
         n = keys.numel()
         st = None
@@ -284,6 +322,11 @@ class HiveTable:
     def insert_noalloc(self, keys, vals, status=True, stream=None):
         """hive_insert_noalloc: the fixed-table insert that allocates nothing
         (for callers that must not call cudaMalloc); at most 2^18 ops."""
+        r = self._N.insert(_fn["hive_insert_noalloc"], self._hp, keys, vals, status, stream)
+        if r is not NotImplemented:
+            if r[0]:
+                _raise(self._L, r[0])
+            return r[1]
         torch = _torch()
         n = keys.numel()
         st = None
@@ -298,6 +341,11 @@ class HiveTable:
 
     def find(self, keys, vals_out=None, found=True, stream=None):
         """Search.  Returns (values, found-flags or None); values are 0 on a miss."""
+        r = self._N.find(_fn["hive_find"], self._hp, keys, vals_out, found, stream)
+        if r is not NotImplemented:
+            if r[0]:
+                _raise(self._L, r[0])
+            return r[1], r[2]
         torch = _torch()
         n = keys.numel()
         if vals_out is None:
@@ -313,6 +361,11 @@ class HiveTable:
         return vals_out, fo
 
     def erase(self, keys, status=True, stream=None):
+        r = self._N.erase(_fn["hive_erase"], self._hp, keys, status, stream)
+        if r is not NotImplemented:
+            if r[0]:
+                _raise(self._L, r[0])
+            return r[1]
         torch = _torch()
         n = keys.numel()
         st = None
@@ -327,6 +380,12 @@ class HiveTable:
     def execute(self, ops, keys, vals=None, stream=None, fused=False):
         """Mixed batch.  Returns (values, status).  fused=True runs it as one
         concurrent kernel (hive_execute_fused) instead of the phased launches."""
+        r = self._N.execute(_fn["hive_execute_fused" if fused else "hive_execute"], self._hp, ops,
+                            keys, vals, stream)
+        if r is not NotImplemented:
+            if r[0]:
+                _raise(self._L, r[0])
+            return r[1], r[2]
         torch = _torch()
         n = keys.numel()
         vo = torch.empty(n, dtype=keys.dtype, device=keys.device)
@@ -472,11 +531,14 @@ class Hive32Table:
         h = C.c_void_p()
         _raise(self._L, self._L.hive32_create(C.byref(cfg), _stream_ptr(stream), C.byref(h)))
         self._h = h
+        self._hp = h.value
+        self._N = _load_native(self._L)
 
     def close(self):
         if getattr(self, "_h", None):
             self._L.hive32_destroy(self._h)
             self._h = None
+            self._hp = 0
 
     def __del__(self):
         try:
@@ -485,6 +547,11 @@ class Hive32Table:
             pass
 
     def insert(self, keys, vals=None, status=True, stream=None):
+        r = self._N.insert(_fn["hive32_insert"], self._hp, keys, vals, status, stream)
+        if r is not NotImplemented:
+            if r[0]:
+                _raise(self._L, r[0])
+            return r[1]
         torch = _torch()
         n = keys.numel()
         st = torch.empty(n, dtype=torch.uint8, device=keys.device) if status is True else (
@@ -495,6 +562,11 @@ class Hive32Table:
         return st
 
     def find(self, keys, vals_out=None, found=True, stream=None):
+        r = self._N.find(_fn["hive32_find"], self._hp, keys, vals_out, found, stream)
+        if r is not NotImplemented:
+            if r[0]:
+                _raise(self._L, r[0])
+            return r[1], r[2]
         torch = _torch()
         n = keys.numel()
         if vals_out is None:
@@ -507,6 +579,11 @@ class Hive32Table:
         return vals_out, fo
 
     def erase(self, keys, status=True, stream=None):
+        r = self._N.erase(_fn["hive32_erase"], self._hp, keys, status, stream)
+        if r is not NotImplemented:
+            if r[0]:
+                _raise(self._L, r[0])
+            return r[1]
         torch = _torch()
         n = keys.numel()
         st = torch.empty(n, dtype=torch.uint8, device=keys.device) if status is True else (
@@ -516,6 +593,11 @@ class Hive32Table:
         return st
 
     def execute(self, ops, keys, vals=None, stream=None):
+        r = self._N.execute(_fn["hive32_execute"], self._hp, ops, keys, vals, stream)
+        if r is not NotImplemented:
+            if r[0]:
+                _raise(self._L, r[0])
+            return r[1], r[2]
         torch = _torch()
         n = keys.numel()
         vo = torch.empty(n, dtype=keys.dtype, device=keys.device)
@@ -575,12 +657,19 @@ class HiveMulti:
                                                   int(max_ops), flags,
                                                   _stream_ptr(stream), C.byref(h)))
         self._h = h
+        self._hp = h.value
+        self._N = _load_native(self._L)
 
     def execute(self, segments, stream=None):
         """segments: iterable of dicts with keys table, ops, keys and optionally
         vals, vals_out, status (CUDA tensors, or pinned CPU tensors that the
         kernels use in place) and n_insert (int)."""
         segs = list(segments)
+        code = self._N.multi(_fn["hive_multi_execute"], self._hp, segs, stream)
+        if code is not NotImplemented:
+            if code:
+                _raise(self._L, code)
+            return
         arr = (Segment * max(len(segs), 1))()
         for i, g in enumerate(segs):
             n = g["keys"].numel()
@@ -606,6 +695,7 @@ class HiveMulti:
         if getattr(self, "_h", None):
             self._L.hive_multi_destroy(self._h)
             self._h = None
+            self._hp = 0
 
     def __del__(self):
         try:
