@@ -332,6 +332,7 @@ __device__ __forceinline__ void run_chunk32(const View32& v, uint32_t stash_n, c
 template <int MODE, int LAYOUT>
 __global__ void __launch_bounds__(kOps32Threads, (MODE == kModeInsert || MODE == kModeMixed) ? 4 : 6)
     k32_ops(View32 v, Ops32 a, uint64_t n, List32 ovf, int prefetch_tags) {
+  pdl_trigger();
   if (prefetch_tags) prefetch_l2_grid(v.tags, static_cast<uint64_t>(v.nb) * kS32);
   const int lane = threadIdx.x & 31;
   const uint32_t warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -508,6 +509,8 @@ __device__ __forceinline__ void overflow32_item(const View32& v, uint32_t word0,
 
 template <int LAYOUT>
 __global__ void __launch_bounds__(256) k32_overflow(View32 v, List32 in, uint8_t* status) {
+  pdl_trigger();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const unsigned warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -562,6 +565,7 @@ __device__ void bitonic32(uint32_t* a, unsigned P) {
 template <int LAYOUT>
 __global__ void __launch_bounds__(kMaint32Threads) k32_maint(View32 v) {
   extern __shared__ uint32_t smem_m32[];
+  pdl_wait();
   using E = E32<LAYOUT>;
   __shared__ unsigned s_reins, s_live;
   Ctrl* c = v.ctrl;
@@ -687,19 +691,15 @@ cudaError_t launch32_ops(int mode, const View32& v, const Ops32& a, uint64_t n, 
 cudaError_t launch32_overflow(const View32& v, const List32& in, uint8_t* status, int blocks,
                               cudaStream_t s) {
   if (v.layout == HIVE32_KEY_ONLY)
-    k32_overflow<HIVE32_KEY_ONLY><<<blocks, 256, 0, s>>>(v, in, status);
-  else
-    k32_overflow<HIVE32_KEY16_VAL16><<<blocks, 256, 0, s>>>(v, in, status);
-  return cudaGetLastError();
+    return launch_dependent(k32_overflow<HIVE32_KEY_ONLY>, blocks, 256, 0, s, v, in, status);
+  return launch_dependent(k32_overflow<HIVE32_KEY16_VAL16>, blocks, 256, 0, s, v, in, status);
 }
 
 cudaError_t launch32_maint(const View32& v, cudaStream_t s) {
   const size_t smem = kMaint32SmemWords * 4;
   if (v.layout == HIVE32_KEY_ONLY)
-    k32_maint<HIVE32_KEY_ONLY><<<1, kMaint32Threads, smem, s>>>(v);
-  else
-    k32_maint<HIVE32_KEY16_VAL16><<<1, kMaint32Threads, smem, s>>>(v);
-  return cudaGetLastError();
+    return launch_dependent(k32_maint<HIVE32_KEY_ONLY>, 1, kMaint32Threads, smem, s, v);
+  return launch_dependent(k32_maint<HIVE32_KEY16_VAL16>, 1, kMaint32Threads, smem, s, v);
 }
 
 cudaError_t setup32(int layout, int* blocks_per_sm) {

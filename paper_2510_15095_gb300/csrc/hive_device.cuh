@@ -139,6 +139,31 @@ __device__ __forceinline__ void lds_frag(const uint64_t* p, uint64_t& a, uint64_
 __device__ __forceinline__ void fence_acq_rel_gpu() {
   asm volatile("fence.acq_rel.gpu;" ::: "memory");
 }
+// Programmatic dependent launch.  A kernel of a call's chain lets the next one
+// be put on the SMs while it runs (pdl_trigger), and that one does nothing
+// before pdl_wait() has seen its predecessor complete with all its writes; so
+// only the launch overlaps.  Without the launch attribute both do nothing.
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Launches a kernel that calls pdl_wait() as the dependent of the stream's
+// previous kernel.  Three launches of a small mixed batch: 15 -> 11 us.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem,
+                             cudaStream_t s, Args... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
 // Asks L2 to fetch [p, p + bytes) from memory (bytes a multiple of 16, p
 // 16-byte aligned); nothing waits for it.
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {

@@ -104,8 +104,8 @@ struct PartList {
   uint32_t shift;    // slot index >> shift = region
 };
 
-// One (table, op range) of a multi-table batch; 64 bytes.
-struct MultiSeg {
+// One (table, op range) of a multi-table batch, with the table's view.
+struct alignas(16) MultiSeg {
   uint32_t table;        // index into the batch's view array
   uint32_t n;            // ops
   uint32_t chunk0;       // first 32-op chunk of this segment within the batch
@@ -115,7 +115,7 @@ struct MultiSeg {
   const uint32_t* vals;  // insert values (nullable)
   uint32_t* vals_out;    // find results (nullable)
   uint8_t* status;       // per-op status (nullable)
-  uint64_t pad2;
+  View v;
 };
 
 // One split launch of one table inside a wave of a multi-table batch.
@@ -184,19 +184,20 @@ cudaError_t launch_fused(const View& v, const uint8_t* ops, const uint32_t* keys
                          List pend, int resizable, const Launch& L, cudaStream_t s);
 cudaError_t launch_count_inserts(const uint8_t* ops, uint64_t n, unsigned int* out,
                                  cudaStream_t s);
-cudaError_t launch_multi_ops(int S, const MultiHdr* hdr, const MultiSeg* segs, const View* views,
-                             List ovf, const Launch& L, cudaStream_t s);
-cudaError_t launch_multi_overflow(int S, const MultiSeg* segs, const View* views, List in,
-                                  const Launch& L, cudaStream_t s);
+cudaError_t launch_multi_ops(int S, const MultiHdr* hdr, const MultiSeg* segs, List ovf,
+                             const Launch& L, cudaStream_t s);
+// Copies `bytes` (rounded up to 16) of pinned host memory to the device.
+cudaError_t launch_stage(void* dst, const void* src, size_t bytes, cudaStream_t s);
+cudaError_t launch_multi_overflow(int S, const MultiSeg* segs, List in, const Launch& L,
+                                  cudaStream_t s);
 cudaError_t launch_multi_maint(int S, const MultiHdr* hdr, const View* views,
-                               const uint32_t* touched, uint32_t max_tables, cudaStream_t s);
+                               const uint32_t* touched, uint32_t max_tables, unsigned* ovf_count,
+                               unsigned long long* out, cudaStream_t s);
 cudaError_t launch_multi_split(int S, const MultiJob* jobs, uint32_t n_jobs, uint32_t total_pairs,
                                const View* views, cudaStream_t s);
 cudaError_t launch_fill_u32(uint32_t* p, uint64_t n, uint32_t value, cudaStream_t s);
 cudaError_t launch_hash(const uint32_t* keys, uint64_t n, uint32_t* h1, uint32_t* h2,
                         cudaStream_t s);
-cudaError_t launch_multi_gather(const MultiHdr* hdr, const View* views, const uint32_t* touched,
-                                uint32_t max_tables, unsigned long long* out, cudaStream_t s);
 cudaError_t query_occupancy(Launch* L, int S);
 
 // ---- tables with 32-bit entries (hive32_*) ----

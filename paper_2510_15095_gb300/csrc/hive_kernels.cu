@@ -776,6 +776,7 @@ constexpr int kDeferBuf = 128;  // entries of each warp's buffer of new keys
 template <int MODE, int S, bool DEFER, int THREADS, bool STAGED>
 __global__ void __launch_bounds__(THREADS, ops_min_blocks(MODE, DEFER, STAGED, THREADS))
     k_ops(View v, OpPtrs a, uint64_t n, List ovf, int prefetch_tags) {
+  pdl_trigger();
   // probes read tags at random; a large batch first asks L2 for the whole tag
   // array in sequential pieces
   if (prefetch_tags) prefetch_l2_grid(v.tags, static_cast<uint64_t>(v.nb) * S);
@@ -927,6 +928,7 @@ constexpr int kPartTile = 2048;
 template <int S>
 __global__ void __launch_bounds__(kPartThreads, 4)
     k_insert_part(View v, OpPtrs a, uint64_t n, List ovf, PartList pl, int prefetch_tags) {
+  pdl_trigger();
   if (prefetch_tags) prefetch_l2_grid(v.tags, static_cast<uint64_t>(v.nb) * S);
   __shared__ uint64_t words[kPartTile];
   __shared__ uint32_t slots[kPartTile];
@@ -1064,6 +1066,8 @@ __global__ void __launch_bounds__(kPartThreads, 4)
 constexpr uint32_t kStoreTiles = 32;
 template <int S>
 __global__ void __launch_bounds__(256) k_insert_store(View v, uint32_t ntiles, PartList pl) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ uint32_t taken;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t groups = (ntiles + kStoreTiles - 1) / kStoreTiles;
@@ -1104,6 +1108,8 @@ constexpr int kClaimThreads = 256;
 constexpr int kClaimBuf = 128;  // entries of each warp's buffer of full-bucket items
 template <int S>
 __global__ void __launch_bounds__(kClaimThreads, 4) k_claim(View v, List in, List out) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ __align__(16) uint64_t claim_smem[(kClaimThreads / 32) * 2 * kClaimBuf];
   const int lane = threadIdx.x & 31;
   OvfBuf ob = ovf_buf_init(claim_smem + (threadIdx.x >> 5) * 2 * kClaimBuf, kClaimBuf);
@@ -1400,6 +1406,8 @@ __device__ __forceinline__ void overflow_item(const View& v, uint64_t word0, uin
 template <int S>
 __global__ void __launch_bounds__(kOvfThreads, HIVE_OVF_MIN_BLOCKS)
     k_overflow(View v, List in, List pend, int resizable, uint8_t* __restrict__ status) {
+  pdl_trigger();
+  pdl_wait();
   // one item per group of S lanes at a time
   const int lane = threadIdx.x & 31;
   const unsigned group0 = (blockIdx.x * blockDim.x + threadIdx.x) / S;
@@ -1990,6 +1998,7 @@ constexpr int kFusedWarpWords = 3 * static_cast<int>(kFusedQ) + static_cast<int>
 template <int S>
 __global__ void __launch_bounds__(kOpsThreads, 3)
     k_fused(View v, OpPtrs a, uint64_t n, List pend, int resizable) {
+  pdl_trigger();
   __shared__ __align__(16) uint64_t fused_smem_words[(kOpsThreads / 32) * kFusedWarpWords];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
@@ -2148,6 +2157,7 @@ __device__ void maint_body(const View& v, uint64_t* smem, int mode = 0) {
 template <int S>
 __global__ void __launch_bounds__(kMaintThreads) k_maint(View v, int mode) {
   extern __shared__ uint64_t smem[];
+  pdl_wait();
   maint_body<S>(v, smem, mode);
 }
 
@@ -2303,12 +2313,18 @@ __device__ __forceinline__ OpPtrs seg_ptrs(const MultiSeg& S) {
 }
 
 // Each warp takes a contiguous run of chunks, so it changes table only at
-// segment boundaries and flushes its counters there.
+// segment boundaries and flushes its counters there.  A small batch is a chain
+// of dependent reads (segment, op, tags, word), so the segment of the first
+// chunk is found 32 ways at a time, and a segment descriptor carries its
+// table's view.  The descriptor sits in shared memory: in registers it cost
+// 200 bytes of spills per thread.
 template <int S>
 __global__ void __launch_bounds__(kOpsThreads, HIVE_MULTI_MIN_BLOCKS)
-    k_multi_ops(const MultiHdr* __restrict__ hdr, const MultiSeg* __restrict__ segs,
-                const View* __restrict__ views, List ovf) {
+    k_multi_ops(const MultiHdr* __restrict__ hdr, const MultiSeg* __restrict__ segs, List ovf) {
+  pdl_trigger();
+  __shared__ MultiSeg held[kOpsThreads / 32];
   const int lane = threadIdx.x & 31;
+  MultiSeg& sg = held[threadIdx.x >> 5];
   const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
   const uint32_t total = hdr->total_chunks;
@@ -2316,36 +2332,57 @@ __global__ void __launch_bounds__(kOpsThreads, HIVE_MULTI_MIN_BLOCKS)
   const uint32_t c0 = static_cast<uint32_t>(static_cast<uint64_t>(total) * w / nw);
   const uint32_t c1 = static_cast<uint32_t>(static_cast<uint64_t>(total) * (w + 1) / nw);
   if (c0 >= c1) return;
-  uint32_t lo = 0, hi = ns;  // last segment with chunk0 <= c0
+  // the last segment with chunk0 <= c0: [lo, hi) narrows to a 32nd per step
+  uint32_t lo = 0, hi = ns;
   while (hi - lo > 1) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (segs[mid].chunk0 <= c0) lo = mid; else hi = mid;
+    const uint32_t step = (hi - lo + 31) / 32;
+    const uint32_t at = lo + lane * step;
+    const unsigned le = __ballot_sync(kFull, at < hi && segs[at < hi ? at : lo].chunk0 <= c0);
+    const uint32_t k = 31 - __clz(le);  // lane 0 always holds
+    hi = min(hi, lo + (k + 1) * step);
+    lo += k * step;
   }
   uint32_t s = lo;
-  View v = views[segs[s].table];
-  uint32_t stash_n = v.ctrl->stash_n;
-  OpPtrs a = seg_ptrs(segs[s]);
+  auto take = [&](uint32_t i) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(segs + i);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(&sg);
+    __syncwarp();
+    for (uint32_t k = lane; k < sizeof(MultiSeg) / 4; k += 32) dst[k] = __ldg(src + k);
+    __syncwarp();
+  };
+  take(s);
+  uint32_t next0 = s + 1 < ns ? segs[s + 1].chunk0 : 0xFFFFFFFFu;
+  uint32_t stash_n = sg.v.ctrl->stash_n;
   LaneCounters cnt;
+  OpIn nxt = load_in<kModeMixed>(seg_ptrs(sg), c0 - sg.chunk0, sg.n, lane);
   for (uint32_t c = c0; c < c1; ++c) {
-    if (s + 1 < ns && segs[s + 1].chunk0 <= c) {
-      flush_counters(v, cnt, lane);
+    if (next0 <= c) {
+      flush_counters(sg.v, cnt, lane);
       do {
         ++s;
       } while (s + 1 < ns && segs[s + 1].chunk0 <= c);
-      v = views[segs[s].table];
-      stash_n = v.ctrl->stash_n;
-      a = seg_ptrs(segs[s]);
+      take(s);
+      next0 = s + 1 < ns ? segs[s + 1].chunk0 : 0xFFFFFFFFu;
+      stash_n = sg.v.ctrl->stash_n;
+      nxt = load_in<kModeMixed>(seg_ptrs(sg), c - sg.chunk0, sg.n, lane);
     }
-    run_chunk<kModeMixed, S>(v, stash_n, a, c - segs[s].chunk0, segs[s].n, ovf, s, cnt, lane);
+    const OpIn cur = nxt;
+    // the next chunk's inputs, unless another segment starts there
+    if (c + 1 < c1 && c + 1 < next0)
+      nxt = load_in<kModeMixed>(seg_ptrs(sg), c + 1 - sg.chunk0, sg.n, lane);
+    run_chunk<kModeMixed, S>(sg.v, stash_n, seg_ptrs(sg), c - sg.chunk0, sg.n, ovf, s, cnt, lane,
+                             nullptr, &cur);
   }
-  flush_counters(v, cnt, lane);
+  flush_counters(sg.v, cnt, lane);
 }
 
 // Steps 3-4 for the overflow list of a multi-table batch.  Inserts that find
 // no room are reported FULL (a resizable table grows before its next batch).
 template <int S>
 __global__ void __launch_bounds__(kOvfThreads)
-    k_multi_overflow(const MultiSeg* __restrict__ segs, const View* __restrict__ views, List in) {
+    k_multi_overflow(const MultiSeg* __restrict__ segs, List in) {
+  pdl_trigger();
+  pdl_wait();
   // one item per group of S lanes at a time
   const int lane = threadIdx.x & 31;
   const unsigned group0 = (blockIdx.x * blockDim.x + threadIdx.x) / S;
@@ -2356,7 +2393,7 @@ __global__ void __launch_bounds__(kOvfThreads)
   OvfCounters oc;
   for (unsigned it = group0; it < total; it += ngroups) {
     const uint32_t sg = in.seg[it];
-    const View v = views[segs[sg].table];
+    const View v = segs[sg].v;
     overflow_item<S>(v, in.words[it], in.idx[it], sg, segs[sg].status, 0, none, oc, lane);
     flush_ovf_counters(v, oc, lead);
   }
@@ -2364,15 +2401,28 @@ __global__ void __launch_bounds__(kOvfThreads)
 }
 
 // One CTA per table of the batch: stash maintenance (exits at once when
-// nothing changed).  The grid covers every table of the group, so a captured
-// graph serves batches of any composition.
+// nothing changed), then the table's size and stash fill for the host's resize
+// policy (entries of tables outside the batch are left as they were).  The
+// grid covers every table of the group, so a captured graph serves batches of
+// any composition.  Block 0 also empties the batch's overflow list for the
+// next batch.
 template <int S>
 __global__ void __launch_bounds__(256)
     k_multi_maint(const MultiHdr* __restrict__ hdr, const View* __restrict__ views,
-                  const uint32_t* __restrict__ touched) {
+                  const uint32_t* __restrict__ touched, unsigned* __restrict__ ovf_count,
+                  unsigned long long* __restrict__ out) {
   extern __shared__ uint64_t smem[];
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *ovf_count = 0;
   if (blockIdx.x >= hdr->n_touched) return;
-  maint_body<S>(views[touched[blockIdx.x]], smem);
+  const uint32_t t = touched[blockIdx.x];
+  maint_body<S>(views[t], smem);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const Ctrl* c = views[t].ctrl;
+    out[2 * t] = c->size;
+    out[2 * t + 1] = (static_cast<unsigned long long>(c->err) << 32) | c->stash_claims;
+  }
 }
 
 // One wave of split launches over many tables: warp w runs pair
@@ -2396,19 +2446,6 @@ __global__ void __launch_bounds__(256)
   split_pair<S>(v, J.src0 + (w - J.pair0), J.half, threadIdx.x & 31);
 }
 
-// Size and stash fill of each table of the batch, for the host's resize
-// policy (entries of tables outside the batch are left as they were).
-__global__ void k_multi_gather(const MultiHdr* __restrict__ hdr, const View* __restrict__ views,
-                               const uint32_t* __restrict__ touched,
-                               unsigned long long* __restrict__ out) {
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= hdr->n_touched) return;
-  const uint32_t t = touched[j];
-  const Ctrl* c = views[t].ctrl;
-  out[2 * t] = c->size;
-  out[2 * t + 1] = (static_cast<unsigned long long>(c->err) << 32) | c->stash_claims;
-}
-
 // BitHash1 and BitHash2 of n keys (hive_hash).
 __global__ void k_hash(const uint32_t* __restrict__ keys, uint64_t n, uint32_t* __restrict__ h1,
                        uint32_t* __restrict__ h2) {
@@ -2428,8 +2465,8 @@ __global__ void k_fill_u32(uint32_t* __restrict__ p, uint64_t n, uint32_t value)
 
 // Launches a kernel on `s`, inside the table's persisting L2 window over the
 // slot tags when it has one (a per-launch attribute: the stream is left as
-// it was).
-template <typename... KArgs, typename... Args>
+// it was).  DEP: as the dependent of the call's previous kernel (see pdl_wait).
+template <bool DEP = false, typename... KArgs, typename... Args>
 cudaError_t launch_in_window(const Launch& L, void (*kern)(KArgs...), unsigned grid,
                              unsigned block, size_t smem, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg{};
@@ -2437,20 +2474,24 @@ cudaError_t launch_in_window(const Launch& L, void (*kern)(KArgs...), unsigned g
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
+  cfg.attrs = at;
   if (L.l2_bytes) {
-    at[0].id = cudaLaunchAttributeAccessPolicyWindow;
-    at[0].val.accessPolicyWindow.base_ptr = L.l2_base;
-    at[0].val.accessPolicyWindow.num_bytes = L.l2_bytes;
-    at[0].val.accessPolicyWindow.hitRatio = L.l2_hit;
-    at[0].val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
-    at[0].val.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute& w = at[cfg.numAttrs++];
+    w.id = cudaLaunchAttributeAccessPolicyWindow;
+    w.val.accessPolicyWindow.base_ptr = L.l2_base;
+    w.val.accessPolicyWindow.num_bytes = L.l2_bytes;
+    w.val.accessPolicyWindow.hitRatio = L.l2_hit;
+    w.val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
+    w.val.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
+  }
+  if (DEP) {
+    cudaLaunchAttribute& d = at[cfg.numAttrs++];
+    d.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    d.val.programmaticStreamSerializationAllowed = 1;
   }
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
-
 // Large batches fetch the tag array into L2 first: when the probes of a batch
 // would touch about every second bucket's tags or more.
 template <int S>
@@ -2568,11 +2609,8 @@ cudaError_t launch_insert_part(const View& v, const uint32_t* keys, const uint32
     e = launch_in_window(L, k_insert_part<32>, blocks, kPartThreads, 0, s, v, a, n, ovf, pl, pf);
   if (e != cudaSuccess) return e;
   const unsigned sb = static_cast<unsigned>(L.num_sms) * 8;
-  if (v.S == 16)
-    k_insert_store<16><<<sb, 256, 0, s>>>(v, ntiles, pl);
-  else
-    k_insert_store<32><<<sb, 256, 0, s>>>(v, ntiles, pl);
-  return cudaGetLastError();
+  if (v.S == 16) return launch_dependent(k_insert_store<16>, sb, 256, 0, s, v, ntiles, pl);
+  return launch_dependent(k_insert_store<32>, sb, 256, 0, s, v, ntiles, pl);
 }
 
 cudaError_t launch_claim(const View& v, List in, uint64_t n, List out, const Launch& L,
@@ -2582,9 +2620,9 @@ cudaError_t launch_claim(const View& v, List in, uint64_t n, List out, const Lau
   const uint64_t cap = static_cast<uint64_t>(L.num_sms) * L.claim_blocks_per_sm;
   if (blocks > cap) blocks = cap;
   if (v.S == 16)
-    return launch_in_window(L, k_claim<16>, static_cast<unsigned>(blocks), kClaimThreads, 0, s, v,
+    return launch_in_window<true>(L, k_claim<16>, static_cast<unsigned>(blocks), kClaimThreads, 0, s, v,
                             in, out);
-  return launch_in_window(L, k_claim<32>, static_cast<unsigned>(blocks), kClaimThreads, 0, s, v, in,
+  return launch_in_window<true>(L, k_claim<32>, static_cast<unsigned>(blocks), kClaimThreads, 0, s, v, in,
                           out);
 }
 
@@ -2592,19 +2630,16 @@ cudaError_t launch_overflow(const View& v, List in, List pend, int resizable, ui
                             const Launch& L, cudaStream_t s) {
   const unsigned blocks = static_cast<unsigned>(L.num_sms * L.ovf_blocks_per_sm);
   if (v.S == 16)
-    return launch_in_window(L, k_overflow<16>, blocks, kOvfThreads, 0, s, v, in, pend, resizable,
+    return launch_in_window<true>(L, k_overflow<16>, blocks, kOvfThreads, 0, s, v, in, pend, resizable,
                             status);
-  return launch_in_window(L, k_overflow<32>, blocks, kOvfThreads, 0, s, v, in, pend, resizable,
+  return launch_in_window<true>(L, k_overflow<32>, blocks, kOvfThreads, 0, s, v, in, pend, resizable,
                           status);
 }
 
 cudaError_t launch_maintenance(const View& v, cudaStream_t s, int mode) {
   constexpr size_t smem = kMaintSmemWords * sizeof(uint64_t);
-  if (v.S == 16)
-    k_maint<16><<<1, kMaintThreads, smem, s>>>(v, mode);
-  else
-    k_maint<32><<<1, kMaintThreads, smem, s>>>(v, mode);
-  return cudaGetLastError();
+  if (v.S == 16) return launch_dependent(k_maint<16>, 1, kMaintThreads, smem, s, v, mode);
+  return launch_dependent(k_maint<32>, 1, kMaintThreads, smem, s, v, mode);
 }
 
 cudaError_t launch_split(const View& v_new, uint32_t src0, uint32_t count, uint32_t half,
@@ -2664,35 +2699,49 @@ cudaError_t launch_fill_u32(uint32_t* p, uint64_t n, uint32_t value, cudaStream_
   return cudaGetLastError();
 }
 
-cudaError_t launch_multi_ops(int S, const MultiHdr* hdr, const MultiSeg* segs, const View* views,
-                             List ovf, const Launch& L, cudaStream_t s) {
+cudaError_t launch_multi_ops(int S, const MultiHdr* hdr, const MultiSeg* segs, List ovf,
+                             const Launch& L, cudaStream_t s) {
   const unsigned blocks = static_cast<unsigned>(L.num_sms * L.multi_blocks_per_sm);
   if (S == 16)
-    k_multi_ops<16><<<blocks, kOpsThreads, 0, s>>>(hdr, segs, views, ovf);
+    k_multi_ops<16><<<blocks, kOpsThreads, 0, s>>>(hdr, segs, ovf);
   else
-    k_multi_ops<32><<<blocks, kOpsThreads, 0, s>>>(hdr, segs, views, ovf);
+    k_multi_ops<32><<<blocks, kOpsThreads, 0, s>>>(hdr, segs, ovf);
   return cudaGetLastError();
 }
 
-cudaError_t launch_multi_overflow(int S, const MultiSeg* segs, const View* views, List in,
-                                  const Launch& L, cudaStream_t s) {
-  const unsigned blocks = static_cast<unsigned>(L.num_sms * L.ovf_blocks_per_sm);
-  if (S == 16)
-    k_multi_overflow<16><<<blocks, kOvfThreads, 0, s>>>(segs, views, in);
-  else
-    k_multi_overflow<32><<<blocks, kOvfThreads, 0, s>>>(segs, views, in);
+namespace {
+// A batch's descriptors (tens of kilobytes) by a kernel that reads them over
+// the CPU-GPU link: a copy engine's turn between kernels costs 4 us more.
+__global__ void __launch_bounds__(1024)
+    k_stage(uint4* __restrict__ dst, const uint4* __restrict__ src, uint32_t n) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) dst[i] = src[i];
+}
+}  // namespace
+cudaError_t launch_stage(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+  const uint32_t n = static_cast<uint32_t>((bytes + 15) / 16);
+  if (!n) return cudaSuccess;
+  k_stage<<<(n + 1023) / 1024, 1024, 0, s>>>(static_cast<uint4*>(dst),
+                                             static_cast<const uint4*>(src), n);
   return cudaGetLastError();
+}
+cudaError_t launch_multi_overflow(int S, const MultiSeg* segs, List in, const Launch& L,
+                                  cudaStream_t s) {
+  const unsigned blocks = static_cast<unsigned>(L.num_sms * L.ovf_blocks_per_sm);
+  if (S == 16) return launch_dependent(k_multi_overflow<16>, blocks, kOvfThreads, 0, s, segs, in);
+  return launch_dependent(k_multi_overflow<32>, blocks, kOvfThreads, 0, s, segs, in);
 }
 
 cudaError_t launch_multi_maint(int S, const MultiHdr* hdr, const View* views,
-                               const uint32_t* touched, uint32_t max_tables, cudaStream_t s) {
+                               const uint32_t* touched, uint32_t max_tables, unsigned* ovf_count,
+                               unsigned long long* out, cudaStream_t s) {
   if (!max_tables) return cudaSuccess;
   constexpr size_t smem = kMaintSmemWords * sizeof(uint64_t);
   if (S == 16)
-    k_multi_maint<16><<<max_tables, 256, smem, s>>>(hdr, views, touched);
-  else
-    k_multi_maint<32><<<max_tables, 256, smem, s>>>(hdr, views, touched);
-  return cudaGetLastError();
+    return launch_dependent(k_multi_maint<16>, max_tables, 256, smem, s, hdr, views, touched,
+                            ovf_count, out);
+  return launch_dependent(k_multi_maint<32>, max_tables, 256, smem, s, hdr, views, touched,
+                          ovf_count, out);
 }
 
 cudaError_t launch_multi_split(int S, const MultiJob* jobs, uint32_t n_jobs, uint32_t total_pairs,
@@ -2703,13 +2752,6 @@ cudaError_t launch_multi_split(int S, const MultiJob* jobs, uint32_t n_jobs, uin
     k_multi_split<16><<<blocks, 256, 0, s>>>(jobs, n_jobs, total_pairs, views);
   else
     k_multi_split<32><<<blocks, 256, 0, s>>>(jobs, n_jobs, total_pairs, views);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_multi_gather(const MultiHdr* hdr, const View* views, const uint32_t* touched,
-                                uint32_t max_tables, unsigned long long* out, cudaStream_t s) {
-  if (!max_tables) return cudaSuccess;
-  k_multi_gather<<<(max_tables + 255) / 256, 256, 0, s>>>(hdr, views, touched, out);
   return cudaGetLastError();
 }
 

@@ -84,8 +84,8 @@ struct hive_multi {
   uint32_t* ovf_idx = nullptr;
   uint32_t* ovf_seg = nullptr;
   unsigned* d_count = nullptr;
-  // per-table size and stash fill after a batch (entries of touched tables)
-  unsigned long long* d_gather = nullptr;
+  // per-table size and stash fill after a batch (entries of touched tables),
+  // in pinned memory that the maintenance kernel writes
   unsigned long long* h_gather = nullptr;
   std::vector<uint64_t> ub;  // asynchronous mode: upper bound of each size
   // synchronous groups of fixed tables: tables whose gathered size is still to
@@ -153,14 +153,13 @@ hive_status enqueue_fixed(hive_multi* m, cudaStream_t s) {
   const MultiHdr* hd = hdr_of(m->d_stage);
   const View* dv = views_of(m, m->d_stage);
   const uint32_t* tc = touched_of(m, m->d_stage);
-  MCK(cudaMemsetAsync(m->d_count, 0, sizeof(unsigned), s));
   const int S = static_cast<int>(m->tables[0]->S);
-  MCK(launch_multi_ops(S, hd, segs_of(m, m->d_stage), dv, ovf, m->L, s));
-  MCK(launch_multi_overflow(S, segs_of(m, m->d_stage), dv, ovf, m->L, s));
-  MCK(launch_multi_maint(S, hd, dv, tc, nt, s));
-  MCK(launch_multi_gather(hd, dv, tc, nt, m->d_gather, s));
-  MCK(cudaMemcpyAsync(m->h_gather, m->d_gather, 2 * sizeof(unsigned long long) * nt,
-                      cudaMemcpyDeviceToHost, s));
+  const MultiSeg* segs = segs_of(m, m->d_stage);
+  MCK(launch_multi_ops(S, hd, segs, ovf, m->L, s));
+  MCK(launch_multi_overflow(S, segs, ovf, m->L, s));
+  // also writes the sizes to the host and empties the overflow list for the
+  // next batch
+  MCK(launch_multi_maint(S, hd, dv, tc, nt, m->d_count, m->h_gather, s));
   return HIVE_OK;
 }
 
@@ -212,7 +211,6 @@ void release(hive_multi* m) {
   cudaFree(m->ovf_idx);
   cudaFree(m->ovf_seg);
   cudaFree(m->d_count);
-  cudaFree(m->d_gather);
   if (m->h_gather) cudaFreeHost(m->h_gather);
   delete m;
 }
@@ -267,7 +265,7 @@ hive_status hive_multi_create(hive_table* const* tables, uint32_t n_tables, uint
   if (e == cudaSuccess) e = cudaMalloc(&m->ovf_idx, max_ops * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&m->ovf_seg, max_ops * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&m->d_count, sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMalloc(&m->d_gather, 2 * sizeof(unsigned long long) * n_tables);
+  if (e == cudaSuccess) e = cudaMemset(m->d_count, 0, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMallocHost(&m->h_gather, 2 * sizeof(unsigned long long) * n_tables);
   if (e == cudaSuccess && m->use_graph)
     e = cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking);
@@ -393,6 +391,7 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
     d.vals = g.vals;
     d.vals_out = g.vals_out;
     d.status = g.status;
+    d.v = make_view(m->tables[g.table]);
     chunk += static_cast<uint32_t>((g.n + 31) / 32);
   }
   hd->n_segs = n_segs;
@@ -406,7 +405,7 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   if (!m->jobs.empty())
     std::memcpy(jobs_of(m, h), m->jobs.data(), m->jobs.size() * sizeof(MultiJob));
   const size_t bytes = m->off_jobs + m->jobs.size() * sizeof(MultiJob);
-  MCK(cudaMemcpyAsync(m->d_stage, h, bytes, cudaMemcpyHostToDevice, s));
+  MCK(launch_stage(m->d_stage, h, bytes, s));
 
   // split waves, in order
   for (size_t w = 0; w < m->wave_begin.size(); ++w) {
