@@ -310,10 +310,9 @@ hive_status grow_for(hive_table* t, uint64_t n_ins, cudaStream_t s) {
 // call does not wait for the GPU here.
 hive_status grow_for_mixed(hive_table* t, const uint8_t* ops, uint64_t n, cudaStream_t s) {
   if (t->nb >= t->nb_max || !over_grow(t, t->size_host + n, t->nb)) return HIVE_OK;
-  HIVE_CK(cudaMemsetAsync(&t->ctrl->n_insert, 0, sizeof(unsigned), s));
-  HIVE_LAUNCH(t, HIVE_K_COUNT, s, launch_count_inserts(ops, n, &t->ctrl->n_insert, s));
-  hive_status st = readback(t, s);
-  if (st != HIVE_OK) return st;
+  HIVE_LAUNCH(t, HIVE_K_COUNT, s,
+              launch_count_inserts(ops, n, t->ctrl, &t->host_ctrl->n_insert, s));
+  HIVE_CK(cudaStreamSynchronize(s));
   return grow_for(t, t->host_ctrl->n_insert, s);
 }
 
@@ -328,9 +327,10 @@ hive_status finish_resizable(hive_table* t, uint8_t* status, cudaStream_t s,
   // waits for the GPU once.
   HIVE_LAUNCH(t, HIVE_K_MAINT, s,
               launch_maintenance(make_view(t), s,
-                                 kMaintStash | (pending_in_b ? kMaintUnlessPend : kMaintUnlessOvf)));
-  hive_status st = readback(t, s);
-  if (st != HIVE_OK) return st;
+                                 kMaintStash | (pending_in_b ? kMaintUnlessPend : kMaintUnlessOvf),
+                                 t->host_ctrl));
+  HIVE_CK(cudaStreamSynchronize(s));
+  hive_status st = HIVE_OK;
   bool in_b = pending_in_b, again = false;
   while ((in_b ? t->host_ctrl->pend_n : t->host_ctrl->ovf_n) != 0) {
     again = true;
@@ -351,9 +351,9 @@ hive_status finish_resizable(hive_table* t, uint8_t* status, cudaStream_t s,
     if (!did) break;
   }
   if (again) {
-    HIVE_LAUNCH(t, HIVE_K_MAINT, s, launch_maintenance(make_view(t), s, kMaintStash));
-    st = readback(t, s);
-    if (st != HIVE_OK) return st;
+    HIVE_LAUNCH(t, HIVE_K_MAINT, s,
+                launch_maintenance(make_view(t), s, kMaintStash, t->host_ctrl));
+    HIVE_CK(cudaStreamSynchronize(s));
   }
   t->size_host = t->host_ctrl->size;
 
@@ -444,9 +444,8 @@ hive_status hive::contract_table(hive_table* t, cudaStream_t s) {
     merged = true;
   }
   if (merged) {
-    HIVE_LAUNCH(t, HIVE_K_MAINT, s, launch_maintenance(make_view(t), s));
-    st = readback(t, s);
-    if (st != HIVE_OK) return st;
+    HIVE_LAUNCH(t, HIVE_K_MAINT, s, launch_maintenance(make_view(t), s, 0, t->host_ctrl));
+    HIVE_CK(cudaStreamSynchronize(s));
     t->size_host = t->host_ctrl->size;
     if (t->vmm) {
       // the work above has completed; buckets past nb are empty and unused,

@@ -57,10 +57,11 @@ struct alignas(128) Ctrl {
   unsigned int pend_n;       // entries in the pending list (no room found)
   unsigned int err;          // sticky error bits
   unsigned int merge_excess; // words a merge batch cannot keep in the low bucket
-  unsigned int n_insert;     // insert ops counted in a mixed batch
+  unsigned int n_insert;     // insert ops counted in a mixed batch (0 between calls)
   unsigned int defer_n;      // new keys of a mixed batch waiting for k_claim
   unsigned int part_next;    // next group of tiles of a store by region
-  unsigned int pad0[3];
+  unsigned int count_blocks; // blocks of that count that are done
+  unsigned int pad0[2];
   unsigned long long stats[kNumStats];
 };
 
@@ -174,7 +175,9 @@ enum : int {
   kMaintUnlessPend = 2,  // do nothing while the pending list (pend_n) holds items
   kMaintUnlessOvf = 4    // do nothing while list A (ovf_n) holds items
 };
-cudaError_t launch_maintenance(const View& v, cudaStream_t s, int mode = 0);
+// host_out (nullable): pinned copy of the control block, written at the end.
+cudaError_t launch_maintenance(const View& v, cudaStream_t s, int mode = 0,
+                               Ctrl* host_out = nullptr);
 cudaError_t launch_split(const View& v_new, uint32_t src0, uint32_t count, uint32_t half,
                          cudaStream_t s);
 cudaError_t launch_merge_excess(const View& v_new, uint32_t count, cudaStream_t s);
@@ -182,7 +185,9 @@ cudaError_t launch_merge(const View& v_new, uint32_t count, List ovf, cudaStream
 cudaError_t launch_fused(const View& v, const uint8_t* ops, const uint32_t* keys,
                          const uint32_t* vals, uint64_t n, uint32_t* vals_out, uint8_t* status,
                          List pend, int resizable, const Launch& L, cudaStream_t s);
-cudaError_t launch_count_inserts(const uint8_t* ops, uint64_t n, unsigned int* out,
+// Counts a batch's inserts into *host_out (pinned); ctrl->n_insert is 0 before
+// and after.
+cudaError_t launch_count_inserts(const uint8_t* ops, uint64_t n, Ctrl* ctrl, unsigned* host_out,
                                  cudaStream_t s);
 cudaError_t launch_multi_ops(int S, const MultiHdr* hdr, const MultiSeg* segs, List ovf,
                              const Launch& L, cudaStream_t s);

@@ -1642,9 +1642,10 @@ struct EvictQ {
 // moves the rest to the front (warp-wide).  Each key first tries both
 // buckets again (slots may have been freed since); the keys still without room
 // take a stash reservation for the warp's chains with one atomic, then run
-// their chains.
+// their chains.  Not inlined: few keys come here, and the chains' registers
+// would spill those of the probes (10^6 ops, S = 32: 80 -> 74 us).
 template <int S>
-__device__ void fused_drain(const View& v, EvictQ& q, uint8_t* status, const List& pend,
+__device__ __noinline__ void fused_drain(const View& v, EvictQ& q, uint8_t* status, const List& pend,
                             int resizable, OvfCounters& oc, int lane) {
   __syncwarp();
   const uint32_t m = q.n < 32 ? q.n : 32u;
@@ -1997,7 +1998,7 @@ constexpr int kFusedWarpWords = 3 * static_cast<int>(kFusedQ) + static_cast<int>
 
 template <int S>
 __global__ void __launch_bounds__(kOpsThreads, 3)
-    k_fused(View v, OpPtrs a, uint64_t n, List pend, int resizable) {
+    k_fused(const __grid_constant__ View v, OpPtrs a, uint64_t n, List pend, int resizable) {
   pdl_trigger();
   __shared__ __align__(16) uint64_t fused_smem_words[(kOpsThreads / 32) * kFusedWarpWords];
   const int lane = threadIdx.x & 31;
@@ -2155,10 +2156,19 @@ __device__ void maint_body(const View& v, uint64_t* smem, int mode = 0) {
 }
 
 template <int S>
-__global__ void __launch_bounds__(kMaintThreads) k_maint(View v, int mode) {
+__global__ void __launch_bounds__(kMaintThreads) k_maint(View v, int mode,
+                                                                Ctrl* __restrict__ host_out) {
   extern __shared__ uint64_t smem[];
   pdl_wait();
   maint_body<S>(v, smem, mode);
+  if (host_out) {
+    // the control block for a host that waits next, written to its pinned copy
+    __syncthreads();
+    constexpr int kWords = sizeof(Ctrl) / sizeof(unsigned long long);
+    if (threadIdx.x < kWords)
+      reinterpret_cast<unsigned long long*>(host_out)[threadIdx.x] =
+          reinterpret_cast<const unsigned long long*>(v.ctrl)[threadIdx.x];
+  }
 }
 
 // ----------------------------------------------------------------------------
@@ -2276,7 +2286,7 @@ __global__ void __launch_bounds__(256) k_merge(View v, uint32_t count, List ovf)
 // atomic per block.  Reads n bytes once: 2^22 codes in 5 us (25 with a byte
 // per load and an atomic per warp).
 __global__ void __launch_bounds__(256)
-    k_count_inserts(const uint8_t* __restrict__ ops, uint64_t n, unsigned* out) {
+    k_count_inserts(const uint8_t* __restrict__ ops, uint64_t n, Ctrl* ctrl, unsigned* host_out) {
   const uint64_t tid = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const uint64_t step = static_cast<uint64_t>(gridDim.x) * blockDim.x;
   uint64_t head = (16 - (reinterpret_cast<uintptr_t>(ops) & 15)) & 15;
@@ -2298,7 +2308,14 @@ __global__ void __launch_bounds__(256)
   c = __reduce_add_sync(kFull, c);
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(&sum, c);
   __syncthreads();
-  if (threadIdx.x == 0 && sum) atomicAdd(out, sum);
+  if (threadIdx.x != 0) return;
+  if (sum) atomicAdd(&ctrl->n_insert, sum);
+  __threadfence();
+  // the last block hands the total to the host and leaves both counts at zero
+  if (atomicAdd(&ctrl->count_blocks, 1u) == gridDim.x - 1) {
+    *host_out = atomicExch(&ctrl->n_insert, 0u);
+    ctrl->count_blocks = 0;
+  }
 }
 
 // ----------------------------------------------------------------------------
@@ -2636,10 +2653,10 @@ cudaError_t launch_overflow(const View& v, List in, List pend, int resizable, ui
                           status);
 }
 
-cudaError_t launch_maintenance(const View& v, cudaStream_t s, int mode) {
+cudaError_t launch_maintenance(const View& v, cudaStream_t s, int mode, Ctrl* host_out) {
   constexpr size_t smem = kMaintSmemWords * sizeof(uint64_t);
-  if (v.S == 16) return launch_dependent(k_maint<16>, 1, kMaintThreads, smem, s, v, mode);
-  return launch_dependent(k_maint<32>, 1, kMaintThreads, smem, s, v, mode);
+  if (v.S == 16) return launch_dependent(k_maint<16>, 1, kMaintThreads, smem, s, v, mode, host_out);
+  return launch_dependent(k_maint<32>, 1, kMaintThreads, smem, s, v, mode, host_out);
 }
 
 cudaError_t launch_split(const View& v_new, uint32_t src0, uint32_t count, uint32_t half,
@@ -2673,12 +2690,13 @@ cudaError_t launch_merge(const View& v_new, uint32_t count, List ovf, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t launch_count_inserts(const uint8_t* ops, uint64_t n, unsigned* out, cudaStream_t s) {
+cudaError_t launch_count_inserts(const uint8_t* ops, uint64_t n, Ctrl* ctrl, unsigned* host_out,
+                                 cudaStream_t s) {
   if (!n) return cudaSuccess;
   uint64_t blocks = (n / 16 + 255) / 256;
   if (blocks > 152 * 4) blocks = 152 * 4;
   if (blocks == 0) blocks = 1;
-  k_count_inserts<<<static_cast<unsigned>(blocks), 256, 0, s>>>(ops, n, out);
+  k_count_inserts<<<static_cast<unsigned>(blocks), 256, 0, s>>>(ops, n, ctrl, host_out);
   return cudaGetLastError();
 }
 
