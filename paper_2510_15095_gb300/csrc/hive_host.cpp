@@ -418,10 +418,8 @@ hive_status hive::contract_table(hive_table* t, cudaStream_t s) {
     trial.p = p;
     trial.nb = nb;
     const View vn = make_view(&trial);
-    HIVE_CK(cudaMemsetAsync(&t->ctrl->merge_excess, 0, sizeof(unsigned), s));
-    HIVE_LAUNCH(t, HIVE_K_MERGE, s, launch_merge_excess(vn, count, s));
-    st = readback(t, s);
-    if (st != HIVE_OK) return st;
+    HIVE_LAUNCH(t, HIVE_K_MERGE, s, launch_merge_excess(vn, count, t->host_ctrl, s));
+    HIVE_CK(cudaStreamSynchronize(s));
     const uint64_t free_stash = t->stash_cap - t->host_ctrl->stash_claims;
     if (t->host_ctrl->merge_excess > free_stash) {
       if (count > t->cfg.resize_batch) {
@@ -433,7 +431,6 @@ hive_status hive::contract_table(hive_table* t, cudaStream_t s) {
     }
     st = ensure_lists(t, static_cast<uint64_t>(count) * t->S);
     if (st != HIVE_OK) return st;
-    HIVE_CK(cudaMemsetAsync(&t->ctrl->ovf_n, 0, sizeof(unsigned), s));
     HIVE_LAUNCH(t, HIVE_K_MERGE, s, launch_merge(vn, count, list_a(t), s));
     t->M = trial.M;
     t->p = trial.p;

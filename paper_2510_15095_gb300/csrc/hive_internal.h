@@ -56,11 +56,11 @@ struct alignas(128) Ctrl {
   unsigned int ovf_n;        // entries in the overflow list (P1 -> P2)
   unsigned int pend_n;       // entries in the pending list (no room found)
   unsigned int err;          // sticky error bits
-  unsigned int merge_excess; // words a merge batch cannot keep in the low bucket
+  unsigned int merge_excess; // words a merge batch cannot keep in the low bucket (0 between calls)
   unsigned int n_insert;     // insert ops counted in a mixed batch (0 between calls)
   unsigned int defer_n;      // new keys of a mixed batch waiting for k_claim
   unsigned int part_next;    // next group of tiles of a store by region
-  unsigned int count_blocks; // blocks of that count that are done
+  unsigned int count_blocks; // blocks of a counting kernel that are done
   unsigned int pad0[2];
   unsigned long long stats[kNumStats];
 };
@@ -180,7 +180,10 @@ cudaError_t launch_maintenance(const View& v, cudaStream_t s, int mode = 0,
                                Ctrl* host_out = nullptr);
 cudaError_t launch_split(const View& v_new, uint32_t src0, uint32_t count, uint32_t half,
                          cudaStream_t s);
-cudaError_t launch_merge_excess(const View& v_new, uint32_t count, cudaStream_t s);
+// Words a merge batch cannot keep in the low buckets and the stash fill, into
+// the pinned host_out; empties list A.
+cudaError_t launch_merge_excess(const View& v_new, uint32_t count, Ctrl* host_out,
+                                cudaStream_t s);
 cudaError_t launch_merge(const View& v_new, uint32_t count, List ovf, cudaStream_t s);
 cudaError_t launch_fused(const View& v, const uint8_t* ops, const uint32_t* keys,
                          const uint32_t* vals, uint64_t n, uint32_t* vals_out, uint8_t* status,

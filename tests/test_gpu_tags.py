@@ -197,3 +197,45 @@ def test_bulk_inserts_stored_by_region(H, bs):
     check(H, t, d, np.concatenate([keys[:100_000], new[:100_000],
                                    W.take_keys(71, c, 100_000)[0]]))
     t.close()
+
+
+@pytest.mark.parametrize("bs", [16, 32])
+@pytest.mark.parametrize("n", [200_001, (1 << 18) - 1])
+def test_new_keys_wait_in_the_warp_queue(H, bs, n):
+    """Mixed batches of several chunks per warp that claim in the bulk kernel:
+    new keys wait in their warp's queue and claim 32 at a time, the last ones
+    at the end; on one table and as ragged segments of a multi-table batch."""
+    slots = 1 << 20
+    rng = np.random.default_rng(n + bs)
+    live, c = W.take_keys(81, 0, slots * 94 // 100)
+    new, _ = W.take_keys(81, c, n // 3)
+    ops, keys, vals = W.mixed_batch(rng, live, new, n // 3, n // 4, n - n // 3 - n // 4, seed=81)
+    o, k, v = torch.from_numpy(ops).cuda(), up(H, keys), up(H, vals)
+    d = oracle.Dict()
+    d.insert(live, W.values_for(live, 81))
+    ev, es = d.execute(ops, keys, vals)
+    t = H.HiveTable(slots, bucket_slots=bs)
+    t.insert(up(H, live), up(H, W.values_for(live, 81)))
+    vo, st = t.execute(o, k, v)
+    assert np.array_equal(st.cpu().numpy(), es) and np.array_equal(H.to_host_u32(vo), ev)
+    check(H, t, d, keys)
+    t.close()
+    # the same ops as segments on two tables, in cuts that end inside a chunk
+    tabs = [H.HiveTable(slots, bucket_slots=bs) for _ in range(2)]
+    for x in tabs:
+        x.insert(up(H, live), up(H, W.values_for(live, 81)))
+    cuts = [0, 1, 33, n // 2, n - 5, n]
+    m = H.HiveMulti(tabs, max_segments=16, max_ops=4 * n)
+    vo = torch.full((2, n), -1, dtype=torch.int32, device="cuda")
+    st = torch.full((2, n), 9, dtype=torch.uint8, device="cuda")
+    segs = [{"table": j, "ops": o[a:b].clone(), "keys": k[a:b].clone(), "vals": v[a:b].clone(),
+             "vals_out": vo[j, a:b], "status": st[j, a:b]}
+            for a, b in zip(cuts, cuts[1:]) for j in range(2)]
+    m.execute(segs)
+    for j in range(2):
+        assert np.array_equal(st[j].cpu().numpy(), es) and np.array_equal(H.to_host_u32(vo[j]), ev)
+        check(H, tabs[j], d, keys)
+    m.close()
+    for x in tabs:
+        assert x.check() == 0
+        x.close()
