@@ -83,6 +83,7 @@ struct View {
   uint32_t placement;    // 0 balanced, 1 BitHash1 first
   uint32_t S;            // slots per bucket: 16 or 32
   uint32_t stage_spin_limit;  // tries of a staged-copy wait before it gives up
+  uint32_t keep_words;   // word reads stay in L2 like the tags, else they leave first
 };
 
 // An op list handed from the bulk kernel to the eviction kernel.

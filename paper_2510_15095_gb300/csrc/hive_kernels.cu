@@ -75,11 +75,11 @@ __device__ __forceinline__ void ld_frag(const uint64_t* p, uint64_t& a, uint64_t
                : "l"(p)
                : "memory");
 }
-// One slot's word; RO as for ld_tags.
+// One slot's word; RO as for ld_tags, `keep` as in View::keep_words.
 template <bool RO>
-__device__ __forceinline__ uint64_t ld_word(const uint64_t* p) {
+__device__ __forceinline__ uint64_t ld_word(const uint64_t* p, bool keep) {
   uint64_t r;
-  const uint64_t pol = policy_pass();
+  const uint64_t pol = keep ? policy_keep() : policy_pass();
   if constexpr (RO)
     asm("ld.global.nc.L2::cache_hint.b64 %0, [%1], %2;" : "=l"(r) : "l"(p), "l"(pol));
   else
@@ -335,14 +335,15 @@ __device__ __forceinline__ void scan_staged(const uint64_t* sbuf, int lane, uint
 // match).
 template <int S, bool RO, class F>
 __device__ __forceinline__ void check_words(const View& v, uint32_t b1, uint32_t b2, uint32_t m1,
-                                            uint32_t m2, uint32_t key, Hit& h, F on_hit) {
+                                            uint32_t m2, uint32_t key, Hit& h, bool keep,
+                                            F on_hit) {
   const uint32_t rot = claim_rot(key);
   while (m1 | m2) {
     const bool in1 = m1 != 0;
     const uint32_t b = in1 ? b1 : b2;
     const uint32_t p = pick_slot(in1 ? m1 : m2, rot);
     const uint32_t slot = slot_of(p);
-    const uint64_t w = ld_word<RO>(v.buckets + static_cast<uint64_t>(b) * S + slot);
+    const uint64_t w = ld_word<RO>(v.buckets + static_cast<uint64_t>(b) * S + slot, keep);
     if (key_of(w) == key) {
       h = Hit{w, b, slot, true};
       on_hit();
@@ -357,8 +358,8 @@ __device__ __forceinline__ void check_words(const View& v, uint32_t b1, uint32_t
 
 template <int S, bool RO>
 __device__ __forceinline__ void check_words(const View& v, uint32_t b1, uint32_t b2, uint32_t m1,
-                                            uint32_t m2, uint32_t key, Hit& h) {
-  check_words<S, RO>(v, b1, b2, m1, m2, key, h, [] {});
+                                            uint32_t m2, uint32_t key, Hit& h, bool keep) {
+  check_words<S, RO>(v, b1, b2, m1, m2, key, h, keep, [] {});
 }
 
 // An erase or replace CAS issued by a probe, checked only at the end of the
@@ -736,7 +737,7 @@ __device__ __forceinline__ void run_chunk(const View& v, uint32_t stash_n, const
       const uint32_t m1 = tag_match<S>(t1, t4);
       const uint32_t m2 = b2 != b1 ? tag_match<S>(t2, t4) : 0u;
       // an erase or replace issues its CAS at once, while the word's line is in L2
-      check_words<S, kRO>(v, b1, b2, m1, m2, key, h,
+      check_words<S, kRO>(v, b1, b2, m1, m2, key, h, v.keep_words,
                           [&] { act_on<MODE, S>(v, h, key, val, op, st, outv, pc); });
       acted = h.ok;
     }
@@ -919,7 +920,7 @@ __global__ void __launch_bounds__(THREADS, ops_min_blocks(MODE, DEFER, STAGED, T
 // floor is 0.82 ms for the 2^25 hits, and false tag matches (30 of 255 per
 // bucket examined) make the rest.  In an L2-resident table the dependent
 // chain key -> tags -> word is the cost: 2^20 slots, 1.7 M lookups 77 -> 27 us.
-template <int S, int THREADS, int G>
+template <int S, int THREADS, int G, bool KEEP>
 __global__ void __launch_bounds__(THREADS, ops_min_blocks(kModeFind, false, false, THREADS))
     k_find(View v, const uint32_t* __restrict__ keys, uint64_t n, uint32_t* __restrict__ vals_out,
            uint8_t* __restrict__ found, int prefetch_tags) {
@@ -959,7 +960,7 @@ __global__ void __launch_bounds__(THREADS, ops_min_blocks(kModeFind, false, fals
         const TagVec<S> t2 = ld_tags<S, true>(v, cd.b2);
         const uint32_t t4 = tag_of(key) * 0x01010101u;
         check_words<S, true>(v, cd.b1, cd.b2, tag_match<S>(t1, t4),
-                             cd.b2 != cd.b1 ? tag_match<S>(t2, t4) : 0u, key, h);
+                             cd.b2 != cd.b1 ? tag_match<S>(t2, t4) : 0u, key, h, KEEP);
       }
       cnt.probes += live;
       cnt.probes += live && (!h.ok || h.b != cd.b1);
@@ -1059,7 +1060,7 @@ __global__ void __launch_bounds__(kPartThreads, 4)
         // key (no key is updated twice in a batch)
         Hit h{0, 0, 0, false};
         check_words<S, false>(v, cd.b1, cd.b2, tag_match<S>(t1, t4),
-                              cd.b2 != cd.b1 ? tag_match<S>(t2, t4) : 0u, key, h);
+                              cd.b2 != cd.b1 ? tag_match<S>(t2, t4) : 0u, key, h, true);
         uint64_t* sp = v.buckets + static_cast<uint64_t>(h.b) * S + h.slot;
         if (!h.ok && stash_n) {
           uint32_t pos;
@@ -1903,7 +1904,7 @@ __device__ void fused_checked(const View& v, uint32_t stash_n, const OpPtrs& a, 
       const TagVec<S> t2 = ld_tags<S, false>(v, b2);
       const uint32_t t4 = tag_of(key) * 0x01010101u;
       check_words<S, false>(v, b1, b2, tag_match<S>(t1, t4),
-                            b2 != b1 ? tag_match<S>(t2, t4) : 0u, key, h);
+                            b2 != b1 ? tag_match<S>(t2, t4) : 0u, key, h, false);
     }
     cnt.probes += active;
     cnt.probes += active && (!h.ok || h.b != b1);
@@ -2041,8 +2042,9 @@ __device__ __forceinline__ void run_chunk_fused(const View& v, uint32_t stash_n,
     const TagVec<S> t1 = ld_tags<S, false>(v, b1);
     const TagVec<S> t2 = ld_tags<S, false>(v, b2);
     const uint32_t t4 = tag_of(key) * 0x01010101u;
+    // the words leave L2 first here (10^6 ops on 2^24 slots: 147 us, 152 kept)
     check_words<S, false>(v, b1, b2, tag_match<S>(t1, t4), b2 != b1 ? tag_match<S>(t2, t4) : 0u,
-                          key, h);
+                          key, h, false);
   }
   cnt.probes += open;
   cnt.probes += open && (!h.ok || h.b != b1);
@@ -2641,12 +2643,10 @@ cudaError_t launch_ops_tt(const View& v, const OpPtrs& a, uint64_t n, List ovf, 
     // groups of four runs once every warp has at least four of them: with
     // fewer, rounding to whole groups leaves warps idle (1.7 M ops on 7296
     // warps: 33 us against 28)
-    if (chunks >= cap * warps_per_block * 16)
-      k_find<S, THREADS, 4><<<static_cast<unsigned>(cap), THREADS, 0, s>>>(
-          v, a.keys, n, a.vals_out, a.found, pf);
-    else
-      k_find<S, THREADS, 1><<<static_cast<unsigned>(blocks), THREADS, 0, s>>>(
-          v, a.keys, n, a.vals_out, a.found, pf);
+    const bool long_batch = chunks >= cap * warps_per_block * 16;
+    auto kern = long_batch ? (v.keep_words ? k_find<S, THREADS, 4, true> : k_find<S, THREADS, 4, false>)
+                           : (v.keep_words ? k_find<S, THREADS, 1, true> : k_find<S, THREADS, 1, false>);
+    kern<<<static_cast<unsigned>(blocks), THREADS, 0, s>>>(v, a.keys, n, a.vals_out, a.found, pf);
     return cudaGetLastError();
   } else
   return launch_in_window(L, k_ops<MODE, S, DEFER, THREADS, STAGED>, static_cast<unsigned>(blocks),
@@ -2654,10 +2654,11 @@ cudaError_t launch_ops_tt(const View& v, const OpPtrs& a, uint64_t n, List ovf, 
 }
 
 template <int MODE, int S, bool DEFER = false>
-cudaError_t launch_ops_t(const View& v, const uint8_t* ops, const uint32_t* keys,
+cudaError_t launch_ops_t(View v, const uint8_t* ops, const uint32_t* keys,
                          const uint32_t* vals, uint64_t n, uint32_t* vals_out, uint8_t* found,
                          uint8_t* status, List ovf, const Launch& L, cudaStream_t s) {
   const OpPtrs a{ops, keys, vals, vals_out, found, status};
+  if (MODE != kModeFind && n * 16 >= static_cast<uint64_t>(v.nb) * S) v.keep_words = 1;
   if constexpr (S == 32) {
     if (L.staged) return launch_ops_tt<MODE, S, DEFER, 256, true>(v, a, n, ovf, L, s);
   }
@@ -2889,7 +2890,7 @@ cudaError_t occupancy_mode(Launch* L) {
   int b = 0;
   cudaError_t e;
   if constexpr (MODE == kModeFind)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_find<S, T, 4>, T, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_find<S, T, 4, false>, T, 0);
   else
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ops<MODE, S, DEFER, T, false>, T, 0);
   L->ops_blocks_per_sm[MODE + (DEFER ? 1 : 0)] = b > 0 ? b : 1;
