@@ -74,6 +74,9 @@ View32 view32(const hive32_table* t) {
   v.stash_cap = t->stash_cap;
   v.max_evictions = t->cfg.max_evictions;
   v.lock_spin_limit = t->cfg.lock_spin_limit;
+  // Entries are worth keeping in L2 while they and the tags fit it (a set of
+  // 20 M slots: 36 M lookups 445 -> 419 us; 2^25 slots: 766 -> 786).
+  v.keep_words = t->nb * kS * (sizeof(uint32_t) + 1) <= (128ull << 20);
   v.layout = static_cast<int>(t->cfg.layout);
   return v;
 }

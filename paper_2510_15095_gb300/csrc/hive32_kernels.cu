@@ -94,11 +94,12 @@ __device__ __forceinline__ void flush32_block(const View32& v, const Counters32&
   }
 }
 
-// A slot's entry, sent through L2 first (RO: no kernel writes the table meanwhile).
+// A slot's entry; `keep` as in View::keep_words (RO: no kernel writes the table
+// meanwhile).
 template <bool RO>
-__device__ __forceinline__ uint32_t ld_entry(const uint32_t* p) {
+__device__ __forceinline__ uint32_t ld_entry(const uint32_t* p, bool keep) {
   uint32_t r;
-  const uint64_t pol = policy_pass();
+  const uint64_t pol = keep ? policy_keep() : policy_pass();
   if constexpr (RO)
     asm("ld.global.nc.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(r) : "l"(p), "l"(pol));
   else
@@ -249,7 +250,8 @@ __device__ __forceinline__ void run_chunk32(const View32& v, uint32_t stash_n, c
       const bool in1 = m1 != 0;
       const uint32_t b = in1 ? b1 : b2;
       const uint32_t p = pick_slot(in1 ? m1 : m2, rot);
-      const uint32_t w = ld_entry<kRO>(v.buckets + static_cast<uint64_t>(b) * kS32 + slot_of(p));
+      const uint32_t w = ld_entry<kRO>(v.buckets + static_cast<uint64_t>(b) * kS32 + slot_of(p),
+                                       v.keep_words);
       if (E::key(w) == key) {
         slot = slot_of(p);
         hb = b;

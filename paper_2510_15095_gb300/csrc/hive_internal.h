@@ -219,6 +219,7 @@ struct View32 {
   Ctrl* ctrl;
   uint32_t M, p, nb, stash_cap, max_evictions, lock_spin_limit;
   int layout;            // HIVE32_KEY16_VAL16 or HIVE32_KEY_ONLY
+  uint32_t keep_words;   // entry reads stay in L2 like the tags, else they leave first
 };
 struct Ops32 {
   const uint8_t* ops;
