@@ -443,10 +443,11 @@ def tables_leg(torch, H, dev, n_tables=1024, steps=8, seed=40):
         for st in range(steps) for t in range(n_tables) for i in range(2))
     caps_same = all(a.capacity() == b.capacity() for a, b in zip(sets[0], sets[1]))
     ops_total = int(nops.sum())
-    # step-level algorithmic bytes of the batched resizable arm (op I/O, every
-    # probed bucket, a written sector per claimed slot) over its wall time
+    # step-level algorithmic bytes of the batched resizable arm (op I/O, the
+    # tags of every probed bucket, a written sector per claimed slot; the words
+    # of hits are left out) over its wall time
     S = knobs["bucket_slots"]
-    byts = 14 * ops_total + 8 * S * probes + 32 * claims
+    byts = 14 * ops_total + S * probes + 32 * claims
     peak_gbs, peak_kind = measured_peak()
     for tabs in sets:
         for tb in tabs:
@@ -564,9 +565,10 @@ def hive32_leg(torch, H, dev, slots=SLOTS, n_find=N_FIND, seed=90, reps=3):
                          f"batch of {n_mix} ops 1:2:1"),
             "insert_gops": n / ins_ms / 1e6, "find_gops": n_find / f_ms / 1e6,
             "mixed_gops": n_mix / m_ms / 1e6, "probes_per_find": probes,
-            # key in, value + flag out, 128 bytes per probed bucket
-            "find_algorithmic_gbs": n_find * (9 + 128 * probes) / f_ms / 1e6,
-            "insert_algorithmic_gbs": n * (4 + 1 + 2 * 128 + 32) / ins_ms / 1e6,
+            # key in, value + flag out, 32 bytes of tags per probed bucket, a
+            # sector per hit (read) or claim (written)
+            "find_algorithmic_gbs": (n_find * (9 + 32 * probes) + 32 * int(hit.sum())) / f_ms / 1e6,
+            "insert_algorithmic_gbs": n * (4 + 1 + 2 * 32 + 32) / ins_ms / 1e6,
             "ms": {"insert": ins_ms, "find": f_ms, "mixed": m_ms}}
 
 
@@ -649,7 +651,8 @@ def sweep_leg(torch, H, dev, table_kw, slots=SLOTS, n_find=N_FIND, seed=70, reps
             assert bool((fv[hit] == v32[hi[hit]]).all())
             row[f"find_{dist_name}_gops"] = n_find / f_ms / 1e6
             row[f"find_{dist_name}_probes"] = probes
-            row[f"find_{dist_name}_algorithmic_gbs"] = n_find * (9 + 8 * S * probes) / f_ms / 1e6
+            row[f"find_{dist_name}_algorithmic_gbs"] = (n_find * (9 + S * probes) +
+                                                        32 * int(hit.sum())) / f_ms / 1e6
         out["loads"][str(L)] = row
     n90, n95 = n_at[90], n_at[95]
     inc_ms = _median_ms(torch, stream, dev,
@@ -782,10 +785,12 @@ def plain_leg(torch, H, dev, seed=80, reps=5):
             "insert_gops": n_ins / ins_ms / 1e6, "find_gops": n_find / f1_ms / 1e6,
             "erase_gops": (n_ins // 2) / er_ms / 1e6, "find_after_erase_gops": n_find / f2_ms / 1e6,
             "ms": {"insert": ins_ms, "find": f1_ms, "erase": er_ms, "find_after_erase": f2_ms},
-            # bytes served from L2: each insert probes both buckets, each find
-            # the buckets it reads (counted by the kernel), plus the op I/O
-            "achieved_l2_gbs": {"insert": (9 + 2 * 8 * S + 32) * n_ins / ins_ms / 1e6,
-                                "find": (9 * n_find + 8 * S * find_probes) / f1_ms / 1e6},
+            # bytes served from L2: the tags of both buckets of an insert and of
+            # the buckets a find examines (counted by the kernel), a sector
+            # per claim or hit, plus the op I/O
+            "achieved_l2_gbs": {"insert": (9 + 2 * S + 32) * n_ins / ins_ms / 1e6,
+                                "find": (9 * n_find + S * find_probes +
+                                         32 * int(hit.sum())) / f1_ms / 1e6},
             "find_probes_per_op": find_probes / n_find}
 
 
@@ -841,13 +846,14 @@ def resize_leg(torch, H, dev, batches=32, n_batch=1 << 22, seed=60):
     st = t.stats()
     size_end = t.size()
     # op-weighted algorithmic bytes: op I/O (op code, key, value in; value,
-    # status out), every probed bucket, a written sector per claimed slot,
-    # and per split or merge pair one bucket read and two written
+    # status out), the tags of every probed bucket, a written sector per
+    # claimed slot (the words of hits are left out), and per split or merge
+    # pair one bucket read and two written
     n_ops = 2 * batches * n_batch
     probes = st["probes"] - s0["probes"]
     claims = (st["claimed_fast"] - s0["claimed_fast"]) + (st["claimed_slow"] - s0["claimed_slow"])
     pairs = (st["splits"] - s0["splits"]) + (st["merges"] - s0["merges"])
-    byts = 14 * n_ops + 8 * S * probes + 32 * claims + 3 * 8 * S * pairs
+    byts = 14 * n_ops + S * probes + 32 * claims + 3 * 8 * S * pairs
     peak_gbs, peak_kind = measured_peak()
     ach = byts / t_total / 1e9
     out["roofline"] = {"bound": "hbm", "algorithmic_bytes": byts, "achieved": ach,
@@ -1150,8 +1156,11 @@ def main():
     s_ins = t.stats()
     t.find(fk, vals_out=f_val, found=f_fnd)
     s_find = t.stats()
-    t.execute(mo, mk, mv)
+    hits_find = int(f_fnd.sum(dtype=torch.int64))
+    _, mix_st = t.execute(mo, mk, mv)
     s_mix = t.stats()
+    hits_mix = int(((mix_st == H.REPLACED) | (mix_st == H.ERASED) | (mix_st == H.FOUND)).sum())
+    del mix_st
     probes_ins = s_ins["probes"]
     probes_find = s_find["probes"] - s_ins["probes"]
     probes_mix = s_mix["probes"] - s_find["probes"]
@@ -1190,20 +1199,20 @@ def main():
     find_ms = prof.get("find", (0.0, 1))
     mix_ms = prof.get("mixed", (0.0, 1))
     claim_ms = prof.get("claim", (0.0, 1))
-    # mixed I/O: op, key, value in; value, status out.  A batch of 2^18 ops or
-    # more claims its new keys in the claim kernel, whose bytes are its own:
-    # a 12-byte list entry and a status byte per new key, a written sector
-    # per claim (the free masks it reads are served by L2)
-    bb = 8 * int(tuned.get("bucket_slots", 32))  # bytes per bucket probe
-    deferred = claim_ms[1] > 0
-    bytes_mix = 14 * n_mix + bb * probes_mix + (0 if deferred else 32 * claimed_mix)
-    bytes_claim = 13 * (claimed_mix + overflowed_mix) + 32 * claimed_mix
-    bytes_find = 9 * n_find + bb * probes_find  # key in, value + flag out, probed buckets
-    bytes_ins = 9 * n_ins + bb * probes_ins + 32 * (n_ins - overflowed)  # + one written sector
-    rl = {}
+    # mixed I/O: op, key, value in; value, status out.  A probe reads the
+    # bucket's tags (a byte per slot), a hit one sector of words, a claim
+    # writes one.  A batch of 2^18 ops or more claims its new keys in the claim
+    # kernel: a 12-byte list entry and both buckets' tags per new key
     sw = int(tuned.get("bucket_slots", 32))
-    for name, (tot, cnt), byts, kname in (("insert", ins_ms, bytes_ins, f"k_ops<insert,S={sw}>"),
-                                            ("find", find_ms, bytes_find, f"k_ops<find,S={sw}>"),
+    deferred = claim_ms[1] > 0
+    bytes_mix = (14 * n_mix + sw * probes_mix + 32 * hits_mix +
+                 (12 * (claimed_mix + overflowed_mix) if deferred else 32 * claimed_mix))
+    bytes_claim = (12 + 2 * sw) * (claimed_mix + overflowed_mix) + 32 * claimed_mix
+    bytes_find = 9 * n_find + sw * probes_find + 32 * hits_find
+    bytes_ins = 9 * n_ins + sw * probes_ins + 32 * (n_ins - overflowed)
+    rl = {}
+    for name, (tot, cnt), byts, kname in (("insert", ins_ms, bytes_ins, f"k_insert_part+store<S={sw}>"),
+                                            ("find", find_ms, bytes_find, f"k_find<S={sw}>"),
                                             ("mixed", mix_ms, bytes_mix, f"k_ops<mixed,S={sw}>"),
                                             ("claim", claim_ms, bytes_claim, f"k_claim<S={sw}>")):
         if name == "claim" and not deferred:
