@@ -186,7 +186,7 @@ cudaError_t launch_split(const View& v_new, uint32_t src0, uint32_t count, uint3
 cudaError_t launch_merge_excess(const View& v_new, uint32_t count, Ctrl* host_out,
                                 cudaStream_t s);
 cudaError_t launch_merge(const View& v_new, uint32_t count, List ovf, cudaStream_t s);
-cudaError_t launch_fused(const View& v, const uint8_t* ops, const uint32_t* keys,
+cudaError_t launch_fused(View v, const uint8_t* ops, const uint32_t* keys,
                          const uint32_t* vals, uint64_t n, uint32_t* vals_out, uint8_t* status,
                          List pend, int resizable, const Launch& L, cudaStream_t s);
 // Counts a batch's inserts into *host_out (pinned); ctrl->n_insert is 0 before

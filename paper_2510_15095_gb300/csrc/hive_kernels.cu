@@ -1904,7 +1904,7 @@ __device__ void fused_checked(const View& v, uint32_t stash_n, const OpPtrs& a, 
       const TagVec<S> t2 = ld_tags<S, false>(v, b2);
       const uint32_t t4 = tag_of(key) * 0x01010101u;
       check_words<S, false>(v, b1, b2, tag_match<S>(t1, t4),
-                            b2 != b1 ? tag_match<S>(t2, t4) : 0u, key, h, false);
+                            b2 != b1 ? tag_match<S>(t2, t4) : 0u, key, h, v.keep_words);
     }
     cnt.probes += active;
     cnt.probes += active && (!h.ok || h.b != b1);
@@ -2042,9 +2042,8 @@ __device__ __forceinline__ void run_chunk_fused(const View& v, uint32_t stash_n,
     const TagVec<S> t1 = ld_tags<S, false>(v, b1);
     const TagVec<S> t2 = ld_tags<S, false>(v, b2);
     const uint32_t t4 = tag_of(key) * 0x01010101u;
-    // the words leave L2 first here (10^6 ops on 2^24 slots: 147 us, 152 kept)
     check_words<S, false>(v, b1, b2, tag_match<S>(t1, t4), b2 != b1 ? tag_match<S>(t2, t4) : 0u,
-                          key, h, false);
+                          key, h, v.keep_words);
   }
   cnt.probes += open;
   cnt.probes += open && (!h.ok || h.b != b1);
@@ -2693,9 +2692,12 @@ cudaError_t launch_ops_s(int mode, const View& v, const uint8_t* ops, const uint
 
 }  // namespace
 
-cudaError_t launch_fused(const View& v, const uint8_t* ops, const uint32_t* keys,
+cudaError_t launch_fused(View v, const uint8_t* ops, const uint32_t* keys,
                          const uint32_t* vals, uint64_t n, uint32_t* vals_out, uint8_t* status,
                          List pend, int resizable, const Launch& L, cudaStream_t s) {
+  // words stay in L2 only for a batch of an op or more per line (2^22 ops on
+  // 2^26 slots 629 -> 616 us; 10^6 ops on 2^24 slots 147 us, 152 kept)
+  v.keep_words = n * 16 >= static_cast<uint64_t>(v.nb) * v.S;
   const uint64_t chunks = (n + 31) / 32;
   const uint64_t warps_per_block = kOpsThreads / 32;
   uint64_t blocks = (chunks + warps_per_block - 1) / warps_per_block;
