@@ -136,7 +136,10 @@ hive_status run32(hive32_table* t, int mode, const uint8_t* ops, const uint32_t*
       return st;
   }
   if (ins && (st = ensure_list32(t, n)) != HIVE_OK) return st;
-  const View32 v = view32(t);
+  View32 v = view32(t);
+  // and in an updating batch that comes back to their lines (2^26 slots: 2^24
+  // mixed ops 1365 -> 1214 us)
+  if (mode != kModeFind && n * 32 >= t->nb * kS) v.keep_words = 1;
   const Ops32 a{ops, keys, vals, vals_out, found, status};
   H32_CK(launch32_ops(mode, v, a, n, list32(t), t->num_sms, s));
   if (ins) H32_CK(launch32_overflow(v, list32(t), status, t->num_sms * 8, s));

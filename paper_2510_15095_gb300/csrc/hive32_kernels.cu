@@ -217,12 +217,81 @@ __device__ __forceinline__ In32 load32(const Ops32& a, uint32_t c, uint64_t n, i
   return in;
 }
 
+// Appends the flagged lanes' items to the eviction list.
+__device__ __forceinline__ void append32(const List32& l, int lane, bool has, uint32_t word,
+                                         uint32_t idx) {
+  const unsigned om = __ballot_sync(kFull, has);
+  if (!om) return;
+  const int leader = __ffs(om) - 1;
+  unsigned base = 0;
+  if (lane == leader) base = atomicAdd(l.count, static_cast<unsigned>(__popc(om)));
+  base = __shfl_sync(kFull, base, leader);
+  if (has) {
+    const unsigned r = base + __popc(om & ((1u << lane) - 1u));
+    l.words[r] = word;
+    l.idx[r] = idx;
+  }
+}
+
+// A warp's queue of a mixed batch's new keys, in shared memory: they wait for
+// 32 of their kind, so that the claims of a batch with one insert in four
+// ops are not made by a quarter of the lanes in each chunk (a set of 2^25
+// slots at 90%, 2^23 ops: 387 -> 325 us; staged buckets took 365).  Their
+// status is written when they are queued (INSERTED; the eviction pass writes
+// it again).
+// `n` is warp-uniform and below 32 between chunks.
+constexpr uint32_t kNewQ32 = 64;
+struct NewQ32 {
+  uint32_t* words;
+  uint32_t* idx;
+  uint32_t n;
+};
+
+// Claims for the first min(n, 32) queued keys (warp-wide); the rest move to
+// the front.
+template <int LAYOUT>
+__device__ __forceinline__ void claim32_queued(const View32& v, NewQ32& q, const List32& ovf,
+                                               Counters32& cnt, int lane) {
+  using E = E32<LAYOUT>;
+  __syncwarp();
+  const uint32_t m = q.n < 32 ? q.n : 32u, rest = q.n - m;
+  const bool has = static_cast<uint32_t>(lane) < m;
+  const uint32_t word = has ? q.words[lane] : kEmpty32;
+  const uint32_t idx = has ? q.idx[lane] : kNoOp;
+  uint32_t mw = 0, mi = 0;
+  if (static_cast<uint32_t>(lane) < rest) {
+    mw = q.words[32 + lane];
+    mi = q.idx[32 + lane];
+  }
+  __syncwarp();
+  if (static_cast<uint32_t>(lane) < rest) {
+    q.words[lane] = mw;
+    q.idx[lane] = mi;
+  }
+  q.n = rest;
+  bool to_ovf = false;
+  if (has) {
+    const uint32_t key = E::key(word);
+    if (place32(v, lh_bucket(bithash1(key), v.M, v.p), lh_bucket(bithash2(key), v.M, v.p), key,
+                word)) {
+      cnt.size_delta += 1;
+      cnt.claimed += 1;
+    } else {
+      to_ovf = true;
+      cnt.overflowed += 1;
+    }
+  }
+  append32(ovf, lane, to_ovf, word, idx);
+}
+
 // Ops [32c, 32c + 32) of a batch, one op per lane: the tags of both candidate
-// buckets in one round trip, then the entries whose tag matches.
+// buckets in one round trip, then the entries whose tag matches.  With a queue
+// `q`, the new keys of a mixed batch wait there for their claims.
 template <int MODE, int LAYOUT>
 __device__ __forceinline__ void run_chunk32(const View32& v, uint32_t stash_n, const Ops32 a,
                                             uint32_t c, uint64_t n, const List32 ovf,
-                                            Counters32& cnt, const In32& in, int lane) {
+                                            Counters32& cnt, const In32& in, int lane,
+                                            NewQ32* q) {
   using E = E32<LAYOUT>;
   constexpr bool kIns = (MODE == kModeInsert || MODE == kModeMixed);
   constexpr bool kRO = MODE == kModeFind;
@@ -289,30 +358,28 @@ __device__ __forceinline__ void run_chunk32(const View32& v, uint32_t stash_n, c
 
   // step 2: claim for absent keys
   bool to_ovf = false;
-  if (kIns && !done && op == OP_INSERT) {
-    const bool placed = place32_from(v, b1, b2, t1, t2, key, E::pack(key, val));
-    if (placed) {
+  if (kIns && q) {
+    const bool fresh = !done && op == OP_INSERT;
+    const unsigned nm = __ballot_sync(kFull, fresh);
+    if (fresh) {
+      const uint32_t r = q->n + __popc(nm & ((1u << lane) - 1u));
+      q->words[r] = E::pack(key, val);
+      q->idx[r] = i;
       st = ST_INSERTED;
-      cnt.size_delta += 1;
-      cnt.claimed += 1;
-    } else {
-      to_ovf = true;
-      cnt.overflowed += 1;
     }
-  }
-  if (kIns) {
-    const unsigned om = __ballot_sync(kFull, to_ovf);
-    if (om) {
-      const int leader = __ffs(om) - 1;
-      unsigned base = 0;
-      if (lane == leader) base = atomicAdd(ovf.count, static_cast<unsigned>(__popc(om)));
-      base = __shfl_sync(kFull, base, leader);
-      if (to_ovf) {
-        const unsigned r = base + __popc(om & ((1u << lane) - 1u));
-        ovf.words[r] = E::pack(key, val);
-        ovf.idx[r] = i;
+    q->n += __popc(nm);
+  } else if (kIns) {
+    if (!done && op == OP_INSERT) {
+      if (place32_from(v, b1, b2, t1, t2, key, E::pack(key, val))) {
+        st = ST_INSERTED;
+        cnt.size_delta += 1;
+        cnt.claimed += 1;
+      } else {
+        to_ovf = true;
+        cnt.overflowed += 1;
       }
     }
+    append32(ovf, lane, to_ovf, E::pack(key, val), i);
   }
   if (valid) {
     if (MODE == kModeFind) {
@@ -323,6 +390,7 @@ __device__ __forceinline__ void run_chunk32(const View32& v, uint32_t stash_n, c
       if (MODE == kModeMixed && a.vals_out) __stcs(a.vals_out + i, outv);
     }
   }
+  if (kIns && q && q->n >= 32) claim32_queued<LAYOUT>(v, *q, ovf, cnt, lane);
 }
 
 // What bounds it (one GB300, a set of 2^25 slots at 90%, 128 MB of entries and
@@ -330,7 +398,9 @@ __device__ __forceinline__ void run_chunk32(const View32& v, uint32_t stash_n, c
 // whole 128-byte buckets staged in shared memory: 30 M inserts 1.58 -> 1.09
 // ms, 60 M lookups (half hits) 1.22 -> 0.86 ms and, with half the keys gone,
 // 1.32 -> 0.76 ms; 15 M erases 0.46 -> 0.62 ms (the entry, its CAS and the tag
-// are three dependent accesses where the old probe had two).
+// are three dependent accesses where the old probe had two).  Mixed batches at
+// four blocks per SM: five and six spill (2^26 slots, 2^24 ops: 1.20 -> 1.32 and
+// 1.45 ms).
 template <int MODE, int LAYOUT>
 __global__ void __launch_bounds__(kOps32Threads, (MODE == kModeInsert || MODE == kModeMixed) ? 4 : 6)
     k32_ops(View32 v, Ops32 a, uint64_t n, List32 ovf, int prefetch_tags) {
@@ -342,14 +412,22 @@ __global__ void __launch_bounds__(kOps32Threads, (MODE == kModeInsert || MODE ==
   const uint32_t nchunks = static_cast<uint32_t>((n + 31) >> 5);
   const uint32_t stash_n = v.ctrl->stash_n;
   Counters32 cnt;
+  constexpr bool kQueue = MODE == kModeMixed;
+  __shared__ uint32_t queue[kQueue ? (kOps32Threads / 32) * 2 * kNewQ32 : 1];
+  uint32_t* mine = queue + (kQueue ? (threadIdx.x >> 5) * 2 * kNewQ32 : 0);
+  NewQ32 nq{mine, mine + kNewQ32, 0};
+  // one chunk per warp: claim at once, with the tags at hand
+  NewQ32* const q = kQueue && nchunks > nwarps ? &nq : nullptr;
   // inputs are loaded one chunk ahead
   In32 nxt{};
   if (warp0 < nchunks) nxt = load32<MODE>(a, warp0, n, lane);
   for (uint32_t c = warp0; c < nchunks; c += nwarps) {
     const In32 in = nxt;
     if (c + nwarps < nchunks) nxt = load32<MODE>(a, c + nwarps, n, lane);
-    run_chunk32<MODE, LAYOUT>(v, stash_n, a, c, n, ovf, cnt, in, lane);
+    run_chunk32<MODE, LAYOUT>(v, stash_n, a, c, n, ovf, cnt, in, lane, q);
   }
+  if constexpr (kQueue)
+    while (nq.n) claim32_queued<LAYOUT>(v, nq, ovf, cnt, lane);
   // an insert examines both buckets of every live op, which ends in one of these
   if (MODE == kModeInsert) cnt.probes = 2 * (cnt.replaced + cnt.claimed + cnt.overflowed);
   flush32_block(v, cnt, lane);

@@ -239,3 +239,36 @@ def test_new_keys_wait_in_the_warp_queue(H, bs, n):
     for x in tabs:
         assert x.check() == 0
         x.close()
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("n", [200_001, 400_000])
+def test_new_keys_wait_in_the_warp_queue_of_32_bit_entries(H, layout, n):
+    """The same queue on tables with 32-bit entries, filled until some of the
+    queued keys find both buckets full."""
+    from test_gpu_hive32 import check_image as check_image32
+
+    rng = np.random.default_rng(n + layout)
+    if layout == 0:
+        pool, slots, n_live, n_new = rng.permutation(0xFFFE).astype(np.uint32), 1 << 16, 50_000, 14_000
+        vmask = 0xFFFF
+    else:
+        slots, n_live, n_new, vmask = 1 << 18, 240_000, 20_000, 0
+        pool, _ = W.take_keys(91, 0, n_live + n_new)
+    live, new = pool[:n_live], pool[n_live:n_live + n_new]
+    lv = (W.values_for(live, 91) & vmask).astype(np.uint32)
+    ops, keys, vals = W.mixed_batch(rng, live, new, n_new, 1_000, n - n_new - 1_000, seed=91)
+    vals = (vals & vmask).astype(np.uint32)
+    t = H.Hive32Table(slots, layout, stash_permille=50)
+    d = oracle.Dict()
+    t.insert(up(H, live), up(H, lv))
+    d.insert(live, lv)
+    before = t.stats()["overflowed"]
+    vo, st = t.execute(torch.from_numpy(ops).cuda(), up(H, keys), up(H, vals))
+    ev, es = d.execute(ops, keys, vals)
+    assert np.array_equal(st.cpu().numpy(), es) and np.array_equal(H.to_host_u32(vo), ev)
+    if layout == 1:
+        assert t.stats()["overflowed"] > before
+    check_image32(t, d)
+    assert t.check() == 0
+    t.close()
