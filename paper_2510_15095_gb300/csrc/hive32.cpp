@@ -137,9 +137,13 @@ hive_status run32(hive32_table* t, int mode, const uint8_t* ops, const uint32_t*
   }
   if (ins && (st = ensure_list32(t, n)) != HIVE_OK) return st;
   View32 v = view32(t);
-  // and in an updating batch that comes back to their lines (2^26 slots: 2^24
-  // mixed ops 1365 -> 1214 us)
-  if (mode != kModeFind && n * 32 >= t->nb * kS) v.keep_words = 1;
+  // and beyond that in a mixed or erase batch that comes back to their lines
+  // (2^26 slots: 2^24 mixed ops 1365 -> 1214 us, 2^25.9 erases 4.52 -> 4.13 ms,
+  // but the same keys inserted again 1.70 -> 2.29 ms; 2^25 slots: 2^24.8
+  // erases 1.27 -> 1.32 ms)
+  if ((mode == kModeMixed || mode == kModeErase) && n * 32 >= t->nb * kS &&
+      t->nb * kS * sizeof(uint32_t) > (128ull << 20))
+    v.keep_words = 1;
   const Ops32 a{ops, keys, vals, vals_out, found, status};
   H32_CK(launch32_ops(mode, v, a, n, list32(t), t->num_sms, s));
   if (ins) H32_CK(launch32_overflow(v, list32(t), status, t->num_sms * 8, s));
