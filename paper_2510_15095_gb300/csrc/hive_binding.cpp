@@ -37,17 +37,31 @@ const at::Tensor& tensor_of(PyObject* o) {
   return THPVariable_Unpack(o);
 }
 
-// Pointer of a contiguous CUDA tensor with >= n items of `item` bytes (or,
-// with `pinned`, of a pinned CPU tensor); NULL for None.
-void* ptr_of(const at::Tensor& t, size_t item, int64_t n, bool pinned = false) {
+// Refuses all but a contiguous CUDA tensor with >= n items of `item` bytes (or,
+// with `pinned`, a pinned CPU tensor).
+void check_plain(const at::Tensor& t, size_t item, int64_t n, bool pinned) {
   if (!t.is_cuda() && !(pinned && t.device().is_cpu() && t.is_pinned())) throw NotPlain();
   if (!t.has_storage() || !t.is_contiguous() || t.element_size() != item || t.numel() < n)
     throw NotPlain();
-  return const_cast<void*>(t.const_data_ptr());
 }
-void* ptr_of(PyObject* o, size_t item, int64_t n, bool pinned = false) {
+// Pointer of an input tensor; NULL for None.
+const void* in_ptr(const at::Tensor& t, size_t item, int64_t n, bool pinned = false) {
+  check_plain(t, item, n, pinned);
+  return t.const_data_ptr();
+}
+const void* in_ptr(PyObject* o, size_t item, int64_t n, bool pinned = false) {
   if (!o || o == Py_None) return nullptr;
-  return ptr_of(tensor_of(o), item, n, pinned);
+  return in_ptr(tensor_of(o), item, n, pinned);
+}
+// Pointer of an output tensor; NULL for None.  A copy-on-write tensor gets its
+// own storage first, as data_ptr() gives it in Python: the kernels write it.
+void* out_ptr(const at::Tensor& t, size_t item, int64_t n, bool pinned = false) {
+  check_plain(t, item, n, pinned);
+  return t.mutable_data_ptr();
+}
+void* out_ptr(PyObject* o, size_t item, int64_t n, bool pinned = false) {
+  if (!o || o == Py_None) return nullptr;
+  return out_ptr(tensor_of(o), item, n, pinned);
 }
 
 void* as_address(PyObject* o) {
@@ -88,7 +102,7 @@ struct Out {
   }
   void make(int64_t n, const at::TensorOptions& opt, size_t item) {
     at::Tensor t = at::empty({n}, opt);
-    ptr = ptr_of(t, item, n);
+    ptr = out_ptr(t, item, n);
     obj = THPVariable_Wrap(std::move(t));
     if (!obj) throw NotPlain();
   }
@@ -96,7 +110,7 @@ struct Out {
     if (o == (required ? Py_None : Py_True)) {
       make(n, opt, item);
     } else if (required || (o != Py_None && o != Py_False)) {
-      ptr = ptr_of(o, item, n);
+      ptr = out_ptr(o, item, n);
       obj = Py_NewRef(o);
     }
   }
@@ -149,8 +163,8 @@ PyObject* py_insert(PyObject*, PyObject* const* a, Py_ssize_t na) {
     const int64_t n = keys.numel();
     Out st;
     st.init(a[4], false, n, bytes_like(keys), 1);
-    const void* k = ptr_of(keys, 4, n);
-    const void* v = ptr_of(a[3], 4, n);
+    const void* k = in_ptr(keys, 4, n);
+    const void* v = in_ptr(a[3], 4, n);
     void* s = stream_of(a[5]);
     const int rc = without_gil([&] { return fn(h, k, v, n, st.ptr, s); });
     return Py_BuildValue("(iN)", rc, st.take());
@@ -166,7 +180,7 @@ PyObject* py_erase(PyObject*, PyObject* const* a, Py_ssize_t na) {
     const int64_t n = keys.numel();
     Out st;
     st.init(a[3], false, n, bytes_like(keys), 1);
-    const void* k = ptr_of(keys, 4, n);
+    const void* k = in_ptr(keys, 4, n);
     void* s = stream_of(a[4]);
     const int rc = without_gil([&] { return fn(h, k, n, st.ptr, s); });
     return Py_BuildValue("(iN)", rc, st.take());
@@ -180,7 +194,7 @@ PyObject* py_find(PyObject*, PyObject* const* a, Py_ssize_t na) {
     void* h = as_address(a[1]);
     const at::Tensor& keys = tensor_of(a[2]);
     const int64_t n = keys.numel();
-    const void* k = ptr_of(keys, 4, n);
+    const void* k = in_ptr(keys, 4, n);
     Out vo, fo;
     vo.init(a[3], true, n, keys.options(), 4);
     fo.init(a[4], false, n, bytes_like(keys), 1);
@@ -197,9 +211,9 @@ PyObject* py_execute(PyObject*, PyObject* const* a, Py_ssize_t na) {
     void* h = as_address(a[1]);
     const at::Tensor& keys = tensor_of(a[3]);
     const int64_t n = keys.numel();
-    const void* k = ptr_of(keys, 4, n);
-    const void* o = ptr_of(a[2], 1, n);
-    const void* v = ptr_of(a[4], 4, n);
+    const void* k = in_ptr(keys, 4, n);
+    const void* o = in_ptr(a[2], 1, n);
+    const void* v = in_ptr(a[4], 4, n);
     Out vo, st;
     vo.make(n, keys.options(), 4);
     st.make(n, bytes_like(keys), 1);
@@ -244,11 +258,11 @@ PyObject* py_multi(PyObject*, PyObject* const* a, Py_ssize_t na) {
       g.reserved0 = 0;
       g.n = static_cast<uint64_t>(n);
       g.n_insert = ins_o ? PyLong_AsUnsignedLongLongMask(ins_o) : g.n;
-      g.ops = static_cast<const uint8_t*>(ptr_of(ops_o, 1, n, true));
-      g.keys = static_cast<const uint32_t*>(ptr_of(keys, 4, n, true));
-      g.vals = static_cast<const uint32_t*>(ptr_of(item(d, k_vals), 4, n, true));
-      g.vals_out = static_cast<uint32_t*>(ptr_of(item(d, k_vals_out), 4, n, true));
-      g.status = static_cast<uint8_t*>(ptr_of(item(d, k_status), 1, n, true));
+      g.ops = static_cast<const uint8_t*>(in_ptr(ops_o, 1, n, true));
+      g.keys = static_cast<const uint32_t*>(in_ptr(keys, 4, n, true));
+      g.vals = static_cast<const uint32_t*>(in_ptr(item(d, k_vals), 4, n, true));
+      g.vals_out = static_cast<uint32_t*>(out_ptr(item(d, k_vals_out), 4, n, true));
+      g.status = static_cast<uint8_t*>(out_ptr(item(d, k_status), 1, n, true));
     }
     void* s = stream_of(a[3]);
     const int rc =
