@@ -118,8 +118,10 @@ struct Out {
 
 at::TensorOptions bytes_like(const at::Tensor& t) { return t.options().dtype(at::kByte); }
 
-// Runs one binding function body: NotPlain and a Python error already set
-// aside, a C++ exception becomes a RuntimeError.
+// Runs one binding function body.  Nothing throws once the C ABI has been
+// called, so after any exception (NotPlain, an output that could not be
+// allocated) the Python code takes the call from its start and raises the
+// error that PyTorch gives there, torch.OutOfMemoryError for instance.
 template <class F>
 PyObject* guarded(Py_ssize_t have, Py_ssize_t want, F body) {
   if (have != want) {
@@ -130,12 +132,10 @@ PyObject* guarded(Py_ssize_t have, Py_ssize_t want, F body) {
     if (modes_active()) throw NotPlain();
     return body();
   } catch (const NotPlain&) {
-    PyErr_Clear();
-    return Py_NewRef(Py_NotImplemented);
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
+  } catch (const std::exception&) {
   }
+  PyErr_Clear();
+  return Py_NewRef(Py_NotImplemented);
 }
 
 template <class F>

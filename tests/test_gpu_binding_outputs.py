@@ -1,4 +1,5 @@
-"""Outputs of the native call path are written through the tensor's own storage."""
+"""Outputs of the native call path: written through the tensor's own storage,
+and the error of an output that cannot be allocated."""
 import numpy as np
 import pytest
 
@@ -48,4 +49,28 @@ def test_copy_on_write_outputs_get_their_own_storage(H, call):
         assert np.array_equal(H.to_host_u32(out), vals) and bool((st != 77).all())
         m.close()
     assert bool((words == -7).all()) and bool((flags == 77).all())
+    t.close()
+
+
+@pytest.mark.parametrize("call", ["find", "insert", "erase", "execute"])
+def test_output_that_cannot_be_allocated(H, call):
+    """torch.OutOfMemoryError, as from torch.empty, and the table untouched."""
+    n = 1 << 24
+    t = H.HiveTable(1 << 12)
+    dk = torch.arange(n, dtype=torch.int32, device="cuda")
+    ops = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    dev = torch.cuda.current_device()
+    total = torch.cuda.get_device_properties(dev).total_memory
+    # 1 MB is left to PyTorch's allocator: an output takes 16 MB or 64
+    torch.cuda.set_per_process_memory_fraction(
+        (torch.cuda.memory_reserved(dev) + (1 << 20)) / total, dev)
+    try:
+        with pytest.raises(torch.OutOfMemoryError):
+            {"find": lambda: t.find(dk), "insert": lambda: t.insert(dk, dk),
+             "erase": lambda: t.erase(dk), "execute": lambda: t.execute(ops, dk, dk)}[call]()
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0, dev)
+    assert t.size() == 0 and t.check() == 0
     t.close()
