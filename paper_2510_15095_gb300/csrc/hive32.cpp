@@ -33,6 +33,7 @@ struct hive32_table {
   Ctrl* host_ctrl = nullptr;
   uint32_t* list_words = nullptr;
   uint32_t* list_idx = nullptr;
+  Retired list_kept;
   uint64_t list_cap = 0;
   int num_sms = 0, blocks_per_sm = 1;
   bool check_contract = false;  // HIVE_DEBUG at creation: update calls check the batch contract
@@ -90,13 +91,15 @@ hive_status check32(const hive32_table* t) {
   return HIVE_OK;
 }
 
-hive_status ensure_list32(hive32_table* t, uint64_t n) {
+hive_status ensure_list32(hive32_table* t, uint64_t n, cudaStream_t s) {
+  if (!t->list_kept.captured) t->list_kept.captured = stream_capturing(s);
   if (n <= t->list_cap) return HIVE_OK;
   uint64_t cap = 1u << 16;
   while (cap < n) cap <<= 1;
   H32_CK(cudaDeviceSynchronize());
-  cudaFree(t->list_words);
-  cudaFree(t->list_idx);
+  t->list_kept.drop(t->list_words, t->list_cap * sizeof(uint32_t));
+  t->list_kept.drop(t->list_idx, t->list_cap * sizeof(uint32_t));
+  t->list_kept.captured = false;
   t->list_words = nullptr;
   t->list_idx = nullptr;
   t->list_cap = 0;
@@ -135,7 +138,7 @@ hive_status run32(hive32_table* t, int mode, const uint8_t* ops, const uint32_t*
         HIVE_OK)
       return st;
   }
-  if (ins && (st = ensure_list32(t, n)) != HIVE_OK) return st;
+  if (ins && (st = ensure_list32(t, n, s)) != HIVE_OK) return st;
   View32 v = view32(t);
   // and beyond that in a mixed or erase batch that comes back to their lines
   // (2^26 slots: 2^24 mixed ops 1365 -> 1214 us, 2^25.9 erases 4.52 -> 4.13 ms,
@@ -160,6 +163,7 @@ void free32(hive32_table* t) {
   cudaFree(t->ctrl);
   cudaFree(t->list_words);
   cudaFree(t->list_idx);
+  t->list_kept.release();
   if (t->host_ctrl) cudaFreeHost(t->host_ctrl);
 }
 

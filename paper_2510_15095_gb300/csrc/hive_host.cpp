@@ -135,10 +135,11 @@ List list_defer(const hive_table* t) {
 List list_b(const hive_table* t) { return List{t->lb_words, t->lb_idx, &t->ctrl->pend_n}; }
 
 void free_lists(hive_table* t) {
-  cudaFree(t->la_words);
-  cudaFree(t->la_idx);
-  cudaFree(t->lb_words);
-  cudaFree(t->lb_idx);
+  t->lists_kept.drop(t->la_words, t->list_cap * sizeof(uint64_t));
+  t->lists_kept.drop(t->la_idx, t->list_cap * sizeof(uint32_t));
+  t->lists_kept.drop(t->lb_words, t->lb_cap * sizeof(uint64_t));
+  t->lists_kept.drop(t->lb_idx, t->lb_cap * sizeof(uint32_t));
+  t->lists_kept.captured = false;
   t->la_words = t->lb_words = nullptr;
   t->la_idx = t->lb_idx = nullptr;
   t->list_cap = t->lb_cap = 0;
@@ -148,7 +149,8 @@ void free_lists(hive_table* t) {
 // merge batch), so they grow to the largest call seen.
 // List B exists for resizable tables (pending items) and once a mixed batch
 // has run (its claim kernel hands full-bucket items from A to B).
-hive_status ensure_lists(hive_table* t, uint64_t n, bool need_b = false) {
+hive_status ensure_lists(hive_table* t, uint64_t n, cudaStream_t s, bool need_b = false) {
+  if (!t->lists_kept.captured) t->lists_kept.captured = stream_capturing(s);
   const bool two = t->cfg.resizable != 0 || need_b || t->lb_cap != 0;
   if (n <= t->list_cap && (!two || n <= t->lb_cap)) return HIVE_OK;
   const uint64_t cap = std::max<uint64_t>(next_pow2(std::max(n, t->list_cap)), 1u << 16);
@@ -167,10 +169,15 @@ hive_status ensure_lists(hive_table* t, uint64_t n, bool need_b = false) {
   return HIVE_OK;
 }
 
+uint64_t part_off_bytes(uint64_t cap) {
+  return part_tiles(cap) * (kPartMaxRegions + 1) * sizeof(uint16_t);
+}
+
 void free_part(hive_table* t) {
-  cudaFree(t->part_words);
-  cudaFree(t->part_slots);
-  cudaFree(t->part_off);
+  t->part_kept.drop(t->part_words, t->part_cap * sizeof(uint64_t));
+  t->part_kept.drop(t->part_slots, t->part_cap * sizeof(uint32_t));
+  t->part_kept.drop(t->part_off, part_off_bytes(t->part_cap));
+  t->part_kept.captured = false;
   t->part_words = nullptr;
   t->part_slots = nullptr;
   t->part_off = nullptr;
@@ -200,30 +207,29 @@ bool want_part(const hive_table* t, uint64_t n) {
 }
 // The list of such an insert.  False (and the plain way is taken) when there
 // is no memory for it, or when the stream is being captured and it would have
-// to be allocated.
+// to be allocated.  It grows like the op lists, to the next power of two, so
+// that calls of slowly rising size seldom wait for an allocation.
 bool ensure_part(hive_table* t, uint64_t n, cudaStream_t s, PartList* out) {
+  const bool capturing = stream_capturing(s);
   if (n > t->part_cap) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-      cudaGetLastError();
-      return false;
-    }
+    if (capturing) return false;
     if (t->part_cap) {
       if (cudaDeviceSynchronize() != cudaSuccess) return false;  // the next launch reports it
       free_part(t);
     }
-    const uint64_t tiles = part_tiles(n);
-    cudaError_t e = dev_alloc(&t->part_words, n * sizeof(uint64_t));
-    if (e == cudaSuccess) e = dev_alloc(&t->part_slots, n * sizeof(uint32_t));
+    const uint64_t cap = next_pow2(n);
+    cudaError_t e = dev_alloc(&t->part_words, cap * sizeof(uint64_t));
+    if (e == cudaSuccess) e = dev_alloc(&t->part_slots, cap * sizeof(uint32_t));
     if (e == cudaSuccess)
-      e = dev_alloc(&t->part_off, tiles * (kPartMaxRegions + 1) * sizeof(uint16_t));
+      e = dev_alloc(&t->part_off, part_off_bytes(cap));
     if (e != cudaSuccess) {
       cudaGetLastError();
       free_part(t);
       return false;
     }
-    t->part_cap = n;
+    t->part_cap = cap;
   }
+  t->part_kept.captured |= capturing;
   const uint32_t shift = part_shift(t);
   *out = PartList{t->part_words, t->part_slots, t->part_off,
                   static_cast<uint32_t>((t->nb * t->S - 1) >> shift) + 1, shift};
@@ -434,7 +440,7 @@ hive_status hive::contract_table(hive_table* t, cudaStream_t s) {
       t->merge_deferred = true;
       break;
     }
-    st = ensure_lists(t, static_cast<uint64_t>(count) * t->S);
+    st = ensure_lists(t, static_cast<uint64_t>(count) * t->S, s);
     if (st != HIVE_OK) return st;
     HIVE_LAUNCH(t, HIVE_K_MERGE, s, launch_merge(vn, count, list_a(t), s));
     t->M = trial.M;
@@ -507,6 +513,32 @@ cudaError_t dev_alloc_raw(void** p, size_t bytes) {
   return cudaMalloc(p, bytes);
 }
 void set_fail_alloc(uint32_t n) { g_fail_alloc.store(n); }
+bool stream_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream while another captures: the launches say so
+    return false;
+  }
+  return cs != cudaStreamCaptureStatusNone;
+}
+void Retired::drop(void* p, uint64_t n) {
+  if (!p) return;
+  if (!captured) {
+    cudaFree(p);
+    return;
+  }
+  try {
+    old.push_back(p);
+  } catch (const std::bad_alloc&) {
+    // not listed, so never freed: a graph may still write it
+  }
+  bytes += n;
+}
+void Retired::release() {
+  for (void* p : old) cudaFree(p);
+  old.clear();
+  bytes = 0;
+}
 bool table_view(const hive_table* t, View* v, Launch* L, bool* resizable) {
   if (!t) return false;
   *v = make_view(t);
@@ -671,6 +703,8 @@ hive_status hive_destroy(hive_table* t) {
   if (t->host_ctrl) cudaFreeHost(t->host_ctrl);
   free_lists(t);
   free_part(t);
+  t->lists_kept.release();
+  t->part_kept.release();
   free_staging(t);
   for (const auto& r : t->recs) {
     cudaEventDestroy(r.a);
@@ -692,7 +726,7 @@ hive_status hive_insert(hive_table* t, const uint32_t* keys, const uint32_t* val
   if (t->check_contract &&
       (st = check_contract_device(nullptr, HIVE_OP_INSERT, keys, n, kReservedKeyMin, s)) != HIVE_OK)
     return st;
-  if ((st = ensure_lists(t, n)) != HIVE_OK) return st;
+  if ((st = ensure_lists(t, n, s)) != HIVE_OK) return st;
   if (t->cfg.resizable && (st = grow_for(t, n, s)) != HIVE_OK) return st;
   const View v = make_view(t);
   PartList pl{};
@@ -740,7 +774,7 @@ hive_status hive_erase(hive_table* t, const uint32_t* keys, uint64_t n, uint8_t*
               launch_ops(kModeErase, v, nullptr, keys, nullptr, n, nullptr, nullptr, status,
                          list_a(t), t->L, s));
   if (t->cfg.resizable) {
-    if ((st = ensure_lists(t, 1)) != HIVE_OK) return st;
+    if ((st = ensure_lists(t, 1, s)) != HIVE_OK) return st;
     return finish_resizable(t, status, s);
   }
   HIVE_LAUNCH(t, HIVE_K_MAINT, s, launch_maintenance(v, s));
@@ -766,7 +800,7 @@ hive_status hive_execute(hive_table* t, const uint8_t* ops, const uint32_t* keys
   if (t->check_contract &&
       (st = check_contract_device(ops, HIVE_OP_FIND, keys, n, kReservedKeyMin, s)) != HIVE_OK)
     return st;
-  if ((st = ensure_lists(t, n, true)) != HIVE_OK) return st;
+  if ((st = ensure_lists(t, n, s, true)) != HIVE_OK) return st;
   if (t->cfg.resizable && (st = grow_for_mixed(t, ops, n, s)) != HIVE_OK) return st;
   const View v = make_view(t);
   // Both op lists are empty here: every mutating call ends with the
@@ -812,7 +846,7 @@ hive_status hive_execute_fused(hive_table* t, const uint8_t* ops, const uint32_t
   if (t->check_contract &&
       (st = check_contract_device(ops, HIVE_OP_FIND, keys, n, kReservedKeyMin, s)) != HIVE_OK)
     return st;
-  if ((st = ensure_lists(t, n)) != HIVE_OK) return st;
+  if ((st = ensure_lists(t, n, s)) != HIVE_OK) return st;
   if (t->cfg.resizable && (st = grow_for_mixed(t, ops, n, s)) != HIVE_OK) return st;
   // inserts that find no room at all go to list B, the pending list that
   // finish_resizable drains
@@ -865,8 +899,8 @@ hive_status hive_memory(hive_table* t, uint64_t* committed, uint64_t* reserved) 
   const uint64_t other = t->nb_max * (t->S + 2 * sizeof(uint32_t)) + t->stash_alloc * sizeof(uint64_t) +
                          t->stash_cap * sizeof(uint32_t) + sizeof(Ctrl) +
                          (t->list_cap + t->lb_cap) * 12 +
-                         t->part_cap * 12 +
-                         part_tiles(t->part_cap) * (kPartMaxRegions + 1) * sizeof(uint16_t);
+                         t->part_cap * 12 + part_off_bytes(t->part_cap) + t->lists_kept.bytes +
+                         t->part_kept.bytes;
   *committed = bucket_now + other;
   *reserved = bucket_max + other;
   return HIVE_OK;

@@ -209,6 +209,21 @@ cudaError_t launch_hash(const uint32_t* keys, uint64_t n, uint32_t* h1, uint32_t
                         cudaStream_t s);
 cudaError_t query_occupancy(Launch* L, int S);
 
+// Whether stream s is being captured into a graph.
+bool stream_capturing(cudaStream_t s);
+// Scratch arrays that a call under stream capture has used: the graph keeps
+// their addresses, so when the arrays grow the old ones are kept until the
+// table goes.  (The arrays grow to powers of two, so the kept ones stay of the
+// order of those in use.)
+struct Retired {
+  bool captured = false;  // the arrays in use are in some graph
+  std::vector<void*> old;
+  uint64_t bytes = 0;  // of the arrays in `old`
+  // Gives up array p of n bytes: frees it, or keeps it for the graphs.
+  void drop(void* p, uint64_t n);
+  void release();  // frees what was kept
+};
+
 // ---- tables with 32-bit entries (hive32_*) ----
 struct View32 {
   uint32_t* buckets;     // [nb * 32] entries
@@ -296,6 +311,7 @@ struct hive_table {
   uint32_t* la_idx = nullptr;
   uint64_t* lb_words = nullptr;  // list B: items that found no room
   uint32_t* lb_idx = nullptr;
+  hive::Retired lists_kept, part_kept;
   // list of a bulk insert that stores by region (allocated on first use)
   uint64_t part_cap = 0;         // ops it holds
   uint64_t* part_words = nullptr;
