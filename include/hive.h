@@ -524,7 +524,8 @@ hive_status hive_check_batch(const uint8_t* h_ops, uint32_t op, const uint32_t* 
  * Neither makes the GPU fault or hang.
  *
  * hive_debug_fail_alloc: the n-th device allocation the library makes from
- * now on (counted over every table of the process, n >= 1) fails as if the
+ * now on (counted over every table of the process, n >= 1, the physical
+ * memory that a map_on_demand table maps as it grows included) fails as if the
  * device were out of memory; n = 0 cancels a pending failure.  The call that
  * made the allocation returns HIVE_ERR_OOM and leaves its table as it was
  * (hive_create frees what it had allocated; an op call queues nothing and

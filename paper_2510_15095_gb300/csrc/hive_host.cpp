@@ -245,10 +245,15 @@ hive_status readback(hive_table* t, cudaStream_t s) {
 // One expansion launch (Section IV-C1).
 hive_status split_step(hive_table* t, cudaStream_t s, bool* did) {
   SplitPlan pl{};
+  const ResizeState before(t);
   *did = plan_split(t, &pl);
   if (!*did) return HIVE_OK;
   hive_status st = ensure_committed(t, s);
-  if (st != HIVE_OK) return st;
+  if (st != HIVE_OK) {
+    before.restore(t);
+    *did = false;
+    return st;
+  }
   View v = make_view(t);
   v.M = pl.M;
   v.p = pl.p;
@@ -502,11 +507,14 @@ namespace hive {
 namespace {
 std::atomic<uint32_t> g_fail_alloc{0};  // 0: off; n: the n-th allocation from now fails
 }  // namespace
-cudaError_t dev_alloc_raw(void** p, size_t bytes) {
+bool alloc_fails() {
   uint32_t c = g_fail_alloc.load();
   while (c != 0 && !g_fail_alloc.compare_exchange_weak(c, c - 1)) {
   }
-  if (c == 1) {
+  return c == 1;
+}
+cudaError_t dev_alloc_raw(void** p, size_t bytes) {
+  if (alloc_fails()) {
     *p = nullptr;
     return cudaErrorMemoryAllocation;
   }

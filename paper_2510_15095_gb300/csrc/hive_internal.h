@@ -346,6 +346,19 @@ struct SplitPlan {
 // Advances the host-side state of t by one split launch and returns its plan;
 // false when the table is at nb_max.
 bool plan_split(hive_table* t, SplitPlan* out);
+// The host-side state that plan_split advances, to put it back when the memory
+// of the new buckets cannot be had (the table would address unmapped ones).
+struct ResizeState {
+  uint32_t M, p;
+  uint64_t nb, splits;
+  explicit ResizeState(const hive_table* t) : M(t->M), p(t->p), nb(t->nb), splits(t->splits) {}
+  void restore(hive_table* t) const {
+    t->M = M;
+    t->p = p;
+    t->nb = nb;
+    t->splits = splits;
+  }
+};
 bool over_grow(const hive_table* t, uint64_t live, uint64_t nb);
 bool under_shrink(const hive_table* t, uint64_t live, uint64_t nb);
 // Contraction loop after a batch (Section IV-C2); reads counters back.
@@ -356,7 +369,9 @@ void free_staging(hive_table* t);  // releases the host-buffer call staging
 hive_status ensure_committed(hive_table* t, cudaStream_t s);
 bool table_view(const hive_table* t, View* v, Launch* L, bool* resizable);
 // Every device allocation of the library goes through here, so that a test
-// can make one of them fail on the host (hive_debug_fail_alloc).
+// can make one of them fail on the host (hive_debug_fail_alloc); grow_commit
+// asks alloc_fails() for its physical allocations.
+bool alloc_fails();
 cudaError_t dev_alloc_raw(void** p, size_t bytes);
 void set_fail_alloc(uint32_t n);  // hive_debug_fail_alloc
 template <class T>

@@ -338,6 +338,13 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   m->jobs.clear();
   m->wave_begin.clear();
   std::vector<std::vector<MultiJob>> waves;
+  std::vector<ResizeState> before;
+  for (uint32_t t : touched) before.emplace_back(m->tables[t]);
+  // a failure before the splits are queued leaves the tables as they were
+  auto undo = [&](hive_status st) {
+    for (size_t i = 0; i < touched.size(); ++i) before[i].restore(m->tables[touched[i]]);
+    return st;
+  };
   for (uint32_t t : touched) {
     hive_table* tb = m->tables[t];
     if (!tb->cfg.resizable || !ins[t]) continue;
@@ -355,12 +362,12 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
     }
     if (any && tb->host_ctrl->stash_n) {
       hive_status st = mark_stash_dirty(tb, s);
-      if (st != HIVE_OK) return st;
+      if (st != HIVE_OK) return undo(st);
     }
   }
   for (uint32_t t : touched) {  // back the buckets the split waves create
     hive_status st = ensure_committed(m->tables[t], s);
-    if (st != HIVE_OK) return st;
+    if (st != HIVE_OK) return undo(st);
   }
   for (auto& w : waves) {
     m->wave_begin.push_back(static_cast<uint32_t>(m->jobs.size()));
@@ -372,7 +379,8 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
     }
   }
   if (m->jobs.size() > m->max_jobs)
-    return mfail(HIVE_ERR_INVALID_ARG, "batch needs more split launches than the staging holds");
+    return undo(
+        mfail(HIVE_ERR_INVALID_ARG, "batch needs more split launches than the staging holds"));
 
   // (2) staging
   uint8_t* h = sl.h_stage;
@@ -405,7 +413,8 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   if (!m->jobs.empty())
     std::memcpy(jobs_of(m, h), m->jobs.data(), m->jobs.size() * sizeof(MultiJob));
   const size_t bytes = m->off_jobs + m->jobs.size() * sizeof(MultiJob);
-  MCK(launch_stage(m->d_stage, h, bytes, s));
+  const cudaError_t staged = launch_stage(m->d_stage, h, bytes, s);
+  if (staged != cudaSuccess) return undo(mcuda(staged, "launch_stage"));
 
   // split waves, in order
   for (size_t w = 0; w < m->wave_begin.size(); ++w) {

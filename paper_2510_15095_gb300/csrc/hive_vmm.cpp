@@ -105,7 +105,7 @@ cudaError_t grow_commit(GrowArray* a, size_t bytes, cudaStream_t s) {
   acc.location = p.location;
   acc.flags = CU_MEM_ACCESS_FLAGS_PROT_READWRITE;
   CUmemGenericAllocationHandle h = 0;
-  if (d.create(&h, delta, &p, 0) != CUDA_SUCCESS) return cudaErrorMemoryAllocation;
+  if (alloc_fails() || d.create(&h, delta, &p, 0) != CUDA_SUCCESS) return cudaErrorMemoryAllocation;
   const CUdeviceptr at = a->base + a->committed;
   if (d.map(at, delta, 0, h, 0) != CUDA_SUCCESS) {
     d.release(h);

@@ -1,0 +1,93 @@
+"""Growth that cannot get memory (the failure is made on the host): the call
+returns OOM, the table keeps its capacity and every key, and the same call
+succeeds once memory can be had."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2510_15095_gb300 import workload as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def H():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_15095_gb300 import hive
+    hive.load_library()
+    yield hive
+    hive.debug_fail_alloc(0)
+
+
+def up(H, a):
+    return H.to_device_u32(a)
+
+
+def check(H, t, d, keys):
+    v, f = t.find(up(H, keys))
+    ev, ef = d.find(keys)
+    assert np.array_equal(H.to_host_u32(v), ev) and np.array_equal(f.cpu().numpy(), ef)
+    img = t.dump()
+    code, where = oracle.check_image(img, img["S"], d, None)
+    assert code == 0, f"invariant {code} fails at {where}"
+    assert t.size() == len(d)
+
+
+def on_demand(H, bs, **kw):
+    # 2^18 slots fill the 2 MB that the driver maps at a time
+    return H.HiveTable(1 << 18, max_slots=1 << 22, resizable=True, bucket_slots=bs,
+                       map_on_demand=True, **kw)
+
+
+@pytest.mark.parametrize("bs", [16, 32])
+def test_reserve_without_memory(H, bs):
+    t, d = on_demand(H, bs), oracle.Dict()
+    keys, _ = W.take_keys(701, 0, 100_000)
+    vals = W.values_for(keys, 701)
+    t.insert(up(H, keys), up(H, vals))
+    d.insert(keys, vals)
+    cap = t.capacity()
+    H.debug_fail_alloc(1)
+    with pytest.raises(H.HiveError) as e:
+        t.reserve(1 << 20)
+    assert "OOM" in str(e.value) and t.capacity() == cap and t.stats()["splits"] == 0
+    check(H, t, d, keys)
+    t.reserve(1 << 20)
+    assert t.capacity() >= 1 << 20
+    check(H, t, d, keys)
+    assert t.check() == 0
+    t.close()
+
+
+@pytest.mark.parametrize("asynchronous", [False, True])
+def test_multi_table_growth_without_memory(H, asynchronous):
+    tabs = [on_demand(H, 16) for _ in range(3)]
+    dicts = [oracle.Dict() for _ in tabs]
+    m = H.HiveMulti(tabs, max_segments=4, max_ops=1 << 20, asynchronous=asynchronous)
+    keys, vals, segs = [], [], []
+    for j in range(3):
+        k, _ = W.take_keys(710 + j, 0, 300_000)
+        keys.append(k)
+        vals.append(W.values_for(k, 710 + j))
+        segs.append({"table": j, "ops": torch.zeros(k.size, dtype=torch.uint8, device="cuda"),
+                     "keys": up(H, k), "vals": up(H, vals[j]),
+                     "status": torch.full((k.size,), 9, dtype=torch.uint8, device="cuda")})
+    caps = [t.capacity() for t in tabs]
+    H.debug_fail_alloc(2)  # the second table's buckets
+    with pytest.raises(H.HiveError) as e:
+        m.execute(segs)
+    assert "OOM" in str(e.value)
+    torch.cuda.synchronize()
+    assert [t.capacity() for t in tabs] == caps and [t.size() for t in tabs] == [0, 0, 0]
+    m.execute(segs)
+    torch.cuda.synchronize()
+    for j, t in enumerate(tabs):
+        assert np.array_equal(segs[j]["status"].cpu().numpy(), dicts[j].insert(keys[j], vals[j]))
+        assert t.capacity() > caps[j]
+        check(H, t, dicts[j], keys[j])
+        assert t.check() == 0
+    m.close()
+    for t in tabs:
+        t.close()
