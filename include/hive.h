@@ -54,7 +54,10 @@ typedef enum {
   HIVE_OK = 0,
   HIVE_ERR_INVALID_ARG = 1,  /* bad pointer, size or configuration */
   HIVE_ERR_RESERVED_KEY = 2, /* sticky: an op used a reserved key */
-  HIVE_ERR_OOM = 3,          /* device allocation failed; table unchanged */
+  HIVE_ERR_OOM = 3,          /* device allocation failed; table unchanged, unless a
+                                resizable table had to grow in the middle of a
+                                batch: then every op has run, and the inserts that
+                                found no room report FULL (also sticky) */
   HIVE_ERR_FULL = 4,         /* sticky: fixed table had no room for some insert */
   HIVE_ERR_TIMEOUT = 5,      /* sticky: a bounded wait gave up (bucket lock) */
   HIVE_ERR_CUDA = 6,         /* a CUDA runtime call failed */

@@ -346,13 +346,13 @@ hive_status finish_resizable(hive_table* t, uint8_t* status, cudaStream_t s,
                                  kMaintStash | (pending_in_b ? kMaintUnlessPend : kMaintUnlessOvf),
                                  t->host_ctrl));
   HIVE_CK(cudaStreamSynchronize(s));
-  hive_status st = HIVE_OK;
+  hive_status st = HIVE_OK, grown = HIVE_OK;
   bool in_b = pending_in_b, again = false;
   while ((in_b ? t->host_ctrl->pend_n : t->host_ctrl->ovf_n) != 0) {
     again = true;
     bool did = false;
-    st = split_step(t, s, &did);
-    if (st != HIVE_OK) return st;
+    // no memory to grow into: as at nb_max, and the call returns the error
+    grown = split_step(t, s, &did);
     View v = make_view(t);
     List in = in_b ? list_b(t) : list_a(t);
     List out = in_b ? list_a(t) : list_b(t);
@@ -367,13 +367,13 @@ hive_status finish_resizable(hive_table* t, uint8_t* status, cudaStream_t s,
     if (!did) break;
   }
   if (again) {
+    // also empties the op lists, whose counts the first pass left alone
     HIVE_LAUNCH(t, HIVE_K_MAINT, s,
                 launch_maintenance(make_view(t), s, kMaintStash, t->host_ctrl));
     HIVE_CK(cudaStreamSynchronize(s));
   }
   t->size_host = t->host_ctrl->size;
-
-  return contract_table(t, s);
+  return grown != HIVE_OK ? grown : contract_table(t, s);
 }
 
 }  // namespace
@@ -446,7 +446,7 @@ hive_status hive::contract_table(hive_table* t, cudaStream_t s) {
       break;
     }
     st = ensure_lists(t, static_cast<uint64_t>(count) * t->S, s);
-    if (st != HIVE_OK) return st;
+    if (st != HIVE_OK) break;  // the waves before this one stand
     HIVE_LAUNCH(t, HIVE_K_MERGE, s, launch_merge(vn, count, list_a(t), s));
     t->M = trial.M;
     t->p = trial.p;
@@ -467,7 +467,7 @@ hive_status hive::contract_table(hive_table* t, cudaStream_t s) {
       if (t->bucket_vm.committed > need + 2 * t->bucket_vm.gran) grow_decommit(&t->bucket_vm, need);
     }
   }
-  return HIVE_OK;
+  return st;
 }
 
 bool hive::plan_split(hive_table* t, SplitPlan* out) {

@@ -91,3 +91,57 @@ def test_multi_table_growth_without_memory(H, asynchronous):
     m.close()
     for t in tabs:
         t.close()
+
+
+@pytest.mark.parametrize("bs", [16, 32])
+@pytest.mark.parametrize("call", ["insert", "execute", "execute_large", "fused"])
+def test_batch_that_cannot_grow_in_the_middle(H, bs, call):
+    """Inserts that fill the last slots find no room, and the table cannot get
+    memory for the split they ask for: every other op of the batch has run, the
+    op lists start empty in the next call, and the same inserts succeed then."""
+    slots = 1 << 18
+    n_new = 60_000
+    keys, c = W.take_keys(721, 0, slots)
+    live, new = keys[:slots - n_new], keys[slots - n_new:]
+    t = on_demand(H, bs, grow=(1, 1), shrink=(1, 10), max_evictions=1, stash_permille=0)
+    d = oracle.Dict()
+    lv = W.values_for(live, 721)
+    for part in np.array_split(np.arange(live.size), 2):
+        t.insert(up(H, live[part]), up(H, lv[part]))
+    d.insert(live, lv)
+    n_find = {"insert": 0, "execute": 100_000, "execute_large": 300_000, "fused": 100_000}[call]
+    rng = np.random.default_rng(bs)
+    mk = np.concatenate([new, rng.choice(live, n_find)])
+    ops = np.concatenate([np.zeros(n_new, np.uint8), np.ones(n_find, np.uint8)])
+    order = rng.permutation(mk.size)
+    mk, ops = mk[order], ops[order]
+    mv = np.where(ops == 0, W.values_for(mk, 722), 0).astype(np.uint32)
+    args = (torch.from_numpy(ops).cuda(), up(H, mk), up(H, mv))
+
+    def run():
+        if call == "insert":
+            return t.insert(args[1], args[2])
+        return t.execute(*args, fused=call == "fused")[1]
+
+    cap = t.capacity()
+    if call.startswith("execute") or call == "fused":  # the lists have the batch's length
+        t.execute(torch.ones_like(args[0]), args[1])
+    else:
+        t.erase(args[1])  # absent
+        t.execute(torch.ones_like(args[0]), args[1])
+    H.debug_fail_alloc(1)
+    with pytest.raises(H.HiveError) as e:
+        run()
+    assert "OOM" in str(e.value) and t.capacity() == cap
+    d.execute(ops, mk, mv)
+    there = t.find(up(H, new))[1].cpu().numpy().astype(bool)
+    assert 0 < (~there).sum() < n_new
+    d.erase(new[~there])
+    check(H, t, d, keys)
+    assert t.check() == 4  # FULL: inserts found no room
+    st = run()
+    assert np.array_equal(st.cpu().numpy(), d.execute(ops, mk, mv)[1])
+    assert t.capacity() > cap
+    check(H, t, d, keys)
+    assert t.check() == 0
+    t.close()
