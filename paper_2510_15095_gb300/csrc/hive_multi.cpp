@@ -84,6 +84,8 @@ struct hive_multi {
   uint32_t* ovf_idx = nullptr;
   uint32_t* ovf_seg = nullptr;
   unsigned* d_count = nullptr;
+  bool count_zero = false;  // the newest batch has left d_count at 0 (not before the
+                            // first one, nor after one that failed half-way)
   // per-table size and stash fill after a batch (entries of touched tables),
   // in pinned memory that the maintenance kernel writes
   unsigned long long* h_gather = nullptr;
@@ -265,7 +267,6 @@ hive_status hive_multi_create(hive_table* const* tables, uint32_t n_tables, uint
   if (e == cudaSuccess) e = cudaMalloc(&m->ovf_idx, max_ops * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&m->ovf_seg, max_ops * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&m->d_count, sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMemset(m->d_count, 0, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMallocHost(&m->h_gather, 2 * sizeof(unsigned long long) * n_tables);
   if (e == cudaSuccess && m->use_graph)
     e = cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking);
@@ -427,6 +428,8 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   }
 
   // (3) the fixed part
+  if (!m->count_zero) MCK(cudaMemsetAsync(m->d_count, 0, sizeof(unsigned), s));
+  m->count_zero = false;
   if (m->use_graph) {
     if (!m->graph) {
       MCK(cudaStreamBeginCapture(m->cap_stream, cudaStreamCaptureModeThreadLocal));
@@ -447,6 +450,7 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
     hive_status st = enqueue_fixed(m, s);
     if (st != HIVE_OK) return st;
   }
+  m->count_zero = true;
   MCK(cudaEventRecord(sl.done, s));
   sl.seq = ++m->seq;
   sl.applied = false;
