@@ -555,6 +555,14 @@ bool table_view(const hive_table* t, View* v, Launch* L, bool* resizable) {
   return true;
 }
 void set_last_error(const std::string& msg) { g_err = msg; }
+cudaError_t take_size(hive_table* t) {
+  if (!t->size_from) return cudaSuccess;
+  const cudaError_t e = cudaEventSynchronize(t->size_from->done[t->size_slot]);
+  if (e != cudaSuccess) return e;
+  t->size_host = t->size_from->sizes[2 * t->size_at];
+  t->size_from.reset();
+  return cudaSuccess;
+}
 }  // namespace hive
 
 extern "C" {
@@ -939,6 +947,7 @@ hive_status hive_clear(hive_table* t, void* stream) {
   t->M = static_cast<uint32_t>(pow2 - 1);
   t->p = static_cast<uint32_t>(t->nb_init - pow2);
   t->size_host = 0;
+  t->size_from.reset();
   t->splits = t->merges = 0;
   std::memset(t->host_ctrl, 0, sizeof(Ctrl));
   return HIVE_OK;

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -209,6 +210,21 @@ cudaError_t launch_hash(const uint32_t* keys, uint64_t n, uint32_t* h1, uint32_t
                         cudaStream_t s);
 cudaError_t query_occupancy(Launch* L, int S);
 
+// Where the batches of a multi-table group leave its tables' sizes: pinned
+// memory that the maintenance kernel writes, and the events of the group's two
+// staging slots.  Tables and the group share it, and either may go first.
+struct SizeSource {
+  unsigned long long* sizes = nullptr;  // per table: size, then error bits and stash fill
+  cudaEvent_t done[2] = {nullptr, nullptr};
+  SizeSource() = default;
+  SizeSource(const SizeSource&) = delete;
+  SizeSource& operator=(const SizeSource&) = delete;
+  ~SizeSource() {
+    if (sizes) cudaFreeHost(sizes);
+    for (cudaEvent_t e : done)
+      if (e) cudaEventDestroy(e);
+  }
+};
 // Whether stream s is being captured into a graph.
 bool stream_capturing(cudaStream_t s);
 // Scratch arrays that a call under stream capture has used: the graph keeps
@@ -318,6 +334,10 @@ struct hive_table {
   uint32_t* part_slots = nullptr;
   uint16_t* part_off = nullptr;
   uint64_t size_host = 0;       // exact after each resizable call
+  // a batch of a synchronous group of fixed tables, not waited for, has gathered
+  // a newer size_host: entry size_at of the source, there when size_slot is done
+  std::shared_ptr<hive::SizeSource> size_from;
+  uint32_t size_at = 0, size_slot = 0;
   uint64_t splits = 0, merges = 0;
   bool merge_deferred = false;
   // profiling hook: events bracketing each launch while enabled
@@ -337,6 +357,9 @@ struct hive_table {
 // Helpers shared by the translation units of the library (hive_host.cpp
 // defines these).
 namespace hive {
+// Takes the size that a batch has gathered for t, if one is to be taken (waits
+// for the batch).
+cudaError_t take_size(hive_table* t);
 View make_view(const hive_table* t);
 // The next expansion launch of a table (Section IV-C1): bucket pairs
 // (src0 + i, src0 + i + half) for i < count, leaving the table at (M, p).

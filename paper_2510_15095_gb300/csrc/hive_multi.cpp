@@ -23,6 +23,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -56,7 +57,7 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // One of the two staging slots: a batch in flight owns one.
 struct Slot {
   uint8_t* h_stage = nullptr;
-  cudaEvent_t done = nullptr;       // recorded after the batch
+  cudaEvent_t done = nullptr;       // recorded after the batch (owned by the group's sizes)
   uint64_t seq = 0;                 // batch number, 0 = never used
   bool applied = true;              // its gathered sizes have been taken
   std::vector<uint32_t> touched;    // tables of the batch
@@ -86,14 +87,9 @@ struct hive_multi {
   unsigned* d_count = nullptr;
   bool count_zero = false;  // the newest batch has left d_count at 0 (not before the
                             // first one, nor after one that failed half-way)
-  // per-table size and stash fill after a batch (entries of touched tables),
-  // in pinned memory that the maintenance kernel writes
-  unsigned long long* h_gather = nullptr;
+  // per-table size and stash fill after a batch (entries of touched tables)
+  std::shared_ptr<SizeSource> sizes;
   std::vector<uint64_t> ub;  // asynchronous mode: upper bound of each size
-  // synchronous groups of fixed tables: tables whose gathered size is still to
-  // be taken, and whether there are any
-  std::vector<char> stale;
-  bool untaken = false;
   cudaGraphExec_t graph = nullptr;
   cudaStream_t cap_stream = nullptr;
   std::vector<MultiJob> jobs;
@@ -161,12 +157,12 @@ hive_status enqueue_fixed(hive_multi* m, cudaStream_t s) {
   MCK(launch_multi_overflow(S, segs, ovf, m->L, s));
   // also writes the sizes to the host and empties the overflow list for the
   // next batch
-  MCK(launch_multi_maint(S, hd, dv, tc, nt, m->d_count, m->h_gather, s));
+  MCK(launch_multi_maint(S, hd, dv, tc, nt, m->d_count, m->sizes->sizes, s));
   return HIVE_OK;
 }
 
 // Asynchronous mode: take the sizes gathered by the newest completed batch.
-// h_gather holds them, or sizes of a later batch in flight that completed
+// The group's sizes hold them, or sizes of a later batch in flight that completed
 // meanwhile; either way gathered size + inserts of later batches bounds the
 // size from above.
 void refresh_bounds(hive_multi* m) {
@@ -179,41 +175,23 @@ void refresh_bounds(hive_multi* m) {
   Slot* later = nullptr;
   for (auto& sl : m->slot)
     if (sl.seq > newest->seq && !sl.applied) later = &sl;
-  for (uint32_t t : newest->touched) m->ub[t] = m->h_gather[2 * t];
+  for (uint32_t t : newest->touched) m->ub[t] = m->sizes->sizes[2 * t];
   if (later)
     for (size_t j = 0; j < later->touched.size(); ++j) m->ub[later->touched[j]] += later->ins[j];
   for (auto& sl : m->slot)
     if (sl.seq && sl.seq <= newest->seq) sl.applied = true;
 }
 
-// Synchronous group of fixed tables: waits for the newest batch and takes the
-// gathered sizes of the tables that batches have touched since.
-cudaError_t take_sizes(hive_multi* m) {
-  if (!m->untaken) return cudaSuccess;
-  const cudaError_t e = cudaEventSynchronize(m->slot[(m->seq - 1) & 1].done);
-  if (e != cudaSuccess) return e;
-  for (size_t t = 0; t < m->tables.size(); ++t)
-    if (m->stale[t]) {
-      m->tables[t]->size_host = m->ub[t] = m->h_gather[2 * t];
-      m->stale[t] = 0;
-    }
-  m->untaken = false;
-  return cudaSuccess;
-}
-
 void release(hive_multi* m) {
   if (m->graph) cudaGraphExecDestroy(m->graph);
   if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
   cudaFree(m->d_stage);
-  for (auto& sl : m->slot) {
+  for (auto& sl : m->slot)
     if (sl.h_stage) cudaFreeHost(sl.h_stage);
-    if (sl.done) cudaEventDestroy(sl.done);
-  }
   cudaFree(m->ovf_words);
   cudaFree(m->ovf_idx);
   cudaFree(m->ovf_seg);
   cudaFree(m->d_count);
-  if (m->h_gather) cudaFreeHost(m->h_gather);
   delete m;
 }
 
@@ -242,10 +220,14 @@ hive_status hive_multi_create(hive_table* const* tables, uint32_t n_tables, uint
       delete m;
       return mfail(HIVE_ERR_INVALID_ARG, "all tables of a group need the same bucket_slots");
     }
+    const cudaError_t e = take_size(tables[i]);
+    if (e != cudaSuccess) {
+      delete m;
+      return mcuda(e, "taking a table's size");
+    }
     m->tables.push_back(tables[i]);
     m->any_resizable |= tables[i]->cfg.resizable != 0;
     m->ub.push_back(tables[i]->size_host);
-    m->stale.push_back(0);
   }
   m->max_segs = max_segments;
   m->max_ops = max_ops;
@@ -258,16 +240,25 @@ hive_status hive_multi_create(hive_table* const* tables, uint32_t n_tables, uint
   m->off_touched = align_up(m->off_views + sizeof(View) * n_tables, 64);
   m->off_jobs = align_up(m->off_touched + sizeof(uint32_t) * n_tables, 64);
   m->stage_bytes = align_up(m->off_jobs + sizeof(MultiJob) * m->max_jobs, 256);
+  try {
+    m->sizes = std::make_shared<SizeSource>();
+  } catch (const std::bad_alloc&) {
+    delete m;
+    return mfail(HIVE_ERR_OOM, "host allocation failed");
+  }
   cudaError_t e = cudaMalloc(&m->d_stage, m->stage_bytes);
-  for (auto& sl : m->slot) {
+  for (int k = 0; k < 2; ++k) {
+    Slot& sl = m->slot[k];
     if (e == cudaSuccess) e = cudaMallocHost(&sl.h_stage, m->stage_bytes);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->sizes->done[k], cudaEventDisableTiming);
+    sl.done = m->sizes->done[k];
   }
   if (e == cudaSuccess) e = cudaMalloc(&m->ovf_words, max_ops * sizeof(uint64_t));
   if (e == cudaSuccess) e = cudaMalloc(&m->ovf_idx, max_ops * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&m->ovf_seg, max_ops * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&m->d_count, sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMallocHost(&m->h_gather, 2 * sizeof(unsigned long long) * n_tables);
+  if (e == cudaSuccess) 
+    e = cudaMallocHost(&m->sizes->sizes, 2 * sizeof(unsigned long long) * n_tables);
   if (e == cudaSuccess && m->use_graph)
     e = cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
@@ -289,11 +280,11 @@ hive_status hive_multi_destroy(hive_multi* m) {
 hive_status hive_multi_bounds(hive_multi* m, uint64_t* out, uint32_t n_tables) {
   if (!m || !out) return mfail(HIVE_ERR_INVALID_ARG, "group and out must not be NULL");
   if (n_tables > m->tables.size()) return mfail(HIVE_ERR_INVALID_ARG, "n_tables above the group's");
-  if (m->async)
-    refresh_bounds(m);
-  else if (!m->any_resizable)
-    MCK(take_sizes(m));
-  for (uint32_t t = 0; t < n_tables; ++t) out[t] = m->async ? m->ub[t] : m->tables[t]->size_host;
+  if (m->async) refresh_bounds(m);
+  for (uint32_t t = 0; t < n_tables; ++t) {
+    if (!m->async) MCK(take_size(m->tables[t]));
+    out[t] = m->async ? m->ub[t] : m->tables[t]->size_host;
+  }
   return HIVE_OK;
 }
 
@@ -464,8 +455,12 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   // nothing of a group of fixed tables depends on the batch's outcome
   // (hive_multi_bounds takes the sizes when it is asked)
   if (!m->async && !m->any_resizable) {
-    for (uint32_t t : touched) m->stale[t] = 1;
-    m->untaken = true;
+    for (uint32_t t : touched) {
+      hive_table* tb = m->tables[t];
+      tb->size_from = m->sizes;
+      tb->size_at = t;
+      tb->size_slot = static_cast<uint32_t>(&sl - m->slot);
+    }
     return HIVE_OK;
   }
   if (m->async) return HIVE_OK;
@@ -475,7 +470,8 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   sl.applied = true;
   for (uint32_t t : touched) {
     hive_table* tb = m->tables[t];
-    tb->size_host = m->h_gather[2 * t];
+    tb->size_host = m->sizes->sizes[2 * t];
+    tb->size_from.reset();
     m->ub[t] = tb->size_host;
     if (tb->cfg.resizable && tb->nb > tb->nb_init && under_shrink(tb, tb->size_host, tb->nb)) {
       hive_status st = contract_table(tb, s);
