@@ -380,12 +380,15 @@ hive_status hive_multi_create(hive_table* const* tables, uint32_t n_tables,
                               uint32_t max_segments, uint64_t max_ops, int flags,
                               void* stream, hive_multi** out);
 
-/* Runs one batch on `stream`.  Consecutive batches of one group go on one
- * stream.  Without HIVE_MULTI_ASYNC, a group holding resizable tables waits
+/* Runs one batch on `stream`.  A batch on another stream than the one before
+ * runs after it.  Without HIVE_MULTI_ASYNC, a group holding resizable tables waits
  * once for the batch (exact sizes, contraction policy applied to its tables);
  * otherwise the call returns after queueing, waiting only for the batch
- * queued two calls earlier.  Errors: INVALID_ARG (bad segment, too many ops,
- * segments or split launches), CUDA. */
+ * queued two calls earlier: results are there, and host arrays may be touched
+ * or freed, once the work on `stream` has completed.  Errors: INVALID_ARG
+ * (bad segment, too many ops, segments or split launches), OOM (no memory for
+ * a table's growth; nothing queued), CUDA (also for a stream that is being
+ * captured, without HIVE_MULTI_ASYNC). */
 hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t n_segs,
                                void* stream);
 

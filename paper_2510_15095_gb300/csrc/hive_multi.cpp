@@ -80,6 +80,7 @@ struct hive_multi {
   uint8_t* d_stage = nullptr;
   Slot slot[2];
   uint64_t seq = 0;
+  cudaStream_t last = nullptr;  // stream of the newest batch
   // overflow list of a batch (entries tagged with their segment)
   uint64_t* ovf_words = nullptr;
   uint32_t* ovf_idx = nullptr;
@@ -294,6 +295,9 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   if (n_segs > m->max_segs) return mfail(HIVE_ERR_INVALID_ARG, "more segments than max_segments");
   if (n_segs && !segs) return mfail(HIVE_ERR_INVALID_ARG, "segs must not be NULL");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  // the descriptors change with every batch, so a graph cannot replay one
+  if (!m->async && stream_capturing(s))
+    return mcuda(cudaErrorStreamCaptureUnsupported, "hive_multi_execute");
   const uint32_t nt = static_cast<uint32_t>(m->tables.size());
   uint64_t total_ops = 0;
   std::vector<uint64_t> ins(nt, 0);
@@ -324,6 +328,10 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   // is done (its staging buffer is then free).
   Slot& sl = m->slot[m->seq & 1];
   MCK(cudaEventSynchronize(sl.done));
+  // The device side of the staging and the tables are shared by all batches:
+  // one on another stream runs after the one before.
+  if (m->seq && (s != m->last || s == cudaStreamPerThread))
+    MCK(cudaStreamWaitEvent(s, m->slot[(m->seq - 1) & 1].done, 0));
   if (m->async) refresh_bounds(m);
 
   // (1) growth, planned as waves of split jobs
@@ -444,6 +452,7 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   m->count_zero = true;
   MCK(cudaEventRecord(sl.done, s));
   sl.seq = ++m->seq;
+  m->last = s;
   sl.applied = false;
   sl.touched = touched;
   sl.ins.clear();

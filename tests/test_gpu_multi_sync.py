@@ -54,3 +54,57 @@ def test_bounds_follow_the_newest_size(H):
     b.close()
     assert tabs[0].size() == 230
     tabs[0].close()
+
+
+def test_batches_on_two_streams_run_in_order(H):
+    """Consecutive batches of a group on different streams, none of them waited
+    for: each one's finds see the batch before."""
+    n, rounds = 150_000, 12
+    keys, _ = W.take_keys(6, 0, n * rounds)
+    tabs = [H.HiveTable(1 << 21, bucket_slots=16) for _ in range(2)]
+    m = H.HiveMulti(tabs, max_segments=4, max_ops=4 * n)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    batches = []
+    for r in range(rounds):
+        part = keys[n * r:n * (r + 1)]
+        segs = [seg(H, 0, part), seg(H, 1, part)]
+        if r:
+            prev = keys[n * (r - 1):n * r]
+            segs += [seg(H, 0, prev, op=H.OP_FIND), seg(H, 1, prev, op=H.OP_FIND)]
+        batches.append(segs)
+    torch.cuda.synchronize()
+    for r, segs in enumerate(batches):
+        m.execute(segs, stream=streams[r % 2])
+    assert m.bounds() == [n * rounds, n * rounds]
+    torch.cuda.synchronize()
+    for segs in batches:
+        for s in segs[:2]:
+            assert bool((s["status"] == H.INSERTED).all())
+        for s in segs[2:]:
+            assert bool((s["status"] == H.FOUND).all()) and bool((s["vals_out"] == s["vals"]).all())
+    m.close()
+    for t in tabs:
+        assert t.check() == 0
+        t.close()
+
+
+def test_capture_is_refused(H):
+    """A captured batch would replay descriptors that later batches replace."""
+    keys, _ = W.take_keys(7, 0, 100)
+    t = H.HiveTable(1 << 12, bucket_slots=16)
+    m = H.HiveMulti([t], max_segments=1, max_ops=1 << 10)
+    s = seg(H, 0, keys)
+    x = torch.zeros(4, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        with pytest.raises(H.HiveError) as e:
+            m.execute([s])
+        x += 1
+    assert "CUDA" in str(e.value)
+    g.replay()
+    m.execute([s])
+    assert m.bounds() == [100] and bool((x == 1).all())
+    assert bool((s["status"] == H.INSERTED).all())
+    m.close()
+    t.close()
