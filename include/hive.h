@@ -402,8 +402,8 @@ hive_status hive_multi_destroy(hive_multi* m);
  * memory uses these, and hive_capacity() of each table, instead of counting
  * inserts itself: erases make the bounds fall again.  Host-side; it queries
  * the batches' events and never waits, except that a synchronous group waits
- * here for the newest batch (of any such group) on each of its fixed tables.
- * INVALID_ARG for NULL pointers
+ * here for its newest batch (and for other groups' newest ones on its fixed
+ * tables).  INVALID_ARG for NULL pointers
  * or n_tables above the group's. */
 hive_status hive_multi_bounds(hive_multi* m, uint64_t* out, uint32_t n_tables);
 

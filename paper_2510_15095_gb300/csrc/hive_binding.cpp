@@ -153,6 +153,7 @@ using FindFn = int (*)(void*, const void*, uint64_t, void*, void*, void*);
 using ExecuteFn = int (*)(void*, const void*, const void*, const void*, uint64_t, void*, void*,
                           void*);
 using MultiFn = int (*)(void*, const hive_segment*, uint32_t, void*);
+using BoundsFn = int (*)(void*, uint64_t*, uint32_t);
 
 // insert(fn, table, keys, vals, status, stream) -> (code, status)
 PyObject* py_insert(PyObject*, PyObject* const* a, Py_ssize_t na) {
@@ -233,14 +234,28 @@ PyObject* item(PyObject* d, PyObject* key) {
   return o;
 }
 
-// multi(fn, group, [segment dicts], stream) -> code
+// multi(fn, group, [segment dicts], stream, bounds) -> (code, arrays)
+// bounds: hive_multi_bounds for a group whose batches are not waited for
+// otherwise, to wait for one that works on host memory (its arrays may be
+// touched when the call returns); 0 for the others.  arrays: the batch's
+// tensors when bounds is given, for the caller to keep while the batch runs.
 PyObject* py_multi(PyObject*, PyObject* const* a, Py_ssize_t na) {
-  return guarded(na, 4, [&]() -> PyObject* {
+  return guarded(na, 5, [&]() -> PyObject* {
     const auto fn = reinterpret_cast<MultiFn>(as_address(a[0]));
     void* h = as_address(a[1]);
+    const auto bounds = reinterpret_cast<BoundsFn>(as_address(a[4]));
     if (!PyList_CheckExact(a[2])) throw NotPlain();
     const Py_ssize_t n_segs = PyList_GET_SIZE(a[2]);
     std::vector<hive_segment> segs(n_segs > 0 ? n_segs : 1);
+    std::vector<PyObject*> arrays;  // borrowed until the tuple is made below
+    if (bounds) arrays.reserve(5 * n_segs);
+    bool host = false;
+    auto seen = [&](PyObject* o) {
+      if (!bounds || !o || o == Py_None) return o;
+      host |= !tensor_of(o).is_cuda();
+      arrays.push_back(o);
+      return o;
+    };
     for (Py_ssize_t i = 0; i < n_segs; ++i) {
       PyObject* d = PyList_GET_ITEM(a[2], i);
       if (!PyDict_CheckExact(d)) throw NotPlain();
@@ -258,16 +273,23 @@ PyObject* py_multi(PyObject*, PyObject* const* a, Py_ssize_t na) {
       g.reserved0 = 0;
       g.n = static_cast<uint64_t>(n);
       g.n_insert = ins_o ? PyLong_AsUnsignedLongLongMask(ins_o) : g.n;
-      g.ops = static_cast<const uint8_t*>(in_ptr(ops_o, 1, n, true));
-      g.keys = static_cast<const uint32_t*>(in_ptr(keys, 4, n, true));
-      g.vals = static_cast<const uint32_t*>(in_ptr(item(d, k_vals), 4, n, true));
-      g.vals_out = static_cast<uint32_t*>(out_ptr(item(d, k_vals_out), 4, n, true));
-      g.status = static_cast<uint8_t*>(out_ptr(item(d, k_status), 1, n, true));
+      g.ops = static_cast<const uint8_t*>(in_ptr(seen(ops_o), 1, n, true));
+      g.keys = static_cast<const uint32_t*>(in_ptr(seen(keys_o), 4, n, true));
+      g.vals = static_cast<const uint32_t*>(in_ptr(seen(item(d, k_vals)), 4, n, true));
+      g.vals_out = static_cast<uint32_t*>(out_ptr(seen(item(d, k_vals_out)), 4, n, true));
+      g.status = static_cast<uint8_t*>(out_ptr(seen(item(d, k_status)), 1, n, true));
     }
     void* s = stream_of(a[3]);
-    const int rc =
-        without_gil([&] { return fn(h, segs.data(), static_cast<uint32_t>(n_segs), s); });
-    return PyLong_FromLong(rc);
+    PyObject* held = PyTuple_New(static_cast<Py_ssize_t>(arrays.size()));
+    if (!held) throw NotPlain();
+    for (size_t i = 0; i < arrays.size(); ++i)
+      PyTuple_SET_ITEM(held, static_cast<Py_ssize_t>(i), Py_NewRef(arrays[i]));
+    const int rc = without_gil([&] {
+      uint64_t none = 0;
+      const int e = fn(h, segs.data(), static_cast<uint32_t>(n_segs), s);
+      return e == HIVE_OK && host ? bounds(h, &none, 0) : e;
+    });
+    return Py_BuildValue("(iN)", rc, held);
   });
 }
 

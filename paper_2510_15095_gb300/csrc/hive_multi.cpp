@@ -6,14 +6,16 @@
 // splits of one linear-hashing round, so the jobs of a wave touch disjoint
 // buckets), (2) writes segment descriptors, per-table views, the list of
 // tables the batch touches and the split jobs into one pinned staging buffer
-// that a single copy moves to the device, then (3) runs the fixed part --
+// that a copy kernel moves to the device, then (3) runs the fixed part --
 // bulk kernel over all segments, eviction kernel, stash maintenance and size
 // gather of the touched tables -- as direct launches or as one replay of a
 // CUDA graph captured on the first call.
 //
 // Two growth modes:
-//  - exact (default): the host waits for each batch, applies the contraction
-//    policy to its resizable tables and knows every size exactly;
+//  - exact (default): a group with resizable tables waits for each batch,
+//    applies the contraction policy and knows every size exactly; a group of
+//    fixed tables has nothing to decide after a batch and returns once it is
+//    queued (hive_multi_bounds waits for the sizes);
 //  - asynchronous (HIVE_MULTI_ASYNC): the host never waits for a batch it just
 //    queued.  Growth is planned from an upper bound of each size: the last
 //    gathered size plus the inserts of the batches queued after it.  Tables
@@ -281,7 +283,10 @@ hive_status hive_multi_destroy(hive_multi* m) {
 hive_status hive_multi_bounds(hive_multi* m, uint64_t* out, uint32_t n_tables) {
   if (!m || !out) return mfail(HIVE_ERR_INVALID_ARG, "group and out must not be NULL");
   if (n_tables > m->tables.size()) return mfail(HIVE_ERR_INVALID_ARG, "n_tables above the group's");
-  if (m->async) refresh_bounds(m);
+  if (m->async)
+    refresh_bounds(m);
+  else if (m->seq)
+    MCK(cudaEventSynchronize(m->slot[(m->seq - 1) & 1].done));
   for (uint32_t t = 0; t < n_tables; ++t) {
     if (!m->async) MCK(take_size(m->tables[t]));
     out[t] = m->async ? m->ub[t] : m->tables[t]->size_host;

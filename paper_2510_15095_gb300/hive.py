@@ -188,8 +188,9 @@ def _load_native(L):
         if not os.path.exists(BINDING_PATH):
             raise RuntimeError(f"{BINDING_PATH} is not built; run __graft_entry__.build()")
         for name in ("hive_insert", "hive_insert_noalloc", "hive_find", "hive_erase",
-                     "hive_execute", "hive_execute_fused", "hive_multi_execute", "hive32_insert",
-                     "hive32_find", "hive32_erase", "hive32_execute"):
+                     "hive_execute", "hive_execute_fused", "hive_multi_execute",
+                     "hive_multi_bounds", "hive32_insert", "hive32_find", "hive32_erase",
+                     "hive32_execute"):
             _fn[name] = C.cast(getattr(L, name), C.c_void_p).value
         spec = importlib.util.spec_from_file_location("hive_binding", BINDING_PATH)
         mod = importlib.util.module_from_spec(spec)
@@ -659,18 +660,41 @@ class HiveMulti:
         self._h = h
         self._hp = h.value
         self._N = _load_native(self._L)
+        # batches that execute() does not wait for, and the arrays they use
+        self._queues = not asynchronous and not any(t.config.resizable for t in self.tables)
+        self._arrays = [(), ()]
 
     def execute(self, segments, stream=None):
         """segments: iterable of dicts with keys table, ops, keys and optionally
         vals, vals_out, status (CUDA tensors, or pinned CPU tensors that the
-        kernels use in place) and n_insert (int)."""
+        kernels use in place) and n_insert (int).
+
+        Returns when the batch is queued on `stream` (default: the current
+        stream), so results are there for work queued behind it or once it has
+        been waited for.  Without asynchronous=True it returns when the batch
+        is done if a table is resizable or an array is in host memory.  Such a
+        group also keeps the arrays of the last two batches, which may still
+        run; bounds() and close() let them go."""
         segs = list(segments)
-        code = self._N.multi(_fn["hive_multi_execute"], self._hp, segs, stream)
-        if code is not NotImplemented:
+        r = self._N.multi(_fn["hive_multi_execute"], self._hp, segs, stream,
+                          _fn["hive_multi_bounds"] if self._queues else 0)
+        if r is NotImplemented:
+            r = self._execute(segs, stream)
+        code, arrays = r
+        if self._queues:
+            # a failed call may have queued part of a batch: its arrays stay
+            # with the ones of the batch before
             if code:
-                _raise(self._L, code)
-            return
+                self._arrays[-1] += arrays
+            else:
+                self._arrays = [self._arrays[-1], arrays]
+        if code:
+            _raise(self._L, code)
+
+    def _execute(self, segs, stream):
+        """The batch by ctypes: (code, arrays to keep)."""
         arr = (Segment * max(len(segs), 1))()
+        arrays = []
         for i, g in enumerate(segs):
             n = g["keys"].numel()
             arr[i].table = int(g["table"])
@@ -681,14 +705,22 @@ class HiveMulti:
             arr[i].vals = _sptr(g.get("vals"), 4, n, "vals")
             arr[i].vals_out = _sptr(g.get("vals_out"), 4, n, "vals_out")
             arr[i].status = _sptr(g.get("status"), 1, n, "status")
-        _raise(self._L, self._L.hive_multi_execute(self._h, arr, len(segs), _stream_ptr(stream)))
+            arrays += [g[k] for k in ("ops", "keys", "vals", "vals_out", "status")
+                       if g.get(k) is not None]
+        code = self._L.hive_multi_execute(self._h, arr, len(segs), _stream_ptr(stream))
+        if not code and self._queues and not all(x.is_cuda for x in arrays):
+            code = self._L.hive_multi_bounds(self._h, (C.c_uint64 * 1)(), 0)
+        return code, tuple(arrays)
 
     def bounds(self) -> list:
-        """hive_multi_bounds: upper bounds of the tables' live sizes (host
-        side; never waits)."""
+        """hive_multi_bounds: upper bounds of the tables' live sizes
+        (asynchronous=True; host side, never waits), or their exact sizes after
+        the newest batch, which it waits for."""
         n = len(self.tables)
         out = (C.c_uint64 * max(n, 1))()
         _raise(self._L, self._L.hive_multi_bounds(self._h, out, n))
+        if self._queues:
+            self._arrays = [(), ()]
         return [int(out[i]) for i in range(n)]
 
     def close(self):
@@ -696,6 +728,7 @@ class HiveMulti:
             self._L.hive_multi_destroy(self._h)
             self._h = None
             self._hp = 0
+            self._arrays = [(), ()]
 
     def __del__(self):
         try:

@@ -108,3 +108,61 @@ def test_capture_is_refused(H):
     assert bool((s["status"] == H.INSERTED).all())
     m.close()
     t.close()
+
+
+@pytest.mark.parametrize("native", [True, False])
+def test_host_arrays_are_done_when_the_call_returns(H, native):
+    """Results in pinned memory are read, and pinned inputs dropped and their
+    memory handed out again, right after execute()."""
+    n = 400_000
+    keys, _ = W.take_keys(8, 0, 4 * n)
+    t = H.HiveTable(1 << 22, bucket_slots=16)
+    m = H.HiveMulti([t], max_segments=2, max_ops=2 * n)
+    if not native:
+        m._N = type("Never", (), {"multi": lambda *a: NotImplemented})()
+    for r in range(4):
+        s = seg(H, 0, keys[n * r:n * (r + 1)], dev="cpu")
+        m.execute([s])
+        status, want = s["status"].numpy().copy(), s["vals"].numpy().copy()
+        assert (status == H.INSERTED).all()
+        del s
+        junk = [torch.full((n,), 1, dtype=torch.int32).pin_memory() for _ in range(4)]
+        f = seg(H, 0, keys[n * r:n * (r + 1)], dev="cpu", op=H.OP_FIND)
+        m.execute([f])
+        assert (f["vals_out"].numpy() == want).all() and (f["status"].numpy() == H.FOUND).all()
+        del f, junk
+    assert m.bounds() == [4 * n]
+    m.close()
+    t.close()
+
+
+@pytest.mark.parametrize("native", [True, False])
+def test_arrays_live_as_long_as_their_batch(H, native):
+    """Temporaries of the current stream in a batch that waits on another one."""
+    n = 100_000
+    keys, _ = W.take_keys(9, 0, 2 * n)
+    t = H.HiveTable(1 << 19, bucket_slots=16)
+    m = H.HiveMulti([t], max_segments=2, max_ops=2 * n)
+    if not native:
+        m._N = type("Never", (), {"multi": lambda *a: NotImplemented})()
+    side = torch.cuda.Stream()
+    warm = seg(H, 0, keys[:1])
+    torch.cuda.synchronize()
+    m.execute([warm], stream=side)
+    for r in range(2):
+        s = seg(H, 0, keys[n * r:n * (r + 1)])
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(200_000_000)  # about 0.1 s
+        m.execute([s], stream=side)
+        del s
+        junk = [torch.full((n,), 7, dtype=torch.int32, device="cuda") for _ in range(4)]
+        junk += [torch.full((n,), 2, dtype=torch.uint8, device="cuda") for _ in range(4)]
+        torch.cuda.synchronize()
+        assert all(bool((x == x[0]).all()) for x in junk)
+        del junk
+    v, f = t.find(H.to_device_u32(keys))
+    assert bool((f == 1).all()) and np.array_equal(H.to_host_u32(v), W.values_for(keys, 5))
+    assert m.bounds() == [2 * n] and m._arrays == [(), ()]
+    m.close()
+    t.close()
