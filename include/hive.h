@@ -256,11 +256,12 @@ hive_status hive_size(hive_table* t, uint64_t* out, void* stream);
 hive_status hive_reserve(hive_table* t, uint64_t slots, void* stream);
 
 /* Device memory of the table in bytes: `committed` is backed by physical
- * memory now, `reserved` is the most it can grow to.  A resizable table keeps
- * its buckets on CUDA virtual memory: it reserves the address range of
- * max_slots at creation, maps physical memory as splits add buckets and
- * returns it after merges, so committed memory follows the capacity (the
- * other arrays are allocated at their maximum).  Host-side, no sync. */
+ * memory now, `reserved` is the most it can grow to.  A map_on_demand table
+ * keeps its buckets and slot tags on CUDA virtual memory: it reserves the
+ * address range of max_slots at creation, maps physical memory as splits add
+ * buckets and returns it after merges, so committed memory follows the
+ * capacity (the other arrays, 8 bytes per bucket and the stash, are allocated
+ * at their maximum, and with l2_persist the tags are).  Host-side, no sync. */
 hive_status hive_memory(hive_table* t, uint64_t* committed, uint64_t* reserved);
 
 /* The two hash mixes of Section III-C on the device: h1_out[i] = BitHash1(keys[i])

@@ -280,10 +280,9 @@ uint64_t grown_nb(const hive_table* t, uint64_t live) {
 // Before a batch with up to n_ins new keys.
 hive_status grow_for(hive_table* t, uint64_t n_ins, cudaStream_t s) {
   // back every bucket the batch's splits create with one mapping call
-  if (t->vmm) {
-    const uint64_t nb = grown_nb(t, t->size_host + n_ins);
-    HIVE_CK(grow_commit(&t->bucket_vm, nb * t->S * sizeof(uint64_t), s));
-  }
+  hive_status st =
+      t->vmm ? commit_buckets(t, grown_nb(t, t->size_host + n_ins), s) : HIVE_OK;
+  if (st != HIVE_OK) return st;
   // K-pair steps of one round touch disjoint buckets and are fused into one
   // launch; the policy still advances K pairs at a time.
   bool any = false, have = false;
@@ -299,7 +298,7 @@ hive_status grow_for(hive_table* t, uint64_t n_ins, cudaStream_t s) {
       continue;
     }
     if (have) {
-      hive_status st = ensure_committed(t, s);
+      st = ensure_committed(t, s);
       if (st != HIVE_OK) return st;
       View v = make_view(t);
       v.M = acc.M;
@@ -310,7 +309,7 @@ hive_status grow_for(hive_table* t, uint64_t n_ins, cudaStream_t s) {
     have = true;
   }
   if (have) {
-    hive_status st = ensure_committed(t, s);
+    st = ensure_committed(t, s);
     if (st != HIVE_OK) return st;
     View v = make_view(t);
     v.M = acc.M;
@@ -395,10 +394,14 @@ hive_status hive::mark_stash_dirty(hive_table* t, cudaStream_t s) {
   return HIVE_OK;
 }
 
-hive_status hive::ensure_committed(hive_table* t, cudaStream_t s) {
+hive_status hive::commit_buckets(hive_table* t, uint64_t nb, cudaStream_t s) {
   if (!t->vmm) return HIVE_OK;
-  HIVE_CK(grow_commit(&t->bucket_vm, t->nb * t->S * sizeof(uint64_t), s));
+  HIVE_CK(grow_commit(&t->bucket_vm, nb * t->S * sizeof(uint64_t), s));
+  if (t->tag_vm.base) HIVE_CK(grow_commit(&t->tag_vm, nb * t->S, s));
   return HIVE_OK;
+}
+hive_status hive::ensure_committed(hive_table* t, cudaStream_t s) {
+  return commit_buckets(t, t->nb, s);
 }
 
 hive_status hive::contract_table(hive_table* t, cudaStream_t s) {
@@ -463,8 +466,10 @@ hive_status hive::contract_table(hive_table* t, cudaStream_t s) {
     if (t->vmm) {
       // the work above has completed; buckets past nb are empty and unused,
       // so whole allocations above them go back
-      const size_t need = t->nb * t->S * sizeof(uint64_t);
-      if (t->bucket_vm.committed > need + 2 * t->bucket_vm.gran) grow_decommit(&t->bucket_vm, need);
+      for (GrowArray* a : {&t->bucket_vm, &t->tag_vm}) {
+        const size_t need = t->nb * t->S * (a == &t->bucket_vm ? sizeof(uint64_t) : 1);
+        if (a->base && a->committed > need + 2 * a->gran) grow_decommit(a, need);
+      }
     }
   }
   return st;
@@ -673,14 +678,18 @@ hive_status hive_create(const hive_config* cfg, void* stream, hive_table** out) 
     if (grow_reserve(&t->bucket_vm, t->nb_max * S * sizeof(uint64_t), t->device) == cudaSuccess) {
       t->vmm = true;
       t->buckets = reinterpret_cast<uint64_t*>(t->bucket_vm.base);
-      e = grow_commit(&t->bucket_vm, t->nb_init * S * sizeof(uint64_t), s);
-    } else {
-      cudaGetLastError();
+      // (a persisting window covers tags that are all there)
+      if (!cfg->l2_persist && grow_reserve(&t->tag_vm, t->nb_max * S, t->device) == cudaSuccess) {
+        t->tag_vm.fill = 0;
+        t->tags = reinterpret_cast<uint32_t*>(t->tag_vm.base);
+      }
+      if (commit_buckets(t, t->nb_init, s) != HIVE_OK) e = cudaErrorMemoryAllocation;
     }
+    cudaGetLastError();
   }
   if (e == cudaSuccess && !t->vmm)
     e = dev_alloc(&t->buckets, t->nb_max * S * sizeof(uint64_t));
-  if (e == cudaSuccess) e = dev_alloc(&t->tags, t->nb_max * S);
+  if (e == cudaSuccess && !t->tag_vm.base) e = dev_alloc(&t->tags, t->nb_max * S);
   if (e == cudaSuccess) e = dev_alloc(&t->locks, 2 * t->nb_max * sizeof(uint32_t));
   if (e == cudaSuccess) e = dev_alloc(&t->stash_kv, t->stash_alloc * sizeof(uint64_t));
   if (e == cudaSuccess) e = dev_alloc(&t->stash_keys, t->stash_cap * sizeof(uint32_t));
@@ -690,7 +699,7 @@ hive_status hive_create(const hive_config* cfg, void* stream, hive_table** out) 
     std::memset(t->host_ctrl, 0, sizeof(Ctrl));
     if (!t->vmm) e = cudaMemsetAsync(t->buckets, 0xFF, t->nb_max * S * sizeof(uint64_t), s);
   }
-  if (e == cudaSuccess) e = cudaMemsetAsync(t->tags, 0, t->nb_max * S, s);
+  if (e == cudaSuccess && !t->tag_vm.base) e = cudaMemsetAsync(t->tags, 0, t->nb_max * S, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(t->locks, 0, 2 * t->nb_max * sizeof(uint32_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(t->stash_kv, 0xFF, t->stash_alloc * sizeof(uint64_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(t->ctrl, 0, sizeof(Ctrl), s);
@@ -711,7 +720,10 @@ hive_status hive_destroy(hive_table* t) {
     grow_free(&t->bucket_vm);
   else
     cudaFree(t->buckets);
-  cudaFree(t->tags);
+  if (t->tag_vm.base)
+    grow_free(&t->tag_vm);
+  else
+    cudaFree(t->tags);
   cudaFree(t->locks);
   cudaFree(t->stash_kv);
   cudaFree(t->stash_keys);
@@ -910,15 +922,16 @@ hive_status hive_memory(hive_table* t, uint64_t* committed, uint64_t* reserved) 
   hive_status st = check_table(t);
   if (st != HIVE_OK) return st;
   if (!committed || !reserved) return fail(HIVE_ERR_INVALID_ARG, "outputs must not be NULL");
-  const uint64_t bucket_max = t->nb_max * t->S * sizeof(uint64_t);
-  const uint64_t bucket_now = t->vmm ? t->bucket_vm.committed : bucket_max;
-  const uint64_t other = t->nb_max * (t->S + 2 * sizeof(uint32_t)) + t->stash_alloc * sizeof(uint64_t) +
+  const uint64_t slots = t->nb_max * t->S;
+  const uint64_t bucket_now = t->vmm ? t->bucket_vm.committed : slots * sizeof(uint64_t);
+  const uint64_t tag_now = t->tag_vm.base ? t->tag_vm.committed : slots;
+  const uint64_t other = t->nb_max * 2 * sizeof(uint32_t) + t->stash_alloc * sizeof(uint64_t) +
                          t->stash_cap * sizeof(uint32_t) + sizeof(Ctrl) +
                          (t->list_cap + t->lb_cap) * 12 +
                          t->part_cap * 12 + part_off_bytes(t->part_cap) + t->lists_kept.bytes +
                          t->part_kept.bytes;
-  *committed = bucket_now + other;
-  *reserved = bucket_max + other;
+  *committed = bucket_now + tag_now + other;
+  *reserved = slots * (sizeof(uint64_t) + 1) + other;
   return HIVE_OK;
 }
 

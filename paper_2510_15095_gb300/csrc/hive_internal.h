@@ -281,11 +281,12 @@ struct GrowArray {
   uint64_t base = 0;
   size_t reserved = 0, committed = 0, gran = 0;
   int device = 0;
+  int fill = 0xFF;  // byte that new chunks are filled with
   std::vector<uint64_t> handles;  // physical allocations, mapped back to back from base
   std::vector<size_t> sizes;      // bytes of each
 };
 cudaError_t grow_reserve(GrowArray* a, size_t max_bytes, int device);
-cudaError_t grow_commit(GrowArray* a, size_t bytes, cudaStream_t s);  // new chunks filled 0xFF
+cudaError_t grow_commit(GrowArray* a, size_t bytes, cudaStream_t s);  // new chunks filled
 void grow_decommit(GrowArray* a, size_t bytes);  // caller ensures no kernel uses the tail
 void grow_free(GrowArray* a);
 }  // namespace hive
@@ -349,7 +350,9 @@ struct hive_table {
   std::vector<Rec> recs;
   std::vector<cudaEvent_t> ev_pool;
   HostIO io;  // host-buffer call staging (allocated on first use)
-  hive::GrowArray bucket_vm;  // resizable tables: buckets on virtual memory
+  // resizable tables: buckets, and unless a window covers them slot tags, on
+  // virtual memory
+  hive::GrowArray bucket_vm, tag_vm;
   bool vmm = false;
   bool check_contract = false;  // HIVE_DEBUG at creation: update calls check the batch contract
 };
@@ -388,7 +391,9 @@ bool under_shrink(const hive_table* t, uint64_t live, uint64_t nb);
 hive_status contract_table(hive_table* t, cudaStream_t s);
 hive_status mark_stash_dirty(hive_table* t, cudaStream_t s);
 void free_staging(hive_table* t);  // releases the host-buffer call staging
-// Resizable tables on virtual memory: back buckets [0, nb) with physical memory.
+// Tables on virtual memory: back buckets [0, nb) (of t by default) with
+// physical memory.
+hive_status commit_buckets(hive_table* t, uint64_t nb, cudaStream_t s);
 hive_status ensure_committed(hive_table* t, cudaStream_t s);
 bool table_view(const hive_table* t, View* v, Launch* L, bool* resizable);
 // Every device allocation of the library goes through here, so that a test

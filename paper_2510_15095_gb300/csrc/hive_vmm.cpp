@@ -119,8 +119,8 @@ cudaError_t grow_commit(GrowArray* a, size_t bytes, cudaStream_t s) {
   a->handles.push_back(h);
   a->sizes.push_back(delta);
   a->committed += delta;
-  // new buckets start empty (all-ones words)
-  return cudaMemsetAsync(reinterpret_cast<void*>(at), 0xFF, delta, s);
+  // new buckets start empty (all-ones words, zero tags)
+  return cudaMemsetAsync(reinterpret_cast<void*>(at), a->fill, delta, s);
 }
 
 // Unmaps whole allocations from the top while what stays mapped still

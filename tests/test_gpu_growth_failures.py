@@ -145,3 +145,44 @@ def test_batch_that_cannot_grow_in_the_middle(H, bs, call):
     check(H, t, d, keys)
     assert t.check() == 0
     t.close()
+
+
+@pytest.mark.parametrize("bs", [16, 32])
+def test_slot_tags_are_mapped_on_demand(H, bs):
+    """A large max_slots costs address space, not memory, beyond 12 bytes a
+    bucket; and a table whose tags cannot be mapped when its buckets can."""
+    nb_max = 1 << 26
+    t = H.HiveTable(1 << 16, max_slots=nb_max * bs, resizable=True, bucket_slots=bs,
+                    map_on_demand=True, stash_permille=0)
+    committed, reserved = t.memory()
+    assert committed < 12 * nb_max + (16 << 20) and reserved >= 9 * bs * nb_max
+    t.close()
+    # 2^21 slots: 16 MB of words and 2 MB of tags are mapped, both full
+    t, d = on_demand(H, bs), oracle.Dict()
+    t.reserve(1 << 21)
+    keys, c = W.take_keys(731, 0, 1 << 20)
+    vals = W.values_for(keys, 731)
+    t.insert(up(H, keys), up(H, vals))
+    d.insert(keys, vals)
+    assert t.capacity() == 1 << 21
+    H.debug_fail_alloc(2)  # the words' mapping succeeds, the tags' fails
+    with pytest.raises(H.HiveError) as e:
+        t.reserve((1 << 21) + 1)
+    assert "OOM" in str(e.value) and t.capacity() == 1 << 21
+    check(H, t, d, keys)
+    more, _ = W.take_keys(731, c, 1 << 21)
+    mv = W.values_for(more, 731)
+    assert np.array_equal(t.insert(up(H, more), up(H, mv)).cpu().numpy(), d.insert(more, mv))
+    assert t.capacity() > 1 << 21
+    check(H, t, d, np.concatenate([keys, more]))
+    # shrink gives the memory back, growth finds it filled anew
+    c0 = t.memory()[0]
+    gone = np.concatenate([keys, more])[: 3 * (1 << 20) - 50_000]
+    assert np.array_equal(t.erase(up(H, gone)).cpu().numpy(), d.erase(gone))
+    assert t.memory()[0] < c0 - (16 << 20)
+    check(H, t, d, keys)
+    t.insert(up(H, gone), up(H, W.values_for(gone, 732)))
+    d.insert(gone, W.values_for(gone, 732))
+    check(H, t, d, gone)
+    assert t.check() == 0
+    t.close()
