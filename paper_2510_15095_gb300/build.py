@@ -3,7 +3,9 @@ native call path of the Python binding (hive_binding.so) with g++.
 
 The translation units compile in parallel: the kernels (CUDA), the host
 library (C++ using the CUDA runtime, linked statically) and the binding, which
-uses the installed torch's headers.
+uses the installed torch's headers.  The binding is optional (the Python code
+makes every call without it, by ctypes): where it does not compile, build()
+says so and goes on.
 """
 from __future__ import annotations
 
@@ -21,6 +23,7 @@ SOURCES = ["hive_kernels.cu", "hive32_kernels.cu", "hive_host.cpp", "hive32.cpp"
            "hive_hostio.cpp", "hive_vmm.cpp", "hive_contract.cpp", "hive_noalloc.cu"]
 HEADERS = ["hive_internal.h", "hive_device.cuh", "hive_tags.cuh"]
 BINDING = os.path.join(OUT_DIR, "hive_binding.so")
+BINDING_STAMP = os.path.join(OUT_DIR, "hive_binding.built_for")
 BINDING_SRC = "hive_binding.cpp"
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -30,14 +33,40 @@ def nvcc() -> str:
     return cand if os.path.exists(cand) else "nvcc"
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(BINDING):
+def _older(path: str, sources) -> bool:
+    if not os.path.exists(path):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
-    deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS + [BINDING_SRC]]
+    t = os.path.getmtime(path)
+    deps = [os.path.join(CSRC, f) for f in sources]
     deps.append(os.path.join(ROOT, "include", "hive.h"))
     deps.append(os.path.abspath(__file__))
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _stale() -> bool:
+    return _older(LIB, SOURCES + HEADERS)
+
+
+def binding_key() -> str:
+    """What a built binding depends on besides its source: torch and Python."""
+    import importlib.metadata
+
+    try:
+        version = importlib.metadata.version("torch")
+    except importlib.metadata.PackageNotFoundError:
+        import torch
+
+        version = torch.__version__
+    return f"torch {version} {sys.implementation.cache_tag}"
+
+
+def binding_fits() -> bool:
+    """Whether the built binding belongs to this torch and Python."""
+    try:
+        with open(BINDING_STAMP) as f:
+            return os.path.exists(BINDING) and f.read() == binding_key()
+    except OSError:
+        return False
 
 
 def build_binding() -> str:
@@ -63,13 +92,26 @@ def build_binding() -> str:
     if r.returncode != 0:
         raise RuntimeError(f"g++ failed for {BINDING_SRC}:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, BINDING)
+    with open(BINDING_STAMP, "w") as f:
+        f.write(binding_key())
     return BINDING
 
 
+def _build_binding() -> None:
+    try:
+        build_binding()
+    except Exception as e:  # noqa: BLE001  (no torch headers, no compiler, ...)
+        sys.stderr.write(f"hive_binding.so was not built, calls go through ctypes: {e}\n")
+
+
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
-    if not force and not _stale():
-        return LIB
+    lib = force or _stale()
+    binding = force or _older(BINDING, [BINDING_SRC]) or not binding_fits()
     os.makedirs(OUT_DIR, exist_ok=True)
+    if not lib:
+        if binding:
+            _build_binding()
+        return LIB
     common = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"),
               "-I", CSRC, *extra_flags]
 
@@ -86,9 +128,9 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         return obj
 
     with ThreadPoolExecutor(len(SOURCES) + 1) as ex:
-        binding = ex.submit(build_binding)
+        if binding:
+            ex.submit(_build_binding)
         objs = list(ex.map(compile_one, SOURCES))
-        binding.result()
     tmp = LIB + f".{os.getpid()}.tmp"
     cmd = [nvcc(), *ARCH, "-shared", "-o", tmp, *objs]
     r = subprocess.run(cmd, capture_output=True, text=True)
