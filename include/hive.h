@@ -115,11 +115,13 @@ typedef struct {
                                limit (a per-process setting, gone when the process
                                exits).  0 = off (default; a tuning knob) */
   uint32_t stage_wait_limit;/* 0 (default): probes read the slot tags.  Otherwise,
-                               with S = 32: probes stage whole 256-byte buckets
-                               through bulk copies that wait on an mbarrier, and
-                               this is the number of tries before such a wait
-                               gives up (TIMEOUT) and the round is redone by
-                               tags; a small value exercises that fallback */
+                               with S = 32: the bulk kernel stages whole 256-byte
+                               buckets through bulk copies that wait on an
+                               mbarrier, which is slower (2^26 lookups on 2^26
+                               slots 3.93 ms, 1.21 by tags), and this is the number of
+                               tries before such a wait gives up (TIMEOUT) and
+                               the round is redone by tags: 1 << 22 is never
+                               reached, a small value exercises that fallback */
   uint32_t block_threads;   /* block shape of the bulk kernels: 128, 256 or 512
                                threads (one op per lane); 0 = 256 (default; a
                                tuning knob) */

@@ -119,7 +119,7 @@ View hive::make_view(const hive_table* t) {
   // updating batch of an op or more per 128-byte line, which launch_ops adds
   // (2^26 slots: 2^24 mixed ops 1317 -> 1263 us, but 2^20 ops 125 -> 128).
   v.keep_words = t->nb * t->S * sizeof(uint64_t) <= (128ull << 20);
-  v.stage_spin_limit = t->cfg.stage_wait_limit ? t->cfg.stage_wait_limit : (1u << 22);
+  v.stage_spin_limit = t->cfg.stage_wait_limit;  // 0: nothing is staged
   return v;
 }
 
