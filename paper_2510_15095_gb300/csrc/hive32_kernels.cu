@@ -716,9 +716,8 @@ cudaError_t launch32_t(const View32& v, const Ops32& a, uint64_t n, const List32
   const uint64_t cap = static_cast<uint64_t>(num_sms) * g_occ32[LAYOUT][MODE];
   if (blocks > cap) blocks = cap;
   if (blocks == 0) blocks = 1;
-  // a batch whose probes touch about every second bucket fetches the tags first
   k32_ops<MODE, LAYOUT><<<static_cast<unsigned>(blocks), kOps32Threads, 0, s>>>(
-      v, a, n, ovf, n * 4 >= v.nb ? 1 : 0);
+      v, a, n, ovf, prefetch_tags_rule(n, v.nb, kS32));
   return cudaGetLastError();
 }
 

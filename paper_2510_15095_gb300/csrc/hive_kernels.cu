@@ -858,8 +858,6 @@ template <int MODE, int S, bool DEFER, int THREADS, bool STAGED>
 __global__ void __launch_bounds__(THREADS, ops_min_blocks(MODE, DEFER, STAGED, THREADS))
     k_ops(View v, OpPtrs a, uint64_t n, List ovf, int prefetch_tags) {
   pdl_trigger();
-  // probes read tags at random; a large batch first asks L2 for the whole tag
-  // array in sequential pieces
   if (prefetch_tags) prefetch_l2_grid(v.tags, static_cast<uint64_t>(v.nb) * S);
   const int lane = threadIdx.x & 31;
   // n < 2^32 per call, so chunk and op indices fit 32 bits
@@ -2618,13 +2616,6 @@ cudaError_t launch_in_window(const Launch& L, void (*kern)(KArgs...), unsigned g
   }
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
-// Large batches fetch the tag array into L2 first: when the probes of a batch
-// would touch about every second bucket's tags or more.
-template <int S>
-int prefetch_rule(uint64_t n, const View& v) {
-  return n * 4 >= v.nb ? 1 : 0;
-}
-
 template <int MODE, int S, bool DEFER, int THREADS, bool STAGED = false>
 cudaError_t launch_ops_tt(const View& v, const OpPtrs& a, uint64_t n, List ovf, const Launch& L,
                           cudaStream_t s) {
@@ -2637,7 +2628,7 @@ cudaError_t launch_ops_tt(const View& v, const OpPtrs& a, uint64_t n, List ovf, 
   if (blocks > cap) blocks = cap;
   if (blocks == 0) blocks = 1;
   const size_t smem = STAGED ? stage_smem(S, THREADS) : 0;
-  const int pf = prefetch_rule<S>(n, v);
+  const int pf = prefetch_tags_rule(n, v.nb, S);
   if constexpr (MODE == kModeFind && !STAGED) {  // finds change no tag: no persisting window
     // groups of four runs once every warp has at least four of them: with
     // fewer, rounding to whole groups leaves warps idle (1.7 M ops on 7296
@@ -2729,7 +2720,7 @@ cudaError_t launch_insert_part(const View& v, const uint32_t* keys, const uint32
   const uint32_t ntiles = static_cast<uint32_t>(part_tiles(n));
   const unsigned cap = static_cast<unsigned>(L.num_sms) * 4;
   const unsigned blocks = ntiles < cap ? ntiles : cap;
-  const int pf = n * 4 >= v.nb ? 1 : 0;
+  const int pf = prefetch_tags_rule(n, v.nb, v.S);
   cudaError_t e;
   if (v.S == 16)
     e = launch_in_window(L, k_insert_part<16>, blocks, kPartThreads, 0, s, v, a, n, ovf, pl, pf);

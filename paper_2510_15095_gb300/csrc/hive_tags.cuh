@@ -54,6 +54,18 @@ __device__ __forceinline__ uint64_t policy_pass() {
   return p;
 }
 
+// Whether a batch of n ops on nb buckets first asks L2 for the whole tag array
+// in sequential pieces: when its probes would touch about every second bucket
+// or more, and while L2 (129 MB) holds the tags beside the words.  Asked for ->
+// left to the probes, 2^22 ops: lookups on 2^26 slots, 64 MB of tags, level
+// (S = 16 81.4 -> 80.1 us, S = 32 88.7 -> 88.4); with 128 MB of tags (2^27
+// slots) and 256 MB, lookups S = 16 151 -> 145 us and 231 -> 204, S = 32
+// 157 -> 150 and 238 -> 211, 32-bit entries 157 -> 151 and 238 -> 210, mixed
+// ops S = 16 1056 -> 1042 and 971 -> 930.
+inline bool prefetch_tags_rule(uint64_t n, uint64_t nb, uint64_t slots_per_bucket) {
+  return n * 4 >= nb && nb * slots_per_bucket <= (96ull << 20);
+}
+
 // The tags of bucket b.  RO: through the read-only path (no kernel writes
 // tags meanwhile); otherwise a relaxed load, which never returns a stale
 // cached copy.
