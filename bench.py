@@ -226,6 +226,44 @@ def recorded_traffic(kernel: str):
     return None, None
 
 
+def rounded(x):
+    """Floats to six digits, in a line that has to stay short."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [rounded(v) for v in x]
+    return x
+
+
+def pick(d, *names):
+    return {k: d[k] for k in names if d and k in d}
+
+
+def result_line(line: dict, extra: dict) -> dict:
+    """The printed line: the contract's fields whole, the headline numbers of
+    the other legs.  (With every leg's tables it was 29 KB long, and readers of
+    the last lines of the output saw a part of it.)"""
+    out = dict(line)
+    out["phases"] = {k: v for k, v in line["phases"].items()
+                     if k not in ("fused_mixed", "paper_default_s32")}
+    rl = dict(line["roofline"])
+    rl["others"] = {k: pick(v, "frac", "avg_ms", "traffic") for k, v in rl.get("others", {}).items()}
+    out["roofline"] = rl
+    legs = {
+        "multi_table": pick(extra.get("multi_table"), "batched_gops", "plain_gops"),
+        "serving": pick(extra.get("serving", {}).get("saturation"), "batched_gops", "fifo_gops"),
+        "resize_stream": pick(extra.get("resize_stream"), "grow_gops", "shrink_gops"),
+        "plain_2e20": pick(extra.get("plain_2e20"), "insert_gops", "find_gops", "erase_gops"),
+        "hive32_key_only": pick(extra.get("hive32_key_only"), "insert_gops", "find_gops",
+                                "mixed_gops"),
+        "cpu_parallel": pick(extra.get("cpu_parallel"), "value", "threads"),
+    }
+    out["legs"] = {k: v for k, v in legs.items() if v}
+    return rounded(out)
+
+
 # ---------------------------------------------------------------------------
 # CPU oracle (baseline and reference arm)
 # ---------------------------------------------------------------------------
@@ -1368,8 +1406,10 @@ def main():
                 "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
                 "dtype": "u32/u64", "data": "synthetic", "config": cfg, "phases": phases,
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "clocks": clocks,
-                "gpu_launches": gpu_launches, **extra}
-        print(json.dumps(line), flush=True)
+                "gpu_launches": gpu_launches}
+        # every leg's tables on stderr, the result in one short line on stdout
+        print("detail " + json.dumps({**line, **extra}), file=sys.stderr, flush=True)
+        print(json.dumps(result_line(line, extra)), flush=True)
     t.close()
     if world > 1:
         dist.destroy_process_group()
