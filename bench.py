@@ -42,7 +42,10 @@ L2_BYTES = 129 * 10**6  # GB300 L2
 # configurations the benchmark's tuner chooses among (fixed table, 95% load)
 BENCH_SPACE = {"bucket_slots": [16, 32], "placement": [0], "max_evictions": [16],
                "block_threads": [128, 256, 512], "l2_persist": [0, 1]}
-KERNEL_SRC = os.path.join(ROOT, "paper_2510_15095_gb300", "csrc", "hive_kernels.cu")
+CSRC = os.path.join(ROOT, "paper_2510_15095_gb300", "csrc")
+# what the step's DRAM traffic depends on: its kernels and the code that picks them
+KERNEL_SRCS = ["hive_kernels.cu", "hive_device.cuh", "hive_tags.cuh", "hive_internal.h",
+               "hive_host.cpp"]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic.txt")
 
 
@@ -210,20 +213,35 @@ def measured_peak():
         return 6800.0, "fallback"
 
 
-def recorded_traffic(kernel: str):
+def source_sha() -> str:
+    h = hashlib.sha256()
+    for name in KERNEL_SRCS:
+        with open(os.path.join(CSRC, name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
+def recorded_traffic(kernel: str, workload: str):
     """DRAM bytes per launch from the committed ncu summary, if it was taken on
-    the current kernel source (else None)."""
+    the current sources and this workload (else None)."""
     try:
-        sha = hashlib.sha256(open(KERNEL_SRC, "rb").read()).hexdigest()[:16]
+        sha = source_sha()
         for line in open(TRAFFIC_FILE):
             if line.startswith("#") or "=" not in line:
                 continue
             kv = dict(tok.split("=", 1) for tok in line.split())
-            if kv.get("kernel") == kernel and kv.get("source_sha") == sha:
-                return float(kv["bytes_per_launch"]), kv
-    except Exception:
+            if (kv.get("kernel"), kv.get("workload"), kv.get("source_sha")) == (kernel, workload, sha):
+                return float(kv["bytes_per_launch"])
+    except (OSError, ValueError, KeyError):
         pass
-    return None, None
+    return None
+
+
+def insert_kernel(slots: int, n: int, sw: int) -> str:
+    """The kernels that a bulk insert of n keys takes (the rule of hive_insert:
+    claims, then stores by region, for dense batches on tables beyond L2)."""
+    by_region = slots * 8 > 256 << 20 and 8 * n >= slots
+    return f"k_insert_part+store<S={sw}>" if by_region else f"k_ops<insert,S={sw}>"
 
 
 def rounded(x):
@@ -1249,15 +1267,17 @@ def main():
     bytes_find = 9 * n_find + sw * probes_find + 32 * hits_find
     bytes_ins = 9 * n_ins + sw * probes_ins + 32 * (n_ins - overflowed)
     rl = {}
-    for name, (tot, cnt), byts, kname in (("insert", ins_ms, bytes_ins, f"k_insert_part+store<S={sw}>"),
-                                            ("find", find_ms, bytes_find, f"k_find<S={sw}>"),
-                                            ("mixed", mix_ms, bytes_mix, f"k_ops<mixed,S={sw}>"),
-                                            ("claim", claim_ms, bytes_claim, f"k_claim<S={sw}>")):
+    for name, (tot, cnt), byts, kname, n_ops in (
+            ("insert", ins_ms, bytes_ins, insert_kernel(args.slots, n_ins, sw), n_ins),
+            ("find", find_ms, bytes_find, f"k_find<S={sw}>", n_find),
+            ("mixed", mix_ms, bytes_mix, f"k_ops<mixed,S={sw}>", n_mix),
+            ("claim", claim_ms, bytes_claim, f"k_claim<S={sw}>", n_mix)):
         if name == "claim" and not deferred:
             continue
         avg = tot / max(cnt, 1)
         ach = byts / (avg / 1e3) / 1e9 if avg > 0 else 0.0
-        traffic, _ = recorded_traffic(kname)
+        batch = "mixed" if name == "claim" else name
+        traffic = recorded_traffic(kname, f"{args.slots}_slots_{batch}_{n_ops}")
         rl[name] = {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
                     "frac": ach / peak, "traffic": traffic, "algorithmic_bytes": byts,
                     "avg_ms": avg, "kernel": kname, "peak_source": peak_kind}

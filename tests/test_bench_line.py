@@ -1,5 +1,6 @@
-"""The benchmark's printed line on the CPU: short, and whole in the fields that its
-readers need."""
+"""The benchmark's printed line on the CPU: short, whole in the fields that its
+readers need, and with recorded DRAM traffic only where it was recorded for the
+same sources and workload."""
 import json
 
 import bench
@@ -52,3 +53,25 @@ def test_line_is_short_and_whole():
     assert d["e2e"]["h2d_bytes_per_step"] == 929457768 and d["roofline"]["kernel"]
     assert d["legs"]["serving"] == {"batched_gops": 9.1, "fifo_gops": 1.2}
     assert bench.json.loads(json.dumps(bench.result_line(line, {})))["legs"] == {}
+
+
+def test_recorded_traffic_needs_the_same_sources_and_workload(monkeypatch, tmp_path):
+    f = tmp_path / "t.txt"
+    f.write_text(f"# c\nkernel=k workload=w bytes_per_launch=5 source_sha={bench.source_sha()}\n"
+                 "kernel=old workload=w bytes_per_launch=7 source_sha=0000\n")
+    monkeypatch.setattr(bench, "TRAFFIC_FILE", str(f))
+    assert bench.recorded_traffic("k", "w") == 5.0
+    assert bench.recorded_traffic("k", "other") is None
+    assert bench.recorded_traffic("old", "w") is None
+    # a change in any of the sources ends it
+    for name in bench.KERNEL_SRCS:
+        monkeypatch.setattr(bench, "KERNEL_SRCS", [n for n in bench.KERNEL_SRCS if n != name])
+        assert bench.recorded_traffic("k", "w") is None
+        monkeypatch.undo()
+        monkeypatch.setattr(bench, "TRAFFIC_FILE", str(f))
+
+
+def test_insert_label_follows_the_path():
+    assert bench.insert_kernel(1 << 26, 60_000_000, 16) == "k_insert_part+store<S=16>"
+    assert bench.insert_kernel(1 << 25, 30_000_000, 16) == "k_ops<insert,S=16>"
+    assert bench.insert_kernel(1 << 26, 1 << 20, 32) == "k_ops<insert,S=32>"
