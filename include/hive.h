@@ -34,7 +34,12 @@
  *    (insert or erase), and in hive_execute no key may be both updated and
  *    searched.  Repeated finds of one key are allowed.  Under this contract
  *    every result is unique and equals applying the ops one by one to a
- *    dictionary.  Outside it the outcome is some serialisation of the batch.
+ *    dictionary.  Outside it the table stays usable, but ops on one key may
+ *    miss one another: two inserts of a new key may both report INSERTED and
+ *    leave two entries (a large insert into a table beyond L2, which stores its
+ *    words after all claims, always does), of which a find or an erase meets
+ *    one.  hive_check() reports CONTRACT where an update saw another one;
+ *    hive_check_batch() and HIVE_DEBUG find every such batch.
  *  - A table is driven by one host thread at a time.  No C++ exception
  *    crosses this interface.  hive_last_error() describes the last failure of
  *    the calling thread.
