@@ -2718,7 +2718,9 @@ cudaError_t launch_insert_part(const View& v, const uint32_t* keys, const uint32
                                const Launch& L, cudaStream_t s) {
   const OpPtrs a{nullptr, keys, vals, nullptr, nullptr, status};
   const uint32_t ntiles = static_cast<uint32_t>(part_tiles(n));
-  const unsigned cap = static_cast<unsigned>(L.num_sms) * 4;
+  // as many warps per SM as the plain insert kernel runs (config blocks_per_sm)
+  const int per_sm = L.ops_blocks_per_sm[kModeInsert] * L.ops_threads / kPartThreads;
+  const unsigned cap = static_cast<unsigned>(L.num_sms) * (per_sm > 4 ? 4 : per_sm < 1 ? 1 : per_sm);
   const unsigned blocks = ntiles < cap ? ntiles : cap;
   const int pf = prefetch_tags_rule(n, v.nb, v.S);
   cudaError_t e;
