@@ -4,12 +4,12 @@
  * The table is the one of "Hive Hash Table: A Warp-Cooperative, Dynamically
  * Resizable Hash Table for GPUs" (arXiv 2510.15095): 32-bit keys and 32-bit
  * values packed into 64-bit words (Section III-A), buckets of S slots with a
- * per-slot tags (the free mask, and a filter for lookups) and a lock per
+ * tag per slot (the free mask, and a filter for lookups) and a lock per
  * bucket plus an overflow stash (Section III-B), two
  * candidate buckets per key from BitHash1/BitHash2 (Section III-C), insert by
  * replace -> claim-then-commit -> bounded cuckoo eviction -> stash
- * (Section IV-A, Algorithms 1-3), lookup and delete by warp match-and-elect
- * (Section IV-B, Algorithm 4), and linear-hashing growth and shrinkage in
+ * (Section IV-A, Algorithms 1-3), lookup and delete of one op per lane by slot
+ * tags (Section IV-B, Algorithm 4), and linear-hashing growth and shrinkage in
  * batches of K bucket pairs (Section IV-C).
  *
  * Conventions shared by every entry point
@@ -19,7 +19,11 @@
  *    the work queued on `stream` has completed.  `stream` is a cudaStream_t
  *    passed as void*; NULL means the legacy default stream.
  *  - Calls are stream-ordered and asynchronous unless stated otherwise.  A
- *    fixed-capacity table never synchronises inside insert/find/erase/execute.
+ *    fixed-capacity table does not synchronise inside insert/find/erase/execute,
+ *    except in a call with more ops than any before it, which may have to
+ *    lengthen the table's scratch lists (to the next power of two).  Once an
+ *    eager call of its size has run, such a call can be captured into a CUDA
+ *    graph; scratch that a graph uses is kept until the table is destroyed.
  *    A resizable table reads a few counters back to the host after each
  *    mutating call (to apply the load-factor policy), so those calls return
  *    after the work on `stream` has completed.

@@ -114,10 +114,13 @@ View hive::make_view(const hive_table* t) {
   v.lock_spin_limit = t->cfg.lock_spin_limit;
   v.placement = t->cfg.placement;
   v.S = t->S;
-  // Words are worth keeping in L2 while they fit it (lookups on 2^23 slots 229
-  // -> 213 us, on 2^25 312 -> 318, on 2^26 420 -> 514), and beyond that in an
-  // updating batch of an op or more per 128-byte line, which launch_ops adds
-  // (2^26 slots: 2^24 mixed ops 1317 -> 1263 us, but 2^20 ops 125 -> 128).
+  // Words are worth keeping in the 129 MB L2 while this table's fit it (lookups
+  // on 2^23 slots 229 -> 213 us, on 2^25 312 -> 318, on 2^26 420 -> 514), and
+  // beyond that in an updating batch of an op or more per 128-byte line, which
+  // launch_ops adds (2^26 slots: 2^24 mixed ops 1317 -> 1263 us, but 2^20 ops
+  // 125 -> 128).  The tables of a group ask one by one, so together they may
+  // keep more than L2 holds; their batches touch a part of it at a time and
+  // gain all the same (256 tables, 1 GB of words: 365 -> 348 us a pair).
   v.keep_words = t->nb * t->S * sizeof(uint64_t) <= (128ull << 20);
   v.stage_spin_limit = t->cfg.stage_wait_limit;  // 0: nothing is staged
   return v;

@@ -68,7 +68,7 @@ __device__ __forceinline__ TagVec<S> ld_tags(const View& v, uint32_t b) {
 // Memory access helpers
 // ----------------------------------------------------------------------------
 
-// 16-byte bucket fragment while other warps may be writing the table.
+// Two words of a bucket while other warps may be writing the table.
 __device__ __forceinline__ void ld_frag(const uint64_t* p, uint64_t& a, uint64_t& b) {
   asm volatile("ld.relaxed.gpu.global.L1::no_allocate.v2.u64 {%0, %1}, [%2];"
                : "=l"(a), "=l"(b)
@@ -1558,7 +1558,7 @@ __global__ void __launch_bounds__(kOvfThreads, HIVE_OVF_MIN_BLOCKS)
 // the version did not move; otherwise the op probes again.  A hit needs no
 // check: the word was observed in place.  Because erases now run beside
 // chains, a chain swaps its victim with a CAS on the word it read (never
-// onto an EMPTY slot); claims then own their slot by its free bit alone.
+// onto an EMPTY slot); claims then own their slot by its tag alone.
 constexpr uint32_t kTransitMask = 0xFFFFu;  // words in transit
 constexpr uint32_t kStep = 1u << 16;         // one finished step
 constexpr uint32_t kFusedRetryLimit = 1u << 14;
@@ -1836,14 +1836,14 @@ struct OpQ {
 
 // The checked probe of the first min(n, 32) queued ops, one per lane
 // (warp-wide); the rest move to the front.  Each attempt reads the version of
-// the BitHash1 bucket of every op still open, probes that bucket and, for the
-// ops still open, the BitHash2 bucket (each round staged in shared memory),
-// then the stash.  A hit is acted on at once: a find takes the staged value
-// (the word was seen in place), an erase or replace CASes the word it saw and
-// probes again if the CAS fails (the word moved).  A miss stands only if no
-// word of that version was in transit and the version did not move;
-// otherwise the op probes again.  New keys then claim a slot by its free bit;
-// keys whose two buckets are full join the warp's eviction queue.
+// the BitHash1 bucket of every op still open, then the tags of both its
+// buckets, the words whose tag matches, and the stash.  A hit is acted on at
+// once: a find takes the value (the word was seen in place), an erase or
+// replace CASes the word it saw and probes again if the CAS fails (the word
+// moved).  A miss stands only if no word of that version was in transit and
+// the version did not move; otherwise the op probes again.  New keys then
+// claim a slot by a CAS on its tag; keys whose two buckets are full join the
+// warp's eviction queue.
 template <int S>
 __device__ void fused_checked(const View& v, uint32_t stash_n, const OpPtrs& a, OpQ& rq,
                               EvictQ& q, const List& pend, int resizable, LaneCounters& cnt,
@@ -2009,13 +2009,11 @@ __device__ void fused_checked(const View& v, uint32_t stash_n, const OpPtrs& a, 
 }
 
 // Ops [32c, 32c + 32) of a mixed batch in the single-kernel mode (one op per
-// lane).  Finds and erases probe first without reading versions, since a hit
-// needs no check (the word was seen in place): the BitHash1 bucket of each,
-// then the BitHash2 bucket of those still open, staged in shared memory.
-// Their misses, and erases whose CAS failed (the word moved), join the warp's
-// queue for the checked probe; so do all inserts, which mostly miss (new
-// keys) and would have to probe again.  The checked probe runs 32 queued ops
-// at a time.
+// lane).  Finds and erases first probe by tags without reading versions,
+// since a hit needs no check (the word was seen in place).  Their misses, and
+// erases whose CAS failed (the word moved), join the warp's queue for the
+// checked probe; so do all inserts, which mostly miss (new keys) and would
+// have to probe again.  The checked probe runs 32 queued ops at a time.
 template <int S>
 __device__ __forceinline__ void run_chunk_fused(const View& v, uint32_t stash_n, const OpPtrs a,
                                                 uint32_t c, uint64_t n, const OpIn& in,
@@ -2339,7 +2337,7 @@ __global__ void __launch_bounds__(256) k_merge_excess(View v, uint32_t count, Ct
 
 // Contraction: warp w merges high bucket (p + w + 2^m) into low bucket p + w,
 // `v` carrying the state after this launch.  Live words take the free slots
-// of the low bucket in rank order (select the r-th free bit); words that do
+// of the low bucket in rank order (the r-th free slot); words that do
 // not fit go to the overflow list and are placed by the eviction kernel.
 template <int S>
 __global__ void __launch_bounds__(256) k_merge(View v, uint32_t count, List ovf) {

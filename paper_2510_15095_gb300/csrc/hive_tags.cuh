@@ -101,7 +101,8 @@ __device__ __forceinline__ TagVec<S> ld_tags_at(const uint32_t* tags, uint32_t b
   return t;
 }
 
-// 0x80 in every byte of x that is zero (exact in every byte).
+// 0x80 in every byte of x that is zero (exact in every byte; this and the
+// shorter test in tag_match are the usual byte-parallel zero tests).
 __device__ __forceinline__ uint32_t zero_bytes(uint32_t x) {
   return ~(((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x | 0x7F7F7F7Fu);
 }
