@@ -386,8 +386,9 @@ enum {
 /* Groups tables (created by hive_create on the current device) for batched
  * calls.  max_segments and max_ops bound one batch.  The tables stay owned by
  * the caller and must outlive the group.  Without HIVE_MULTI_ASYNC they may
- * still be used one by one between batches (same stream); with it, drive them
- * only through the group. */
+ * still be used one by one between batches, or in another such group (a call on
+ * another stream waits for the batch on the GPU); with it, drive them only
+ * through the group. */
 hive_status hive_multi_create(hive_table* const* tables, uint32_t n_tables,
                               uint32_t max_segments, uint64_t max_ops, int flags,
                               void* stream, hive_multi** out);

@@ -503,6 +503,12 @@ hive_status check_table(hive_table* t) {
   if (!t) return fail(HIVE_ERR_INVALID_ARG, "table is NULL");
   return HIVE_OK;
 }
+// The same for a call that works on the table's memory on `stream`.
+hive_status check_table(hive_table* t, void* stream) {
+  if (!t) return fail(HIVE_ERR_INVALID_ARG, "table is NULL");
+  if (t->size_from) HIVE_CK(join_batch(t, static_cast<cudaStream_t>(stream)));
+  return HIVE_OK;
+}
 
 hive_status check_n(uint64_t n) {
   if (n >= (1ull << 32)) return fail(HIVE_ERR_INVALID_ARG, "n must be below 2^32 per call");
@@ -570,6 +576,16 @@ cudaError_t take_size(hive_table* t) {
   t->size_host = t->size_from->sizes[2 * t->size_at];
   t->size_from.reset();
   return cudaSuccess;
+}
+cudaError_t join_batch(hive_table* t, cudaStream_t s) {
+  if (!t->size_from || (s == t->size_stream && s != cudaStreamPerThread) || stream_capturing(s))
+    return cudaSuccess;
+  const cudaEvent_t done = t->size_from->done[t->size_slot];
+  const cudaError_t e = cudaEventQuery(done);
+  if (e == cudaSuccess) return take_size(t);
+  if (e != cudaErrorNotReady) return e;
+  cudaGetLastError();
+  return cudaStreamWaitEvent(s, done, 0);
 }
 }  // namespace hive
 
@@ -748,7 +764,7 @@ hive_status hive_destroy(hive_table* t) {
 
 hive_status hive_insert(hive_table* t, const uint32_t* keys, const uint32_t* vals, uint64_t n,
                         uint8_t* status, void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   if ((st = check_n(n)) != HIVE_OK) return st;
   if (n == 0) return HIVE_OK;
@@ -777,7 +793,7 @@ hive_status hive_insert(hive_table* t, const uint32_t* keys, const uint32_t* val
 
 hive_status hive_find(hive_table* t, const uint32_t* keys, uint64_t n, uint32_t* vals_out,
                       uint8_t* found, void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   if ((st = check_n(n)) != HIVE_OK) return st;
   if (n == 0) return HIVE_OK;
@@ -791,7 +807,7 @@ hive_status hive_find(hive_table* t, const uint32_t* keys, uint64_t n, uint32_t*
 
 hive_status hive_erase(hive_table* t, const uint32_t* keys, uint64_t n, uint8_t* status,
                        void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   if ((st = check_n(n)) != HIVE_OK) return st;
   if (n == 0) return HIVE_OK;
@@ -822,7 +838,7 @@ constexpr uint64_t kDeferMin = 1u << 18;
 hive_status hive_execute(hive_table* t, const uint8_t* ops, const uint32_t* keys,
                          const uint32_t* vals, uint64_t n, uint32_t* vals_out, uint8_t* status,
                          void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   if ((st = check_n(n)) != HIVE_OK) return st;
   if (n == 0) return HIVE_OK;
@@ -868,7 +884,7 @@ hive_status hive_execute(hive_table* t, const uint8_t* ops, const uint32_t* keys
 hive_status hive_execute_fused(hive_table* t, const uint8_t* ops, const uint32_t* keys,
                                const uint32_t* vals, uint64_t n, uint32_t* vals_out,
                                uint8_t* status, void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   if ((st = check_n(n)) != HIVE_OK) return st;
   if (n == 0) return HIVE_OK;
@@ -890,7 +906,7 @@ hive_status hive_execute_fused(hive_table* t, const uint8_t* ops, const uint32_t
 }
 
 hive_status hive_size(hive_table* t, uint64_t* out, void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   if (!out) return fail(HIVE_ERR_INVALID_ARG, "out must not be NULL");
   if ((st = readback(t, static_cast<cudaStream_t>(stream))) != HIVE_OK) return st;
@@ -947,7 +963,7 @@ hive_status hive_capacity(hive_table* t, uint64_t* slots_out) {
 }
 
 hive_status hive_clear(hive_table* t, void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // Buckets at or past nb are kept empty by construction; only [0, nb) and
@@ -970,7 +986,7 @@ hive_status hive_clear(hive_table* t, void* stream) {
 }
 
 hive_status hive_check(hive_table* t, void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if ((st = readback(t, s)) != HIVE_OK) return st;
@@ -1000,7 +1016,7 @@ hive_status hive_debug_fail_alloc(uint32_t n) {
 }
 
 hive_status hive_debug_hold_lock(hive_table* t, uint64_t bucket, int held, void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   if (bucket != UINT64_MAX && bucket >= t->nb)
     return fail(HIVE_ERR_INVALID_ARG, "bucket is not in use");
@@ -1015,7 +1031,7 @@ hive_status hive_debug_hold_lock(hive_table* t, uint64_t bucket, int held, void*
 }
 
 hive_status hive_debug_set_versions(hive_table* t, uint32_t value, void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   if (value & 0xFFFFu)
     return fail(HIVE_ERR_INVALID_ARG, "the low 16 bits (words in transit) must be 0");
@@ -1025,7 +1041,7 @@ hive_status hive_debug_set_versions(hive_table* t, uint32_t value, void* stream)
 }
 
 hive_status hive_stats(hive_table* t, hive_stats_t* out, void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   if (!out) return fail(HIVE_ERR_INVALID_ARG, "out must not be NULL");
   if ((st = readback(t, static_cast<cudaStream_t>(stream))) != HIVE_OK) return st;
@@ -1075,7 +1091,7 @@ hive_status hive_profile_read(hive_table* t, hive_profile_t* out) {
 }
 
 hive_status hive_dump(hive_table* t, hive_image* img, void* stream) {
-  hive_status st = check_table(t);
+  hive_status st = check_table(t, stream);
   if (st != HIVE_OK) return st;
   if (!img) return fail(HIVE_ERR_INVALID_ARG, "img must not be NULL");
   cudaStream_t s = static_cast<cudaStream_t>(stream);

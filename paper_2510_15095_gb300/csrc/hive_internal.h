@@ -339,6 +339,7 @@ struct hive_table {
   // a newer size_host: entry size_at of the source, there when size_slot is done
   std::shared_ptr<hive::SizeSource> size_from;
   uint32_t size_at = 0, size_slot = 0;
+  cudaStream_t size_stream = nullptr;  // the batch's stream
   uint64_t splits = 0, merges = 0;
   bool merge_deferred = false;
   // profiling hook: events bracketing each launch while enabled
@@ -363,6 +364,10 @@ namespace hive {
 // Takes the size that a batch has gathered for t, if one is to be taken (waits
 // for the batch).
 cudaError_t take_size(hive_table* t);
+// Makes work queued on s next wait for a batch of a group that is not waited for
+// otherwise and works on t on another stream.  (A stream under capture cannot
+// wait for what is outside its graph; whoever replays the graph does.)
+cudaError_t join_batch(hive_table* t, cudaStream_t s);
 View make_view(const hive_table* t);
 // The next expansion launch of a table (Section IV-C1): bucket pairs
 // (src0 + i, src0 + i + half) for i < count, leaving the table at (M, p).

@@ -337,6 +337,8 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   // one on another stream runs after the one before.
   if (m->seq && (s != m->last || s == cudaStreamPerThread))
     MCK(cudaStreamWaitEvent(s, m->slot[(m->seq - 1) & 1].done, 0));
+  for (uint32_t t : touched)  // and after another group's batch on its tables
+    if (m->tables[t]->size_from != m->sizes) MCK(join_batch(m->tables[t], s));
   if (m->async) refresh_bounds(m);
 
   // (1) growth, planned as waves of split jobs
@@ -474,6 +476,7 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
       tb->size_from = m->sizes;
       tb->size_at = t;
       tb->size_slot = static_cast<uint32_t>(&sl - m->slot);
+      tb->size_stream = s;
     }
     return HIVE_OK;
   }

@@ -88,6 +88,56 @@ def test_batches_on_two_streams_run_in_order(H):
         t.close()
 
 
+@pytest.mark.parametrize("late", ["find", "size", "insert", "noalloc", "execute", "erase", "stats",
+                                  "dump", "clear", "group"])
+def test_single_calls_on_another_stream_follow_the_batch(H, late):
+    """A batch that is still queued on a side stream, and a call on one of its
+    tables on the current stream right after it."""
+    n = 50_000
+    keys, _ = W.take_keys(10, 0, n)
+    t = H.HiveTable(1 << 17, bucket_slots=16)
+    m = H.HiveMulti([t], max_segments=1, max_ops=n)
+    other = H.HiveMulti([t], max_segments=1, max_ops=n)
+    s, f = seg(H, 0, keys), seg(H, 0, keys, op=H.OP_FIND)
+    dk, dv = s["keys"].clone(), s["vals"].clone()
+    t.insert(dk, dv)  # scratch has its size
+    t.execute(f["ops"], dk, dv)
+    t.clear()
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(200_000_000)  # about 0.1 s
+    m.execute([s], stream=side)
+    if late == "find":
+        v, found = t.find(dk)
+        assert bool((found == 1).all()) and bool((v == dv).all())
+    elif late == "size":
+        assert t.size() == n
+    elif late in ("insert", "noalloc"):
+        st = (t.insert if late == "insert" else t.insert_noalloc)(dk, dv)
+        assert bool((st == H.REPLACED).all())
+    elif late == "execute":
+        assert bool((t.execute(f["ops"], dk, dv)[1] == H.FOUND).all())
+    elif late == "erase":
+        assert bool((t.erase(dk) == H.ERASED).all())
+    elif late == "stats":
+        assert t.stats()["claimed_fast"] >= n
+    elif late == "dump":
+        assert t.dump()["size"] == n
+    elif late == "clear":
+        t.clear()
+        assert t.size() == 0 and m.bounds() == [0]
+    else:
+        other.execute([f])
+        torch.cuda.current_stream().synchronize()
+        assert bool((f["status"] == H.FOUND).all())
+    torch.cuda.synchronize()
+    assert bool((s["status"] == H.INSERTED).all())
+    assert t.check() == 0
+    for x in (m, other, t):
+        x.close()
+
+
 def test_capture_is_refused(H):
     """A captured batch would replay descriptors that later batches replace."""
     keys, _ = W.take_keys(7, 0, 100)
