@@ -38,30 +38,33 @@ const at::Tensor& tensor_of(PyObject* o) {
 }
 
 // Refuses all but a contiguous CUDA tensor with >= n items of `item` bytes (or,
-// with `pinned`, a pinned CPU tensor).
-void check_plain(const at::Tensor& t, size_t item, int64_t n, bool pinned) {
-  if (!t.is_cuda() && !(pinned && t.device().is_cpu() && t.is_pinned())) throw NotPlain();
+// with `host`, which is then set, a pinned CPU tensor).
+void check_plain(const at::Tensor& t, size_t item, int64_t n, bool* host) {
+  if (!t.is_cuda()) {
+    if (!host || !t.device().is_cpu() || !t.is_pinned()) throw NotPlain();
+    *host = true;
+  }
   if (!t.has_storage() || !t.is_contiguous() || t.element_size() != item || t.numel() < n)
     throw NotPlain();
 }
 // Pointer of an input tensor; NULL for None.
-const void* in_ptr(const at::Tensor& t, size_t item, int64_t n, bool pinned = false) {
-  check_plain(t, item, n, pinned);
+const void* in_ptr(const at::Tensor& t, size_t item, int64_t n, bool* host = nullptr) {
+  check_plain(t, item, n, host);
   return t.const_data_ptr();
 }
-const void* in_ptr(PyObject* o, size_t item, int64_t n, bool pinned = false) {
+const void* in_ptr(PyObject* o, size_t item, int64_t n, bool* host = nullptr) {
   if (!o || o == Py_None) return nullptr;
-  return in_ptr(tensor_of(o), item, n, pinned);
+  return in_ptr(tensor_of(o), item, n, host);
 }
 // Pointer of an output tensor; NULL for None.  A copy-on-write tensor gets its
 // own storage first, as data_ptr() gives it in Python: the kernels write it.
-void* out_ptr(const at::Tensor& t, size_t item, int64_t n, bool pinned = false) {
-  check_plain(t, item, n, pinned);
+void* out_ptr(const at::Tensor& t, size_t item, int64_t n, bool* host = nullptr) {
+  check_plain(t, item, n, host);
   return t.mutable_data_ptr();
 }
-void* out_ptr(PyObject* o, size_t item, int64_t n, bool pinned = false) {
+void* out_ptr(PyObject* o, size_t item, int64_t n, bool* host = nullptr) {
   if (!o || o == Py_None) return nullptr;
-  return out_ptr(tensor_of(o), item, n, pinned);
+  return out_ptr(tensor_of(o), item, n, host);
 }
 
 void* as_address(PyObject* o) {
@@ -234,11 +237,31 @@ PyObject* item(PyObject* d, PyObject* key) {
   return o;
 }
 
+// References to a batch's arrays, in a list with room for `most` of them.
+struct Held {
+  PyObject* list;
+  Py_ssize_t n = 0;
+  explicit Held(Py_ssize_t most) : list(PyList_New(most)) {
+    if (!list) throw NotPlain();
+  }
+  Held(const Held&) = delete;
+  Held& operator=(const Held&) = delete;
+  ~Held() { Py_XDECREF(list); }
+  void add(PyObject* o) { PyList_SET_ITEM(list, n++, Py_NewRef(o)); }
+  PyObject* take() {
+    Py_SET_SIZE(reinterpret_cast<PyVarObject*>(list), n);  // the rest was never filled
+    PyObject* r = list;
+    list = nullptr;
+    return r;
+  }
+};
+
 // multi(fn, group, [segment dicts], stream, bounds) -> (code, arrays)
 // bounds: hive_multi_bounds for a group whose batches are not waited for
 // otherwise, to wait for one that works on host memory (its arrays may be
 // touched when the call returns); 0 for the others.  arrays: the batch's
-// tensors when bounds is given, for the caller to keep while the batch runs.
+// tensors when bounds is given (a list), for the caller to keep while the batch
+// runs.
 PyObject* py_multi(PyObject*, PyObject* const* a, Py_ssize_t na) {
   return guarded(na, 5, [&]() -> PyObject* {
     const auto fn = reinterpret_cast<MultiFn>(as_address(a[0]));
@@ -247,13 +270,10 @@ PyObject* py_multi(PyObject*, PyObject* const* a, Py_ssize_t na) {
     if (!PyList_CheckExact(a[2])) throw NotPlain();
     const Py_ssize_t n_segs = PyList_GET_SIZE(a[2]);
     std::vector<hive_segment> segs(n_segs > 0 ? n_segs : 1);
-    std::vector<PyObject*> arrays;  // borrowed until the tuple is made below
-    if (bounds) arrays.reserve(5 * n_segs);
+    Held held(bounds ? 5 * n_segs : 0);
     bool host = false;
-    auto seen = [&](PyObject* o) {
-      if (!bounds || !o || o == Py_None) return o;
-      host |= !tensor_of(o).is_cuda();
-      arrays.push_back(o);
+    auto keep = [&](PyObject* o) {
+      if (bounds && o && o != Py_None) held.add(o);
       return o;
     };
     for (Py_ssize_t i = 0; i < n_segs; ++i) {
@@ -273,23 +293,19 @@ PyObject* py_multi(PyObject*, PyObject* const* a, Py_ssize_t na) {
       g.reserved0 = 0;
       g.n = static_cast<uint64_t>(n);
       g.n_insert = ins_o ? PyLong_AsUnsignedLongLongMask(ins_o) : g.n;
-      g.ops = static_cast<const uint8_t*>(in_ptr(seen(ops_o), 1, n, true));
-      g.keys = static_cast<const uint32_t*>(in_ptr(seen(keys_o), 4, n, true));
-      g.vals = static_cast<const uint32_t*>(in_ptr(seen(item(d, k_vals)), 4, n, true));
-      g.vals_out = static_cast<uint32_t*>(out_ptr(seen(item(d, k_vals_out)), 4, n, true));
-      g.status = static_cast<uint8_t*>(out_ptr(seen(item(d, k_status)), 1, n, true));
+      g.ops = static_cast<const uint8_t*>(in_ptr(keep(ops_o), 1, n, &host));
+      g.keys = static_cast<const uint32_t*>(in_ptr(keep(keys_o), 4, n, &host));
+      g.vals = static_cast<const uint32_t*>(in_ptr(keep(item(d, k_vals)), 4, n, &host));
+      g.vals_out = static_cast<uint32_t*>(out_ptr(keep(item(d, k_vals_out)), 4, n, &host));
+      g.status = static_cast<uint8_t*>(out_ptr(keep(item(d, k_status)), 1, n, &host));
     }
     void* s = stream_of(a[3]);
-    PyObject* held = PyTuple_New(static_cast<Py_ssize_t>(arrays.size()));
-    if (!held) throw NotPlain();
-    for (size_t i = 0; i < arrays.size(); ++i)
-      PyTuple_SET_ITEM(held, static_cast<Py_ssize_t>(i), Py_NewRef(arrays[i]));
     const int rc = without_gil([&] {
       uint64_t none = 0;
       const int e = fn(h, segs.data(), static_cast<uint32_t>(n_segs), s);
-      return e == HIVE_OK && host ? bounds(h, &none, 0) : e;
+      return e == HIVE_OK && host && bounds ? bounds(h, &none, 0) : e;
     });
-    return Py_BuildValue("(iN)", rc, held);
+    return Py_BuildValue("(iN)", rc, held.take());
   });
 }
 

@@ -322,6 +322,11 @@ struct hive_table {
   uint32_t* stash_keys = nullptr;
   hive::Ctrl* ctrl = nullptr;
   hive::Ctrl* host_ctrl = nullptr;  // pinned readback buffer
+  // a batch of a synchronous group of fixed tables, not waited for, has gathered
+  // a newer size_host: entry size_at of the source, there when size_slot is done
+  std::shared_ptr<hive::SizeSource> size_from;
+  uint32_t size_at = 0, size_slot = 0;
+  cudaStream_t size_stream = nullptr;  // the batch's stream
   uint64_t list_cap = 0;         // entries of list A
   uint64_t lb_cap = 0;           // entries of list B (0: not allocated)
   uint64_t* la_words = nullptr;  // list A: bulk kernel -> eviction kernel
@@ -335,11 +340,6 @@ struct hive_table {
   uint32_t* part_slots = nullptr;
   uint16_t* part_off = nullptr;
   uint64_t size_host = 0;       // exact after each resizable call
-  // a batch of a synchronous group of fixed tables, not waited for, has gathered
-  // a newer size_host: entry size_at of the source, there when size_slot is done
-  std::shared_ptr<hive::SizeSource> size_from;
-  uint32_t size_at = 0, size_slot = 0;
-  cudaStream_t size_stream = nullptr;  // the batch's stream
   uint64_t splits = 0, merges = 0;
   bool merge_deferred = false;
   // profiling hook: events bracketing each launch while enabled

@@ -346,10 +346,11 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   m->wave_begin.clear();
   std::vector<std::vector<MultiJob>> waves;
   std::vector<ResizeState> before;
-  for (uint32_t t : touched) before.emplace_back(m->tables[t]);
+  if (m->any_resizable)
+    for (uint32_t t : touched) before.emplace_back(m->tables[t]);
   // a failure before the splits are queued leaves the tables as they were
   auto undo = [&](hive_status st) {
-    for (size_t i = 0; i < touched.size(); ++i) before[i].restore(m->tables[touched[i]]);
+    for (size_t i = 0; i < before.size(); ++i) before[i].restore(m->tables[touched[i]]);
     return st;
   };
   for (uint32_t t : touched) {
@@ -393,6 +394,8 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   uint8_t* h = sl.h_stage;
   MultiHdr* hd = hdr_of(h);
   MultiSeg* sg = segs_of(m, h);
+  View* vw = views_of(m, h);
+  for (uint32_t t : touched) vw[t] = make_view(m->tables[t]);  // no kernel reads the others
   uint32_t chunk = 0;
   for (uint32_t i = 0; i < n_segs; ++i) {
     const hive_segment& g = segs[i];
@@ -406,15 +409,13 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
     d.vals = g.vals;
     d.vals_out = g.vals_out;
     d.status = g.status;
-    d.v = make_view(m->tables[g.table]);
+    d.v = vw[g.table];
     chunk += static_cast<uint32_t>((g.n + 31) / 32);
   }
   hd->n_segs = n_segs;
   hd->total_chunks = chunk;
   hd->n_tables = nt;
   hd->n_touched = static_cast<uint32_t>(touched.size());
-  View* vw = views_of(m, h);
-  for (uint32_t t = 0; t < nt; ++t) vw[t] = make_view(m->tables[t]);
   if (!touched.empty())
     std::memcpy(touched_of(m, h), touched.data(), touched.size() * sizeof(uint32_t));
   if (!m->jobs.empty())
@@ -473,7 +474,7 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   if (!m->async && !m->any_resizable) {
     for (uint32_t t : touched) {
       hive_table* tb = m->tables[t];
-      tb->size_from = m->sizes;
+      if (tb->size_from != m->sizes) tb->size_from = m->sizes;
       tb->size_at = t;
       tb->size_slot = static_cast<uint32_t>(&sl - m->slot);
       tb->size_stream = s;

@@ -682,7 +682,7 @@ class HiveMulti:
         self._N = _load_native(self._L)
         # batches that execute() does not wait for, and the arrays they use
         self._queues = not asynchronous and not any(t.config.resizable for t in self.tables)
-        self._arrays = [(), ()]
+        self._arrays = [[], []]
 
     def execute(self, segments, stream=None):
         """segments: iterable of dicts with keys table, ops, keys and optionally
@@ -730,7 +730,7 @@ class HiveMulti:
         code = self._L.hive_multi_execute(self._h, arr, len(segs), _stream_ptr(stream))
         if not code and self._queues and not all(x.is_cuda for x in arrays):
             code = self._L.hive_multi_bounds(self._h, (C.c_uint64 * 1)(), 0)
-        return code, tuple(arrays)
+        return code, arrays
 
     def bounds(self) -> list:
         """hive_multi_bounds: upper bounds of the tables' live sizes
@@ -740,7 +740,7 @@ class HiveMulti:
         out = (C.c_uint64 * max(n, 1))()
         _raise(self._L, self._L.hive_multi_bounds(self._h, out, n))
         if self._queues:
-            self._arrays = [(), ()]
+            self._arrays = [[], []]
         return [int(out[i]) for i in range(n)]
 
     def close(self):
@@ -748,7 +748,7 @@ class HiveMulti:
             self._L.hive_multi_destroy(self._h)
             self._h = None
             self._hp = 0
-            self._arrays = [(), ()]
+            self._arrays = [[], []]
 
     def __del__(self):
         try:

@@ -213,6 +213,6 @@ def test_arrays_live_as_long_as_their_batch(H, native):
         del junk
     v, f = t.find(H.to_device_u32(keys))
     assert bool((f == 1).all()) and np.array_equal(H.to_host_u32(v), W.values_for(keys, 5))
-    assert m.bounds() == [2 * n] and m._arrays == [(), ()]
+    assert m.bounds() == [2 * n] and m._arrays == [[], []]
     m.close()
     t.close()
