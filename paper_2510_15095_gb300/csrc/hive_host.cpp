@@ -221,7 +221,8 @@ bool ensure_part(hive_table* t, uint64_t n, cudaStream_t s, PartList* out) {
       free_part(t);
     }
     const uint64_t cap = next_pow2(n);
-    cudaError_t e = dev_alloc(&t->part_words, cap * sizeof(uint64_t));
+    cudaError_t e = prepare_insert_part(static_cast<int>(t->S));
+    if (e == cudaSuccess) e = dev_alloc(&t->part_words, cap * sizeof(uint64_t));
     if (e == cudaSuccess) e = dev_alloc(&t->part_slots, cap * sizeof(uint32_t));
     if (e == cudaSuccess)
       e = dev_alloc(&t->part_off, part_off_bytes(cap));

@@ -167,6 +167,9 @@ cudaError_t launch_insert_part(const View& v, const uint32_t* keys, const uint32
                                uint64_t n, uint8_t* status, List ovf, const PartList& pl,
                                const Launch& L, cudaStream_t s);
 uint64_t part_tiles(uint64_t n);
+// Loads both kernels (a lazy load may find no memory): the second one must not
+// fail once the first has claimed slots whose words it is to store.
+cudaError_t prepare_insert_part(int S);
 // Claims for the new keys of a mixed batch of n ops, listed in `in` by the bulk
 // kernel; items with both buckets full go to `out`.
 cudaError_t launch_claim(const View& v, List in, uint64_t n, List out, const Launch& L,

@@ -2711,6 +2711,16 @@ cudaError_t launch_ops(int mode, const View& v, const uint8_t* ops, const uint32
 
 uint64_t part_tiles(uint64_t n) { return (n + kPartTile - 1) / kPartTile; }
 
+template <int S>
+static cudaError_t load_part_kernels() {
+  cudaFuncAttributes a;
+  const cudaError_t e = cudaFuncGetAttributes(&a, k_insert_part<S>);
+  return e != cudaSuccess ? e : cudaFuncGetAttributes(&a, k_insert_store<S>);
+}
+cudaError_t prepare_insert_part(int S) {
+  return S == 16 ? load_part_kernels<16>() : load_part_kernels<32>();
+}
+
 cudaError_t launch_insert_part(const View& v, const uint32_t* keys, const uint32_t* vals,
                                uint64_t n, uint8_t* status, List ovf, const PartList& pl,
                                const Launch& L, cudaStream_t s) {
