@@ -28,6 +28,7 @@
 #include <memory>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "hive.h"
@@ -337,20 +338,20 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   // one on another stream runs after the one before.
   if (m->seq && (s != m->last || s == cudaStreamPerThread))
     MCK(cudaStreamWaitEvent(s, m->slot[(m->seq - 1) & 1].done, 0));
-  for (uint32_t t : touched)  // and after another group's batch on its tables
-    if (m->tables[t]->size_from != m->sizes) MCK(join_batch(m->tables[t], s));
+  for (uint32_t t : touched) {  // and after another group's batch on its tables
+    hive_table* tb = m->tables[t];
+    if (tb->size_from && tb->size_from != m->sizes) MCK(join_batch(tb, s));
+  }
   if (m->async) refresh_bounds(m);
 
   // (1) growth, planned as waves of split jobs
   m->jobs.clear();
   m->wave_begin.clear();
   std::vector<std::vector<MultiJob>> waves;
-  std::vector<ResizeState> before;
-  if (m->any_resizable)
-    for (uint32_t t : touched) before.emplace_back(m->tables[t]);
   // a failure before the splits are queued leaves the tables as they were
+  std::vector<std::pair<hive_table*, ResizeState>> before;  // the tables that split
   auto undo = [&](hive_status st) {
-    for (size_t i = 0; i < before.size(); ++i) before[i].restore(m->tables[touched[i]]);
+    for (auto& b : before) b.second.restore(b.first);
     return st;
   };
   for (uint32_t t : touched) {
@@ -360,6 +361,7 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
     uint32_t wave = 0;
     bool any = false;
     while (over_grow(tb, size_now + ins[t], tb->nb) && tb->nb < tb->nb_max) {
+      if (!any) before.emplace_back(tb, ResizeState(tb));
       const uint32_t M_before = tb->M;
       SplitPlan pl{};
       if (!plan_split(tb, &pl)) break;
@@ -374,6 +376,7 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
     }
   }
   for (uint32_t t : touched) {  // back the buckets the split waves create
+    if (!m->tables[t]->vmm) continue;
     hive_status st = ensure_committed(m->tables[t], s);
     if (st != HIVE_OK) return undo(st);
   }
@@ -400,8 +403,8 @@ hive_status hive_multi_execute(hive_multi* m, const hive_segment* segs, uint32_t
   for (uint32_t i = 0; i < n_segs; ++i) {
     const hive_segment& g = segs[i];
     MultiSeg& d = sg[i];
-    std::memset(&d, 0, sizeof(d));
     d.table = g.table;
+    d.pad = 0;
     d.n = static_cast<uint32_t>(g.n);
     d.chunk0 = chunk;
     d.ops = g.ops;
